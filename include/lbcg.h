@@ -150,6 +150,13 @@ int lb_destroy(lb_handle* h);
  * Drops any captured step graph. */
 int lb_set_stream(lb_handle* h, void* stream);
 
+/* The cudaStream_t that the handle's work is issued on: the one given to
+ * lb_set_stream, or the handle's own (a stream that synchronises with the
+ * legacy stream) when none or NULL was given.  A caller whose allocator reuses
+ * memory by stream needs it to keep device arrays that it hands to the calls
+ * below alive until that stream has passed them. */
+void* lb_get_stream(const lb_handle* h);
+
 /* Droplet initial state: phi = +1 within distance R_j of centre j (periodic
  * distance on open axes, union over droplets), -1 elsewhere; with width > 0,
  * phi = max_j tanh((R_j - d_j)/width).  rho = 1, u = 0, populations at the
@@ -177,14 +184,13 @@ int lb_init_fields(lb_handle* h, const float* phi, const float* rho, const float
  * Runs of 12 steps are replayed from a captured CUDA graph. */
 int lb_step(lb_handle* h, int64_t nsteps);
 
-/* Choose the tile shape of the step kernel (0..5: 32x8x4, 32x8x8, 32x8x4
- * with a register cap for 3 CTAs per SM, 32x8x6 capped for 3 CTAs per SM,
- * 32x4x4 capped for 6 CTAs per SM, nodes per CTA; 5: 32x8x8 with the
- * near-contact scan of each interface node inside the node loop instead of
- * a phase of its own); used by the autotuner.  Results do not depend on the
- * tile (bit for bit).  Lattices too large for 32-bit population offsets
- * (2 x 27 x nodes >= 2^32) step with tile 0 whatever the setting.
- * lb_get_tile returns the current index. */
+/* Choose the tile shape of the step kernel (0..5: 32x8x4, 32x8x8, 32x8x2,
+ * 32x8x1, 32x4x4 and, as 1, 32x8x8 nodes per CTA); used by autotuners.  Without
+ * this call the step picks a shape by the lattice's size.  Results do not
+ * depend on the tile (bit for bit).  The widest staging halo (h_max >= 4),
+ * FP64 storage, the Shan-Chen model and lattices whose z planes exceed 32-bit
+ * byte offsets step with tile 0 whatever the setting.  lb_get_tile returns
+ * the index last set (0 if none). */
 int lb_set_tile(lb_handle* h, int tile);
 int lb_get_tile(const lb_handle* h);
 

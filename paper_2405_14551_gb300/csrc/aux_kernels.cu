@@ -56,23 +56,6 @@ cudaError_t launch_init_droplets(const Geo& g, int n, const double* d_centres, c
   return cudaGetLastError();
 }
 
-// phi side array for the first step, taken from the initial phi field
-template <typename R>
-__global__ void __launch_bounds__(256) k_phi_from_init(long long N, const float* __restrict__ phi0, R* __restrict__ phi) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x)
-    phi[i] = (R)phi0[i];
-}
-
-cudaError_t launch_phi_from_init(int storage, const Geo& g, const float* phi0, void* phi, cudaStream_t st) {
-  const long long need = (g.N + 255) / 256;
-  const int blocks = (int)(need < 65535 ? need : 65535);
-  if (storage_is_f64(storage))
-    k_phi_from_init<double><<<blocks, 256, 0, st>>>(g.N, phi0, reinterpret_cast<double*>(phi));
-  else
-    k_phi_from_init<float><<<blocks, 256, 0, st>>>(g.N, phi0, reinterpret_cast<float*>(phi));
-  return cudaGetLastError();
-}
-
 // ---------------------------------------------------------------------------
 // deterministic FP64 reductions over the fields buffer
 // ---------------------------------------------------------------------------
@@ -239,9 +222,15 @@ __device__ __forceinline__ int cc_find_local(int* L, int i) {
   return -1;
 }
 
+// phi: value of node (x, y, z) at base[x + sy y + sz z].
 template <typename R>
-__global__ void __launch_bounds__(256) k_cc_local(Geo g, const R* __restrict__ phi, int* __restrict__ Lg,
-                                                  unsigned* status) {
+struct PhiView {
+  const R* base;
+  long long sy, sz;
+};
+
+template <typename R>
+__global__ void __launch_bounds__(256) k_cc_local(Geo g, PhiView<R> phi, int* __restrict__ Lg, unsigned* status) {
   __shared__ int L[CC_TN];
   const int x0 = blockIdx.x * CC_TX, y0 = blockIdx.y * CC_TY, z0 = blockIdx.z * CC_TZ;
   for (int k = threadIdx.x; k < CC_TN; k += blockDim.x) {
@@ -249,7 +238,7 @@ __global__ void __launch_bounds__(256) k_cc_local(Geo g, const R* __restrict__ p
     bool on = false;
     if (x < g.nx && y < g.ny && z < g.nz) {
       const long long i = (long long)x + (long long)g.nx * ((long long)y + (long long)g.ny * z);
-      on = !node_solid(g, i) && phi[i] > R(0);
+      on = !node_solid(g, i) && phi.base[(long long)x + phi.sy * y + phi.sz * z] > R(0);
     }
     L[k] = on ? k : -1;
   }
@@ -375,15 +364,12 @@ __global__ void k_cc_count(Geo g, int* __restrict__ Lp, int* count) {
   if (local) atomicAdd(count, local);
 }
 
-cudaError_t launch_cc(int storage, const Geo& g, const void* fields, int* labels, int* count, unsigned* status,
-                      cudaStream_t st) {
+template <typename R>
+static cudaError_t launch_cc_t(const Geo& g, PhiView<R> phi, int* labels, int* count, unsigned* status, cudaStream_t st) {
   const long long need = (g.N + 255) / 256;
   const int blocks = (int)(need < 8192 ? need : 8192);
   const dim3 tiles((g.nx + CC_TX - 1) / CC_TX, (g.ny + CC_TY - 1) / CC_TY, (g.nz + CC_TZ - 1) / CC_TZ);
-  if (storage_is_f64(storage))
-    k_cc_local<double><<<tiles, 256, 0, st>>>(g, reinterpret_cast<const double*>(fields), labels, status);
-  else
-    k_cc_local<float><<<tiles, 256, 0, st>>>(g, reinterpret_cast<const float*>(fields), labels, status);
+  k_cc_local<R><<<tiles, 256, 0, st>>>(g, phi, labels, status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_cc_union<<<blocks, 256, 0, st>>>(g, labels, status);
@@ -393,9 +379,17 @@ cudaError_t launch_cc(int storage, const Geo& g, const void* fields, int* labels
   return cudaGetLastError();
 }
 
+cudaError_t launch_cc(int storage, const Geo& g, const void* padded, const PadGeo& pg, int* labels, int* count,
+                      unsigned* status, cudaStream_t st) {
+  const long long first = pg.hx + (long long)pg.px * (pg.h + (long long)pg.py * pg.h), sz = (long long)pg.px * pg.py;
+  if (storage_is_f64(storage))
+    return launch_cc_t(g, PhiView<double>{reinterpret_cast<const double*>(padded) + first, pg.px, sz}, labels, count, status, st);
+  return launch_cc_t(g, PhiView<float>{reinterpret_cast<const float*>(padded) + first, pg.px, sz}, labels, count, status, st);
+}
+
 cudaError_t launch_phi_monitor(const Geo& g, const float* phi, int* labels, int* count, double* partials,
                                double* volume, unsigned* status, cudaStream_t st) {
-  cudaError_t e = launch_cc(0, g, phi, labels, count, status, st);  // phi is the first (only) field
+  cudaError_t e = launch_cc_t(g, PhiView<float>{phi, g.nx, (long long)g.nx * g.ny}, labels, count, status, st);
   if (e != cudaSuccess) return e;
   const int nb = reduce_blocks(g.N);
   k_phi_volume_partial<<<nb, RED_THREADS, 0, st>>>(g, phi, partials);

@@ -34,10 +34,11 @@ struct Phys {
   double psi0;    // Shan-Chen pseudo-potential scale rho_0
 };
 
-// Device pointers of one population lattice.  Two-set storage: f holds
-// f^A [27][N] followed by f^B [27][N].  Reduced storage: f holds f* [27][N]
-// (FP32 or FP16 deviations) and sv holds the colour scalars (s, vx, vy, vz)
-// of each node as one float4.
+// Device pointers of one population lattice.  Two-set storage: f holds f^A
+// and f^B in blocks of 32 nodes of a row, [z][y][x / 32][54 directions][32]
+// (the last block of a row is padded).  Reduced storage: f holds f* (FP32 or
+// FP16 deviations) in blocks of 27 directions and sv holds the colour scalars
+// (s, vx, vy, vz) of each node as one float4, [z][y][x].
 struct StateBuf {
   void* f;
   float4* sv;
@@ -53,13 +54,58 @@ struct InitBuf {
 
 enum Loader { LOAD_PULL = 0, LOAD_FIELDS = 1 };
 
-// Where a step reads phi(t): the accumulator of the previous step, or a
-// plain array of the compute type (the initial fields' phi).  Exactly one is
-// non-null.
+// The same parameters in the compute type of the kernels.
+template <typename R>
+struct PhysR {
+  R tau_a, tau_b, A2, beta, A_h, h_min, h_max, phi_I, G, psi0;
+  R g[3];
+  int equal_tau, K, g_mode, collision;
+};
+template <typename R>
+inline PhysR<R> phys_as(const Phys& p) {
+  return PhysR<R>{R(p.tau_a), R(p.tau_b), R(p.A2),    R(p.beta), R(p.A_h), R(p.h_min), R(p.h_max), R(p.phi_I), R(p.G), R(p.psi0),
+                  {R(p.g[0]), R(p.g[1]), R(p.g[2])}, p.equal_tau, p.K, p.g_mode, p.collision};
+}
+
+// The padded array of phi (Shan-Chen: phi, psi_A, psi_B) that k_phi writes
+// every step: nodes -hx..., -h... of the lattice first, rows a multiple of 32
+// bytes, extents that cover the halo of every tile (tiles are at most 32 x 8 x
+// 8 nodes).
+constexpr int pad_hx(int h) { return h > 4 ? 8 : 4; }
+struct PadGeo {
+  int px, py, pz, hx, h;
+};
+inline PadGeo pad_geo(const Geo& g, int halo) {
+  PadGeo p;
+  p.hx = pad_hx(halo);
+  p.h = halo;
+  p.px = (g.nx + 31) / 32 * 32 + 2 * p.hx;
+  p.py = g.ny + 7 + 2 * halo;
+  p.pz = g.nz + 7 + 2 * halo;
+  return p;
+}
+
+// Where k_phi reads the phase field: the accumulator of the previous step, or
+// the initial phi.  Exactly one is non-null.
 struct PhiSrc {
-  const void* phi;
+  const float* phi;
   const unsigned long long* acc;
 };
+
+// Where the fields kernel writes: field k at p + slot[k] N, or nowhere (-1).
+struct FieldOut {
+  void* p = nullptr;
+  signed char slot[16] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1};
+};
+// the fields of mask, each at its own index (packed: in increasing order)
+inline FieldOut field_out(void* p, uint32_t mask, bool packed) {
+  FieldOut o;
+  o.p = p;
+  int n = 0;
+  for (int k = 0; k < 14; ++k)
+    if ((mask >> k) & 1u) o.slot[k] = (signed char)(packed ? n++ : k);
+  return o;
+}
 
 // Accumulators written by a step: out receives the component densities of
 // the next time level (all zero before the step); the step zeroes its own
@@ -76,15 +122,17 @@ inline int acc_words(int storage) { return storage == 3 ? 2 : 1; }
 // One run of a batch, as seen by the batched persistent kernel.
 struct RunDesc {
   Geo g;
-  Phys p;
+  PhysR<float> p;
   StateBuf S[2];
   unsigned long long* acc[3];  // accumulator rotation (see AccBufs)
-  int tiles_x, tiles_y, tiles_z;
-  long long tile_begin;  // first work item of this run
+  float* phi;                  // padded phase field
+  PadGeo pg;
+  long long tile_begin;        // first work items of this run: tiles and
+  long long row_begin;         // groups of eight rows
 };
 
 // Tile shapes of the fused step kernel (x, y extent of the thread block and z
-// nodes per thread).  Tile 5 scans near contact inside the node loop.
+// nodes per thread).
 struct Tile {
   int tx, ty, tz;
 };
@@ -95,6 +143,8 @@ size_t elem_bytes(int storage);
 // population-like arrays of a state: 2 x 27 (two sets), 27 (single set) or
 // the 10 quadratic-form coefficients of the moment storage
 int state_arrays(int storage);
+// elements of f as the device holds it (padded rows)
+size_t state_elems(int storage, const Geo& g);
 bool storage_is_twoset(int storage);
 bool storage_is_f64(int storage);
 
@@ -103,38 +153,50 @@ bool storage_is_f64(int storage);
 // length K <= 3) or 7 (K <= 6)
 inline int stage_halo(const Phys& p) { return p.A_h == 0.0 ? 1 : (p.K <= 3 ? 4 : 7); }
 // rebuild the accumulator of the current time level from the populations of in
+// one direction of a state (not the moment storage) from its blocks to a plain
+// [z][y][x] array (gather) or back
+cudaError_t launch_direction(int storage, const Geo& g, void* f, int dir, void* plain, bool gather, cudaStream_t st);
 cudaError_t launch_phi_acc(int storage, const Geo& g, const StateBuf& in, unsigned long long* acc, cudaStream_t st);
-// one step (write_state) and/or the fields of the current level (write_fields);
-// tile indexes kTiles (only tile 0 for the variants that are not hot)
+// one step (write_state) or the fields of the current level (write_fields): two
+// launches, k_phi into the padded array phi (for a halo of `halo` nodes), then
+// the tiles; tile indexes kTiles (only tile 0 for the variants that are not hot)
 cudaError_t launch_step(int storage, int loader, bool write_state, bool write_fields, int tile, const Geo& g,
                         const Phys& p, const StateBuf& in, const InitBuf& init, PhiSrc src, AccBufs ab, StateBuf out,
-                        void* fields, unsigned* status, cudaStream_t st);
+                        void* phi, int halo, const FieldOut& fields, unsigned* status, cudaStream_t st);
+// phi of the current level into the padded array, nothing else
+cudaError_t launch_phi_only(int storage, const Geo& g, const Phys& p, const InitBuf& init, PhiSrc src, void* phi, int halo,
+                            cudaStream_t st);
+// PHI_SOLID into the whole padded array of `fields` fields (once, at its creation)
+cudaError_t launch_phi_fill(int storage, const PadGeo& pg, int fields, void* phi, cudaStream_t st);
+// the padded phi as a plain [z][y][x] array, 0 at solid nodes
+cudaError_t launch_phi_plain(int storage, const Geo& g, const PadGeo& pg, const void* phi, void* plain, cudaStream_t st);
 // export pre-collision populations of a box, canonical order, as double
 cudaError_t launch_export(int storage, int loader, const Geo& g, const Phys& p, const StateBuf& in,
                           const InitBuf& init, int x0, int y0, int z0, int bx, int by, int bz, double* outA,
                           double* outB, cudaStream_t st);
 
-// batched step over runs[0..nruns): one persistent launch of blocks_per_sm x
-// SMs CTAs; parity selects S[parity] as input, k the accumulator phase
-// (runs read acc[k], add into acc[(k+1)%3], clear acc[(k+2)%3]); halo is the
-// largest stage_halo of the runs
-cudaError_t launch_batched(int storage, const RunDesc* d_runs, int nruns, long long ntiles, int tile, int halo,
-                           long long max_nodes, int parity, int k, int blocks_per_sm, unsigned* status,
+// batched step (run_of: the run of every tile, then of every row group): k_phi_batched over ngroups groups of eight
+// rows, then one persistent launch of blocks_per_sm x SMs CTAs over the
+// tiles; parity selects S[parity] as input, k the accumulator phase (runs read
+// acc[k], add into acc[(k+1)%3], clear acc[(k+2)%3]); halo is the staging halo
+// that every run of the batch was created with, max_rows the most population blocks in a z plane of a run
+cudaError_t launch_batched(int storage, const RunDesc* d_runs, const int* run_of, long long ntiles, long long ngroups, int tile,
+                           int halo, long long max_rows, int parity, int k, int blocks_per_sm, unsigned* status,
                            cudaStream_t st);
 int sm_count_host();
 
 // --- aux_kernels.cu ----------------------------------------------------------
 cudaError_t launch_init_droplets(const Geo& g, int n, const double* d_centres, const double* d_radii, double width,
                                  float* phi0, float* rho0, float* u0, cudaStream_t st);
-cudaError_t launch_phi_from_init(int storage, const Geo& g, const float* phi0, void* phi, cudaStream_t st);
 // deterministic FP64 sums of the fields buffer; partials needs nblocks*8 doubles
 int reduce_blocks(long long N);
 cudaError_t launch_reduce(int storage, const Geo& g, const void* fields, double* partials, double* out8,
                           cudaStream_t st);
 cudaError_t launch_laplace(int storage, const Geo& g, const void* fields, double cut, double* partials,
                            double* out4, cudaStream_t st);
-cudaError_t launch_cc(int storage, const Geo& g, const void* fields, int* labels, int* count, unsigned* status,
-                      cudaStream_t st);
+// droplet count of the padded phi
+cudaError_t launch_cc(int storage, const Geo& g, const void* padded, const PadGeo& pg, int* labels, int* count,
+                      unsigned* status, cudaStream_t st);
 // droplet count and dispersed volume of a float phase-field array [N]
 cudaError_t launch_phi_monitor(const Geo& g, const float* phi, int* labels, int* count, double* partials,
                                double* volume, unsigned* status, cudaStream_t st);

@@ -16,6 +16,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <fstream>
+#include <mutex>
 #include <sstream>
 #include <string>
 #include <vector>
@@ -53,6 +54,35 @@ int cuda_err(cudaError_t e, const char* where) {
     if (e_ != cudaSuccess) return cuda_err(e_, #call);  \
   } while (0)
 
+// The streams that handles and batches own.  A caller's allocator may still hold
+// events to record on such a stream (memory handed to lb_fields and freed
+// later) after the handle is gone, so streams are given back here and used
+// again instead of being destroyed: as many as were ever in use at once.
+std::mutex g_streams_mutex;
+std::vector<std::pair<int, cudaStream_t>> g_idle_streams;  // (device, stream)
+
+cudaError_t take_stream(cudaStream_t* st) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  {
+    std::lock_guard<std::mutex> lock(g_streams_mutex);
+    for (size_t k = 0; k < g_idle_streams.size(); ++k) {
+      if (g_idle_streams[k].first != dev) continue;
+      *st = g_idle_streams[k].second;
+      g_idle_streams.erase(g_idle_streams.begin() + (long)k);
+      return cudaSuccess;
+    }
+  }
+  return cudaStreamCreate(st);
+}
+// st: idle (synchronised) and on device dev
+void give_stream(int dev, cudaStream_t st) {
+  if (!st) return;
+  std::lock_guard<std::mutex> lock(g_streams_mutex);
+  g_idle_streams.emplace_back(dev, st);
+}
+
 template <typename T>
 __global__ void k_convert(long long n, const T* __restrict__ src, float* __restrict__ dst) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -79,6 +109,7 @@ struct lb_handle {
   int storage;
   cudaStream_t stream = nullptr;   // stream all work is issued on
   cudaStream_t own_stream = nullptr;
+  int device = 0;
   lb_alloc alloc{};
   bool have_alloc = false;
   std::vector<std::pair<void*, size_t>> owned;
@@ -86,10 +117,11 @@ struct lb_handle {
 
   StateBuf S[2]{};
   int cur = 0;
-  void* phi = nullptr;      // R[N]: phi of the initial fields
+  void* phi = nullptr;      // padded phase field of the step in progress (PadGeo), 3 fields with Shan-Chen
+  int halo = 1;             // staging halo the padded array is laid out for
   // accumulators of the component densities: acc[phi_acc] holds phi of the
   // current time level, acc[(phi_acc + 1) % 3] is all zero; phi_acc = -1:
-  // phi is in the phi array (initial state) and all three are zero
+  // phi is the initial field and all three are zero
   unsigned long long* acc[3] = {nullptr, nullptr, nullptr};
   int phi_acc = -1;
   float* init_phi = nullptr;
@@ -106,6 +138,7 @@ struct lb_handle {
   bool initialised = false;
   int64_t t = 0;
   int tile = 0;
+  bool tile_chosen = false;  // lb_set_tile was called; otherwise step_tile_of picks by size
   cudaGraphExec_t graph[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};  // [cur * 3 + phi_acc]
   uint64_t graph_launches = 0;  // kernel launches in one replay
   lbcg::SurrogateState* surrogate = nullptr;  // its device buffers are owned like the rest
@@ -161,27 +194,61 @@ void dev_free(lb_handle* h, void* p) {
 
 size_t real_bytes(int storage) { return storage_is_f64(storage) ? 8 : 4; }
 
-size_t state_bytes(const lb_handle* h) {
-  const size_t N = (size_t)h->g.N;
-  const size_t fbytes = (size_t)state_arrays(h->storage) * N * elem_bytes(h->storage);
-  if (storage_is_twoset(h->storage)) return fbytes;
-  return fbytes + 4 * N * sizeof(float);
+// Bytes of the population arrays of a state as a checkpoint holds them
+// ([dir][z][y][x]; colour scalars apart), and as the device holds them.
+size_t file_pop_bytes(const lb_handle* h) {
+  return (size_t)state_arrays(h->storage) * (size_t)h->g.N * elem_bytes(h->storage);
+}
+size_t dev_pop_bytes(const lb_handle* h) { return state_elems(h->storage, h->g) * elem_bytes(h->storage); }
+size_t file_state_bytes(const lb_handle* h) {
+  return file_pop_bytes(h) + (storage_is_twoset(h->storage) ? 0 : 4 * (size_t)h->g.N * sizeof(float));
 }
 
 bool alloc_state(lb_handle* h, StateBuf& s) {
   const size_t N = (size_t)h->g.N;
   if (storage_is_twoset(h->storage)) {
-    s.f = dev_alloc(h, (size_t)state_arrays(h->storage) * N * elem_bytes(h->storage));
+    s.f = dev_alloc(h, dev_pop_bytes(h));
     return s.f != nullptr;
   }
   // one allocation: f* (or the moment coefficients) then the float4 colour
   // scalars (256-byte aligned)
-  const size_t fb = ((size_t)state_arrays(h->storage) * N * elem_bytes(h->storage) + 255) & ~(size_t)255;
+  const size_t fb = (dev_pop_bytes(h) + 255) & ~(size_t)255;
   char* base = (char*)dev_alloc(h, fb + N * sizeof(float4));
   if (!base) return false;
   s.f = base;
   s.sv = (float4*)(base + fb);
   return true;
+}
+
+// Copy the current populations (and colour scalars) to or from a host buffer
+// in checkpoint order, one direction at a time through a buffer of N values.
+// Synchronises the stream.
+int copy_state_host(lb_handle* h, char* host, bool to_host) {
+  const StateBuf& s = h->S[h->cur];
+  const size_t N = (size_t)h->g.N, eb = elem_bytes(h->storage), nd = (size_t)state_arrays(h->storage);
+  const cudaMemcpyKind kind = to_host ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice;
+  cudaError_t e = cudaSuccess;
+  if (h->storage == LB_STORAGE_MOMENT_F32) {  // records, same order on the device
+    e = to_host ? cudaMemcpyAsync(host, s.f, nd * N * eb, kind, h->stream) : cudaMemcpyAsync(s.f, host, nd * N * eb, kind, h->stream);
+  } else {
+    void* tmp = dev_alloc(h, N * eb);
+    if (!tmp) return set_err(LB_ENOMEM, "checkpoint buffer allocation failed");
+    for (size_t d = 0; d < nd && e == cudaSuccess; ++d) {
+      char* at = host + d * N * eb;
+      if (!to_host) e = cudaMemcpyAsync(tmp, at, N * eb, kind, h->stream);
+      if (e == cudaSuccess) e = launch_direction(h->storage, h->g, s.f, (int)d, tmp, to_host, h->stream);
+      g_launches += 1;
+      if (to_host && e == cudaSuccess) e = cudaMemcpyAsync(at, tmp, N * eb, kind, h->stream);
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    dev_free(h, tmp);
+  }
+  if (e == cudaSuccess && !storage_is_twoset(h->storage)) {
+    char* at = host + nd * N * eb;
+    e = to_host ? cudaMemcpyAsync(at, s.sv, N * sizeof(float4), kind, h->stream) : cudaMemcpyAsync(s.sv, at, N * sizeof(float4), kind, h->stream);
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  return cuda_err(e, "checkpoint copy");
 }
 
 InitBuf init_buf(const lb_handle* h) {
@@ -237,7 +304,7 @@ int validate(const lb_grid* gr, const lb_params* p) {
 
 size_t acc_bytes(const lb_handle* h) { return (size_t)h->g.N * (size_t)acc_words(h->storage) * 8; }
 
-// Clear the three accumulators (phi then lives in the phi array).
+// Clear the three accumulators (phi is then the initial field).
 cudaError_t reset_acc(lb_handle* h) {
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaMemsetAsync(h->acc[k], 0, acc_bytes(h), h->stream);
@@ -257,21 +324,41 @@ cudaError_t rebuild_acc(lb_handle* h) {
 
 // Where the current phi is read from, and the accumulators a step writes.
 PhiSrc phi_src(const lb_handle* h) {
-  if (h->phi_acc < 0) return PhiSrc{h->phi, nullptr};
+  if (h->phi_acc < 0) return PhiSrc{h->init_phi, nullptr};
   return PhiSrc{nullptr, h->acc[h->phi_acc]};
 }
 AccBufs acc_bufs(const lb_handle* h) {
-  const int k = h->phi_acc < 0 ? 2 : h->phi_acc;  // from the phi array: every accumulator is zero
+  const int k = h->phi_acc < 0 ? 2 : h->phi_acc;  // from the initial field: every accumulator is zero
   return AccBufs{h->acc[(k + 1) % 3], h->acc[(k + 2) % 3]};
+}
+
+// Tile of a handle whose caller chose none: the deepest tile (fewest halo nodes
+// staged and partial sums flushed per node) that gives every SM a CTA, two for
+// the shallower ones; on small lattices the tile that spreads the
+// nodes over the most SMs, since a step then lasts as long as one tile's chain
+// of nodes.  Measured us per step, x8 / x4 / x2 / x1: 32^3 29 / 25 / 17 / 13 (4 to
+// 32 times fewer CTAs than SM slots), 64x64x128 55 / 58 / 59 / 64, 256x256x512
+// 2560 / 2660 / 2890 / 3350.
+int step_tile_of(const lb_handle* h) {
+  if (h->tile_chosen) return h->tile;
+  const int order[4] = {1, 0, 2, 3};  // 32x8x8, x4, x2, x1
+  const long long sms = sm_count_host();
+  for (int k = 0; k < 4; ++k) {
+    const Tile& T = kTiles[order[k]];
+    const long long ctas = (long long)((h->g.nx + T.tx - 1) / T.tx) * ((h->g.ny + T.ty - 1) / T.ty) * ((h->g.nz + T.tz - 1) / T.tz);
+    if (ctas >= (k == 0 ? 1 : 2) * sms) return order[k];
+  }
+  return order[3];
 }
 
 // Issue one step (no graph).
 int issue_step(lb_handle* h) {
   const int nxt = h->cur ^ 1;
   const bool fresh = h->mode == 0;
-  LB_CUDA(launch_step(h->storage, fresh ? LOAD_FIELDS : LOAD_PULL, true, false, fresh ? 0 : h->tile, h->g, h->p,
-                      h->S[h->cur], init_buf(h), phi_src(h), acc_bufs(h), h->S[nxt], nullptr, h->status, h->stream));
-  g_launches += 1;
+  LB_CUDA(launch_step(h->storage, fresh ? LOAD_FIELDS : LOAD_PULL, true, false, fresh ? 0 : step_tile_of(h), h->g, h->p,
+                      h->S[h->cur], init_buf(h), phi_src(h), acc_bufs(h), h->S[nxt], h->phi, h->halo, FieldOut{}, h->status,
+                      h->stream));
+  g_launches += 2;
   h->phi_acc = ((h->phi_acc < 0 ? 2 : h->phi_acc) + 1) % 3;
   h->cur = nxt;
   h->mode = 1;
@@ -313,45 +400,28 @@ int ensure_fields(lb_handle* h) {
   return LB_OK;
 }
 
-// Fill the fields buffer at the current time level.
-int compute_fields(lb_handle* h) {
+// Write the fields of mask at the current time level: into the fields buffer
+// (field k at k N), or packed into dst (compute type).
+int compute_fields(lb_handle* h, uint32_t mask, void* dst = nullptr) {
   if (!h->initialised) return set_err(LB_ESTATE, "handle not initialised");
-  int rc = ensure_fields(h);
-  if (rc) return rc;
-  LB_CUDA(launch_step(h->storage, h->mode == 0 ? LOAD_FIELDS : LOAD_PULL, false, true, 0, h->g, h->p, h->S[h->cur],
-                      init_buf(h), phi_src(h), AccBufs{nullptr, nullptr}, h->S[h->cur ^ 1], h->fields, h->status,
-                      h->stream));
-  g_launches += 1;
+  if (!dst) {
+    const int rc = ensure_fields(h);
+    if (rc) return rc;
+  }
+  if (dst && mask == LB_F_PHI) {  // no population enters phi
+    LB_CUDA(launch_phi_only(h->storage, h->g, h->p, init_buf(h), phi_src(h), h->phi, h->halo, h->stream));
+    LB_CUDA(launch_phi_plain(h->storage, h->g, pad_geo(h->g, h->halo), h->phi, dst, h->stream));
+  } else {
+    LB_CUDA(launch_step(h->storage, h->mode == 0 ? LOAD_FIELDS : LOAD_PULL, false, true, 0, h->g, h->p, h->S[h->cur],
+                        init_buf(h), phi_src(h), AccBufs{nullptr, nullptr}, h->S[h->cur ^ 1], h->phi, h->halo,
+                        field_out(dst ? dst : h->fields, mask, dst != nullptr), h->status, h->stream));
+  }
+  g_launches += 2;
   return LB_OK;
 }
 
-}  // namespace
-
-extern "C" {
-
-const char* lb_strerror(int code) {
-  switch (code) {
-    case LB_OK: return "ok";
-    case LB_EINVAL: return "invalid argument";
-    case LB_ENOMEM: return "out of memory";
-    case LB_ECUDA: return "CUDA error";
-    case LB_EUNSTABLE: return "unstable: non-finite or non-positive density";
-    case LB_ETIMEOUT: return "bounded device wait gave up";
-    case LB_ESTATE: return "invalid state for this call";
-    case LB_EIO: return "file error or incompatible checkpoint";
-  }
-  return "unknown error";
-}
-
-const char* lb_last_error(void) { return g_last_error.c_str(); }
-
-uint64_t lb_launch_count(void) { return g_launches.load(); }
-
-size_t lb_device_bytes(const lb_handle* h) { return h ? h->bytes : 0; }
-
-int64_t lb_time(const lb_handle* h) { return h ? h->t : -1; }
-
-int lb_create(const lb_grid* grid, const lb_params* params, const lb_alloc* alloc, lb_handle** out) {
+// lb_create with a staging halo of at least min_halo (1, 4 or 7) nodes.
+int create_handle(const lb_grid* grid, const lb_params* params, const lb_alloc* alloc, int min_halo, lb_handle** out) {
   if (!out) return set_err(LB_EINVAL, "out is null");
   *out = nullptr;
   int rc = validate(grid, params);
@@ -393,15 +463,19 @@ int lb_create(const lb_grid* grid, const lb_params* params, const lb_alloc* allo
     h->alloc = *alloc;
     h->have_alloc = true;
   }
-  cudaError_t e = cudaStreamCreate(&h->own_stream);
+  cudaGetDevice(&h->device);
+  cudaError_t e = take_stream(&h->own_stream);
   if (e != cudaSuccess) {
     delete h;
-    return cuda_err(e, "cudaStreamCreate");
+    return cuda_err(e, "stream");
   }
   h->stream = h->own_stream;
   const size_t N = (size_t)h->g.N;
+  h->halo = std::max(min_halo, stage_halo(h->p));
+  const PadGeo pg = pad_geo(h->g, h->halo);
+  const size_t padded = (size_t)pg.px * pg.py * pg.pz * (h->p.model == LB_MODEL_SHAN_CHEN ? 3 : 1);
   bool ok = alloc_state(h, h->S[0]) && alloc_state(h, h->S[1]);
-  ok = ok && (h->phi = dev_alloc(h, N * real_bytes(h->storage))) != nullptr;
+  ok = ok && (h->phi = dev_alloc(h, padded * real_bytes(h->storage))) != nullptr;
   for (int k = 0; k < 3; ++k) ok = ok && (h->acc[k] = (unsigned long long*)dev_alloc(h, acc_bytes(h))) != nullptr;
   ok = ok && (h->init_phi = (float*)dev_alloc(h, N * sizeof(float))) != nullptr;
   ok = ok && (h->red = (double*)dev_alloc(h, ((size_t)reduce_blocks(h->g.N) * 8 + 16) * sizeof(double))) != nullptr;
@@ -412,6 +486,7 @@ int lb_create(const lb_grid* grid, const lb_params* params, const lb_alloc* allo
     return set_err(LB_ENOMEM, "device allocation failed");
   }
   if ((e = cudaMemsetAsync(h->status, 0, sizeof(unsigned), h->stream)) != cudaSuccess ||
+      (e = launch_phi_fill(h->storage, pg, h->p.model == LB_MODEL_SHAN_CHEN ? 3 : 1, h->phi, h->stream)) != cudaSuccess ||
       (e = reset_acc(h)) != cudaSuccess) {
     lb_destroy(h);
     return cuda_err(e, "cudaMemsetAsync");
@@ -420,13 +495,46 @@ int lb_create(const lb_grid* grid, const lb_params* params, const lb_alloc* allo
   return LB_OK;
 }
 
+}  // namespace
+
+extern "C" {
+
+const char* lb_strerror(int code) {
+  switch (code) {
+    case LB_OK: return "ok";
+    case LB_EINVAL: return "invalid argument";
+    case LB_ENOMEM: return "out of memory";
+    case LB_ECUDA: return "CUDA error";
+    case LB_EUNSTABLE: return "unstable: non-finite or non-positive density";
+    case LB_ETIMEOUT: return "bounded device wait gave up";
+    case LB_ESTATE: return "invalid state for this call";
+    case LB_EIO: return "file error or incompatible checkpoint";
+  }
+  return "unknown error";
+}
+
+const char* lb_last_error(void) { return g_last_error.c_str(); }
+
+uint64_t lb_launch_count(void) { return g_launches.load(); }
+
+size_t lb_device_bytes(const lb_handle* h) { return h ? h->bytes : 0; }
+
+int64_t lb_time(const lb_handle* h) { return h ? h->t : -1; }
+
+int lb_create(const lb_grid* grid, const lb_params* params, const lb_alloc* alloc, lb_handle** out) {
+  return create_handle(grid, params, alloc, 1, out);
+}
+
 int lb_destroy(lb_handle* h) {
   if (!h) return LB_OK;
   if (h->stream) cudaStreamSynchronize(h->stream);
   drop_graphs(h);
   if (h->surrogate) destroy_surrogate(h->surrogate);
   while (!h->owned.empty()) dev_free(h, h->owned.back().first);
-  if (h->own_stream) cudaStreamDestroy(h->own_stream);
+  if (h->own_stream) {
+    cudaStreamSynchronize(h->own_stream);
+    give_stream(h->device, h->own_stream);
+  }
   delete h;
   return LB_OK;
 }
@@ -447,6 +555,8 @@ int lb_set_stream(lb_handle* h, void* stream) {
   drop_graphs(h);
   return LB_OK;
 }
+
+void* lb_get_stream(const lb_handle* h) { return h ? (void*)h->stream : nullptr; }
 
 int lb_init_droplets(lb_handle* h, int32_t n, const double* centres, const double* radii, double width) {
   if (!h) return set_err(LB_EINVAL, "null handle");
@@ -471,9 +581,8 @@ int lb_init_droplets(lb_handle* h, int32_t n, const double* centres, const doubl
   }
   cudaError_t e = launch_init_droplets(h->g, n, dbuf, dbuf ? dbuf + 3 * n : nullptr, width, h->init_phi, nullptr,
                                        nullptr, h->stream);
-  if (e == cudaSuccess) e = launch_phi_from_init(h->storage, h->g, h->init_phi, h->phi, h->stream);
   if (e == cudaSuccess) e = reset_acc(h);
-  g_launches += 2;
+  g_launches += 1;
   if (dbuf) {
     cudaStreamSynchronize(h->stream);
     dev_free(h, dbuf);
@@ -504,9 +613,7 @@ int lb_init_fields(lb_handle* h, const float* phi, const float* rho, const float
       return set_err(LB_ENOMEM, "u buffer allocation failed");
     LB_CUDA(cudaMemcpyAsync(h->init_u, u, 3 * N * sizeof(float), kind, h->stream));
   }
-  LB_CUDA(launch_phi_from_init(h->storage, h->g, h->init_phi, h->phi, h->stream));
   LB_CUDA(reset_acc(h));
-  g_launches += 1;
   if (!is_device) LB_CUDA(cudaStreamSynchronize(h->stream));
   h->use_rho = rho != nullptr;
   h->use_u = u != nullptr;
@@ -571,8 +678,9 @@ int lb_step_timed(lb_handle* h, int64_t nsteps, double* ms) {
 int lb_set_tile(lb_handle* h, int tile) {
   if (!h) return set_err(LB_EINVAL, "null handle");
   if (tile < 0 || tile >= NUM_TILES) return set_err(LB_EINVAL, "tile index out of range");
-  if (tile != h->tile) drop_graphs(h);
+  if (tile != h->tile || !h->tile_chosen) drop_graphs(h);
   h->tile = tile;
+  h->tile_chosen = true;
   return LB_OK;
 }
 
@@ -582,10 +690,11 @@ static int fields_out(lb_handle* h, uint32_t mask, void* dst, int dst_is_device,
   if (!h) return set_err(LB_EINVAL, "null handle");
   if (!dst) return set_err(LB_EINVAL, "dst is null");
   if (mask == 0 || (mask >> NFIELDS)) return set_err(LB_EINVAL, "field mask must select fields 0..13");
-  int rc = compute_fields(h);
+  const bool f64 = storage_is_f64(h->storage);
+  if (dst_is_device && f64 == dbl) return compute_fields(h, mask, dst);  // straight to the caller's array
+  int rc = compute_fields(h, mask);
   if (rc) return rc;
   const size_t N = (size_t)h->g.N;
-  const bool f64 = storage_is_f64(h->storage);
   const size_t ob = dbl ? sizeof(double) : sizeof(float);
   void* tmp = nullptr;
   if (f64 != dbl) {  // need a converted copy
@@ -653,7 +762,7 @@ int lb_get_populations(lb_handle* h, int32_t x0, int32_t y0, int32_t z0, int32_t
 
 int lb_reduce_f64(lb_handle* h, double* out) {
   if (!h || !out) return set_err(LB_EINVAL, "null argument");
-  int rc = compute_fields(h);
+  int rc = compute_fields(h, LB_F_PHI | LB_F_RHO | LB_F_UX | LB_F_UY | LB_F_UZ | LB_F_RHOA | LB_F_RHOB | LB_F_H);
   if (rc) return rc;
   const int nb = reduce_blocks(h->g.N);
   double* res = h->red + (size_t)nb * 8;
@@ -667,7 +776,7 @@ int lb_reduce_f64(lb_handle* h, double* out) {
 int lb_laplace_f64(lb_handle* h, double cut, double* dp) {
   if (!h || !dp) return set_err(LB_EINVAL, "null argument");
   if (!(cut >= 0.0 && cut < 1.0)) return set_err(LB_EINVAL, "cut must lie in [0, 1)");
-  int rc = compute_fields(h);
+  int rc = compute_fields(h, LB_F_PHI | LB_F_RHO);
   if (rc) return rc;
   const int nb = reduce_blocks(h->g.N);
   double* res = h->red + (size_t)nb * 8;
@@ -683,11 +792,11 @@ int lb_laplace_f64(lb_handle* h, double cut, double* dp) {
 
 int lb_droplet_count(lb_handle* h, int32_t* count) {
   if (!h || !count) return set_err(LB_EINVAL, "null argument");
-  int rc = compute_fields(h);
-  if (rc) return rc;
+  if (!h->initialised) return set_err(LB_ESTATE, "handle not initialised");
   if (!h->labels && !(h->labels = (int*)dev_alloc(h, (size_t)h->g.N * sizeof(int))))
     return set_err(LB_ENOMEM, "label buffer allocation failed");
-  LB_CUDA(launch_cc(h->storage, h->g, h->fields, h->labels, h->count, h->status, h->stream));
+  LB_CUDA(launch_phi_only(h->storage, h->g, h->p, init_buf(h), phi_src(h), h->phi, h->halo, h->stream));
+  LB_CUDA(launch_cc(h->storage, h->g, h->phi, pad_geo(h->g, h->halo), h->labels, h->count, h->status, h->stream));
   g_launches += 3;
   int c = 0;
   unsigned st = 0;
@@ -705,7 +814,7 @@ int lb_phi_monitor(lb_handle* h, const float* phi, int32_t* count, double* volum
     return set_err(LB_ENOMEM, "label buffer allocation failed");
   double* vol_dev = h->red + (size_t)reduce_blocks(h->g.N) * 8;  // past the partials
   LB_CUDA(launch_phi_monitor(h->g, phi, h->labels, h->count, h->red, vol_dev, h->status, h->stream));
-  g_launches += 5;
+  g_launches += 4;
   int c = 0;
   unsigned st = 0;
   double v = 0.0;
@@ -735,21 +844,16 @@ int lb_save(lb_handle* h, const char* path) {
   FILE* fp = std::fopen(path, "wb");
   if (!fp) return set_err(LB_EIO, std::string("cannot open ") + path);
   const size_t N = (size_t)h->g.N;
-  const size_t sb = state_bytes(h);
-  std::vector<char> buf(h->mode == 1 ? sb : N * sizeof(float) * 5);
+  std::vector<char> buf(h->mode == 1 ? file_state_bytes(h) : N * sizeof(float) * 5);
   cudaError_t e = cudaSuccess;
   int32_t hdr[4] = {(int32_t)CKPT_MAGIC, (int32_t)CKPT_VERSION, h->mode, h->regularised};
   bool ok = std::fwrite(hdr, sizeof(hdr), 1, fp) == 1 && std::fwrite(&h->grid, sizeof(lb_grid), 1, fp) == 1 &&
             std::fwrite(&h->params, sizeof(lb_params), 1, fp) == 1 && std::fwrite(&h->t, sizeof(int64_t), 1, fp) == 1;
   if (ok && h->mode == 1) {
-    const StateBuf& s = h->S[h->cur];
-    if (storage_is_twoset(h->storage)) {
-      e = cudaMemcpyAsync(buf.data(), s.f, sb, cudaMemcpyDeviceToHost, h->stream);
-    } else {
-      const size_t fb = (size_t)state_arrays(h->storage) * N * elem_bytes(h->storage);
-      e = cudaMemcpyAsync(buf.data(), s.f, fb, cudaMemcpyDeviceToHost, h->stream);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(buf.data() + fb, s.sv, N * sizeof(float4), cudaMemcpyDeviceToHost, h->stream);
+    const int rc = copy_state_host(h, buf.data(), true);
+    if (rc) {
+      std::fclose(fp);
+      return rc;
     }
   } else if (ok) {
     int32_t flags[2] = {h->use_rho, h->use_u};
@@ -788,20 +892,13 @@ int lb_load(lb_handle* h, const char* path) {
   const size_t N = (size_t)h->g.N;
   cudaError_t e = cudaSuccess;
   if (hdr[2] == 1) {
-    const size_t sb = state_bytes(h);
+    const size_t sb = file_state_bytes(h);
     std::vector<char> buf(sb);
     ok = std::fread(buf.data(), 1, sb, fp) == sb;
     std::fclose(fp);
     if (!ok) return set_err(LB_EIO, "truncated checkpoint");
-    const StateBuf& s = h->S[h->cur];
-    if (storage_is_twoset(h->storage)) {
-      e = cudaMemcpyAsync(s.f, buf.data(), sb, cudaMemcpyHostToDevice, h->stream);
-    } else {
-      const size_t fb = (size_t)state_arrays(h->storage) * N * elem_bytes(h->storage);
-      e = cudaMemcpyAsync(s.f, buf.data(), fb, cudaMemcpyHostToDevice, h->stream);
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(s.sv, buf.data() + fb, N * sizeof(float4), cudaMemcpyHostToDevice, h->stream);
-    }
+    const int rc = copy_state_host(h, buf.data(), false);
+    if (rc) return rc;
     if (e == cudaSuccess) e = rebuild_acc(h);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_err(e, "checkpoint upload");
@@ -835,13 +932,9 @@ int lb_copy_state(lb_handle* dst, lb_handle* src) {
   if (e == cudaSuccess && src->mode == 1) {
     const StateBuf& a = src->S[src->cur];
     const StateBuf& b = dst->S[dst->cur];
-    if (storage_is_twoset(src->storage)) {
-      e = cudaMemcpyAsync(b.f, a.f, state_bytes(src), cudaMemcpyDeviceToDevice, dst->stream);
-    } else {
-      const size_t fb = (size_t)state_arrays(src->storage) * N * elem_bytes(src->storage);
-      e = cudaMemcpyAsync(b.f, a.f, fb, cudaMemcpyDeviceToDevice, dst->stream);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(b.sv, a.sv, N * sizeof(float4), cudaMemcpyDeviceToDevice, dst->stream);
-    }
+    e = cudaMemcpyAsync(b.f, a.f, dev_pop_bytes(src), cudaMemcpyDeviceToDevice, dst->stream);
+    if (e == cudaSuccess && !storage_is_twoset(src->storage))
+      e = cudaMemcpyAsync(b.sv, a.sv, N * sizeof(float4), cudaMemcpyDeviceToDevice, dst->stream);
     if (e == cudaSuccess) e = rebuild_acc(dst);
   } else if (e == cudaSuccess) {
     e = cudaMemcpyAsync(dst->init_phi, src->init_phi, N * sizeof(float), cudaMemcpyDeviceToDevice, dst->stream);
@@ -855,7 +948,6 @@ int lb_copy_state(lb_handle* dst, lb_handle* src) {
         return set_err(LB_ENOMEM, "field buffer allocation failed");
       e = cudaMemcpyAsync(dst->init_u, src->init_u, 3 * N * sizeof(float), cudaMemcpyDeviceToDevice, dst->stream);
     }
-    if (e == cudaSuccess) e = launch_phi_from_init(dst->storage, dst->g, dst->init_phi, dst->phi, dst->stream);
     if (e == cudaSuccess) e = reset_acc(dst);
   }
   if (e != cudaSuccess) return cuda_err(e, "copy state");
@@ -879,10 +971,13 @@ struct lb_batch {
   int storage = 0;
   cudaStream_t stream = nullptr;
   cudaStream_t own_stream = nullptr;
+  int device = 0;
   RunDesc* d_runs = nullptr;
   std::vector<RunDesc> h_runs;
-  long long ntiles = 0, max_nodes = 0, total_nodes = 0;
-  int halo = 1;  // largest staging halo of the runs
+  int* d_run_of = nullptr;  // run of every tile, then of every row group (owned by run 0)
+  size_t run_of_cap = 0;
+  long long ntiles = 0, ngroups = 0, max_rows = 0, total_nodes = 0;
+  int halo = 1;  // staging halo of every run: the largest any of them needs
   int tile = 0;
   int blocks_per_sm = 2;
   bool dirty = true;
@@ -903,27 +998,42 @@ void batch_drop_graphs(lb_batch* b) {
 
 int batch_descriptors(lb_batch* b) {
   const Tile& T = kTiles[b->tile];
-  long long tb = 0;
-  b->halo = 1;
-  b->max_nodes = 0;
+  long long tb = 0, rb = 0;
+  b->max_rows = 0;
   b->h_runs.resize(b->runs.size());
   for (size_t r = 0; r < b->runs.size(); ++r) {
     lb_handle* h = b->runs[r];
     RunDesc& d = b->h_runs[r];
     d.g = h->g;
-    d.p = h->p;
+    d.p = phys_as<float>(h->p);
     d.S[0] = h->S[0];
     d.S[1] = h->S[1];
     for (int k = 0; k < 3; ++k) d.acc[k] = h->acc[k];
-    d.tiles_x = (h->g.nx + T.tx - 1) / T.tx;
-    d.tiles_y = (h->g.ny + T.ty - 1) / T.ty;
-    d.tiles_z = (h->g.nz + T.tz - 1) / T.tz;
+    d.phi = (float*)h->phi;
+    d.pg = pad_geo(h->g, h->halo);
     d.tile_begin = tb;
-    tb += (long long)d.tiles_x * d.tiles_y * d.tiles_z;
-    b->halo = std::max(b->halo, stage_halo(h->p));
-    b->max_nodes = std::max(b->max_nodes, h->g.N);
+    d.row_begin = rb;
+    tb += (long long)((h->g.nx + T.tx - 1) / T.tx) * ((h->g.ny + T.ty - 1) / T.ty) * ((h->g.nz + T.tz - 1) / T.tz);
+    rb += ((long long)h->g.ny * h->g.nz + 7) / 8;
+    b->max_rows = std::max(b->max_rows, (long long)((h->g.nx + BLK - 1) / BLK) * h->g.ny);
   }
   b->ntiles = tb;
+  b->ngroups = rb;
+  std::vector<int> run_of((size_t)(tb + rb));
+  for (size_t r = 0; r < b->h_runs.size(); ++r) {
+    const bool last = r + 1 == b->h_runs.size();
+    std::fill(run_of.begin() + b->h_runs[r].tile_begin, run_of.begin() + (last ? tb : b->h_runs[r + 1].tile_begin), (int)r);
+    std::fill(run_of.begin() + tb + b->h_runs[r].row_begin, run_of.begin() + tb + (last ? rb : b->h_runs[r + 1].row_begin), (int)r);
+  }
+  if (run_of.size() > b->run_of_cap) {
+    LB_CUDA(cudaStreamSynchronize(b->stream));  // steps in flight read the old table
+    dev_free(b->runs[0], b->d_run_of);
+    b->run_of_cap = 0;
+    b->d_run_of = (int*)dev_alloc(b->runs[0], run_of.size() * sizeof(int));
+    if (!b->d_run_of) return set_err(LB_ENOMEM, "work list allocation failed");
+    b->run_of_cap = run_of.size();
+  }
+  LB_CUDA(cudaMemcpyAsync(b->d_run_of, run_of.data(), run_of.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
   LB_CUDA(cudaMemcpyAsync(b->d_runs, b->h_runs.data(), sizeof(RunDesc) * b->h_runs.size(), cudaMemcpyHostToDevice,
                           b->stream));
   LB_CUDA(cudaStreamSynchronize(b->stream));
@@ -933,9 +1043,9 @@ int batch_descriptors(lb_batch* b) {
 
 // one batched step from lattice parity `parity` and accumulator phase k
 int batch_issue(lb_batch* b, int parity, int k) {
-  LB_CUDA(launch_batched(b->storage, b->d_runs, (int)b->runs.size(), b->ntiles, b->tile, b->halo, b->max_nodes,
-                         parity, k, b->blocks_per_sm, b->runs[0]->status, b->stream));
-  g_launches += 1;
+  LB_CUDA(launch_batched(b->storage, b->d_runs, b->d_run_of, b->ntiles, b->ngroups, b->tile, b->halo,
+                         b->max_rows, parity, k, b->blocks_per_sm, b->runs[0]->status, b->stream));
+  g_launches += 2;
   return LB_OK;
 }
 
@@ -1041,15 +1151,18 @@ int lb_batch_create(int32_t nruns, const lb_grid* grids, const lb_params* params
     return set_err(LB_EINVAL, "batches support the two-set and reduced FP32/FP16 storages only");
   lb_batch* b = new lb_batch();
   b->storage = params[0].storage;
-  cudaError_t e = cudaStreamCreate(&b->own_stream);
+  cudaGetDevice(&b->device);
+  cudaError_t e = take_stream(&b->own_stream);
   if (e != cudaSuccess) {
     delete b;
-    return cuda_err(e, "cudaStreamCreate");
+    return cuda_err(e, "stream");
   }
   b->stream = b->own_stream;
+  for (int r = 0; r < nruns; ++r)
+    if (params[r].A_h != 0.0) b->halo = std::max(b->halo, params[r].h_max < 4.0 ? 4 : 7);  // stage_halo
   for (int r = 0; r < nruns; ++r) {
     lb_handle* h = nullptr;
-    int rc = lb_create(&grids[r], &params[r], alloc, &h);
+    int rc = create_handle(&grids[r], &params[r], alloc, b->halo, &h);
     if (rc) {
       lb_batch_destroy(b);
       return rc;
@@ -1072,7 +1185,10 @@ int lb_batch_destroy(lb_batch* b) {
   if (b->stream) cudaStreamSynchronize(b->stream);
   batch_drop_graphs(b);
   for (size_t r = b->runs.size(); r-- > 0;) lb_destroy(b->runs[r]);  // run 0 owns the descriptors
-  if (b->own_stream) cudaStreamDestroy(b->own_stream);
+  if (b->own_stream) {
+    cudaStreamSynchronize(b->own_stream);
+    give_stream(b->device, b->own_stream);
+  }
   delete b;
   return LB_OK;
 }
@@ -1171,9 +1287,7 @@ int lb_batch_autotune(lb_batch* b, int32_t steps, int use_cache, double* result)
   int rc = batch_tune(b, steps, use_cache, result);
   // the timed steps advanced the runs: return every run to its initial state
   for (lb_handle* h : b->runs) {
-    cudaError_t e = launch_phi_from_init(h->storage, h->g, h->init_phi, h->phi, h->stream);
-    if (e == cudaSuccess) e = reset_acc(h);
-    g_launches += 1;
+    cudaError_t e = reset_acc(h);
     if (e != cudaSuccess && rc == LB_OK) rc = cuda_err(e, "autotune reset");
     h->mode = 0;
     h->t = 0;

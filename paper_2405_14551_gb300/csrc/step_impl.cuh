@@ -160,19 +160,19 @@ __device__ __forceinline__ R eval_moment(const float4& qa, const float4& qb, con
 // Stored post-collision total population f*_dir of node src (single set
 // storages).  Reduced: the stored value.  Moment storage: the node's
 // quadratic form (eval_moment); only the records that c_i touches are read.
-template <int ST, typename I>
-__device__ __forceinline__ typename Store<ST>::R load_fs(const typename Store<ST>::E* __restrict__ f, I N, I dir, I src,
-                                                         int i, bool bb) {
+template <int ST>
+__device__ __forceinline__ typename Store<ST>::R load_fs(const typename Store<ST>::E* __restrict__ f, size_t N, int dir,
+                                                         size_t src, int i, bool bb) {
   using R = typename Store<ST>::R;
   if constexpr (Store<ST>::MOMENT) {
     const float4 qa = reinterpret_cast<const float4*>(f)[src];
     float4 qb = make_float4(0.f, 0.f, 0.f, 0.f);
     float2 qc = make_float2(0.f, 0.f);
-    if (cx(i) || cy(i) || cz(i)) qb = reinterpret_cast<const float4*>(f + (I)4 * N)[src];
-    if ((cx(i) && cz(i)) || (cy(i) && cz(i))) qc = reinterpret_cast<const float2*>(f + (I)8 * N)[src];
+    if (cx(i) || cy(i) || cz(i)) qb = reinterpret_cast<const float4*>(f + 4 * N)[src];
+    if ((cx(i) && cz(i)) || (cy(i) && cz(i))) qc = reinterpret_cast<const float2*>(f + 8 * N)[src];
     return eval_moment<R>(qa, qb, qc, i, bb);
   } else {
-    return decode<ST>(f[dir * N + src], i);
+    return decode<ST>(f[src + dir * BLK], i);  // src: Lay::at of the node
   }
 }
 
@@ -183,18 +183,18 @@ __device__ __forceinline__ double round_(double v) { return round(v); }
 __device__ __forceinline__ bool finite_(float v) { return isfinite(v); }
 __device__ __forceinline__ bool finite_(double v) { return isfinite(v); }
 
-// A collision's output apart from the relaxed populations, as a quadratic form
-// in the lattice velocity: w_i (alpha + beta.c_i + c_i.Gamma.c_i).  The
-// equilibrium, the perturbation (B_i = w_i (|c_i|^2 - 2/3)), the Guo source and
-// the projected non-equilibrium part are all of this shape, so a node forms
-// these ten coefficients once and each opposite pair (p, 26 - p) takes its even
-// part w (alpha + c.Gamma.c) and its odd part w beta.c with one or two
-// additions from sums that the pairs share, in place of three scalar products
-// and their products per pair.  The step is bound by instruction issue more
-// than by bytes; measured per step, before -> after: Shan-Chen 128x128x256 441
-// -> 408 us, regularised reduced FP32 150x93x203 427 -> 400 us, FP16 128x128x256
-// 433 -> 415 us.  xy, xz, yz hold 2 Gamma.  The roundings are explicit, so every
-// instantiation of the step forms the same values.
+// The output of a Shan-Chen collision apart from the relaxed populations, as a
+// quadratic form in the lattice velocity: w_i (alpha + beta.c_i +
+// c_i.Gamma.c_i).  The equilibrium and the Guo source are of this shape, so a
+// node forms these ten coefficients once per component and each opposite pair
+// (p, 26 - p) takes its even part w (alpha + c.Gamma.c) and its odd part
+// w beta.c with one or two additions from sums that the pairs share, in place
+// of scalar products and their products per direction.  128x128x256: 441 ->
+// 408 us per step when it came in.  xy, xz, yz hold 2 Gamma.  The roundings are
+// explicit, so every instantiation of the step forms the same values.  (The
+// colour-gradient collision keeps its products per pair: the same change there
+// gained 3 to 6 %, but near contact turns a last-bit difference into other
+// scan decisions within tens of steps.)
 template <typename R>
 struct QForm {
   R a, bx, by, bz, xx, yy, zz, xy, xz, yz;
@@ -303,6 +303,37 @@ __device__ __forceinline__ bool region_walled(const Geo& g, int x0, int y0, int 
          (g.wz && (z0 - d <= 0 || z0 + tz - 1 + d >= g.nz - 1));
 }
 
+// Populations of a state (all storages but the moment records) are stored in
+// blocks of 32 nodes of a row: block (x / 32, y, z) holds its ND directions
+// one after the other, 32 values each.  A node's 27 (54) values then sit at
+// constant offsets from one address, and so do the values that one neighbour
+// row contributes, so that the pulls and stores of a node take their
+// direction from the instruction's immediate offset; a warp's store of a
+// whole node row is 32 x ND consecutive values.  With one array per direction
+// ([dir][z][y][x]) every access carried its own 64-bit address, some fifty
+// registers of them: 2.84 -> 2.57 ms per step of the 256x256x512 emulsion, 385
+// -> 358 us of Shan-Chen 128x128x256.
+// Rows are padded to whole blocks.
+template <int ST>
+struct Lay {
+  using E = typename Store<ST>::E;
+  static constexpr bool MOMENT = Store<ST>::MOMENT;
+  static constexpr int ND = Store<ST>::TWOSET ? 2 * Q : Q;
+  static constexpr int DS = MOMENT ? 1 : BLK;         // stride of the directions
+  // elements of one row, and element of node x of a row at direction 0 (moment
+  // storage: the node index)
+  __host__ __device__ __forceinline__ static size_t row(const Geo& g) {
+    return MOMENT ? (size_t)g.nx : (size_t)((g.nx + BLK - 1) / BLK) * (ND * BLK);
+  }
+  template <typename I>
+  __host__ __device__ __forceinline__ static I in_row(I x) {
+    return MOMENT ? x : x / BLK * (I)(ND * BLK) + x % BLK;
+  }
+  __host__ __device__ __forceinline__ static size_t at(const Geo& g, int x, int y, int z) {
+    return row(g) * ((size_t)y + (size_t)g.ny * z) + in_row((size_t)x);
+  }
+};
+
 template <int ST>
 struct View {
   using E = typename Store<ST>::E;
@@ -355,16 +386,17 @@ __device__ __forceinline__ void pull_node(const View<ST>& S, const Geo& g, const
   for (int i = 0; i < Q; ++i) {
     const int a = 1 - cx(i), b = 1 - cy(i), c = 1 - cz(i);
     const bool bb = n.sx[a] | n.sy[b] | n.sz[c];
-    const long long src = bb ? self : (long long)n.xs[a] + (long long)g.nx * ((long long)n.ys[b] + (long long)g.ny * n.zs[c]);
+    const int sx = bb ? n.xs[1] : n.xs[a], sy = bb ? n.ys[1] : n.ys[b], sz = bb ? n.zs[1] : n.zs[c];
+    const size_t src = Lay<ST>::at(g, sx, sy, sz);
     const int dir = bb ? opp(i) : i;
     R va, vb;
     if constexpr (Store<ST>::TWOSET) {
-      va = decode<ST>(S.f[(size_t)dir * N + src], i);
-      vb = decode<ST>(S.f[(size_t)(Q + dir) * N + src], i);
+      va = decode<ST>(S.f[src + (size_t)dir * BLK], i);
+      vb = decode<ST>(S.f[src + (size_t)(Q + dir) * BLK], i);
       f[i] = va + vb;
     } else {
-      const R fs = load_fs<ST, size_t>(S.f, N, (size_t)dir, (size_t)src, i, bb);
-      colour_split<R, true>(fs, S.sv[src], i, bb, va, vb);
+      const R fs = load_fs<ST>(S.f, N, dir, src, i, bb);
+      colour_split<R, true>(fs, S.sv[(size_t)sx + (size_t)g.nx * ((size_t)sy + (size_t)g.ny * sz)], i, bb, va, vb);
       f[i] = fs;
     }
     rA += va;
@@ -379,7 +411,7 @@ __device__ __forceinline__ void pull_node(const View<ST>& S, const Geo& g, const
 // Pre-collision populations from fields (initial state or reconstruction):
 // f_i = f^eq_i(rho, u) (Eq. disteq) [+ w_i/(2 cs^4) Q_i:Pi^neq], f^A = (rhoA/rho) f.
 template <typename R, bool COMP>
-__device__ __forceinline__ void fields_node(const InitBuf& I, const Geo& g, const Phys& P, const Nbr& n,
+__device__ __forceinline__ void fields_node(const InitBuf& I, const Geo& g, const PhysR<R>& P, const Nbr& n,
                                             long long self, R f[Q], R& rA, R& rB, R* fa, R* fb) {
   const R ph = I.phi[self];
   const R rho = I.rho ? R(I.rho[self]) : R(1);
@@ -447,87 +479,106 @@ __device__ __forceinline__ void fields_node(const InitBuf& I, const Geo& g, cons
   }
 }
 
-// Pull for the hot path: totals f_i and component densities.  WALLFREE: no
-// neighbour of the node is solid (no bounce-back test).  IDX32: every
-// population offset fits in 32 bits.  TOTALS (single-set storages): only the
-// totals f_i; the neighbours' colour scalars are not read and rA, rB are left
-// to the caller.
-template <int ST, bool WALLFREE, bool IDX32, bool TOTALS>
-__device__ __forceinline__ void pull_fast(const View<ST>& S, const Geo& g, const Nbr& n, int self,
-                                          typename Store<ST>::R f[Q], typename Store<ST>::R& rA,
-                                          typename Store<ST>::R& rB) {
+// A value that is the same in every lane, in a form the compiler knows to be
+// uniform (a warp reduction's result), so that base addresses made from it
+// take the uniform path as kernel parameters do.
+__device__ __forceinline__ int uniform(int v) { return (int)__reduce_or_sync(0xffffffffu, (unsigned)v); }
+__device__ __forceinline__ float uniform(float v) { return __int_as_float(uniform(__float_as_int(v))); }
+template <typename T>
+__device__ __forceinline__ T* uniform(T* p) {
+  const unsigned long long v = reinterpret_cast<unsigned long long>(p);
+  const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)v), hi = __reduce_or_sync(0xffffffffu, (unsigned)(v >> 32));
+  return reinterpret_cast<T*>(((unsigned long long)hi << 32) | lo);
+}
+// Where a node of a tile without solid neighbours (WALLFREE) reads its
+// neighbours' values.  The z plane of a source is the same for the whole CTA,
+// so a thread keeps nine offsets within a plane (3 x 3 neighbours in x and y)
+// for all its nodes; 27 addresses serve all pulls.  IDX32: the byte offsets
+// within one z plane fit in 32 bits.
+template <int ST, bool IDX32>
+struct PlaneIdx {
+  using I = typename std::conditional<IDX32, unsigned, size_t>::type;
+  I o[3][3];  // [y + 1][x + 1] element offset within a plane (moment storage: node offset)
+  __device__ __forceinline__ static I at(const Geo& g, int x, int y) { return (I)Lay<ST>::row(g) * (I)y + Lay<ST>::in_row((I)x); }
+  __device__ __forceinline__ void init(const Geo& g, int x, int y) {
+    int xs[3], ys[3];
+#pragma unroll
+    for (int d = -1; d <= 1; ++d) {
+      int a = x + d, b = y + d;
+      xs[d + 1] = a < 0 ? a + g.nx : (a >= g.nx ? a - g.nx : a);
+      ys[d + 1] = b < 0 ? b + g.ny : (b >= g.ny ? b - g.ny : b);
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) o[b][a] = at(g, xs[a], ys[b]);
+  }
+};
+// value at element offset o of a plane whose first element is base
+template <typename T, typename I>
+__device__ __forceinline__ T plane_ld(const T* __restrict__ base, I o) {
+  return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + (I)(o * (I)sizeof(T)));
+}
+// The raw stored values a node pulls (both sets, or the single set's totals),
+// loaded before anything is decoded so that independent work (gradient, scan)
+// runs while they are in flight.
+template <int ST, bool IDX32>
+__device__ __forceinline__ void pull_plane(const View<ST>& S, const Geo& g, const PlaneIdx<ST, IDX32>& ix, const int zs[3],
+                                           typename Store<ST>::E ra[Q], typename Store<ST>::E rb[Q]) {
+  using E = typename Store<ST>::E;
+  const size_t plane = Lay<ST>::row(g) * (size_t)g.ny;
+  const E* zp[3] = {S.f + (size_t)zs[0] * plane, S.f + (size_t)zs[1] * plane, S.f + (size_t)zs[2] * plane};
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const auto o = ix.o[1 - cy(i)][1 - cx(i)];
+    const E* p = reinterpret_cast<const E*>(reinterpret_cast<const char*>(zp[1 - cz(i)]) + o * (unsigned)sizeof(E));
+    ra[i] = p[i * BLK];
+    if constexpr (Store<ST>::TWOSET) rb[i] = p[(Q + i) * BLK];
+  }
+}
+// moment storage: the quadratic forms of the neighbours, evaluated
+template <int ST, bool IDX32>
+__device__ __forceinline__ void pull_plane_moment(const View<ST>& S, size_t N, size_t plane, const PlaneIdx<ST, IDX32>& ix,
+                                                  const int zs[3], typename Store<ST>::R f[Q]) {
   using R = typename Store<ST>::R;
-  using I = typename std::conditional<IDX32, unsigned, size_t>::type;
-  const I N = (I)g.N;
-  int rb[3][3];
-#pragma unroll
-  for (int b = 0; b < 3; ++b)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) rb[b][c] = g.nx * (n.ys[b] + g.ny * n.zs[c]);
-  rA = R(0);
-  rB = R(0);
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
-    const int a = 1 - cx(i), b = 1 - cy(i), c = 1 - cz(i);
-    int src = n.xs[a] + rb[b][c];
-    I dir = (I)i;
-    bool bb = false;
-    if constexpr (!WALLFREE) {
-      bb = n.sx[a] | n.sy[b] | n.sz[c];
-      src = bb ? self : src;
-      dir = bb ? (I)opp(i) : dir;
-    }
-    if constexpr (Store<ST>::TWOSET) {
-      const R va = decode<ST>(S.f[dir * N + (I)src], i);
-      const R vb = decode<ST>(S.f[((I)Q + dir) * N + (I)src], i);
-      f[i] = va + vb;
-      rA += va;
-      rB += vb;
-    } else if constexpr (TOTALS) {
-      f[i] = load_fs<ST, I>(S.f, N, dir, (I)src, i, bb);
-    } else {
-      const R fs = load_fs<ST, I>(S.f, N, dir, (I)src, i, bb);
-      R va, vb;
-      colour_split<R, !WALLFREE>(fs, S.sv[src], i, bb, va, vb);
-      f[i] = fs;
-      rA += va;
-      rB += vb;
-    }
+    const size_t zp = (size_t)zs[1 - cz(i)] * plane;
+    const auto o = ix.o[1 - cy(i)][1 - cx(i)];
+    const float4 qa = plane_ld(reinterpret_cast<const float4*>(S.f) + zp, o);
+    float4 qb = make_float4(0.f, 0.f, 0.f, 0.f);
+    float2 qc = make_float2(0.f, 0.f);
+    if (i != REST) qb = plane_ld(reinterpret_cast<const float4*>(S.f + 4 * N) + zp, o);
+    if ((cx(i) && cz(i)) || (cy(i) && cz(i))) qc = plane_ld(reinterpret_cast<const float2*>(S.f + 8 * N) + zp, o);
+    f[i] = eval_moment<R>(qa, qb, qc, i, false);
   }
 }
-
-// The pull of pull_fast split in two: the raw stored values (both sets, or
-// the single set's totals) are loaded first and decoded and summed later, so
-// that independent work (the near-contact scan) runs while the loads are in
-// flight.  Same values and the same order of additions as pull_fast.
-template <int ST, bool WALLFREE, bool IDX32>
-__device__ __forceinline__ void pull_raw(const View<ST>& S, const Geo& g, const Nbr& n, int self,
-                                         typename Store<ST>::E ra[Q], typename Store<ST>::E rb[Q]) {
-  using I = typename std::conditional<IDX32, unsigned, size_t>::type;
-  const I N = (I)g.N;
-  int rbo[3][3];
-#pragma unroll
-  for (int b = 0; b < 3; ++b)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) rbo[b][c] = g.nx * (n.ys[b] + g.ny * n.zs[c]);
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const int a = 1 - cx(i), b = 1 - cy(i), c = 1 - cz(i);
-    int src = n.xs[a] + rbo[b][c];
-    I dir = (I)i;
-    if constexpr (!WALLFREE) {
-      const bool bb = n.sx[a] | n.sy[b] | n.sz[c];
-      src = bb ? self : src;
-      dir = bb ? (I)opp(i) : dir;
-    }
-    ra[i] = S.f[dir * N + (I)src];
-    if constexpr (Store<ST>::TWOSET) rb[i] = S.f[((I)Q + dir) * N + (I)src];
-  }
-}
+// The same loads of a node with solid neighbours in reach (halfway
+// bounce-back from the node itself, Lay::at element self), any offset width.
 template <int ST>
-__device__ __forceinline__ void pull_raw_finish(const typename Store<ST>::E ra[Q], const typename Store<ST>::E rb[Q],
-                                                typename Store<ST>::R f[Q], typename Store<ST>::R& rA,
-                                                typename Store<ST>::R& rB) {
+__device__ __forceinline__ void pull_walled(const View<ST>& S, const Geo& g, const Nbr& n, size_t self,
+                                            typename Store<ST>::E ra[Q], typename Store<ST>::E rb[Q],
+                                            typename Store<ST>::R f[Q]) {
+  const size_t N = (size_t)g.N;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const int a = 1 - cx(i), b = 1 - cy(i), c = 1 - cz(i);
+    const bool bb = n.sx[a] | n.sy[b] | n.sz[c];
+    const size_t src = bb ? self : Lay<ST>::at(g, n.xs[a], n.ys[b], n.zs[c]);
+    const int dir = bb ? opp(i) : i;
+    if constexpr (Store<ST>::MOMENT) {
+      f[i] = load_fs<ST>(S.f, N, dir, src, i, bb);
+    } else {
+      ra[i] = S.f[src + dir * BLK];
+      if constexpr (Store<ST>::TWOSET) rb[i] = S.f[src + (Q + dir) * BLK];
+    }
+  }
+}
+// Decode the raw values: totals f_i and, for two sets, the component densities.
+template <int ST>
+__device__ __forceinline__ void pull_finish(const typename Store<ST>::E ra[Q], const typename Store<ST>::E rb[Q],
+                                            typename Store<ST>::R f[Q], typename Store<ST>::R& rA,
+                                            typename Store<ST>::R& rB) {
   using R = typename Store<ST>::R;
   rA = R(0);
   rB = R(0);
@@ -682,29 +733,29 @@ struct Acc<double> {
 
 // The integer sums of the component populations a node pulls (the same
 // values, hence the same sums, as the senders accumulated).
-template <int ST, bool WALLFREE, bool IDX32>
-__device__ __forceinline__ void pull_acc(const View<ST>& S, const Geo& g, const Nbr& n, int self,
+template <int ST, bool WALLFREE>
+__device__ __forceinline__ void pull_acc(const View<ST>& S, const Geo& g, const Nbr& n,
                                          typename Acc<typename Store<ST>::R>::S& sa,
                                          typename Acc<typename Store<ST>::R>::S& sb) {
   using R = typename Store<ST>::R;
   using A = Acc<R>;
-  using I = typename std::conditional<IDX32, unsigned, size_t>::type;
-  const I N = (I)g.N;
+  const size_t N = (size_t)g.N;
   sa = 0;
   sb = 0;
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const int a = 1 - cx(i), b = 1 - cy(i), c = 1 - cz(i);
     const bool bb = WALLFREE ? false : (n.sx[a] | n.sy[b] | n.sz[c]);
-    const I src = bb ? (I)self : (I)n.xs[a] + (I)g.nx * ((I)n.ys[b] + (I)g.ny * (I)n.zs[c]);
-    const I dir = bb ? (I)opp(i) : (I)i;
+    const int sx = bb ? n.xs[1] : n.xs[a], sy = bb ? n.ys[1] : n.ys[b], sz = bb ? n.zs[1] : n.zs[c];
+    const size_t src = Lay<ST>::at(g, sx, sy, sz);
+    const int dir = bb ? opp(i) : i;
     R va, vb;
     if constexpr (Store<ST>::TWOSET) {
-      va = decode<ST>(S.f[dir * N + src], i);
-      vb = decode<ST>(S.f[((I)Q + dir) * N + src], i);
+      va = decode<ST>(S.f[src + dir * BLK], i);
+      vb = decode<ST>(S.f[src + (Q + dir) * BLK], i);
     } else {
-      const R fs = load_fs<ST, I>(S.f, N, dir, src, i, bb);
-      colour_split<R, !WALLFREE>(fs, S.sv[src], i, bb, va, vb);
+      const R fs = load_fs<ST>(S.f, N, dir, src, i, bb);
+      colour_split<R, !WALLFREE>(fs, S.sv[(size_t)sx + (size_t)g.nx * ((size_t)sy + (size_t)g.ny * sz)], i, bb, va, vb);
     }
     sa += A::q(va);
     sb += A::q(vb);
@@ -713,7 +764,7 @@ __device__ __forceinline__ void pull_acc(const View<ST>& S, const Geo& g, const 
 
 // Rebuild the accumulator of the current time level from stored populations
 // (after a checkpoint load or a state copy): one node per thread.
-template <int ST, bool IDX32>
+template <int ST>
 __global__ void __launch_bounds__(256) k_phi_acc(View<ST> S, Geo g, unsigned long long* __restrict__ acc) {
   using A = Acc<typename Store<ST>::R>;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -730,155 +781,174 @@ __global__ void __launch_bounds__(256) k_phi_acc(View<ST> S, Geo g, unsigned lon
     make_nbr(g, x, y, z, n);
     typename A::S sa, sb;
     if (near_wall(g, x, y, z))
-      pull_acc<ST, false, IDX32>(S, g, n, (int)idx, sa, sb);
+      pull_acc<ST, false>(S, g, n, sa, sb);
     else
-      pull_acc<ST, true, IDX32>(S, g, n, (int)idx, sa, sb);
+      pull_acc<ST, true>(S, g, n, sa, sb);
     A::store(acc, (size_t)idx, sa, sb);
   }
 }
 
 // ---------------------------------------------------------------------------
+// phase field of the current level
+// ---------------------------------------------------------------------------
+// k_phi decodes the staged scalars of the whole lattice once per step into a
+// padded array (PadGeo), so that a tile stages its halo with plain 16-byte
+// asynchronous copies: no wrap, no solid test and no decoding in the tile.
+// The decoding of one value (two integer-to-float conversions and a
+// reciprocal) used to be repeated for every tile that holds the node in its
+// halo, 5 times per node for a 32x8x8 tile with near contact.
+// Fields: phi, or (Shan-Chen) phi, psi_A, psi_B.  A warp takes a row of nodes,
+// reads each word once and stores it to every padded position that wraps onto
+// it; positions beyond a wall and solid layers hold PHI_SOLID from the array's
+// creation (k_phi_fill) on.  It also zeroes the accumulator two steps ahead
+// (AccBufs::zero, or null).
+// Bound: bytes (8 B read, 4 B written, 8 B zeroed per node).
+template <typename R>
+__device__ __forceinline__ R sc_psi(R r, R psi0) {
+  if constexpr (sizeof(R) == 4) return psi0 * (1.0f - expf(-r / psi0));
+  else return psi0 * (1.0 - exp(-r / psi0));
+}
+
+// The launches of a step (k_phi, k_step, k_phi of the next, ...) follow one
+// another with programmatic dependent launch: a kernel lets its successor
+// start filling free SMs once all its own CTAs run, and touches global memory
+// only after its predecessor has completed.  That hides the launch latency,
+// the larger part of a step on small lattices.  Together with k_phi reading each
+// word once: 58.1 -> 54.5 us per step at 64x64x128, 2.57 -> 2.50 ms at
+// 256x256x512.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Source coordinate of padded coordinate c - h on an axis of n nodes; -1
+// where the position is solid or beyond a wall.
+__device__ __forceinline__ int pad_source(int c, int h, int n, int wall) {
+  int v = c - h;
+  if (wall) return v <= 0 || v >= n - 1 ? -1 : v;
+  if ((unsigned)v < (unsigned)n) return v;
+  v += v < 0 ? n : -n;
+  if ((unsigned)v < (unsigned)n) return v;
+  return ((v % n) + n) % n;
+}
+
+template <typename R, bool SC>
+__device__ __forceinline__ void phi_row(const PhiSrc& src, const InitBuf& init, const Geo& g, const PadGeo& pg, R psi0,
+                                        R* __restrict__ out, unsigned long long* __restrict__ zero, int y, int z) {
+  if ((g.wy && (y == 0 || y == g.ny - 1)) || (g.wz && (z == 0 || z == g.nz - 1))) return;
+  const int lane = threadIdx.x;
+  const size_t fld = (size_t)pg.px * pg.py * pg.pz;
+  const size_t base = (size_t)g.nx * ((size_t)y + (size_t)g.ny * z);
+  const int xa = g.wx ? 1 : 0, xb = g.wx ? g.nx - 1 : g.nx;  // fluid nodes of the row
+  // padded coordinates that wrap onto the row: its own first
+  const int ey = g.wy ? 0 : g.ny, ez = g.wz ? 0 : g.nz, limy = g.ny + 2 * pg.h, limz = g.nz + 2 * pg.h;
+  int cy0 = y + pg.h, cz0 = z + pg.h;
+  while (ey && cy0 >= ey) cy0 -= ey;
+  while (ez && cz0 >= ez) cz0 -= ez;
+  for (int x0 = xa; x0 < xb; x0 += 128) {
+    R v[4][SC ? 3 : 1];
+    // four positions a lane, 32 apart: their loads are in flight together
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int x = x0 + 32 * j + lane;
+      if (x >= xb) continue;
+      if constexpr (SC) {
+        R ra, rb;
+        if (src.acc) {
+          Acc<R>::densities(src.acc, base + x, ra, rb);
+        } else {
+          const R ph = R(src.phi[base + x]);
+          const R rho = init.rho ? R(init.rho[base + x]) : R(1);
+          ra = rho * (R(1) + ph) * R(0.5);
+          rb = rho * (R(1) - ph) * R(0.5);
+        }
+        v[j][0] = (ra - rb) / (ra + rb);
+        v[j][1] = sc_psi(ra, psi0);
+        v[j][2] = sc_psi(rb, psi0);
+      } else {
+        v[j][0] = src.acc ? Acc<R>::phi(src.acc, base + x) : R(src.phi[base + x]);
+      }
+    }
+    if (zero) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (x0 + 32 * j + lane < xb) Acc<R>::zero(zero, base + x0 + 32 * j + lane);
+    }
+    for (int cz = cz0; cz < limz; cz += ez ? ez : limz) {
+      for (int cy = cy0; cy < limy; cy += ey ? ey : limy) {
+        R* row = out + (size_t)pg.px * ((size_t)cy + (size_t)pg.py * cz);
+        auto put = [&](int c, const R* w) {
+          row[c] = w[0];
+          if constexpr (SC) {
+            row[fld + c] = w[1];
+            row[2 * fld + c] = w[2];
+          }
+        };
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int x = x0 + 32 * j + lane;
+          if (x >= xb) continue;
+          const int c = x + pg.hx;
+          put(c, v[j]);
+          if (!g.wx) {
+            for (int d = c - g.nx; d >= 0; d -= g.nx) put(d, v[j]);
+            for (int d = c + g.nx; d < g.nx + 2 * pg.hx; d += g.nx) put(d, v[j]);
+          }
+        }
+      }
+    }
+  }
+}
+
+template <typename R, bool SC>
+__global__ void __launch_bounds__(256) k_phi(PhiSrc src, InitBuf init, Geo g, PadGeo pg, R psi0, R* __restrict__ out,
+                                             unsigned long long* __restrict__ zero) {
+  launch_dependents();
+  wait_primary();
+  const long long rows = (long long)g.ny * g.nz;
+  for (long long row = (long long)blockIdx.x * 8 + threadIdx.y; row < rows; row += (long long)gridDim.x * 8)
+    phi_row<R, SC>(src, init, g, pg, psi0, out, zero, (int)(row % g.ny), (int)(row / g.ny));
+}
+
+// ---------------------------------------------------------------------------
 // shared-memory layout of a tile
 // ---------------------------------------------------------------------------
-// phi of the tile plus a halo of H nodes (HX along x: 1 without near
-// contact, else H rounded up to a multiple of 4 so that rows start on 16-byte
-// vectors), the component partial sums over the tile plus a one-node ring,
-// and with near contact the scan queue, the distance h of each tile node and
-// the queue counter.
+// The staged scalar fields (NPH of them) of the tile plus a halo of H nodes
+// (pad_hx(H) along x, so that rows are whole 16-byte pieces of the padded
+// array) and the component partial sums over the tile plus a one-node ring.
 constexpr size_t align16(size_t b) { return (b + 15) / 16 * 16; }
 
-template <typename R, int TX, int TY, int TZ, int H, int NPH = 1, bool QH = true>
+template <typename R, int TX, int TY, int TZ, int H, int NPH = 1>
 struct Layout {
-  static constexpr int HX = H == 1 ? 1 : (H + 3) / 4 * 4;
+  static constexpr int HX = pad_hx(H);
   static constexpr int SX = TX + 2 * HX, SY = TY + 2 * H, SZ = TZ + 2 * H, SXY = SX * SY, NS = SXY * SZ;
   static constexpr int EX = TX + 2, EY = TY + 2, EZ = TZ + 2, EXY = EX * EY, E = EXY * EZ;
-  static constexpr int NT = TX * TY * TZ;
-  // NPH staged scalar fields of NS values each (phi; the Shan-Chen model
-  // adds psi_A and psi_B)
   static constexpr size_t off_acc = align16(sizeof(R) * (size_t)NS * NPH);
-  // the scan's queue and h (QH: a tile that scans in its own phase)
-  static constexpr size_t off_queue = off_acc + align16(8 * (size_t)Acc<R>::W * (size_t)E);
-  static constexpr size_t off_h = off_queue + (H > 1 && QH ? align16(2 * (size_t)NT) : 0);
-  static constexpr size_t off_count = off_h + (H > 1 && QH ? align16((size_t)NT) : 0);
-  static constexpr size_t bytes = off_count + 16;
+  static constexpr size_t bytes = off_acc + align16(8 * (size_t)Acc<R>::W * (size_t)E);
 };
 
-template <typename R, bool FROM_ACC>
-struct PhiLoad {
-  // nodes per 16-byte vector
-  static constexpr int V = FROM_ACC ? 16 / (8 * Acc<R>::W) : 16 / (int)sizeof(R);
-  using Raw = typename std::conditional<FROM_ACC, ulonglong2,
-                                        typename std::conditional<sizeof(R) == 4, float4, double2>::type>::type;
-  __device__ static __forceinline__ R one(const PhiSrc& s, size_t node) {
-    if constexpr (FROM_ACC) return Acc<R>::phi(s.acc, node);
-    else return reinterpret_cast<const R*>(s.phi)[node];
-  }
-  // the V consecutive nodes from `node` (a multiple of V) as one load ...
-  __device__ static __forceinline__ Raw ld(const PhiSrc& s, size_t node) {
-    if constexpr (FROM_ACC) return acc_ld2(s.acc + Acc<R>::W * node);
-    else return *reinterpret_cast<const Raw*>(reinterpret_cast<const R*>(s.phi) + node);
-  }
-  // ... and their phi
-  __device__ static __forceinline__ void dec(const Raw& w, R* out) {
-    if constexpr (FROM_ACC) {
-      if constexpr (Acc<R>::W == 1) {
-        out[0] = Acc<float>::phi_word(w.x);
-        out[1] = Acc<float>::phi_word(w.y);
-      } else {
-        out[0] = Acc<double>::phi_words(w.x, w.y);
-      }
-    } else {
-      const R* r = reinterpret_cast<const R*>(&w);
-#pragma unroll
-      for (int j = 0; j < V; ++j) out[j] = r[j];
-    }
-  }
-};
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Stage phi of the tile plus its halo (Layout) in shared memory; solid and
-// beyond-wall nodes get the marker PHI_SOLID, periodic axes wrap.  The block
-// is walked as one flat list (of 16-byte vectors when the rows allow it), so
-// no lane idles on a short row.  No barrier.
-template <typename R, bool FROM_ACC, int TX, int TY, int TZ, int H>
-__device__ __forceinline__ void stage_phi(const PhiSrc& src, const Geo& g, R* sp, int x0, int y0, int z0) {
-  using L = Layout<R, TX, TY, TZ, H>;
-  using PL = PhiLoad<R, FROM_ACC>;
-  constexpr int V = PL::V;
+// Issue the copies of the tile's staged fields (the caller waits for them
+// with cp_async_wait_all and a barrier).
+template <typename R, int TX, int TY, int TZ, int H, int NPH>
+__device__ __forceinline__ void stage_tile(const R* __restrict__ phi, const PadGeo& pg, R* sp, int x0, int y0, int z0) {
+  using L = Layout<R, TX, TY, TZ, H, NPH>;
+  constexpr int V = 16 / (int)sizeof(R), QR = L::SX / V, ROWS = L::SY * L::SZ, NT = TX * TY;
+  const size_t fld = (size_t)pg.px * pg.py * pg.pz;
+  const R* base = phi + (size_t)x0 + (size_t)pg.px * ((size_t)y0 + (size_t)pg.py * z0);
   const int tid = threadIdx.y * TX + threadIdx.x;
-  if constexpr (H > 1) {
-    static_assert(L::HX % V == 0 && TX % V == 0, "vector staging needs whole vectors per row");
-  }
-  if (H > 1 && g.nx % V == 0) {
-    // every vector lies wholly inside or wholly outside the box along x; NB
-    // vectors per thread are loaded before any is decoded, so their latencies
-    // overlap
-    constexpr int QR = (H > 1 ? L::SX : V) / V, NQ = QR * L::SY * L::SZ, NB = 4;
-    using Raw = typename PL::Raw;
-    for (int q0 = tid; q0 < NQ; q0 += NB * TX * TY) {
-      Raw raw[NB];
-      int meta[NB];  // row * QR + qx, or -1 beyond the block
-      unsigned fill = 0;  // bit b: vector b is solid or beyond a wall (no load)
 #pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        const int q = q0 + b * TX * TY;
-        meta[b] = -1;
-        if (q >= NQ) continue;
-        meta[b] = q;
-        const int qx = q % QR, row = q / QR;
-        const int ly = row % L::SY, lz = row / L::SY;
-        int gy = y0 - H + ly, gz = z0 - H + lz;
-        bool rsolid = false;
-        if (g.wy) rsolid |= (gy <= 0 || gy >= g.ny - 1);
-        else if ((unsigned)gy >= (unsigned)g.ny) gy = ((gy % g.ny) + g.ny) % g.ny;
-        if (g.wz) rsolid |= (gz <= 0 || gz >= g.nz - 1);
-        else if ((unsigned)gz >= (unsigned)g.nz) gz = ((gz % g.nz) + g.nz) % g.nz;
-        const int gx0 = x0 - L::HX + qx * V;
-        bool inside = gx0 >= 0 && gx0 < g.nx;
-        int gxl = gx0;
-        if (!inside && !g.wx) {
-          gxl = ((gx0 % g.nx) + g.nx) % g.nx;
-          inside = true;
-        }
-        if (inside && !rsolid) raw[b] = PL::ld(src, (size_t)gxl + (size_t)g.nx * ((size_t)gy + (size_t)g.ny * gz));
-        else fill |= 1u << b;
-        if (rsolid) fill |= 1u << (NB + b);
-      }
+  for (int k = 0; k < (QR * ROWS + NT - 1) / NT; ++k) {
+    const int q = tid + k * NT;
+    if (q >= QR * ROWS) break;
+    const int row = q / QR, c = (q - row * QR) * V;
+    const int lz = row / L::SY, ly = row - lz * L::SY;
+    const size_t o = (size_t)pg.px * ((size_t)ly + (size_t)pg.py * lz) + c;
 #pragma unroll
-      for (int b = 0; b < NB; ++b) {
-        if (meta[b] < 0) continue;
-        const int qx = meta[b] % QR, row = meta[b] / QR;
-        R v[V];
-        if ((fill >> b) & 1u) {
-#pragma unroll
-          for (int j = 0; j < V; ++j) v[j] = R(PHI_SOLID);
-        } else {
-          PL::dec(raw[b], v);
-        }
-        const bool rsolid = (fill >> (NB + b)) & 1u;
-        const int gx0 = x0 - L::HX + qx * V;
-        R* dst = sp + (size_t)row * L::SX + qx * V;
-#pragma unroll
-        for (int j = 0; j < V; ++j) {
-          const int xj = gx0 + j;
-          const bool solid = rsolid || (g.wx && (xj <= 0 || xj >= g.nx - 1));
-          dst[j] = solid ? R(PHI_SOLID) : v[j];
-        }
-      }
-    }
-  } else {
-    for (int q = tid; q < L::NS; q += TX * TY) {
-      const int lx = q % L::SX, row = q / L::SX;
-      const int ly = row % L::SY, lz = row / L::SY;
-      int gx = x0 - L::HX + lx, gy = y0 - H + ly, gz = z0 - H + lz;
-      bool solid = false;
-      if (g.wx) solid |= (gx <= 0 || gx >= g.nx - 1);
-      else if ((unsigned)gx >= (unsigned)g.nx) gx = ((gx % g.nx) + g.nx) % g.nx;
-      if (g.wy) solid |= (gy <= 0 || gy >= g.ny - 1);
-      else if ((unsigned)gy >= (unsigned)g.ny) gy = ((gy % g.ny) + g.ny) % g.ny;
-      if (g.wz) solid |= (gz <= 0 || gz >= g.nz - 1);
-      else if ((unsigned)gz >= (unsigned)g.nz) gz = ((gz % g.nz) + g.nz) % g.nz;
-      sp[q] = solid ? R(PHI_SOLID) : PL::one(src, (size_t)gx + (size_t)g.nx * ((size_t)gy + (size_t)g.ny * gz));
-    }
+    for (int f = 0; f < NPH; ++f) cp_async16(sp + f * L::NS + row * L::SX + c, base + f * fld + o);
   }
 }
 
@@ -886,53 +956,60 @@ __device__ __forceinline__ void stage_phi(const PhiSrc& src, const Geo& g, R* sp
 // colour gradient and near-contact scan on the staged tile
 // ---------------------------------------------------------------------------
 // Colour gradient grad phi(p) = (1/cs2) sum_i w_i c_i phi(p + c_i) on the
-// shared tile; a solid neighbour contributes phi(p) (neutral wetting).  Tiles
-// whose halo holds no solid node skip the solid test (WALLFREE).  The D3Q27
-// weights factor: for c_a = +-1, w(c) = v(c_b) v(c_c) / 216 with v(0) = 4,
-// v(+-1) = 1 on the two other axes, so each component is the central
+// shared tile; a solid neighbour contributes phi(p) (neutral wetting).  The
+// D3Q27 weights factor: for c_a = +-1, w(c) = v(c_b) v(c_c) / 216 with v(0) =
+// 4, v(+-1) = 1 on the two other axes, so each component is the central
 // difference along its axis smoothed by (1, 4, 1) x (1, 4, 1) across the
-// others, times 3/216 = 1/72.  Evaluated one z plane of the 3x3x3 block at a
-// time.
+// others, times 3/216 = 1/72.  One z plane of the 3x3x3 block contributes its
+// smoothed x and y differences and its smoothed sum (GradPlane).
+template <typename R>
+struct GradPlane {
+  R ex, ey, sm;
+};
+template <typename R, bool WALLFREE, bool CENTRE>
+__device__ __forceinline__ GradPlane<R> grad_plane(const R* sp, int c, int SX, R p0) {
+  R p[3][3];
+#pragma unroll
+  for (int dy = -1; dy <= 1; ++dy) {
+#pragma unroll
+    for (int dx = -1; dx <= 1; ++dx) {
+      R v = sp[c + dx + SX * dy];
+      if constexpr (!WALLFREE) v = (v > R(0.5) * R(PHI_SOLID)) ? p0 : v;
+      p[dy + 1][dx + 1] = v;
+    }
+  }
+  GradPlane<R> o;
+  o.ex = fma_rn(R(4), p[1][2] - p[1][0], (p[0][2] - p[0][0]) + (p[2][2] - p[2][0]));
+  o.ey = fma_rn(R(4), p[2][1] - p[0][1], (p[2][0] - p[0][0]) + (p[2][2] - p[0][2]));
+  // the plane smoothed over x and y enters the z difference
+  o.sm = R(0);
+  if constexpr (CENTRE)
+    o.sm = fma_rn(R(4), fma_rn(R(4), p[1][1], p[1][0] + p[1][2]),
+                  fma_rn(R(4), p[0][1], p[0][0] + p[0][2]) + fma_rn(R(4), p[2][1], p[2][0] + p[2][2]));
+  return o;
+}
+template <typename R>
+__device__ __forceinline__ void grad_from(const GradPlane<R>& lo, const GradPlane<R>& mid, const GradPlane<R>& hi,
+                                          R gr[3]) {
+  constexpr R k72 = R(1) / R(72);
+  gr[0] = mul_rn(fma_rn(R(4), mid.ex, lo.ex) + hi.ex, k72);
+  gr[1] = mul_rn(fma_rn(R(4), mid.ey, lo.ey) + hi.ey, k72);
+  gr[2] = mul_rn(hi.sm - lo.sm, k72);
+}
 template <typename R, bool WALLFREE>
 __device__ __forceinline__ void tile_grad(const R* sp, int c, int SX, int SXY, R gr[3]) {
   const R p0 = sp[c];
-  R gx = R(0), gy = R(0), gz = R(0);
-#pragma unroll
-  for (int dz = -1; dz <= 1; ++dz) {
-    R p[3][3];
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy) {
-#pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        if (dz == 0 && dy == 0 && dx == 0) {
-          p[1][1] = p0;
-          continue;
-        }
-        R v = sp[c + dx + SX * dy + SXY * dz];
-        if constexpr (!WALLFREE) v = (v > R(0.5) * R(PHI_SOLID)) ? p0 : v;
-        p[dy + 1][dx + 1] = v;
-      }
-    }
-    // x differences smoothed over y, y differences smoothed over x
-    const R ex = (p[0][2] - p[0][0]) + (p[2][2] - p[2][0]) + R(4) * (p[1][2] - p[1][0]);
-    const R ey = (p[2][0] - p[0][0]) + (p[2][2] - p[0][2]) + R(4) * (p[2][1] - p[0][1]);
-    if (dz == 0) {
-      gx += R(4) * ex;
-      gy += R(4) * ey;
-    } else {
-      gx += ex;
-      gy += ey;
-      // the plane smoothed over x and y enters the z difference
-      const R sm = (p[0][0] + p[0][2] + R(4) * p[0][1]) + (p[2][0] + p[2][2] + R(4) * p[2][1]) +
-                   R(4) * (p[1][0] + p[1][2] + R(4) * p[1][1]);
-      gz += dz > 0 ? sm : -sm;
-    }
-  }
-  constexpr R k72 = R(1) / R(72);
-  gr[0] = gx * k72;
-  gr[1] = gy * k72;
-  gr[2] = gz * k72;
+  const GradPlane<R> lo = grad_plane<R, WALLFREE, true>(sp, c - SXY, SX, p0);
+  const GradPlane<R> mid = grad_plane<R, WALLFREE, false>(sp, c, SX, p0);
+  const GradPlane<R> hi = grad_plane<R, WALLFREE, true>(sp, c + SXY, SX, p0);
+  grad_from(lo, mid, hi, gr);
 }
+
+// round(v) to an int, half away from zero: v + 0.5 sign(v) towards zero, then
+// truncated (the sum rounded towards zero keeps its integer part).  Not
+// finite: 0.
+__device__ __forceinline__ int iround(float v) { return __float2int_rz(__fadd_rz(v, copysignf(0.5f, v))); }
+__device__ __forceinline__ int iround(double v) { return __double2int_rz(__dadd_rz(v, copysign(0.5, v))); }
 
 // Near-contact scan of one interface node (Eqs. stress_jump, near_cont_force):
 // step along the outward normal n_out = -grad phi/|grad phi| by round(k n_out),
@@ -943,16 +1020,15 @@ __device__ __forceinline__ void tile_grad(const R* sp, int c, int SX, int SXY, R
 // gg = |gr| its gradient.
 template <typename R, bool WALLFREE>
 __device__ __forceinline__ int nc_scan(const R* sp, int c, int SX, int SXY, int K, int x, int y, int z, const Geo& g,
-                                       const Phys& P, const R gr[3], R gg) {
-  const R phi_I = R(P.phi_I);
+                                       R phi_I, const R gr[3], R gg) {
   const R inv = R(-1) / gg;
-  const R no0 = gr[0] * inv, no1 = gr[1] * inv, no2 = gr[2] * inv;
+  // components within [-1, 1] (the clamp also maps a normal that is not a
+  // number into it), so a target lies at most k <= K nodes away on each axis
+  const R no0 = fmax(R(-1), fmin(R(1), gr[0] * inv)), no1 = fmax(R(-1), fmin(R(1), gr[1] * inv)),
+          no2 = fmax(R(-1), fmin(R(1), gr[2] * inv));
 #pragma unroll 1
   for (int k = 1; k <= K; ++k) {
-    // |n_out| = 1, so |d| <= k <= K; the clamp also covers non-finite normals
-    const int dx = max(-k, min(k, (int)round_(R(k) * no0)));
-    const int dy = max(-k, min(k, (int)round_(R(k) * no1)));
-    const int dz = max(-k, min(k, (int)round_(R(k) * no2)));
+    const int dx = iround(R(k) * no0), dy = iround(R(k) * no1), dz = iround(R(k) * no2);
     if constexpr (!WALLFREE) {
       if (g.wx && (x + dx <= 0 || x + dx >= g.nx - 1)) break;
       if (g.wy && (y + dy <= 0 || y + dy >= g.ny - 1)) break;
@@ -970,55 +1046,14 @@ __device__ __forceinline__ int nc_scan(const R* sp, int c, int SX, int SXY, int 
   return 0;
 }
 
-// Near-contact distance of every node of the tile into hs (Layout::NT bytes,
-// 0 for nodes without a partner): queue the tile's interface nodes (|phi| <
-// phi_I; solid nodes hold PHI_SOLID and are never queued) by warp-aggregated
-// appends, then all threads take queue entries in turn, so no lane idles on a
-// bulk node.  The counter was cleared before the staging barrier.  Ends with
-// a barrier.
-template <typename R, int TX, int TY, int TZ, int H, bool WALLFREE>
-__device__ __forceinline__ void nc_tile(const R* sp, const Geo& g, const Phys& P, unsigned char* hs,
-                                        unsigned short* queue, int* count, int x0, int y0, int z0) {
-  using L = Layout<R, TX, TY, TZ, H>;
-  const int tid = threadIdx.y * TX + threadIdx.x;
-  const int lane = tid & 31;
-  const R phi_I = R(P.phi_I);
-  for (int lz = 0; lz < TZ; ++lz) {
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + lz;
-    const bool in = x < g.nx && y < g.ny && z < g.nz;
-    const int o = (lz * TY + threadIdx.y) * TX + threadIdx.x;
-    const int c = (lz + H) * L::SXY + (threadIdx.y + H) * L::SX + (threadIdx.x + L::HX);
-    const bool iface = in && fabs(sp[c]) < phi_I;
-    hs[o] = 0;
-    const unsigned m = __ballot_sync(0xffffffffu, iface);
-    if (m) {
-      const int leader = __ffs(m) - 1;
-      int base = 0;
-      if (lane == leader) base = atomicAdd(count, __popc(m));
-      base = __shfl_sync(0xffffffffu, base, leader);
-      if (iface) queue[base + __popc(m & ((1u << lane) - 1u))] = (unsigned short)o;
-    }
-  }
-  __syncthreads();
-  const int n = *count;
-  for (int q = tid; q < n; q += TX * TY) {
-    const int o = queue[q];
-    const int lx = o % TX, ly = (o / TX) % TY, lz = o / (TX * TY);
-    const int c = (lz + H) * L::SXY + (ly + H) * L::SX + (lx + L::HX);
-    R gr[3];
-    tile_grad<R, WALLFREE>(sp, c, L::SX, L::SXY, gr);
-    const R gg = sqrt_(gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2]);
-    int h = 0;
-    if (gg >= R(NC_GRAD_MIN))
-      h = nc_scan<R, WALLFREE>(sp, c, L::SX, L::SXY, P.K, x0 + lx, y0 + ly, z0 + lz, g, P, gr, gg);
-    hs[o] = (unsigned char)h;
-  }
-  __syncthreads();
-}
-
 // ---------------------------------------------------------------------------
 // the nodes of one tile
 // ---------------------------------------------------------------------------
+template <typename R>
+__device__ __forceinline__ void put_field(const FieldOut& o, int k, size_t N, size_t self, R v) {
+  if (o.slot[k] >= 0) reinterpret_cast<R*>(o.p)[(size_t)o.slot[k] * N + self] = v;
+}
+
 // Send the component populations (a, b) of direction i of the node at
 // accumulator index e0 to the node that pulls them: x + c_i, or the node
 // itself when x + c_i is solid (halfway bounce-back).
@@ -1033,73 +1068,93 @@ __device__ __forceinline__ void send(unsigned long long* sw, int e0, const Nbr& 
 
 // Pull, collide, recolour and store every node of the tile; with WS also
 // send the post-collision component populations to the tile's partial sums.
-// sp holds phi of the tile and its halo (Layout), hs the near-contact
-// distance of each tile node (read when A_h != 0).
-// INL: the near-contact scan of an interface node runs here, between the
-// loads and the sums of its pull, instead of in a separate phase of the tile
-// (same h: the same scan from the same gradient).  zero_acc (non-null): the
-// accumulator two steps ahead, zeroed here node by node.
-template <int ST, int LOADER, bool WS, bool WF, int TX, int TY, int TZ, int H, bool WALLFREE, bool IDX32, bool REG,
-          bool INL = false>
+// sp holds phi of the tile and its halo (Layout), accin the accumulator of the
+// current level (null: the densities come from phi).  The near-contact scan of
+// an interface node runs between the loads and the sums of its pull, while
+// the loads are in flight (EARLY), or before the loads in the tiles whose
+// registers cannot hold a node's raw values through it.
+template <int ST, int LOADER, bool WS, bool WF, int TX, int TY, int TZ, int H, bool WALLFREE, bool IDX32, bool REG, bool EARLY>
 __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O, const InitBuf& init, const Geo& g,
-                                           const Phys& P, const unsigned char* hs,
-                                           typename Store<ST>::R* __restrict__ fields,
+                                           const PhysR<typename Store<ST>::R>& P,
+                                           const FieldOut& fields,
                                            unsigned* __restrict__ status, const typename Store<ST>::R* sp,
                                            unsigned long long* sw, const unsigned long long* __restrict__ accin,
-                                           int x0, int y0, int z0, unsigned long long* __restrict__ zero_acc = nullptr) {
+                                           int x0, int y0, int z0) {
   using R = typename Store<ST>::R;
   using L = Layout<R, TX, TY, TZ, H>;
-  using I = typename std::conditional<IDX32, unsigned, size_t>::type;
+  using E = typename Store<ST>::E;
   const R tau_a = R(P.tau_a), tau_b = R(P.tau_b);
-  const R A2 = R(P.A2), beta = R(P.beta), A_h = R(P.A_h);
-  const I N = (I)g.N;
-  const size_t NF = (size_t)g.N;
-
-  for (int lz = 0; lz < TZ; ++lz) {
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + lz;
-    if (x >= g.nx || y >= g.ny || z >= g.nz) continue;
-    const int self = x + g.nx * (y + g.ny * z);
-    if (zero_acc) Acc<R>::zero(zero_acc, (size_t)self);  // the accumulator two steps ahead
+  const R A2 = R(P.A2), beta = R(P.beta), A_h = R(P.A_h), phi_I = R(P.phi_I);
+  const size_t N = (size_t)g.N, plane = (size_t)g.nx * (size_t)g.ny;
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int x = x0 + tx, y = y0 + ty;
+  if (x >= g.nx || y >= g.ny) return;
+  using PI = PlaneIdx<ST, IDX32>;
+  PI ix;
+  if constexpr (WALLFREE) ix.init(g, x, y);
+  else ix.o[1][1] = PI::at(g, x, y);
+  const auto self_o = ix.o[1][1];
+  const size_t plane_e = Lay<ST>::row(g) * (size_t)g.ny;  // elements of a z plane
+  int c = H * L::SXY + (ty + H) * L::SX + (tx + L::HX);
+  int e0 = L::EXY + (ty + 1) * L::EX + (tx + 1);
+  // gradient planes at z - 1 and z: a wall-free column takes one new plane a node
+  GradPlane<R> glo, gmid;
+  if constexpr (WALLFREE) {
+    glo = grad_plane<R, true, true>(sp, c - L::SXY, L::SX, R(0));
+    gmid = grad_plane<R, true, true>(sp, c, L::SX, R(0));
+  }
+#pragma unroll 1
+  for (int lz = 0; lz < TZ; ++lz, c += L::SXY, e0 += L::EXY) {
+    const int z = z0 + lz;
+    if (z >= g.nz) break;
+    const size_t self = (size_t)z * plane + (size_t)g.nx * (size_t)y + (size_t)x;
     if (!WALLFREE && is_solid(g, x, y, z)) {
       if constexpr (WF) {
-        for (int k = 0; k < NFIELDS; ++k) fields[(size_t)k * NF + self] = R(0);
+        for (int k = 0; k < NFIELDS; ++k) put_field<R>(fields, k, N, self, R(0));
       }
       continue;
     }
     Nbr n;
-    make_nbr(g, x, y, z, n);
+    if constexpr (!WALLFREE || LOADER != LOAD_PULL) make_nbr(g, x, y, z, n);
     R f[Q], rA, rB;
-    const int c = (lz + H) * L::SXY + (threadIdx.y + H) * L::SX + (threadIdx.x + L::HX);
-    const int e0 = (lz + 1) * L::EXY + (threadIdx.y + 1) * L::EX + (threadIdx.x + 1);
+    E ra[Q], rb[Q];
+    auto pull = [&]() {
+      if constexpr (WALLFREE) {
+        const int zs[3] = {z > 0 ? z - 1 : g.nz - 1, z, z + 1 < g.nz ? z + 1 : 0};
+        if constexpr (Store<ST>::MOMENT) pull_plane_moment<ST, IDX32>(S, N, plane, ix, zs, f);
+        else pull_plane<ST, IDX32>(S, g, ix, zs, ra, rb);
+      } else {
+        pull_walled<ST>(S, g, n, (size_t)z * plane_e + self_o, ra, rb, f);
+      }
+    };
+    if constexpr (LOADER == LOAD_PULL && EARLY) pull();
     const R phx = sp[c];
     // colour gradient from the tile; near-contact distance from the scan
-    R gr[3], gg;
-    int h = 0;
-    constexpr bool SPLIT = INL && LOADER == LOAD_PULL && !Store<ST>::MOMENT;
-    if constexpr (SPLIT) {
-      typename Store<ST>::E ra[Q], rb[Q];
-      pull_raw<ST, WALLFREE, IDX32>(S, g, n, self, ra, rb);
-      tile_grad<R, WALLFREE>(sp, c, L::SX, L::SXY, gr);
-      gg = sqrt_(gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2]);
-      if (H > 1 && A_h != R(0) && fabs(phx) < R(P.phi_I) && gg >= R(NC_GRAD_MIN))
-        h = nc_scan<R, WALLFREE>(sp, c, L::SX, L::SXY, P.K, x, y, z, g, P, gr, gg);
-      pull_raw_finish<ST>(ra, rb, f, rA, rB);
+    R gr[3];
+    if constexpr (WALLFREE) {
+      const GradPlane<R> ghi = grad_plane<R, true, true>(sp, c + L::SXY, L::SX, R(0));
+      grad_from(glo, gmid, ghi, gr);
+      glo = gmid;
+      gmid = ghi;
+    } else {
+      tile_grad<R, false>(sp, c, L::SX, L::SXY, gr);
     }
-    if constexpr (SPLIT && Store<ST>::TWOSET) {
-      // pulled and summed above
-    } else if constexpr (LOADER == LOAD_PULL) {
-      if constexpr (Store<ST>::TWOSET) {
-        pull_fast<ST, WALLFREE, IDX32, false>(S, g, n, self, f, rA, rB);
-      } else {
+    const R gg = sqrt_(gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2]);
+    int h = 0;
+    if (H > 1 && A_h != R(0) && fabs(phx) < phi_I && gg >= R(NC_GRAD_MIN))
+      h = nc_scan<R, WALLFREE>(sp, c, L::SX, L::SXY, P.K, x, y, z, g, phi_I, gr, gg);
+    if constexpr (LOADER == LOAD_PULL) {
+      if constexpr (!EARLY) pull();
+      if constexpr (!Store<ST>::MOMENT) pull_finish<ST>(ra, rb, f, rA, rB);
+      if constexpr (!Store<ST>::TWOSET) {
         // single set: rhoA of the node is the sum the senders accumulated
         // (what a pull of the rebuilt f^A_i gives), so the neighbours' colour
         // scalars need not be read
-        if constexpr (!SPLIT) pull_fast<ST, WALLFREE, IDX32, true>(S, g, n, self, f, rA, rB);
         R rt = R(0);
 #pragma unroll
         for (int i = 0; i < Q; ++i) rt += f[i];
         if (accin) {
-          Acc<R>::densities(accin, (size_t)self, rA, rB);
+          Acc<R>::densities(accin, self, rA, rB);
         } else {  // phi given as an array: split the pulled total by it
           rA = R(0.5) * rt * (R(1) + phx);
         }
@@ -1119,19 +1174,6 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
       if (cx(p)) j0 += R(cx(p)) * d;
       if (cy(p)) j1 += R(cy(p)) * d;
       if (cz(p)) j2 += R(cz(p)) * d;
-    }
-
-    if constexpr (!SPLIT) {
-      tile_grad<R, WALLFREE>(sp, c, L::SX, L::SXY, gr);
-      gg = sqrt_(gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2]);
-      if (H > 1 && A_h != R(0)) {
-        if constexpr (INL) {
-          if (fabs(phx) < R(P.phi_I) && gg >= R(NC_GRAD_MIN))
-            h = nc_scan<R, WALLFREE>(sp, c, L::SX, L::SXY, P.K, x, y, z, g, P, gr, gg);
-        } else {
-          h = hs[(lz * TY + threadIdx.y) * TX + threadIdx.x];
-        }
-      }
     }
     R Ahh = R(0);
     if (H > 1 && A_h != R(0)) {
@@ -1165,20 +1207,20 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
     if (!(rho > R(0) && rho < R(Acc<R>::RHO_MAX))) atomicOr(status, 1u);
 
     if constexpr (WF) {
-      fields[(size_t)F_PHI * NF + self] = phx;
-      fields[(size_t)F_RHO * NF + self] = rho;
-      fields[(size_t)F_UX * NF + self] = u0;
-      fields[(size_t)F_UY * NF + self] = u1;
-      fields[(size_t)F_UZ * NF + self] = u2;
-      fields[(size_t)F_RHOA * NF + self] = rA;
-      fields[(size_t)F_RHOB * NF + self] = rB;
-      fields[(size_t)F_FRX * NF + self] = Fr0;
-      fields[(size_t)F_FRY * NF + self] = Fr1;
-      fields[(size_t)F_FRZ * NF + self] = Fr2;
-      fields[(size_t)F_H * NF + self] = R(h);
-      fields[(size_t)F_GX * NF + self] = gr[0];
-      fields[(size_t)F_GY * NF + self] = gr[1];
-      fields[(size_t)F_GZ * NF + self] = gr[2];
+      put_field<R>(fields, F_PHI, N, self, phx);
+      put_field<R>(fields, F_RHO, N, self, rho);
+      put_field<R>(fields, F_UX, N, self, u0);
+      put_field<R>(fields, F_UY, N, self, u1);
+      put_field<R>(fields, F_UZ, N, self, u2);
+      put_field<R>(fields, F_RHOA, N, self, rA);
+      put_field<R>(fields, F_RHOB, N, self, rB);
+      put_field<R>(fields, F_FRX, N, self, Fr0);
+      put_field<R>(fields, F_FRY, N, self, Fr1);
+      put_field<R>(fields, F_FRZ, N, self, Fr2);
+      put_field<R>(fields, F_H, N, self, R(h));
+      put_field<R>(fields, F_GX, N, self, gr[0]);
+      put_field<R>(fields, F_GY, N, self, gr[1]);
+      put_field<R>(fields, F_GZ, N, self, gr[2]);
     }
     if constexpr (!WS) continue;
 
@@ -1205,10 +1247,16 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
     const R gn = gg > R(NORMAL_FLOOR) ? gg : R(NORMAL_FLOOR);
     const R segamp = beta * rA * rB * irho / gn;
     const R sA = rA * irho;
-    // f* = keep f + w_i (alpha + beta.c + c.Gamma.c) (QForm): equilibrium (Eq.
-    // disteq), perturbation and Guo source.  BGK relaxes f towards feq: keep f
-    // + omega feq.  The regularised collision (collision == 1) keeps feq and
-    // relaxes the non-equilibrium part projected on Hermite orders 1 and 2,
+    // equilibrium (Eq. disteq) and Guo source split into parts even and odd
+    // under c -> -c: feq = w [rho(1 - 1.5 uu) + 4.5 rho (c.u)^2] + 3 w rho (c.u),
+    // S = guo w [9 (c.u)(c.F) - 3 u.F] + 3 guo w (c.F)
+    const R r0 = rho * (R(1) - R(1.5) * uu);
+    const R r45 = R(4.5) * rho;
+    const R r3 = R(3) * rho;
+    const R g9 = R(9) * guo, g3 = R(3) * guo, gm3uF = -R(3) * guo * uF;
+    // BGK relaxes f towards feq: keep f + omega feq.  The regularised
+    // collision (collision == 1) keeps feq and relaxes the non-equilibrium
+    // part projected on Hermite orders 1 and 2:
     //   feq + keep w [3 c.J + 4.5 (c.Pi.c - tr(Pi)/3)],
     //   J = j - rho u = -F/2,  Pi = sum_i c c f_i - rho (u u + I/3).
     constexpr bool reg = REG;
@@ -1234,36 +1282,6 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
       Pyz -= rho * u1 * u2;
       trP = Pxx + Pyy + Pzz;
     }
-    QForm<R> qf;
-    {
-      const R r45 = R(4.5) * wf * rho, r3 = R(3) * wf * rho, hg9 = R(4.5) * guo;
-      const R bF = reg ? R(3) * guo - R(1.5) * keep : R(3) * guo;
-      // Gamma = r45 u u + hg9 (u F + F u) + A2ig g g - A2g I: each row a times (u, F, g) of b
-      const R v0 = fma_rn(r45, u0, mul_rn(hg9, F0)), v1 = fma_rn(r45, u1, mul_rn(hg9, F1)),
-              v2 = fma_rn(r45, u2, mul_rn(hg9, F2));
-      const R k0 = mul_rn(hg9, u0), k1 = mul_rn(hg9, u1), k2 = mul_rn(hg9, u2);
-      const R m0 = mul_rn(A2ig, gr[0]), m1 = mul_rn(A2ig, gr[1]), m2 = mul_rn(A2ig, gr[2]);
-      qf.a = fma_rn(R(-3) * guo, uF, fma_rn(R(2) / R(3), A2g, wf * rho * (R(1) - R(1.5) * uu)));
-      qf.bx = fma_rn(r3, u0, mul_rn(bF, F0));
-      qf.by = fma_rn(r3, u1, mul_rn(bF, F1));
-      qf.bz = fma_rn(r3, u2, mul_rn(bF, F2));
-      qf.xx = fma_rn(v0, u0, fma_rn(k0, F0, fma_rn(m0, gr[0], -A2g)));
-      qf.yy = fma_rn(v1, u1, fma_rn(k1, F1, fma_rn(m1, gr[1], -A2g)));
-      qf.zz = fma_rn(v2, u2, fma_rn(k2, F2, fma_rn(m2, gr[2], -A2g)));
-      qf.xy = R(2) * fma_rn(v0, u1, fma_rn(k0, F1, mul_rn(m0, gr[1])));
-      qf.xz = R(2) * fma_rn(v0, u2, fma_rn(k0, F2, mul_rn(m0, gr[2])));
-      qf.yz = R(2) * fma_rn(v1, u2, fma_rn(k1, F2, mul_rn(m1, gr[2])));
-      if constexpr (reg) {
-        const R kP = keep * R(4.5);
-        qf.a = fma_rn(R(-1.5) * keep, trP, qf.a);
-        qf.xx = fma_rn(kP, Pxx, qf.xx);
-        qf.yy = fma_rn(kP, Pyy, qf.yy);
-        qf.zz = fma_rn(kP, Pzz, qf.zz);
-        qf.xy = fma_rn(R(2) * kP, Pxy, qf.xy);
-        qf.xz = fma_rn(R(2) * kP, Pxz, qf.xz);
-        qf.yz = fma_rn(R(2) * kP, Pyz, qf.yz);
-      }
-    }
     // colour scalars of the single-set storages, as stored
     float4 svo = make_float4(0.f, 0.f, 0.f, 0.f);
     if constexpr (!Store<ST>::TWOSET) {
@@ -1271,14 +1289,25 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
       O.sv[self] = svo;
     }
     if constexpr (Store<ST>::MOMENT) {
-      // the form itself is what this storage keeps (the host admits it with the
-      // regularised collision only; Eqs. disteq, distnoneq, LBpostmom)
-      const float4 qa = make_float4(qf.a, qf.bx, qf.by, qf.bz);
-      const float4 qb = make_float4(qf.xx, qf.yy, qf.zz, qf.xy);
-      const float2 qc = make_float2(qf.xz, qf.yz);
+      // f*_i = w_i (alpha + beta.c_i + c_i.Gamma.c_i): the equilibrium, the
+      // relaxed Hermite orders 1-2, the perturbation (B_i = w_i (|c_i|^2 - 2/3))
+      // and the Guo source below are each w_i times a quadratic form in c_i
+      // (Eqs. disteq, distnoneq, LBpostmom; the host admits this storage with
+      // the regularised collision only)
+      const R kP = keep * R(4.5), hg9 = R(0.5) * g9;
+      const R bF = g3 - R(1.5) * keep;  // beta = 3 rho u + (3 guo - 1.5 keep) F
+      const float4 qa = make_float4(r0 + gm3uF - R(1.5) * keep * trP + (R(2) / R(3)) * A2g, r3 * u0 + bF * F0,
+                                    r3 * u1 + bF * F1, r3 * u2 + bF * F2);
+      const float4 qb = make_float4(r45 * u0 * u0 + g9 * u0 * F0 + A2ig * gr[0] * gr[0] - A2g + kP * Pxx,
+                                    r45 * u1 * u1 + g9 * u1 * F1 + A2ig * gr[1] * gr[1] - A2g + kP * Pyy,
+                                    r45 * u2 * u2 + g9 * u2 * F2 + A2ig * gr[2] * gr[2] - A2g + kP * Pzz,
+                                    R(2) * (r45 * u0 * u1 + hg9 * (u0 * F1 + F0 * u1) + A2ig * gr[0] * gr[1] + kP * Pxy));
+      const float2 qc =
+          make_float2(R(2) * (r45 * u0 * u2 + hg9 * (u0 * F2 + F0 * u2) + A2ig * gr[0] * gr[2] + kP * Pxz),
+                      R(2) * (r45 * u1 * u2 + hg9 * (u1 * F2 + F1 * u2) + A2ig * gr[1] * gr[2] + kP * Pyz));
       reinterpret_cast<float4*>(O.f)[self] = qa;
-      reinterpret_cast<float4*>(O.f + (I)4 * N)[self] = qb;
-      reinterpret_cast<float2*>(O.f + (I)8 * N)[self] = qc;
+      reinterpret_cast<float4*>(O.f + 4 * N)[self] = qb;
+      reinterpret_cast<float2*>(O.f + 8 * N)[self] = qc;
       // what the neighbours will pull: the quadratic form at each c_i
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
@@ -1288,171 +1317,118 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
       }
       continue;
     }
+    E* op = O.f + ((size_t)z * plane_e + self_o);
     {  // rest direction
-      const R wa = mul_rn(wgt<R>(REST), qf.a);
-      const R fs = reg ? wa : fma_rn(keep, f[REST], wa);
+      const R W = wgt<R>(REST);
+      const R rel = reg ? R(-1.5) * W * trP : f[REST];
+      const R fs = keep * rel + wf * W * r0 - bweight<R>(REST) * A2g + W * gm3uF;
       if constexpr (Store<ST>::TWOSET) {
-        const R fa = mul_rn(sA, fs);
+        const R fa = sA * fs;
         const R fb = fs - fa;
-        O.f[(I)REST * N + (I)self] = encode<ST>(fa, REST);
-        O.f[(I)(Q + REST) * N + (I)self] = encode<ST>(fb, REST);
+        op[REST * BLK] = encode<ST>(fa, REST);
+        op[(Q + REST) * BLK] = encode<ST>(fb, REST);
         send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, REST, fa, fb);
       } else {
         const typename Store<ST>::E enc = encode<ST>(fs, REST);
-        O.f[(I)REST * N + (I)self] = enc;
+        op[REST * BLK] = enc;
         R va, vb;
         colour_split<R, false>(decode<ST>(enc, REST), svo, REST, false, va, vb);
         send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, REST, va, vb);
       }
     }
-    auto pairs = [&](auto cls) {
-      constexpr int CLS = decltype(cls)::value;
-      const QClass<R, CLS> qc(qf);
-      // segregation amplitude of the class: w/|c| beta rhoA rhoB/rho n
-      constexpr R ks = CLS == 1 ? wgt<R>(4) * inv_norm<R>(4) : CLS == 2 ? wgt<R>(1) * inv_norm<R>(1) : wgt<R>(0) * inv_norm<R>(0);
-      const R kseg = mul_rn(ks, segamp);
-      const R g0 = mul_rn(kseg, gr[0]), g1 = mul_rn(kseg, gr[1]), g2 = mul_rn(kseg, gr[2]);
 #pragma unroll
-      for (int p = 0; p < REST; ++p) {
-        if (cnorm2(p) != CLS) continue;
-        const int q = opp(p);
-        const R even = qc.even(p), odd = qc.odd(p);
-        R fsp = even + odd, fsq = even - odd;
-        if constexpr (!reg) {
-          fsp = fma_rn(keep, f[p], fsp);
-          fsq = fma_rn(keep, f[q], fsq);
-        }
-        if constexpr (Store<ST>::TWOSET) {
-          const R seg = QClass<R, CLS>::along(p, g0, g1, g2);
-          const R fap = fma_rn(sA, fsp, seg);
-          const R faq = fma_rn(sA, fsq, -seg);
-          const R fbp = fsp - fap, fbq = fsq - faq;
-          O.f[(I)p * N + (I)self] = encode<ST>(fap, p);
-          O.f[(I)q * N + (I)self] = encode<ST>(faq, q);
-          O.f[(I)(Q + p) * N + (I)self] = encode<ST>(fbp, p);
-          O.f[(I)(Q + q) * N + (I)self] = encode<ST>(fbq, q);
-          send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, p, fap, fbp);
-          send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, q, faq, fbq);
-        } else {
-          const typename Store<ST>::E ep = encode<ST>(fsp, p), eq = encode<ST>(fsq, q);
-          O.f[(I)p * N + (I)self] = ep;
-          O.f[(I)q * N + (I)self] = eq;
-          // colour_split of p and of its opposite q: c_q.v = -(c_p.v) exactly,
-          // so the segregation term is formed once and negated (bit for bit
-          // what colour_split gives for q)
-          R cv = R(0);
-          if (cx(p)) cv += R(cx(p)) * R(svo.y);
-          if (cy(p)) cv += R(cy(p)) * R(svo.z);
-          if (cz(p)) cv += R(cz(p)) * R(svo.w);
-          const R seg = mul_rn(wgt<R>(p) * inv_norm<R>(p), cv);
-          const R dp = decode<ST>(ep, p), dq = decode<ST>(eq, q);
-          const R vap = fma_rn(R(svo.x), dp, seg), vaq = fma_rn(R(svo.x), dq, -seg);
-          send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, p, vap, dp - vap);
-          send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, q, vaq, dq - vaq);
-        }
+    for (int p = 0; p < REST; ++p) {
+      const int q = opp(p);
+      const R W = wgt<R>(p);
+      R cu = R(0), cF = R(0), cg = R(0);
+      if (cx(p)) { cu += R(cx(p)) * u0; cF += R(cx(p)) * F0; cg += R(cx(p)) * gr[0]; }
+      if (cy(p)) { cu += R(cy(p)) * u1; cF += R(cy(p)) * F1; cg += R(cy(p)) * gr[1]; }
+      if (cz(p)) { cu += R(cz(p)) * u2; cF += R(cz(p)) * F2; cg += R(cz(p)) * gr[2]; }
+      R even = W * (wf * (r0 + r45 * cu * cu) + g9 * cu * cF + gm3uF + A2ig * cg * cg) - bweight<R>(p) * A2g;
+      R odd = W * (wf * r3 * cu + g3 * cF);
+      R bp = f[p], bq = f[q];
+      if constexpr (reg) {
+        // c.Pi.c and c.J = -(c.F)/2 for this pair's velocity
+        R cpc = R(0);
+        if (cx(p)) cpc += Pxx;
+        if (cy(p)) cpc += Pyy;
+        if (cz(p)) cpc += Pzz;
+        if (cx(p) && cy(p)) cpc += R(2 * cx(p) * cy(p)) * Pxy;
+        if (cx(p) && cz(p)) cpc += R(2 * cx(p) * cz(p)) * Pxz;
+        if (cy(p) && cz(p)) cpc += R(2 * cy(p) * cz(p)) * Pyz;
+        even += keep * W * R(4.5) * (cpc - trP * (R(1) / R(3)));
+        odd += keep * W * R(-1.5) * cF;
+        bp = R(0);
+        bq = R(0);
       }
-    };
-    pairs(std::integral_constant<int, 1>{});
-    pairs(std::integral_constant<int, 2>{});
-    pairs(std::integral_constant<int, 3>{});
+      const R fsp = keep * bp + even + odd;
+      const R fsq = keep * bq + even - odd;
+      if constexpr (Store<ST>::TWOSET) {
+        const R seg = segamp * W * inv_norm<R>(p) * cg;
+        const R fap = sA * fsp + seg;
+        const R faq = sA * fsq - seg;
+        const R fbp = fsp - fap, fbq = fsq - faq;
+        op[p * BLK] = encode<ST>(fap, p);
+        op[q * BLK] = encode<ST>(faq, q);
+        op[(Q + p) * BLK] = encode<ST>(fbp, p);
+        op[(Q + q) * BLK] = encode<ST>(fbq, q);
+        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, p, fap, fbp);
+        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, q, faq, fbq);
+      } else {
+        const typename Store<ST>::E ep = encode<ST>(fsp, p), eq = encode<ST>(fsq, q);
+        op[p * BLK] = ep;
+        op[q * BLK] = eq;
+        // colour_split of p and of its opposite q: c_q.v = -(c_p.v) exactly,
+        // so the segregation term is formed once and negated (bit for bit
+        // what colour_split gives for q)
+        R cv = R(0);
+        if (cx(p)) cv += R(cx(p)) * R(svo.y);
+        if (cy(p)) cv += R(cy(p)) * R(svo.z);
+        if (cz(p)) cv += R(cz(p)) * R(svo.w);
+        const R seg = mul_rn(W * inv_norm<R>(p), cv);
+        const R dp = decode<ST>(ep, p), dq = decode<ST>(eq, q);
+        const R vap = fma_rn(R(svo.x), dp, seg), vaq = fma_rn(R(svo.x), dq, -seg);
+        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, p, vap, dp - vap);
+        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, q, vaq, dq - vaq);
+      }
+    }
   }
 }
 
 // Add the tile's partial sums (tile plus a one-node ring) to the global
 // accumulator; entries beyond a wall are never sent to, periodic axes wrap.
-template <typename R, int TX, int TY, int TZ, int H>
+// A warp takes whole rows of the ring (its y and z are then the warp's), the
+// two columns past the 32 lanes come last.
+template <typename R, int TX, int TY, int TZ, typename L>
 __device__ __forceinline__ void flush_partials(const unsigned long long* sw, unsigned long long* __restrict__ acc,
                                                const Geo& g, int x0, int y0, int z0) {
-  using L = Layout<R, TX, TY, TZ, H>;
-  for (int e = threadIdx.y * TX + threadIdx.x; e < L::E; e += TX * TY) {
+  static_assert(TX == 32, "one lane per column");
+  constexpr int ROWS = L::EY * L::EZ;
+  // node of ring column ex, or -1 beyond a wall (pad_source also drops the
+  // solid layers, whose sums are zero)
+  auto row_base = [&](int row) -> long long {
+    const int ez = row / L::EY, ey = row - ez * L::EY;
+    const int gy = pad_source(y0 + ey, 1, g.ny, g.wy), gz = pad_source(z0 + ez, 1, g.nz, g.wz);
+    return gy < 0 || gz < 0 ? -1 : (long long)g.nx * ((long long)gy + (long long)g.ny * gz);
+  };
+  const int gx = pad_source(x0 + (int)threadIdx.x, 1, g.nx, g.wx);
+  for (int row = threadIdx.y; row < ROWS; row += TY) {
+    const int e = row * L::EX + (int)threadIdx.x;
+    const long long rb = row_base(row);
+    if (rb >= 0 && gx >= 0 && !Acc<R>::shared_zero(sw, L::E, e)) Acc<R>::flush_shared(acc, (size_t)(rb + gx), sw, L::E, e);
+  }
+  for (int k = threadIdx.y * TX + threadIdx.x; k < 2 * ROWS; k += TX * TY) {
+    const int row = k >> 1, ex = TX + (k & 1), e = row * L::EX + ex;
     if (Acc<R>::shared_zero(sw, L::E, e)) continue;
-    const int ex = e % L::EX, ey = (e / L::EX) % L::EY, ez = e / L::EXY;
-    int gx = x0 - 1 + ex, gy = y0 - 1 + ey, gz = z0 - 1 + ez;
-    if ((unsigned)gx >= (unsigned)g.nx) {
-      if (g.wx) continue;
-      gx = ((gx % g.nx) + g.nx) % g.nx;
-    }
-    if ((unsigned)gy >= (unsigned)g.ny) {
-      if (g.wy) continue;
-      gy = ((gy % g.ny) + g.ny) % g.ny;
-    }
-    if ((unsigned)gz >= (unsigned)g.nz) {
-      if (g.wz) continue;
-      gz = ((gz % g.nz) + g.nz) % g.nz;
-    }
-    Acc<R>::flush_shared(acc, (size_t)gx + (size_t)g.nx * ((size_t)gy + (size_t)g.ny * gz), sw, L::E, e);
+    const long long rb = row_base(row);
+    const int gt = pad_source(x0 + ex, 1, g.nx, g.wx);
+    if (rb >= 0 && gt >= 0) Acc<R>::flush_shared(acc, (size_t)(rb + gt), sw, L::E, e);
   }
 }
 
 // ---------------------------------------------------------------------------
 // Shan-Chen multicomponent model (Sec. III.C.3, lattice pseudo-potential)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float sc_psi(float r, float psi0) { return psi0 * (1.0f - expf(-r / psi0)); }
-__device__ __forceinline__ double sc_psi(double r, double psi0) { return psi0 * (1.0 - exp(-r / psi0)); }
-
-// Stage phi, psi_A and psi_B (pseudo-potential psi(rho) = rho_0 (1 -
-// exp(-rho/rho_0)) of each component) of the tile plus a one-node halo; solid
-// and beyond-wall nodes get the marker.  The component densities come from
-// the accumulator of the step before, or (first step) from the initial
-// fields: rho_k = rho (1 +- phi)/2.  No barrier.
-template <typename R, bool FROM_ACC, int TX, int TY, int TZ>
-__device__ __forceinline__ void stage_sc(const PhiSrc& src, const InitBuf& init, const Geo& g, R psi0, R* sp,
-                                         R* spa, R* spb, int x0, int y0, int z0) {
-  using L = Layout<R, TX, TY, TZ, 1, 3>;
-  for (int q = threadIdx.y * TX + threadIdx.x; q < L::NS; q += TX * TY) {
-    const int lx = q % L::SX, row = q / L::SX;
-    const int ly = row % L::SY, lz = row / L::SY;
-    int gx = x0 - 1 + lx, gy = y0 - 1 + ly, gz = z0 - 1 + lz;
-    bool solid = false;
-    if (g.wx) solid |= (gx <= 0 || gx >= g.nx - 1);
-    else if ((unsigned)gx >= (unsigned)g.nx) gx = ((gx % g.nx) + g.nx) % g.nx;
-    if (g.wy) solid |= (gy <= 0 || gy >= g.ny - 1);
-    else if ((unsigned)gy >= (unsigned)g.ny) gy = ((gy % g.ny) + g.ny) % g.ny;
-    if (g.wz) solid |= (gz <= 0 || gz >= g.nz - 1);
-    else if ((unsigned)gz >= (unsigned)g.nz) gz = ((gz % g.nz) + g.nz) % g.nz;
-    if (solid) {
-      sp[q] = spa[q] = spb[q] = R(PHI_SOLID);
-      continue;
-    }
-    const size_t node = (size_t)gx + (size_t)g.nx * ((size_t)gy + (size_t)g.ny * gz);
-    R ra, rb;
-    if constexpr (FROM_ACC) {
-      Acc<R>::densities(src.acc, node, ra, rb);
-    } else {
-      const R ph = reinterpret_cast<const R*>(src.phi)[node];
-      const R rho = init.rho ? R(init.rho[node]) : R(1);
-      ra = rho * (R(1) + ph) * R(0.5);
-      rb = rho * (R(1) - ph) * R(0.5);
-    }
-    sp[q] = (ra - rb) / (ra + rb);
-    spa[q] = sc_psi(ra, psi0);
-    spb[q] = sc_psi(rb, psi0);
-  }
-}
-
-// Pull of both component sets (two-set storages): f^A_i, f^B_i and their sums.
-template <int ST, bool WALLFREE, bool IDX32>
-__device__ __forceinline__ void pull_comp(const View<ST>& S, const Geo& g, const Nbr& n, int self,
-                                          typename Store<ST>::R fa[Q], typename Store<ST>::R fb[Q],
-                                          typename Store<ST>::R& rA, typename Store<ST>::R& rB) {
-  using R = typename Store<ST>::R;
-  using I = typename std::conditional<IDX32, unsigned, size_t>::type;
-  const I N = (I)g.N;
-  rA = R(0);
-  rB = R(0);
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const int a = 1 - cx(i), b = 1 - cy(i), c = 1 - cz(i);
-    const bool bb = WALLFREE ? false : (n.sx[a] | n.sy[b] | n.sz[c]);
-    const I src = bb ? (I)self : (I)n.xs[a] + (I)g.nx * ((I)n.ys[b] + (I)g.ny * (I)n.zs[c]);
-    const I dir = bb ? (I)opp(i) : (I)i;
-    fa[i] = decode<ST>(S.f[dir * N + src], i);
-    fb[i] = decode<ST>(S.f[((I)Q + dir) * N + src], i);
-    rA += fa[i];
-    rB += fb[i];
-  }
-}
-
 // The nodes of one tile in the Shan-Chen model: pull both components, the
 // pseudo-potential forces F_A = -psi_A G sum_i w_i psi_B(x + c_i) c_i (= -psi_A
 // (G/3) times the stencil gradient of psi_B; a solid neighbour contributes the
@@ -1461,48 +1437,88 @@ __device__ __forceinline__ void pull_comp(const View<ST>& S, const Geo& g, const
 // towards f^eq(rho_k, u') with the Guo source of F_k, store and send.
 template <int ST, int LOADER, bool WS, bool WF, int TX, int TY, int TZ, bool WALLFREE, bool IDX32>
 __device__ __forceinline__ void step_nodes_sc(const View<ST>& S, const View<ST>& O, const InitBuf& init,
-                                              const Geo& g, const Phys& P, typename Store<ST>::R* __restrict__ fields,
+                                              const Geo& g, const PhysR<typename Store<ST>::R>& P,
+                                              const FieldOut& fields,
                                               unsigned* __restrict__ status, const typename Store<ST>::R* sp,
                                               const typename Store<ST>::R* spa, const typename Store<ST>::R* spb,
                                               unsigned long long* sw, int x0, int y0, int z0) {
   using R = typename Store<ST>::R;
-  using L = Layout<R, TX, TY, TZ, 1, 3>;
-  using I = typename std::conditional<IDX32, unsigned, size_t>::type;
-  const I N = (I)g.N;
-  const size_t NF = (size_t)g.N;
+  using L = Layout<R, TX, TY, TZ, 1, WF ? 3 : 2>;
+  const size_t N = (size_t)g.N, plane = (size_t)g.nx * (size_t)g.ny;
   const R wa = R(1) / R(P.tau_a), wb = R(1) / R(P.tau_b);
   const R G3 = R(P.G) / R(3);
-  for (int lz = 0; lz < TZ; ++lz) {
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + lz;
-    if (x >= g.nx || y >= g.ny || z >= g.nz) continue;
-    const int self = x + g.nx * (y + g.ny * z);
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int x = x0 + tx, y = y0 + ty;
+  if (x >= g.nx || y >= g.ny) return;
+  using PI = PlaneIdx<ST, IDX32>;
+  PI ix;
+  if constexpr (WALLFREE) ix.init(g, x, y);
+  else ix.o[1][1] = PI::at(g, x, y);
+  const auto self_o = ix.o[1][1];
+  const size_t plane_e = Lay<ST>::row(g) * (size_t)g.ny;  // elements of a z plane
+  int c = L::SXY + (ty + 1) * L::SX + (tx + L::HX);
+  int e0 = L::EXY + (ty + 1) * L::EX + (tx + 1);
+  GradPlane<R> alo, amid, blo, bmid;
+  if constexpr (WALLFREE) {
+    alo = grad_plane<R, true, true>(spa, c - L::SXY, L::SX, R(0));
+    amid = grad_plane<R, true, true>(spa, c, L::SX, R(0));
+    blo = grad_plane<R, true, true>(spb, c - L::SXY, L::SX, R(0));
+    bmid = grad_plane<R, true, true>(spb, c, L::SX, R(0));
+  }
+#pragma unroll 1
+  for (int lz = 0; lz < TZ; ++lz, c += L::SXY, e0 += L::EXY) {
+    const int z = z0 + lz;
+    if (z >= g.nz) break;
+    const size_t self = (size_t)z * plane + (size_t)g.nx * (size_t)y + (size_t)x;
     if (!WALLFREE && is_solid(g, x, y, z)) {
       if constexpr (WF) {
-        for (int k = 0; k < NFIELDS; ++k) fields[(size_t)k * NF + self] = R(0);
+        for (int k = 0; k < NFIELDS; ++k) put_field<R>(fields, k, N, self, R(0));
       }
       continue;
     }
     Nbr n;
-    make_nbr(g, x, y, z, n);
-    R fa[Q], fb[Q], rA, rB;
+    if constexpr (!WALLFREE || LOADER != LOAD_PULL) make_nbr(g, x, y, z, n);
+    R fa[Q], fb[Q], rA = R(0), rB = R(0);
+    if constexpr (LOADER == LOAD_PULL) {  // two-set storages: the stored values are the populations
+      if constexpr (WALLFREE) {
+        const int zs[3] = {z > 0 ? z - 1 : g.nz - 1, z, z + 1 < g.nz ? z + 1 : 0};
+        pull_plane<ST, IDX32>(S, g, ix, zs, fa, fb);
+      } else {
+        pull_walled<ST>(S, g, n, (size_t)z * plane_e + self_o, fa, fb, nullptr);
+      }
+    }
+    R gA[3], gB[3], gphi[3];
+    if constexpr (WALLFREE) {
+      const GradPlane<R> ahi = grad_plane<R, true, true>(spa, c + L::SXY, L::SX, R(0));
+      grad_from(alo, amid, ahi, gA);
+      alo = amid;
+      amid = ahi;
+      const GradPlane<R> bhi = grad_plane<R, true, true>(spb, c + L::SXY, L::SX, R(0));
+      grad_from(blo, bmid, bhi, gB);
+      blo = bmid;
+      bmid = bhi;
+    } else {
+      tile_grad<R, false>(spa, c, L::SX, L::SXY, gA);
+      tile_grad<R, false>(spb, c, L::SX, L::SXY, gB);
+    }
     if constexpr (LOADER == LOAD_PULL) {
-      pull_comp<ST, WALLFREE, IDX32>(S, g, n, self, fa, fb, rA, rB);
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        rA += fa[i];
+        rB += fb[i];
+      }
     } else {
       R f[Q];
       fields_node<R, true>(init, g, P, n, (long long)self, f, rA, rB, fa, fb);
     }
-    const int c = (lz + 1) * L::SXY + (threadIdx.y + 1) * L::SX + (threadIdx.x + 1);
-    const int e0 = (lz + 1) * L::EXY + (threadIdx.y + 1) * L::EX + (threadIdx.x + 1);
     R jA[3] = {R(0), R(0), R(0)}, jB[3] = {R(0), R(0), R(0)};
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      if (cx(i)) { jA[0] += R(cx(i)) * fa[i]; jB[0] += R(cx(i)) * fb[i]; }
-      if (cy(i)) { jA[1] += R(cy(i)) * fa[i]; jB[1] += R(cy(i)) * fb[i]; }
-      if (cz(i)) { jA[2] += R(cz(i)) * fa[i]; jB[2] += R(cz(i)) * fb[i]; }
+    for (int i = 0; i < REST; ++i) {  // opposite pairs
+      const R da = fa[i] - fa[opp(i)], db = fb[i] - fb[opp(i)];
+      if (cx(i)) { jA[0] += R(cx(i)) * da; jB[0] += R(cx(i)) * db; }
+      if (cy(i)) { jA[1] += R(cy(i)) * da; jB[1] += R(cy(i)) * db; }
+      if (cz(i)) { jA[2] += R(cz(i)) * da; jB[2] += R(cz(i)) * db; }
     }
-    R gA[3], gB[3], gphi[3];
-    tile_grad<R, WALLFREE>(spa, c, L::SX, L::SXY, gA);
-    tile_grad<R, WALLFREE>(spb, c, L::SX, L::SXY, gB);
     R FA[3], FB[3], Fs[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -1530,20 +1546,20 @@ __device__ __forceinline__ void step_nodes_sc(const View<ST>& S, const View<ST>&
     if constexpr (WF) {
       tile_grad<R, WALLFREE>(sp, c, L::SX, L::SXY, gphi);
       const R irho = R(1) / rho;
-      fields[(size_t)F_PHI * NF + self] = sp[c];
-      fields[(size_t)F_RHO * NF + self] = rho;
-      fields[(size_t)F_UX * NF + self] = (jA[0] + jB[0] + R(0.5) * (FA[0] + FB[0])) * irho;
-      fields[(size_t)F_UY * NF + self] = (jA[1] + jB[1] + R(0.5) * (FA[1] + FB[1])) * irho;
-      fields[(size_t)F_UZ * NF + self] = (jA[2] + jB[2] + R(0.5) * (FA[2] + FB[2])) * irho;
-      fields[(size_t)F_RHOA * NF + self] = rA;
-      fields[(size_t)F_RHOB * NF + self] = rB;
-      fields[(size_t)F_FRX * NF + self] = Fs[0];
-      fields[(size_t)F_FRY * NF + self] = Fs[1];
-      fields[(size_t)F_FRZ * NF + self] = Fs[2];
-      fields[(size_t)F_H * NF + self] = R(0);
-      fields[(size_t)F_GX * NF + self] = gphi[0];
-      fields[(size_t)F_GY * NF + self] = gphi[1];
-      fields[(size_t)F_GZ * NF + self] = gphi[2];
+      put_field<R>(fields, F_PHI, N, self, sp[c]);
+      put_field<R>(fields, F_RHO, N, self, rho);
+      put_field<R>(fields, F_UX, N, self, (jA[0] + jB[0] + R(0.5) * (FA[0] + FB[0])) * irho);
+      put_field<R>(fields, F_UY, N, self, (jA[1] + jB[1] + R(0.5) * (FA[1] + FB[1])) * irho);
+      put_field<R>(fields, F_UZ, N, self, (jA[2] + jB[2] + R(0.5) * (FA[2] + FB[2])) * irho);
+      put_field<R>(fields, F_RHOA, N, self, rA);
+      put_field<R>(fields, F_RHOB, N, self, rB);
+      put_field<R>(fields, F_FRX, N, self, Fs[0]);
+      put_field<R>(fields, F_FRY, N, self, Fs[1]);
+      put_field<R>(fields, F_FRZ, N, self, Fs[2]);
+      put_field<R>(fields, F_H, N, self, R(0));
+      put_field<R>(fields, F_GX, N, self, gphi[0]);
+      put_field<R>(fields, F_GY, N, self, gphi[1]);
+      put_field<R>(fields, F_GZ, N, self, gphi[2]);
     }
     if constexpr (!WS) continue;
     const R uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
@@ -1571,9 +1587,10 @@ __device__ __forceinline__ void step_nodes_sc(const View<ST>& S, const View<ST>&
     };
     const QForm<R> qa = form(wa, rA, FA), qb = form(wb, rB, FB);
     const R ka = R(1) - wa, kb = R(1) - wb;
+    auto* op = O.f + ((size_t)z * plane_e + self_o);
     auto put = [&](int i, R oa, R ob) {
-      O.f[(I)i * N + (I)self] = encode<ST>(oa, i);
-      O.f[(I)(Q + i) * N + (I)self] = encode<ST>(ob, i);
+      op[i * BLK] = encode<ST>(oa, i);
+      op[(Q + i) * BLK] = encode<ST>(ob, i);
       send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, i, oa, ob);
     };
     put(REST, fma_rn(ka, fa[REST], mul_rn(wgt<R>(REST), qa.a)), fma_rn(kb, fb[REST], mul_rn(wgt<R>(REST), qb.a)));
@@ -1595,166 +1612,155 @@ __device__ __forceinline__ void step_nodes_sc(const View<ST>& S, const View<ST>&
   }
 }
 
-// One tile of the Shan-Chen step: clear, stage, step, flush.  Ends with a
-// barrier.
-template <int ST, int LOADER, bool WS, bool WF, int TX, int TY, int TZ, bool IDX32>
-__device__ __forceinline__ void step_tile_sc(const View<ST>& S, const View<ST>& O, const InitBuf& init,
-                                             const PhiSrc& src, const AccBufs& ab, const Geo& g, const Phys& P,
-                                             typename Store<ST>::R* __restrict__ fields,
-                                             unsigned* __restrict__ status, unsigned char* smem, int x0, int y0,
-                                             int z0) {
-  using R = typename Store<ST>::R;
-  using L = Layout<R, TX, TY, TZ, 1, 3>;
-  R* sp = reinterpret_cast<R*>(smem);
-  R* spa = sp + L::NS;
-  R* spb = spa + L::NS;
-  unsigned long long* sw = reinterpret_cast<unsigned long long*>(smem + L::off_acc);
-  const int tid = threadIdx.y * TX + threadIdx.x;
-  if constexpr (WS) {
-    for (int lz = 0; lz < TZ; ++lz) {
-      const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + lz;
-      if (x < g.nx && y < g.ny && z < g.nz) Acc<R>::zero(ab.zero, (size_t)x + (size_t)g.nx * ((size_t)y + (size_t)g.ny * z));
-    }
-    for (int e = tid; e < Acc<R>::W * L::E; e += TX * TY) sw[e] = 0ull;
-  }
-  if (src.acc) stage_sc<R, true, TX, TY, TZ>(src, init, g, R(P.psi0), sp, spa, spb, x0, y0, z0);
-  else stage_sc<R, false, TX, TY, TZ>(src, init, g, R(P.psi0), sp, spa, spb, x0, y0, z0);
-  __syncthreads();
-  if (!region_walled(g, x0, y0, z0, TX, TY, TZ, 1))
-    step_nodes_sc<ST, LOADER, WS, WF, TX, TY, TZ, true, IDX32>(S, O, init, g, P, fields, status, sp, spa, spb, sw, x0,
-                                                               y0, z0);
-  else
-    step_nodes_sc<ST, LOADER, WS, WF, TX, TY, TZ, false, IDX32>(S, O, init, g, P, fields, status, sp, spa, spb, sw,
-                                                                x0, y0, z0);
-  __syncthreads();
-  if constexpr (WS) {
-    flush_partials<R, TX, TY, TZ, 1>(sw, ab.out, g, x0, y0, z0);
-    __syncthreads();
-  }
-}
-
-template <int ST, int LOADER, bool WS, bool WF, int TX, int TY, int TZ, bool IDX32>
-__global__ void __launch_bounds__(TX* TY, (ST == 3) ? 1 : 2)
-    k_step_sc(View<ST> S, View<ST> O, InitBuf init, PhiSrc src, AccBufs ab, Geo g, Phys P,
-              typename Store<ST>::R* __restrict__ fields, unsigned* __restrict__ status) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  step_tile_sc<ST, LOADER, WS, WF, TX, TY, TZ, IDX32>(S, O, init, src, ab, g, P, fields, status, smem_raw,
-                                                      blockIdx.x * TX, blockIdx.y * TY, blockIdx.z * TZ);
-}
-
-// One tile of the step: clear, stage, scan, step, flush.  Ends with a
-// barrier, so the caller may reuse the shared memory.
-template <int ST, int LOADER, bool WS, bool WF, int TX, int TY, int TZ, int H, bool IDX32, bool INL = false>
-__device__ __forceinline__ void step_tile(const View<ST>& S, const View<ST>& O, const InitBuf& init, const PhiSrc& src,
-                                          const AccBufs& ab, const Geo& g, const Phys& P,
-                                          typename Store<ST>::R* __restrict__ fields, unsigned* __restrict__ status,
+// A tile of either model: clear the partial sums while the staged fields are
+// copied in, step the nodes, flush.  Ends with a barrier when AGAIN (the caller
+// reuses the shared memory).
+template <int ST, int LOADER, bool WS, bool WF, int TX, int TY, int TZ, int H, bool IDX32, bool SC, bool EARLY, bool AGAIN>
+__device__ __forceinline__ void step_tile(const View<ST>& S, const View<ST>& O, const InitBuf& init,
+                                          const unsigned long long* __restrict__ accin, unsigned long long* __restrict__ accout,
+                                          const typename Store<ST>::R* __restrict__ phi, const PadGeo& pg, const Geo& g,
+                                          const PhysR<typename Store<ST>::R>& P,
+                                          const FieldOut& fields, unsigned* __restrict__ status,
                                           unsigned char* smem, int x0, int y0, int z0) {
   using R = typename Store<ST>::R;
-  using L = Layout<R, TX, TY, TZ, H, 1, !INL>;
+  constexpr int NPH = SC ? (WF ? 3 : 2) : 1;
+  using L = Layout<R, TX, TY, TZ, H, NPH>;
   R* sp = reinterpret_cast<R*>(smem);
   unsigned long long* sw = reinterpret_cast<unsigned long long*>(smem + L::off_acc);
-  unsigned short* queue = reinterpret_cast<unsigned short*>(smem + L::off_queue);
-  unsigned char* hs = smem + L::off_h;
-  int* count = reinterpret_cast<int*>(smem + L::off_count);
   const int tid = threadIdx.y * TX + threadIdx.x;
-  if constexpr (WS) {
-    // this tile's nodes of the accumulator two steps ahead (INL: in the node loop)
-    if constexpr (!INL) {
-      for (int lz = 0; lz < TZ; ++lz) {
-        const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + lz;
-        if (x < g.nx && y < g.ny && z < g.nz)
-          Acc<R>::zero(ab.zero, (size_t)x + (size_t)g.nx * ((size_t)y + (size_t)g.ny * z));
-      }
-    }
+  if constexpr (WS && !AGAIN) {
+    for (int e = tid; e < Acc<R>::W * L::E; e += TX * TY) sw[e] = 0ull;
+    wait_primary();
+  }
+  // a step of the Shan-Chen model needs psi_A, psi_B only (fields 1 and 2)
+  stage_tile<R, TX, TY, TZ, H, NPH>(SC && !WF ? phi + (size_t)pg.px * pg.py * pg.pz : phi, pg, sp, x0, y0, z0);
+  if constexpr (WS && AGAIN) {
     for (int e = tid; e < Acc<R>::W * L::E; e += TX * TY) sw[e] = 0ull;
   }
-  if (H > 1 && tid == 0) *count = 0;
-  if (src.acc) stage_phi<R, true, TX, TY, TZ, H>(src, g, sp, x0, y0, z0);
-  else stage_phi<R, false, TX, TY, TZ, H>(src, g, sp, x0, y0, z0);
+  cp_async_wait_all();
   __syncthreads();
-  const bool nc = H > 1 && P.A_h != 0.0;
-  if constexpr (H > 1 && !INL) {
-    if (nc) {
-      if (region_walled(g, x0, y0, z0, TX, TY, TZ, P.K + 1))
-        nc_tile<R, TX, TY, TZ, H, false>(sp, g, P, hs, queue, count, x0, y0, z0);
-      else
-        nc_tile<R, TX, TY, TZ, H, true>(sp, g, P, hs, queue, count, x0, y0, z0);
+  // a tile whose one-node halo (with near contact: the scan's halo of K + 1
+  // nodes) holds no solid node needs no bounce-back or wall tests
+  const bool wallfree = !region_walled(g, x0, y0, z0, TX, TY, TZ, (H > 1 && P.A_h != R(0)) ? P.K + 1 : 1);
+  if constexpr (SC) {
+    R* spa = sp + (NPH - 2) * L::NS;
+    R* spb = spa + L::NS;
+    if (wallfree)
+      step_nodes_sc<ST, LOADER, WS, WF, TX, TY, TZ, true, IDX32>(S, O, init, g, P, fields, status, sp, spa, spb, sw, x0,
+                                                                 y0, z0);
+    else
+      step_nodes_sc<ST, LOADER, WS, WF, TX, TY, TZ, false, IDX32>(S, O, init, g, P, fields, status, sp, spa, spb, sw,
+                                                                  x0, y0, z0);
+  } else {
+    auto nodes = [&](auto wf, auto reg) {
+      step_nodes<ST, LOADER, WS, WF, TX, TY, TZ, H, decltype(wf)::value, IDX32, decltype(reg)::value, EARLY>(
+          S, O, init, g, P, fields, status, sp, sw, accin, x0, y0, z0);
+    };
+    if (P.collision == 1) {  // regularised collision
+      if (wallfree) nodes(std::true_type{}, std::true_type{});
+      else nodes(std::false_type{}, std::true_type{});
+    } else {
+      if (wallfree) nodes(std::true_type{}, std::false_type{});
+      else nodes(std::false_type{}, std::false_type{});
     }
   }
-  // a tile whose one-node halo holds no solid node needs no bounce-back or
-  // wall tests (INL: nor the scan's halo of K + 1 nodes)
-  const bool wallfree = !region_walled(g, x0, y0, z0, TX, TY, TZ, (INL && nc) ? P.K + 1 : 1);
-  unsigned long long* zacc = INL ? ab.zero : nullptr;
-  if (P.collision == 1) {  // regularised collision
-    if (wallfree)
-      step_nodes<ST, LOADER, WS, WF, TX, TY, TZ, H, true, IDX32, true, INL>(S, O, init, g, P, hs, fields, status, sp,
-                                                                            sw, src.acc, x0, y0, z0, zacc);
-    else
-      step_nodes<ST, LOADER, WS, WF, TX, TY, TZ, H, false, IDX32, true, INL>(S, O, init, g, P, hs, fields, status, sp,
-                                                                             sw, src.acc, x0, y0, z0, zacc);
-  } else {
-    if (wallfree)
-      step_nodes<ST, LOADER, WS, WF, TX, TY, TZ, H, true, IDX32, false, INL>(S, O, init, g, P, hs, fields, status, sp,
-                                                                             sw, src.acc, x0, y0, z0, zacc);
-    else
-      step_nodes<ST, LOADER, WS, WF, TX, TY, TZ, H, false, IDX32, false, INL>(S, O, init, g, P, hs, fields, status,
-                                                                              sp, sw, src.acc, x0, y0, z0, zacc);
-  }
-  __syncthreads();
   if constexpr (WS) {
-    flush_partials<R, TX, TY, TZ, H>(sw, ab.out, g, x0, y0, z0);
     __syncthreads();
+    flush_partials<R, TX, TY, TZ, L>(sw, accout, g, x0, y0, z0);
   }
+  if constexpr (AGAIN) __syncthreads();
 }
 
-template <int ST, int LOADER, bool WS, bool WF, int TX, int TY, int TZ, int H, bool IDX32, int MINB = 2,
-          bool INL = false>
+template <int ST, int LOADER, bool WS, bool WF, int TX, int TY, int TZ, int H, bool IDX32, int MINB, bool SC>
 __global__ void __launch_bounds__(TX* TY, (ST == 3) ? 1 : MINB)
-    k_step(View<ST> S, View<ST> O, InitBuf init, PhiSrc src, AccBufs ab, Geo g, Phys P,
-           typename Store<ST>::R* __restrict__ fields, unsigned* __restrict__ status) {
+    k_step(View<ST> S, View<ST> O, InitBuf init, const unsigned long long* accin, unsigned long long* accout,
+           const typename Store<ST>::R* phi, PadGeo pg, Geo g, PhysR<typename Store<ST>::R> P,
+           FieldOut fields, unsigned* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  step_tile<ST, LOADER, WS, WF, TX, TY, TZ, H, IDX32, INL>(S, O, init, src, ab, g, P, fields, status, smem_raw,
-                                                           blockIdx.x * TX, blockIdx.y * TY, blockIdx.z * TZ);
+  launch_dependents();
+  if constexpr (!WS) wait_primary();
+  constexpr bool EARLY = ST == 3 || TX * TY * MINB <= 512;  // 128 registers a thread or more
+  step_tile<ST, LOADER, WS, WF, TX, TY, TZ, H, IDX32, SC, EARLY, false>(S, O, init, accin, accout, phi, pg, g, P, fields, status,
+                                                                 smem_raw, blockIdx.x * TX, blockIdx.y * TY,
+                                                                 blockIdx.z * TZ);
 }
 
 // ---------------------------------------------------------------------------
-// batched persistent kernel: many independent runs of uneven sizes and
-// parameters, one launch per step.  Work items are (run, tile); persistent
-// CTAs stride over the item list and find the run of an item by binary
-// search over the runs' prefix offsets.  Every run's accumulators are at the
-// same phase k of their rotation.
+// batched persistent kernels: many independent runs of uneven sizes and
+// parameters, one k_phi_batched and one k_step_batched launch per step.  Work
+// items are (run, row group) and (run, tile); persistent CTAs stride over the
+// item list and look the run of an item up in a table (run_of; a binary search
+// over the runs' prefix offsets put six dependent loads before every tile).  Every run's accumulators are at the same phase k of their
+// rotation.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int find_run(const RunDesc* runs, int nruns, long long item) {
-  int lo = 0, hi = nruns - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (runs[mid].tile_begin <= item) lo = mid;
-    else hi = mid - 1;
+__device__ __forceinline__ Geo uniform(const Geo& d) {
+  Geo g;
+  g.nx = uniform(d.nx);
+  g.ny = uniform(d.ny);
+  g.nz = uniform(d.nz);
+  const int w = uniform(d.wx | d.wy << 1 | d.wz << 2);
+  g.wx = w & 1;
+  g.wy = w >> 1 & 1;
+  g.wz = w >> 2 & 1;
+  g.N = (long long)g.nx * g.ny * g.nz;
+  return g;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256) k_phi_batched(const RunDesc* __restrict__ runs, const int* __restrict__ run_of,
+                                                     long long ngroups, int k) {
+  launch_dependents();
+  wait_primary();
+  for (long long t = blockIdx.x; t < ngroups; t += gridDim.x) {
+    const RunDesc& d = runs[run_of[t]];
+    const PhiSrc src{nullptr, d.acc[k]};
+    const InitBuf none{nullptr, nullptr, nullptr, 0};
+    // eight rows of the run, one a warp
+    const long long row = (t - d.row_begin) * 8 + threadIdx.y;
+    if (row < (long long)d.g.ny * d.g.nz)
+      phi_row<R, false>(src, none, d.g, d.pg, R(0), d.phi, d.acc[(k + 2) % 3], (int)(row % d.g.ny), (int)(row / d.g.ny));
   }
-  return lo;
 }
 
-template <int ST, int TX, int TY, int TZ, int H, bool IDX32, int MINB = 2, bool INL = false>
+template <int ST, int TX, int TY, int TZ, int H, bool IDX32, int MINB>
 __global__ void __launch_bounds__(TX* TY, MINB)
-    k_step_batched(const RunDesc* __restrict__ runs, int nruns, long long ntiles, int parity, int k,
+    k_step_batched(const RunDesc* __restrict__ runs, const int* __restrict__ run_of, long long ntiles, int parity, int k,
                    unsigned* __restrict__ status) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   InitBuf none{nullptr, nullptr, nullptr, 0};
+  launch_dependents();
+  wait_primary();
+  int next = run_of[blockIdx.x < ntiles ? blockIdx.x : 0];
   for (long long t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int r = find_run(runs, nruns, t);
-    const RunDesc& d = runs[r];
-    const long long lt = t - d.tile_begin;
-    const int bx = (int)(lt % d.tiles_x);
-    const int by = (int)((lt / d.tiles_x) % d.tiles_y);
-    const int bz = (int)(lt / ((long long)d.tiles_x * d.tiles_y));
-    const Geo g = d.g;
-    const Phys P = d.p;
-    const PhiSrc src{nullptr, d.acc[k]};
-    const AccBufs ab{d.acc[(k + 1) % 3], d.acc[(k + 2) % 3]};
-    step_tile<ST, LOAD_PULL, true, false, TX, TY, TZ, H, IDX32, INL>(view<ST>(d.S[parity]),
-                                                                     view<ST>(d.S[parity ^ 1]), none, src, ab, g, P,
-                                                                     nullptr, status, smem_raw, bx * TX, by * TY,
-                                                                     bz * TZ);
+    const RunDesc& d = runs[next];
+    if (t + gridDim.x < ntiles) next = run_of[t + gridDim.x];  // its load runs through the tile
+    const int lt = uniform((int)(t - d.tile_begin));
+    const Geo g = uniform(d.g);
+    const int tiles_x = (g.nx + TX - 1) / TX, tiles_y = (g.ny + TY - 1) / TY;
+    const int bx = lt % tiles_x, by = (lt / tiles_x) % tiles_y, bz = lt / (tiles_x * tiles_y);
+    PadGeo pg = d.pg;
+    View<ST> S = view<ST>(d.S[parity]), O = view<ST>(d.S[parity ^ 1]);
+    S.f = uniform(S.f);
+    O.f = uniform(O.f);
+    O.sv = uniform(O.sv);
+    PhysR<float> P = d.p;
+    P.tau_a = uniform(P.tau_a);
+    P.tau_b = uniform(P.tau_b);
+    P.A2 = uniform(P.A2);
+    P.beta = uniform(P.beta);
+    P.A_h = uniform(P.A_h);
+    P.h_min = uniform(P.h_min);
+    P.h_max = uniform(P.h_max);
+    P.phi_I = uniform(P.phi_I);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) P.g[a] = uniform(P.g[a]);
+    const int bits = uniform(P.equal_tau | P.K << 1 | P.g_mode << 4 | P.collision << 6);
+    P.equal_tau = bits & 1;
+    P.K = bits >> 1 & 7;
+    P.g_mode = bits >> 4 & 3;
+    P.collision = bits >> 6;
+    step_tile<ST, LOAD_PULL, true, false, TX, TY, TZ, H, IDX32, false, (TX * TY * MINB <= 512 && !Store<ST>::TWOSET), true>(
+        S, O, none, d.acc[k], d.acc[(k + 1) % 3], d.phi, pg, g, P, FieldOut{}, status, smem_raw, bx * TX, by * TY, bz * TZ);
   }
 }
 
@@ -1762,7 +1768,7 @@ __global__ void __launch_bounds__(TX* TY, MINB)
 // population export (pre-collision, both components, canonical order, double)
 // ---------------------------------------------------------------------------
 template <int ST, int LOADER>
-__global__ void __launch_bounds__(128) k_export(View<ST> S, InitBuf init, Geo g, Phys P, int x0, int y0, int z0,
+__global__ void __launch_bounds__(128) k_export(View<ST> S, InitBuf init, Geo g, PhysR<typename Store<ST>::R> P, int x0, int y0, int z0,
                                                 int bx, int by, int bz, double* outA, double* outB) {
   using R = typename Store<ST>::R;
   const long long M = (long long)bx * by * bz;

@@ -4,21 +4,19 @@
 
 namespace lbcg {
 
-// tile 2: the 32x8x4 tile with registers capped for 3 CTAs per SM; tile 3: a
-// 32x8x6 tile capped for 3 CTAs per SM; tile 4: 32x4x4 (128 threads) capped
-// for 6 CTAs per SM; tile 5: 32x8x8 with the near-contact scan inside the
-// node loop
-const Tile kTiles[NUM_TILES] = {{32, 8, 4}, {32, 8, 8}, {32, 8, 4}, {32, 8, 6}, {32, 4, 4}, {32, 8, 8}};
+const Tile kTiles[NUM_TILES] = {{32, 8, 4}, {32, 8, 8}, {32, 8, 2}, {32, 8, 1}, {32, 4, 4}, {32, 8, 8}};
 
 template <int ST>
 cudaError_t launch_phi_acc_t(const Geo& g, const StateBuf& in, unsigned long long* acc, cudaStream_t st);
 template <int ST>
 cudaError_t launch_step_s(int loader, bool ws, bool wf, int tile, const Geo& g, const Phys& p, const StateBuf& in,
-                          const InitBuf& init, PhiSrc src, AccBufs ab, StateBuf out, void* fields, unsigned* status,
+                          const InitBuf& init, PhiSrc src, AccBufs ab, StateBuf out, void* phi, int halo, const FieldOut& fields, unsigned* status,
                           cudaStream_t st);
 template <int ST>
-cudaError_t launch_batched_t(const RunDesc* d_runs, int nruns, long long ntiles, int tile, int halo,
-                             long long max_nodes, int parity, int k, int blocks_per_sm, unsigned* status,
+cudaError_t launch_phi_s(const Geo& g, const Phys& p, const InitBuf& init, PhiSrc src, void* phi, int halo, cudaStream_t st);
+template <int ST>
+cudaError_t launch_batched_t(const RunDesc* d_runs, const int* run_of, long long ntiles, long long ngroups, int tile, int halo,
+                             long long max_rows, int parity, int k, int blocks_per_sm, unsigned* status,
                              cudaStream_t st);
 template <int ST>
 cudaError_t launch_export_t(int loader, const Geo& g, const Phys& p, const StateBuf& in, const InitBuf& init, int x0,
@@ -36,16 +34,59 @@ cudaError_t launch_phi_acc(int storage, const Geo& g, const StateBuf& in, unsign
 }
 
 cudaError_t launch_step(int storage, int loader, bool write_state, bool write_fields, int tile, const Geo& g,
-                        const Phys& p, const StateBuf& in, const InitBuf& init, PhiSrc src, AccBufs ab, StateBuf out,
-                        void* fields, unsigned* status, cudaStream_t st) {
+                        const Phys& p, const StateBuf& in, const InitBuf& init, PhiSrc src, AccBufs ab, StateBuf out, void* phi, int halo, const FieldOut& fields, unsigned* status, cudaStream_t st) {
   switch (storage) {
-    case 0: return launch_step_s<0>(loader, write_state, write_fields, tile, g, p, in, init, src, ab, out, fields, status, st);
-    case 1: return launch_step_s<1>(loader, write_state, write_fields, tile, g, p, in, init, src, ab, out, fields, status, st);
-    case 2: return launch_step_s<2>(loader, write_state, write_fields, tile, g, p, in, init, src, ab, out, fields, status, st);
-    case 3: return launch_step_s<3>(loader, write_state, write_fields, tile, g, p, in, init, src, ab, out, fields, status, st);
-    case 4: return launch_step_s<4>(loader, write_state, write_fields, tile, g, p, in, init, src, ab, out, fields, status, st);
+    case 0: return launch_step_s<0>(loader, write_state, write_fields, tile, g, p, in, init, src, ab, out, phi, halo, fields, status, st);
+    case 1: return launch_step_s<1>(loader, write_state, write_fields, tile, g, p, in, init, src, ab, out, phi, halo, fields, status, st);
+    case 2: return launch_step_s<2>(loader, write_state, write_fields, tile, g, p, in, init, src, ab, out, phi, halo, fields, status, st);
+    case 3: return launch_step_s<3>(loader, write_state, write_fields, tile, g, p, in, init, src, ab, out, phi, halo, fields, status, st);
+    case 4: return launch_step_s<4>(loader, write_state, write_fields, tile, g, p, in, init, src, ab, out, phi, halo, fields, status, st);
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_phi_only(int storage, const Geo& g, const Phys& p, const InitBuf& init, PhiSrc src, void* phi, int halo,
+                            cudaStream_t st) {
+  switch (storage) {
+    case 0: return launch_phi_s<0>(g, p, init, src, phi, halo, st);
+    case 1: return launch_phi_s<1>(g, p, init, src, phi, halo, st);
+    case 2: return launch_phi_s<2>(g, p, init, src, phi, halo, st);
+    case 3: return launch_phi_s<3>(g, p, init, src, phi, halo, st);
+    case 4: return launch_phi_s<4>(g, p, init, src, phi, halo, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256) k_phi_fill(size_t n, R* __restrict__ phi) {
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) phi[i] = R(PHI_SOLID);
+}
+cudaError_t launch_phi_fill(int storage, const PadGeo& pg, int fields, void* phi, cudaStream_t st) {
+  const size_t n = (size_t)pg.px * pg.py * pg.pz * (size_t)fields;
+  const unsigned blocks = (unsigned)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
+  if (storage == 3) k_phi_fill<<<blocks, 256, 0, st>>>(n, (double*)phi);
+  else k_phi_fill<<<blocks, 256, 0, st>>>(n, (float*)phi);
+  return cudaGetLastError();
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256) k_phi_plain(Geo g, PadGeo pg, const R* __restrict__ phi, R* __restrict__ plain) {
+  const long long rows = (long long)g.ny * g.nz;
+  for (long long row = (long long)blockIdx.x * 8 + threadIdx.y; row < rows; row += (long long)gridDim.x * 8) {
+    const long long y = row % g.ny, z = row / g.ny;
+    const R* src = phi + pg.hx + (long long)pg.px * (pg.h + y + (long long)pg.py * (pg.h + z));
+    for (int x = threadIdx.x; x < g.nx; x += 32) {
+      const R v = src[x];
+      plain[row * g.nx + x] = v > R(0.5) * R(PHI_SOLID) ? R(0) : v;
+    }
+  }
+}
+cudaError_t launch_phi_plain(int storage, const Geo& g, const PadGeo& pg, const void* phi, void* plain, cudaStream_t st) {
+  const long long groups = ((long long)g.ny * g.nz + 7) / 8;
+  const unsigned blocks = (unsigned)(groups < 8192 ? groups : 8192);
+  if (storage == 3) k_phi_plain<<<blocks, dim3(32, 8), 0, st>>>(g, pg, (const double*)phi, (double*)plain);
+  else k_phi_plain<<<blocks, dim3(32, 8), 0, st>>>(g, pg, (const float*)phi, (float*)plain);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_export(int storage, int loader, const Geo& g, const Phys& p, const StateBuf& in,
@@ -61,13 +102,13 @@ cudaError_t launch_export(int storage, int loader, const Geo& g, const Phys& p, 
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_batched(int storage, const RunDesc* d_runs, int nruns, long long ntiles, int tile, int halo,
-                           long long max_nodes, int parity, int k, int blocks_per_sm, unsigned* status,
+cudaError_t launch_batched(int storage, const RunDesc* d_runs, const int* run_of, long long ntiles, long long ngroups, int tile,
+                           int halo, long long max_rows, int parity, int k, int blocks_per_sm, unsigned* status,
                            cudaStream_t st) {
   switch (storage) {
-    case 0: return launch_batched_t<0>(d_runs, nruns, ntiles, tile, halo, max_nodes, parity, k, blocks_per_sm, status, st);
-    case 1: return launch_batched_t<1>(d_runs, nruns, ntiles, tile, halo, max_nodes, parity, k, blocks_per_sm, status, st);
-    case 2: return launch_batched_t<2>(d_runs, nruns, ntiles, tile, halo, max_nodes, parity, k, blocks_per_sm, status, st);
+    case 0: return launch_batched_t<0>(d_runs, run_of, ntiles, ngroups, tile, halo, max_rows, parity, k, blocks_per_sm, status, st);
+    case 1: return launch_batched_t<1>(d_runs, run_of, ntiles, ngroups, tile, halo, max_rows, parity, k, blocks_per_sm, status, st);
+    case 2: return launch_batched_t<2>(d_runs, run_of, ntiles, ngroups, tile, halo, max_rows, parity, k, blocks_per_sm, status, st);
   }
   return cudaErrorInvalidValue;  // no batched FP64 or moment instantiation
 }
@@ -83,8 +124,35 @@ int sm_count_host() {
   return n;
 }
 
+template <typename E>
+__global__ void __launch_bounds__(256) k_direction(Geo g, E* __restrict__ f, int nd, int dir, E* __restrict__ plain, bool gather) {
+  const long long nbx = (g.nx + BLK - 1) / BLK;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.N; i += (long long)gridDim.x * blockDim.x) {
+    const long long row = i / g.nx;
+    const int x = (int)(i - row * g.nx);
+    E& v = f[((row * nbx + x / BLK) * nd + dir) * BLK + x % BLK];
+    if (gather) plain[i] = v;
+    else v = plain[i];
+  }
+}
+
+cudaError_t launch_direction(int storage, const Geo& g, void* f, int dir, void* plain, bool gather, cudaStream_t st) {
+  const long long need = (g.N + 255) / 256;
+  const int blocks = (int)(need < 8192 ? need : 8192), nd = state_arrays(storage);
+  switch (elem_bytes(storage)) {
+    case 2: k_direction<<<blocks, 256, 0, st>>>(g, (uint16_t*)f, nd, dir, (uint16_t*)plain, gather); break;
+    case 4: k_direction<<<blocks, 256, 0, st>>>(g, (uint32_t*)f, nd, dir, (uint32_t*)plain, gather); break;
+    default: k_direction<<<blocks, 256, 0, st>>>(g, (uint64_t*)f, nd, dir, (uint64_t*)plain, gather); break;
+  }
+  return cudaGetLastError();
+}
+
 size_t elem_bytes(int storage) { return storage == 3 ? 8 : (storage == 2 ? 2 : 4); }
 int state_arrays(int storage) { return storage == 4 ? MOMENT_COEFS : (storage == 0 || storage == 3 ? 2 * Q : Q); }
+size_t state_elems(int storage, const Geo& g) {
+  if (storage == 4) return (size_t)MOMENT_COEFS * (size_t)g.N;
+  return (size_t)((g.nx + BLK - 1) / BLK) * BLK * (size_t)g.ny * (size_t)g.nz * (size_t)state_arrays(storage);
+}
 bool storage_is_twoset(int storage) { return storage == 0 || storage == 3; }
 bool storage_is_f64(int storage) { return storage == 3; }
 

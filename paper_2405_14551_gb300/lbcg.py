@@ -67,6 +67,7 @@ _SIGS = {
                                  ctypes.POINTER(ctypes.c_void_p)]),
     "lb_destroy": (ctypes.c_int, [ctypes.c_void_p]),
     "lb_set_stream": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p]),
+    "lb_get_stream": (ctypes.c_void_p, [ctypes.c_void_p]),
     "lb_init_droplets": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p,
                                         ctypes.c_double]),
     "lb_init_fields": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
@@ -231,6 +232,16 @@ def lb_set_stream(h, stream_ptr: int):
     _check(load_library().lb_set_stream(h, ctypes.c_void_p(stream_ptr)), "lb_set_stream")
 
 
+def _used_by(h, *tensors):
+    """Device tensors handed to a call on handle h: the caching allocator must
+    not give their memory away before the handle's stream, which need not be
+    the tensors' own, has passed the call."""
+    import torch
+    s = torch.cuda.ExternalStream(load_library().lb_get_stream(h) or 0)
+    for t in tensors:
+        t.record_stream(s)
+
+
 def lb_init_droplets(h, centres, radii, width=0.0):
     c = np.ascontiguousarray(np.asarray(centres, dtype=np.float64).reshape(-1, 3))
     r = np.ascontiguousarray(np.asarray(radii, dtype=np.float64).reshape(-1))
@@ -258,6 +269,8 @@ def lb_init_fields(h, phi, rho=None, u=None, regularised=False):
 
     _check(load_library().lb_init_fields(h, ptr(phi), ptr(rho), ptr(u), int(bool(regularised)), int(is_dev)),
            "lb_init_fields")
+    if is_dev:
+        _used_by(h, *keep)
 
 
 def lb_step(h, nsteps: int):
@@ -288,6 +301,8 @@ def lb_surrogate_load(h, path: str):
 def lb_surrogate_predict(h, out=None):
     _check(load_library().lb_surrogate_predict(h, ctypes.c_void_p(out.data_ptr()) if out is not None else None),
            "lb_surrogate_predict")
+    if out is not None:
+        _used_by(h, out)
 
 
 def lb_surrogate_cycle(h, judge, K: int, vol_tol: float, phi_tol: float):
@@ -322,6 +337,8 @@ def lb_fields(h, mask: int, dst, dst_is_device: bool, f64: bool = False):
     p = dst.data_ptr() if dst_is_device else dst.ctypes.data
     fn = L.lb_fields_f64 if f64 else L.lb_fields
     _check(fn(h, int(mask), p, int(bool(dst_is_device))), "lb_fields")
+    if dst_is_device:
+        _used_by(h, dst)
 
 
 def lb_get_populations(h, box):
