@@ -4,6 +4,7 @@
 // partial sums in a fixed partition and a fixed tree order, then one block
 // sums the partials in a fixed order, so results are bitwise reproducible.
 #include "../../include/lbcg.h"
+#include "exact_sum.cuh"
 #include "internal.h"
 #include "lattice.cuh"
 
@@ -72,13 +73,13 @@ int reduce_blocks(long long N) {
   return (int)b;
 }
 
+// (a lattice has fewer than 2^31 nodes: 32-bit divisions, none without walls)
 __device__ __forceinline__ bool node_solid(const Geo& g, long long idx) {
-  const int x = (int)(idx % g.nx);
-  const long long yz = idx / g.nx;
-  const int y = (int)(yz % g.ny);
-  const int z = (int)(yz / g.ny);
+  if (!(g.wx | g.wy | g.wz)) return false;
+  const unsigned yz = (unsigned)idx / (unsigned)g.nx, z = yz / (unsigned)g.ny;
+  const int x = (int)((unsigned)idx - yz * (unsigned)g.nx), y = (int)(yz - z * (unsigned)g.ny);
   return (g.wx && (x == 0 || x == g.nx - 1)) || (g.wy && (y == 0 || y == g.ny - 1)) ||
-         (g.wz && (z == 0 || z == g.nz - 1));
+         (g.wz && ((int)z == 0 || (int)z == g.nz - 1));
 }
 
 // fixed-order tree sum of NV values per thread into s[0..NV)
@@ -92,6 +93,11 @@ __device__ void block_tree(double (*s)[RED_THREADS], double v[NV]) {
     __syncthreads();
   }
 }
+
+// Sum over fluid nodes of (1 + phi)/2 from the sum of phi and the node count.
+__device__ __forceinline__ double volume_of(const Sum3& phi, int nodes) { return 0.5 * ((double)nodes + phi.value()); }
+// the kinetic term is formed from velocities scaled by SQUARE_SCALE
+constexpr double KE_UNSCALE = 0.5 * SQUARE_UNSCALE;
 
 template <typename R>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_partial(Geo g, const R* __restrict__ fl, double* partials) {
@@ -119,6 +125,62 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_partial(Geo g, const R* 
     for (int k = 0; k < 8; ++k) partials[(size_t)blockIdx.x * 8 + k] = s[k][0];
 }
 
+// The same sums of FP32 fields, a thread's share in Sum3 terms, then FP64 for
+// the tree: the FP64 pipe (22 operations and conversions a node) bounded the
+// kernel above, 174 -> 86 us at 128x128x256.  A thread whose terms
+// overflow FP32 repeats its share in FP64.
+__global__ void __launch_bounds__(RED_THREADS) k_reduce_partial_f32(Geo g, const float* __restrict__ fl, double* partials) {
+  __shared__ double s[8][RED_THREADS];
+  const size_t N = (size_t)g.N;
+  const long long chunk = (g.N + gridDim.x - 1) / gridDim.x;
+  const long long beg = (long long)blockIdx.x * chunk;
+  const long long end = beg + chunk < g.N ? beg + chunk : g.N;
+  Sum3 a, b, j[3], ph, ke;
+  int active = 0, nodes = 0;
+  for (long long i = beg + threadIdx.x; i < end; i += RED_THREADS) {
+    if (node_solid(g, i)) continue;
+    ++nodes;
+    const float rho = fl[F_RHO * N + i];
+    const float u[3] = {fl[F_UX * N + i], fl[F_UY * N + i], fl[F_UZ * N + i]};
+    a.add(fl[F_RHOA * N + i]);
+    b.add(fl[F_RHOB * N + i]);
+    ph.add(fl[F_PHI * N + i]);
+    active += fl[F_H * N + i] > 0.f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float p = __fmul_rn(rho, u[k]), e = __fmaf_rn(rho, u[k], -p);  // rho u = p + e
+      j[k].add(p);
+      j[k].add(e);
+      const float w = __fmul_rn(u[k], SQUARE_SCALE);
+      const float ps = __fmul_rn(p, SQUARE_SCALE), es = __fmul_rn(e, SQUARE_SCALE);
+      ke.add_product(ps, w);
+      ke.add(__fmul_rn(es, w));
+    }
+  }
+  double v[8] = {a.value(),   b.value(),          j[0].value(),   j[1].value(),
+                 j[2].value(), volume_of(ph, nodes), (double)active, KE_UNSCALE * ke.value()};
+  if (!(a.finite() && b.finite() && ph.finite() && j[0].finite() && j[1].finite() && j[2].finite() && ke.finite())) {
+    for (int k = 0; k < 8; ++k) v[k] = 0.0;
+    for (long long i = beg + threadIdx.x; i < end; i += RED_THREADS) {
+      if (node_solid(g, i)) continue;
+      const double rho = fl[F_RHO * N + i];
+      const double ux = fl[F_UX * N + i], uy = fl[F_UY * N + i], uz = fl[F_UZ * N + i];
+      v[0] += fl[F_RHOA * N + i];
+      v[1] += fl[F_RHOB * N + i];
+      v[2] += rho * ux;
+      v[3] += rho * uy;
+      v[4] += rho * uz;
+      v[5] += 0.5 * (1.0 + (double)fl[F_PHI * N + i]);
+      v[6] += fl[F_H * N + i] > 0.f ? 1.0 : 0.0;
+      v[7] += 0.5 * rho * (ux * ux + uy * uy + uz * uz);
+    }
+    if (ph.finite()) v[5] = volume_of(ph, nodes);
+  }
+  block_tree<8>(s, v);
+  if (threadIdx.x == 0)
+    for (int k = 0; k < 8; ++k) partials[(size_t)blockIdx.x * 8 + k] = s[k][0];
+}
+
 template <int NV>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_final(int nblocks, const double* __restrict__ partials,
                                                               double* out) {
@@ -138,7 +200,7 @@ cudaError_t launch_reduce(int storage, const Geo& g, const void* fields, double*
   if (storage_is_f64(storage))
     k_reduce_partial<double><<<nb, RED_THREADS, 0, st>>>(g, reinterpret_cast<const double*>(fields), partials);
   else
-    k_reduce_partial<float><<<nb, RED_THREADS, 0, st>>>(g, reinterpret_cast<const float*>(fields), partials);
+    k_reduce_partial_f32<<<nb, RED_THREADS, 0, st>>>(g, reinterpret_cast<const float*>(fields), partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_reduce_final<8><<<1, RED_THREADS, 0, st>>>(nb, partials, out8);
@@ -146,17 +208,25 @@ cudaError_t launch_reduce(int storage, const Geo& g, const void* fields, double*
 }
 
 // dispersed volume sum over fluid nodes of (1 + phi)/2 of a phase-field array,
-// in the partition and order of k_reduce_partial (same value as its v[5])
+// in the partition and order of k_reduce_partial_f32 (same value as its v[5])
 __global__ void __launch_bounds__(RED_THREADS) k_phi_volume_partial(Geo g, const float* __restrict__ phi,
                                                                     double* partials) {
   __shared__ double s[1][RED_THREADS];
   const long long chunk = (g.N + gridDim.x - 1) / gridDim.x;
   const long long beg = (long long)blockIdx.x * chunk;
   const long long end = beg + chunk < g.N ? beg + chunk : g.N;
-  double v[1] = {0};
+  Sum3 ph;
+  int nodes = 0;
   for (long long i = beg + threadIdx.x; i < end; i += RED_THREADS) {
     if (node_solid(g, i)) continue;
-    v[0] += 0.5 * (1.0 + (double)phi[i]);
+    ++nodes;
+    ph.add(phi[i]);
+  }
+  double v[1] = {volume_of(ph, nodes)};
+  if (!ph.finite()) {
+    v[0] = 0.0;
+    for (long long i = beg + threadIdx.x; i < end; i += RED_THREADS)
+      if (!node_solid(g, i)) v[0] += 0.5 * (1.0 + (double)phi[i]);
   }
   block_tree<1>(s, v);
   if (threadIdx.x == 0) partials[blockIdx.x] = s[0][0];
@@ -206,8 +276,12 @@ cudaError_t launch_laplace(int storage, const Geo& g, const void* fields, double
 // atomicCAS; every loop is bounded and reports through the status word.
 // A first pass joins the links inside 32 x 8 x 8 tiles in shared memory and
 // writes, per node, the global index of its tile-local root (the smallest
-// index of its tile-local component); the global pass then joins only the
-// links that cross tile faces.
+// index of its tile-local component); the global pass then visits only the
+// nodes on a tile's upper faces and joins the links that cross them.  The
+// count is the tile-local roots less the joins that succeeded: a hook only
+// ever puts a root under a smaller label, so each one merges two trees.
+// With a pass over all nodes for the faces and one for the roots:
+// 128x128x256, 123 -> 92 us for the passes.
 // ---------------------------------------------------------------------------
 constexpr int CC_TX = 32, CC_TY = 8, CC_TZ = 8, CC_TN = CC_TX * CC_TY * CC_TZ;
 
@@ -230,7 +304,8 @@ struct PhiView {
 };
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_cc_local(Geo g, PhiView<R> phi, int* __restrict__ Lg, unsigned* status) {
+__global__ void __launch_bounds__(256) k_cc_local(Geo g, PhiView<R> phi, int* __restrict__ Lg, int* count,
+                                                  unsigned* status) {
   __shared__ int L[CC_TN];
   const int x0 = blockIdx.x * CC_TX, y0 = blockIdx.y * CC_TY, z0 = blockIdx.z * CC_TZ;
   for (int k = threadIdx.x; k < CC_TN; k += blockDim.x) {
@@ -275,11 +350,13 @@ __global__ void __launch_bounds__(256) k_cc_local(Geo g, PhiView<R> phi, int* __
   }
   if (!ok) atomicOr(status, 2u);
   __syncthreads();
+  int roots = 0;
   for (int k = threadIdx.x; k < CC_TN; k += blockDim.x) {
     const int x = x0 + k % CC_TX, y = y0 + (k / CC_TX) % CC_TY, z = z0 + k / (CC_TX * CC_TY);
     if (x >= g.nx || y >= g.ny || z >= g.nz) continue;
     const long long i = (long long)x + (long long)g.nx * ((long long)y + (long long)g.ny * z);
     int r = L[k] < 0 ? -1 : cc_find_local(L, k);
+    roots += r == k;
     if (L[k] >= 0 && r < 0) {
       atomicOr(status, 2u);
       r = k;
@@ -289,6 +366,8 @@ __global__ void __launch_bounds__(256) k_cc_local(Geo g, PhiView<R> phi, int* __
                           (long long)g.nx * ((long long)(y0 + (r / CC_TX) % CC_TY) +
                                              (long long)g.ny * (z0 + r / (CC_TX * CC_TY))));
   }
+  roots = __reduce_add_sync(0xffffffffu, roots);
+  if ((threadIdx.x & 31) == 0 && roots) atomicAdd(count, roots);
 }
 
 // Root of i.  Every parent label is smaller than its child's (the tile pass
@@ -311,71 +390,70 @@ __device__ __forceinline__ int cc_find(volatile int* L, int i, long long limit) 
   return -1;
 }
 
-__global__ void k_cc_union(Geo g, int* __restrict__ Lp, unsigned* status) {
+__device__ __forceinline__ bool cc_join(int* Lp, int i, int j, long long limit, int& joined) {
   volatile int* L = Lp;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.N; i += (long long)gridDim.x * blockDim.x) {
-    if (L[i] < 0) continue;
-    const int x = (int)(i % g.nx);
-    const long long yz = i / g.nx;
-    const int y = (int)(yz % g.ny);
-    const int z = (int)(yz / g.ny);
-    for (int a = 0; a < 3; ++a) {
-      int v[3] = {x, y, z};
-      const int nn[3] = {g.nx, g.ny, g.nz};
-      const int wall[3] = {g.wx, g.wy, g.wz};
-      const int tile[3] = {CC_TX, CC_TY, CC_TZ};
-      if ((v[a] + 1) % tile[a] != 0 && v[a] + 1 < nn[a]) continue;  // joined by the tile pass
-      v[a] += 1;
-      if (v[a] >= nn[a]) {
-        if (wall[a]) continue;
-        v[a] -= nn[a];
-      }
-      const long long j = (long long)v[0] + (long long)g.nx * ((long long)v[1] + (long long)g.ny * v[2]);
-      if (L[j] < 0) continue;
-      int ra = (int)i, rb = (int)j;
-      bool done = false;
-      for (int it = 0; it < (1 << 22) && !done; ++it) {
-        ra = cc_find(L, ra, g.N);
-        rb = cc_find(L, rb, g.N);
-        if (ra < 0 || rb < 0) break;
-        if (ra == rb) {
-          done = true;
-          break;
-        }
-        if (ra < rb) {
-          const int t = ra;
-          ra = rb;
-          rb = t;
-        }
-        const int old = atomicCAS(Lp + ra, ra, rb);
-        if (old == ra) done = true;
-        else ra = old;
-      }
-      if (!done) atomicOr(status, 2u);
+  int ra = i, rb = j;
+  for (int it = 0; it < (1 << 22); ++it) {
+    ra = cc_find(L, ra, limit);
+    rb = cc_find(L, rb, limit);
+    if (ra < 0 || rb < 0) return false;
+    if (ra == rb) return true;
+    if (ra < rb) {
+      const int t = ra;
+      ra = rb;
+      rb = t;
     }
+    const int old = atomicCAS(Lp + ra, ra, rb);
+    if (old == ra) {
+      ++joined;
+      return true;
+    }
+    ra = old;
   }
+  return false;
 }
 
-__global__ void k_cc_count(Geo g, int* __restrict__ Lp, int* count) {
-  volatile int* L = Lp;
-  int local = 0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.N; i += (long long)gridDim.x * blockDim.x)
-    if (L[i] == (int)i) ++local;
-  if (local) atomicAdd(count, local);
+// One CTA per tile: the links from the nodes of its upper x, y and z faces (its
+// last layer in the box) to the next tile, periodic on open axes.
+__global__ void __launch_bounds__(256) k_cc_union(Geo g, int* __restrict__ Lp, int* count, unsigned* status) {
+  const int o[3] = {(int)blockIdx.x * CC_TX, (int)blockIdx.y * CC_TY, (int)blockIdx.z * CC_TZ};
+  const int nn[3] = {g.nx, g.ny, g.nz}, wall[3] = {g.wx, g.wy, g.wz}, tile[3] = {CC_TX, CC_TY, CC_TZ};
+  int joined = 0;
+  bool ok = true;
+  constexpr int FX = CC_TY * CC_TZ, FY = CC_TX * CC_TZ, FZ = CC_TX * CC_TY;
+  for (int q = threadIdx.x; q < FX + FY + FZ; q += blockDim.x) {
+    const int a = q < FZ ? 2 : (q < FZ + FY ? 1 : 0);
+    const int k = a == 2 ? q : (a == 1 ? q - FZ : q - FZ - FY);
+    int v[3];
+    const int last = o[a] + tile[a] < nn[a] ? o[a] + tile[a] - 1 : nn[a] - 1;
+    if (a == 2) { v[0] = o[0] + k % CC_TX; v[1] = o[1] + k / CC_TX; v[2] = last; }
+    else if (a == 1) { v[0] = o[0] + k % CC_TX; v[1] = last; v[2] = o[2] + k / CC_TX; }
+    else { v[0] = last; v[1] = o[1] + k % CC_TY; v[2] = o[2] + k / CC_TY; }
+    if (v[0] >= g.nx || v[1] >= g.ny || v[2] >= g.nz) continue;
+    const long long i = (long long)v[0] + (long long)g.nx * ((long long)v[1] + (long long)g.ny * v[2]);
+    v[a] += 1;
+    if (v[a] >= nn[a]) {
+      if (wall[a]) continue;
+      v[a] -= nn[a];
+    }
+    const long long j = (long long)v[0] + (long long)g.nx * ((long long)v[1] + (long long)g.ny * v[2]);
+    const volatile int* L = Lp;
+    if (L[i] < 0 || L[j] < 0) continue;
+    ok = cc_join(Lp, (int)i, (int)j, g.N, joined) && ok;
+  }
+  if (!ok) atomicOr(status, 2u);
+  joined = __reduce_add_sync(0xffffffffu, joined);
+  if ((threadIdx.x & 31) == 0 && joined) atomicSub(count, joined);
 }
 
 template <typename R>
 static cudaError_t launch_cc_t(const Geo& g, PhiView<R> phi, int* labels, int* count, unsigned* status, cudaStream_t st) {
-  const long long need = (g.N + 255) / 256;
-  const int blocks = (int)(need < 8192 ? need : 8192);
   const dim3 tiles((g.nx + CC_TX - 1) / CC_TX, (g.ny + CC_TY - 1) / CC_TY, (g.nz + CC_TZ - 1) / CC_TZ);
-  k_cc_local<R><<<tiles, 256, 0, st>>>(g, phi, labels, status);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), st);
   if (e != cudaSuccess) return e;
-  k_cc_union<<<blocks, 256, 0, st>>>(g, labels, status);
+  k_cc_local<R><<<tiles, 256, 0, st>>>(g, phi, labels, count, status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(count, 0, sizeof(int), st)) != cudaSuccess) return e;
-  k_cc_count<<<blocks, 256, 0, st>>>(g, labels, count);
+  k_cc_union<<<tiles, 256, 0, st>>>(g, labels, count, status);
   return cudaGetLastError();
 }
 
