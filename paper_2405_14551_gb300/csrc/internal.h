@@ -183,6 +183,9 @@ cudaError_t launch_export(int storage, int loader, const Geo& g, const Phys& p, 
 cudaError_t launch_batched(int storage, const RunDesc* d_runs, const int* run_of, long long ntiles, long long ngroups, int tile,
                            int halo, long long max_rows, int parity, int k, int blocks_per_sm, unsigned* status,
                            cudaStream_t st);
+// the tile shape that launch_batched takes for tile: the wide halos and planes
+// beyond 32-bit byte offsets have one shape only
+int batched_tile(int storage, int tile, int halo, long long max_rows);
 int sm_count_host();
 
 // --- aux_kernels.cu ----------------------------------------------------------

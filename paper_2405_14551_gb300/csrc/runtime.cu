@@ -979,6 +979,7 @@ struct lb_batch {
   long long ntiles = 0, ngroups = 0, max_rows = 0, total_nodes = 0;
   int halo = 1;  // staging halo of every run: the largest any of them needs
   int tile = 0;
+  int shape = 0;  // the tile shape of the work list (batched_tile)
   int blocks_per_sm = 2;
   bool dirty = true;
   uint64_t graph_launches = 0;  // kernel launches in one replay
@@ -997,9 +998,11 @@ void batch_drop_graphs(lb_batch* b) {
 }
 
 int batch_descriptors(lb_batch* b) {
-  const Tile& T = kTiles[b->tile];
   long long tb = 0, rb = 0;
   b->max_rows = 0;
+  for (lb_handle* h : b->runs) b->max_rows = std::max(b->max_rows, (long long)((h->g.nx + BLK - 1) / BLK) * h->g.ny);
+  b->shape = batched_tile(b->storage, b->tile, b->halo, b->max_rows);
+  const Tile& T = kTiles[b->shape];
   b->h_runs.resize(b->runs.size());
   for (size_t r = 0; r < b->runs.size(); ++r) {
     lb_handle* h = b->runs[r];
@@ -1015,7 +1018,6 @@ int batch_descriptors(lb_batch* b) {
     d.row_begin = rb;
     tb += (long long)((h->g.nx + T.tx - 1) / T.tx) * ((h->g.ny + T.ty - 1) / T.ty) * ((h->g.nz + T.tz - 1) / T.tz);
     rb += ((long long)h->g.ny * h->g.nz + 7) / 8;
-    b->max_rows = std::max(b->max_rows, (long long)((h->g.nx + BLK - 1) / BLK) * h->g.ny);
   }
   b->ntiles = tb;
   b->ngroups = rb;
@@ -1043,7 +1045,7 @@ int batch_descriptors(lb_batch* b) {
 
 // one batched step from lattice parity `parity` and accumulator phase k
 int batch_issue(lb_batch* b, int parity, int k) {
-  LB_CUDA(launch_batched(b->storage, b->d_runs, b->d_run_of, b->ntiles, b->ngroups, b->tile, b->halo,
+  LB_CUDA(launch_batched(b->storage, b->d_runs, b->d_run_of, b->ntiles, b->ngroups, b->shape, b->halo,
                          b->max_rows, parity, k, b->blocks_per_sm, b->runs[0]->status, b->stream));
   g_launches += 2;
   return LB_OK;

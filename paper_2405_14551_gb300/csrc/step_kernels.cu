@@ -113,6 +113,11 @@ cudaError_t launch_batched(int storage, const RunDesc* d_runs, const int* run_of
   return cudaErrorInvalidValue;  // no batched FP64 or moment instantiation
 }
 
+int batched_tile(int storage, int tile, int halo, long long max_rows) {
+  const unsigned long long plane = (unsigned long long)max_rows * BLK * (unsigned long long)state_arrays(storage) * elem_bytes(storage);
+  return halo >= 7 || plane >= (1ull << 32) ? 0 : tile;
+}
+
 int sm_count_host() {
   static int n = 0;
   if (!n) {

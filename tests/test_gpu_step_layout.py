@@ -137,3 +137,25 @@ def test_batch_of_uneven_runs_follows_its_work_list():
         fb, fs = b.fields(r), s.fields()
         for k in fs:
             np.testing.assert_array_equal(fb[k], fs[k], err_msg=f"run {r} field {k}")
+
+
+@pytest.mark.parametrize("h_max", [4.5, 5.9, 6.0])
+def test_batch_with_wide_scan_steps_every_node(h_max):
+    """Scan lengths beyond 3 have one tile shape, whatever the batch's setting."""
+    import paper_2405_14551_gb300.lbcg as L
+    from paper_2405_14551_gb300 import workloads as W
+    p = dict(W.BASE, A_h=0.1, h_min=2.0, h_max=h_max)
+    runs = [W.Workload(f"r{k}", s, 0b010 * k, p, 5, phi=_phi(s, k)) for k, s in enumerate([(40, 24, 20), (33, 17, 21)])]
+    b = L.Batch(runs)
+    L.lb_batch_set_tile(b.b, 5, 2)
+    b.step(6)
+    for r, w in enumerate(runs):
+        for tile in (None, 0, 5):
+            s = L.Sim(*w.shape, walls=w.walls, **w.params)
+            s.init_fields(w.phi)
+            if tile is not None:
+                L.lb_set_tile(s.h, tile)
+            s.step(6)
+            fb, fs = b.fields(r), s.fields()
+            for k in fs:
+                np.testing.assert_array_equal(fb[k], fs[k], err_msg=f"run {r} tile {tile} field {k}")
