@@ -42,7 +42,10 @@ extern "C" {
 #define LB_EIO -7       /* file read/write failed or the file is not a checkpoint of this grid */
 
 /* ---- population storage formats ---------------------------------------- */
-/* Two population sets f^A, f^B in FP32, [comp][27][nz][ny][nx]; 432 B per node update. */
+/* Two population sets f^A, f^B in FP32; 432 B per node update.  (On the device
+ * the populations of every storage but the moments lie in blocks of 32 nodes of
+ * a row, [nz][ny][ceil(nx / 32)][comp * 27][32]; files and lb_get_populations
+ * hold [comp][27][nz][ny][nx].) */
 #define LB_STORAGE_TWOSET_F32 0
 /* Exact single-set form: total post-collision f* (27 x FP32) plus the colour
  * scalars s = rhoA/rho and v = beta rhoA rhoB/rho n (one float4); the pulling
@@ -139,8 +142,8 @@ typedef struct {
  * the host (LB_EINVAL, nothing allocated), then allocates two population
  * lattices in the chosen storage, three accumulators of the component
  * densities (8 bytes per node each, 16 in FP64 storage) that carry phi from
- * one step to the next, and the initial-field arrays.  *out receives the
- * handle (caller-owned; release with lb_destroy). */
+ * one step to the next, the phase field of the current level padded by the
+ * scan's reach, and the initial-field arrays.  *out receives the handle (caller-owned; release with lb_destroy). */
 int lb_create(const lb_grid* grid, const lb_params* params, const lb_alloc* alloc, lb_handle** out);
 
 /* Release all device memory of the handle (after synchronising its stream). */
@@ -175,8 +178,8 @@ int lb_init_fields(lb_handle* h, const float* phi, const float* rho, const float
                    int is_device);
 
 /* Advance nsteps >= 0 time steps, asynchronously on the handle's stream.
- * Each step is one kernel over tiles of nodes: it stages phi of the tile and
- * a halo, runs the near-contact scan of Eqs. stress_jump / near_cont_force
+ * A step is one pass that decodes phi from the density sums and one kernel
+ * over tiles of nodes: it stages phi of the tile and a halo, runs the near-contact scan of Eqs. stress_jump / near_cont_force
  * for the tile's interface nodes (with A_h != 0), pulls, collides, recolours
  * and stores every node (one read and one write of the population state),
  * and adds each stored component population to the density sums of the node
@@ -195,8 +198,8 @@ int lb_set_tile(lb_handle* h, int tile);
 int lb_get_tile(const lb_handle* h);
 
 /* Advance nsteps >= 1 steps without graph replay, recording a CUDA event on
- * the handle's stream after every step kernel.  Synchronises the stream;
- * *ms receives the mean duration of one step kernel in milliseconds. */
+ * the handle's stream after every step.  Synchronises the stream; *ms receives
+ * the mean duration of one step (both kernels) in milliseconds. */
 int lb_step_timed(lb_handle* h, int64_t nsteps, double* ms);
 
 /* Steps taken since the last initialisation. */
@@ -317,9 +320,9 @@ int32_t lb_batch_size(const lb_batch* b);
 int64_t lb_batch_nodes(const lb_batch* b);
 int lb_batch_set_stream(lb_batch* b, void* stream);
 
-/* Advance every run by nsteps: per step one persistent launch over the work
- * list of all runs' (run, tile) items (the step of lb_step on each tile),
- * replayed from a captured CUDA graph.  All runs must be initialised and at
+/* Advance every run by nsteps: per step one launch that decodes phi of all runs
+ * and one persistent launch over the work list of all runs' (run, tile) items
+ * (the step of lb_step on each tile), replayed from a captured CUDA graph.  All runs must be initialised and at
  * the same lattice parity; the first step of freshly initialised runs is
  * taken per run. */
 int lb_batch_step(lb_batch* b, int64_t nsteps);
@@ -327,7 +330,9 @@ int lb_batch_step(lb_batch* b, int64_t nsteps);
 /* The one-run-at-a-time baseline: lb_step on each run in turn. */
 int lb_batch_step_sequential(lb_batch* b, int64_t nsteps);
 
-/* Tile shape (0..5, as lb_set_tile) and persistent CTAs per SM (1..16). */
+/* Tile shape (0..5, as lb_set_tile) and persistent CTAs per SM (1..16).  Runs
+ * that scan 4 nodes or further, or whose z planes exceed 32-bit byte offsets,
+ * put the whole batch on tile 0. */
 int lb_batch_set_tile(lb_batch* b, int tile, int blocks_per_sm);
 
 /* Autotuner: time `steps` batched steps for every tile shape and CTAs-per-SM

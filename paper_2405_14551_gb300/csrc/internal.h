@@ -150,8 +150,12 @@ bool storage_is_f64(int storage);
 
 // --- step_kernels.cu -------------------------------------------------------
 // halo of the phi tile a step stages: 1 without near contact, else 4 (scan
-// length K <= 3) or 7 (K <= 6)
-inline int stage_halo(const Phys& p) { return p.A_h == 0.0 ? 1 : (p.K <= 3 ? 4 : 7); }
+// length K <= 3), 6 (K <= 5) or 7 (K = 6).  The wide halos have one tile, 32x8x4:
+// deeper ones stage fewer values a node but leave one CTA an SM less to hide the
+// scan behind (K = 5 on 150x93x203, us/step: 314 with 32x8x4, 336 with 32x8x8;
+// two-set 339 against 430).  6 instead of 7 for K <= 5: 315 -> 303 us a step
+// of the reduced storage there.
+inline int stage_halo(const Phys& p) { return p.A_h == 0.0 ? 1 : (p.K <= 3 ? 4 : p.K <= 5 ? 6 : 7); }
 // rebuild the accumulator of the current time level from the populations of in
 // one direction of a state (not the moment storage) from its blocks to a plain
 // [z][y][x] array (gather) or back

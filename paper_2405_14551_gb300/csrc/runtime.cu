@@ -2,9 +2,10 @@
 //
 // A handle owns two population lattices (ping-pong), three accumulators of
 // the component densities that carry phi from one step to the next (see
-// step_impl.cuh), the initial-field arrays and small scratch buffers.  Steps
-// are issued asynchronously on the handle's stream, one kernel per step; runs
-// of steps replay a captured CUDA graph of STEPS_PER_GRAPH steps, one graph
+// step_impl.cuh), the padded phase field of the current level, the
+// initial-field arrays and small scratch buffers.  Steps are issued
+// asynchronously on the handle's stream, two kernels per step; runs of steps
+// replay a captured CUDA graph of STEPS_PER_GRAPH steps, one graph
 // per (lattice parity, accumulator phase).
 #include <cuda_runtime.h>
 #include <sys/stat.h>
@@ -1161,7 +1162,7 @@ int lb_batch_create(int32_t nruns, const lb_grid* grids, const lb_params* params
   }
   b->stream = b->own_stream;
   for (int r = 0; r < nruns; ++r)
-    if (params[r].A_h != 0.0) b->halo = std::max(b->halo, params[r].h_max < 4.0 ? 4 : 7);  // stage_halo
+    if (params[r].A_h != 0.0) b->halo = std::max(b->halo, params[r].h_max < 4.0 ? 4 : params[r].h_max < 6.0 ? 6 : 7);  // stage_halo
   for (int r = 0; r < nruns; ++r) {
     lb_handle* h = nullptr;
     int rc = create_handle(&grids[r], &params[r], alloc, b->halo, &h);

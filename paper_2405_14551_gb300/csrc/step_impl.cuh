@@ -2,13 +2,13 @@
 // Device code of the time step of the two-component colour-gradient LB scheme on D3Q27
 // (arXiv 2405.14551, Sec. III.B-III.D) for sm_103a.
 //
-// A step is one kernel, k_step, over CTA tiles of TX x TY x TZ nodes (TX x TY
-// threads, TZ nodes per thread):
-//   1. stage phi(t) of the tile plus a halo of H nodes in shared memory.  phi
-//      is not stored between steps as an array of its own: the step before
-//      accumulated the component densities rhoA, rhoB of every node on the
-//      write side (item 4), and the staging decodes
-//      phi = (rhoA - rhoB)/(rhoA + rhoB) (Eq. order_param) from them;
+// A step is two kernels.  k_phi decodes the phase field of the current level
+// from the component densities that the step before accumulated (item 4), once
+// per node, into an array padded by the staging halo, and zeroes the
+// accumulator two steps ahead.  k_step works on CTA tiles of TX x TY x TZ nodes
+// (TX x TY threads, TZ nodes per thread):
+//   1. stage phi(t) of the tile plus a halo of H nodes in shared memory
+//      (16-byte asynchronous copies from k_phi's array);
 //   2. with near contact (A_h != 0, halo H > K): every interface node of the
 //      tile scans along its outward normal (Eqs. stress_jump,
 //      near_cont_force); the distance h stays in shared memory.  The
@@ -30,12 +30,14 @@
 //      CTA schedule, batching), and it equals what a pull of the stored
 //      populations gives (k_phi_acc rebuilds it that way after a load).
 // The accumulators rotate over three buffers: a step reads phi(t) from one,
-// adds phi(t+1) into the next (zeroed by the step before) and zeroes its own
-// nodes of the third (read by the step before and not read again).  The
-// populations are read and written once per step; the accumulators add 8 B
-// read, 16 B atomically updated and 8 B zeroed per node (FP32 storages).
-// Populations are structure-of-arrays [dir][z][y][x]: for a fixed direction
-// consecutive threads read consecutive addresses (coalesced).
+// adds phi(t+1) into the next (zeroed by the step before) and zeroes the third
+// (read by the step before and not read again).  The populations are read and
+// written once per step; the accumulators and the phase field add 8 B read,
+// 16 B atomically updated, 8 B zeroed and 4 B written and read per node (FP32
+// storages).
+// Populations lie in blocks of 32 nodes of a row, [z][y][x / 32][dir][32]
+// (Lay<ST>): for a fixed direction a warp reads one 128-byte line, and all
+// directions of a node are a constant offset apart.
 #include <cstdio>
 #include <cstdlib>
 #include <type_traits>
@@ -640,7 +642,14 @@ struct Acc<float> {
   static constexpr int W = 1;  // 64-bit words per node, in global and in shared memory
   using S = int;               // sum of one component
   static constexpr float RHO_MAX = 4.0f;
-  __device__ static __forceinline__ S q(float v) { return __float2int_rn(v * 268435456.0f); }
+  static constexpr float SCALE = 268435456.0f;
+  __device__ static __forceinline__ S q(float v) { return __float2int_rn(v * SCALE); }
+  // the same for values that are already multiplied by SCALE (exact: a power of two)
+  __device__ static __forceinline__ void send_shared_scaled(unsigned long long* sw, int E, int e, float a, float b) {
+    int* p = reinterpret_cast<int*>(sw);
+    atomicAdd(p + e, __float2int_rn(a));
+    atomicAdd(p + E + e, __float2int_rn(b));
+  }
   // add one node's contributions (a, b) to the shared partial sums of node e:
   // two planes of E 32-bit words (rhoA, then rhoB) in the E 64-bit words of
   // sw; 32-bit shared atomics (one packed 64-bit shared atomic per direction
@@ -1057,13 +1066,43 @@ __device__ __forceinline__ void put_field(const FieldOut& o, int k, size_t N, si
 // Send the component populations (a, b) of direction i of the node at
 // accumulator index e0 to the node that pulls them: x + c_i, or the node
 // itself when x + c_i is solid (halfway bounce-back).
-template <typename R, bool WALLFREE, int EX, int EXY, int E>
-__device__ __forceinline__ void send(unsigned long long* sw, int e0, const Nbr& n, int i, R a, R b) {
+template <bool WALLFREE, int EX, int EXY>
+__device__ __forceinline__ int send_to(int e0, const Nbr& n, int i) {
   int e = e0 + cx(i) + EX * cy(i) + EXY * cz(i);
   if constexpr (!WALLFREE) {
     if (n.sx[1 + cx(i)] | n.sy[1 + cy(i)] | n.sz[1 + cz(i)]) e = e0;
   }
-  Acc<R>::send_shared(sw, E, e, a, b);
+  return e;
+}
+template <typename R, bool WALLFREE, int EX, int EXY, int E>
+__device__ __forceinline__ void send(unsigned long long* sw, int e0, const Nbr& n, int i, R a, R b) {
+  Acc<R>::send_shared(sw, E, send_to<WALLFREE, EX, EXY>(e0, n, i), a, b);
+}
+
+// Single-set storages: what colour_split gives the puller of the stored total
+// fs (with the colour scalars sv), formed from fs already multiplied by the
+// fixed-point scale.  A power of two passes through every rounding, so these
+// are the bits of colour_split's values times the scale, and the two
+// multiplications a direction fall away (bound by issue; FP16 storage at
+// 128x128x256: 329 -> 322 us a step).
+template <bool WALLFREE, typename L>
+__device__ __forceinline__ void send_split(unsigned long long* sw, int e0, const Nbr& n, int i, float fs, const float4& sv,
+                                           float seg) {
+  const float va = fma_rn(sv.x, fs, seg);
+  Acc<float>::send_shared_scaled(sw, L::E, send_to<WALLFREE, L::EX, L::EXY>(e0, n, i), va, fs - va);
+}
+// the scaled segregation term w_i c_i.v/|c_i| of colour_split
+__device__ __forceinline__ float split_seg(const float4& sv, int i) {
+  float cv = 0.f;
+  if (cx(i)) cv += (float)cx(i) * sv.y;
+  if (cy(i)) cv += (float)cy(i) * sv.z;
+  if (cz(i)) cv += (float)cz(i) * sv.w;
+  return mul_rn(wgt<float>(i) * inv_norm<float>(i) * Acc<float>::SCALE, cv);
+}
+template <int ST>
+__device__ __forceinline__ float decode_scaled(typename Store<ST>::E v, int i) {
+  if constexpr (ST == 2) return fma_rn(__half2float(v), F16_INV_SCALE * Acc<float>::SCALE, wgt<float>(i) * Acc<float>::SCALE);
+  else return mul_rn((float)v, Acc<float>::SCALE);
 }
 
 // Pull, collide, recolour and store every node of the tile; with WS also
@@ -1311,9 +1350,8 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
       // what the neighbours will pull: the quadratic form at each c_i
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
-        R va, vb;
-        colour_split<R, false>(eval_moment<R>(qa, qb, qc, i, false), svo, i, false, va, vb);
-        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, i, va, vb);
+        const float fs = mul_rn(eval_moment<R>(qa, qb, qc, i, false), Acc<float>::SCALE);
+        send_split<WALLFREE, L>(sw, e0, n, i, fs, svo, i == REST ? 0.f : split_seg(svo, i));
       }
       continue;
     }
@@ -1331,9 +1369,7 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
       } else {
         const typename Store<ST>::E enc = encode<ST>(fs, REST);
         op[REST * BLK] = enc;
-        R va, vb;
-        colour_split<R, false>(decode<ST>(enc, REST), svo, REST, false, va, vb);
-        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, REST, va, vb);
+        send_split<WALLFREE, L>(sw, e0, n, REST, decode_scaled<ST>(enc, REST), svo, 0.f);
       }
     }
 #pragma unroll
@@ -1346,7 +1382,7 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
       if (cz(p)) { cu += R(cz(p)) * u2; cF += R(cz(p)) * F2; cg += R(cz(p)) * gr[2]; }
       R even = W * (wf * (r0 + r45 * cu * cu) + g9 * cu * cF + gm3uF + A2ig * cg * cg) - bweight<R>(p) * A2g;
       R odd = W * (wf * r3 * cu + g3 * cF);
-      R bp = f[p], bq = f[q];
+      const R bp = f[p], bq = f[q];
       if constexpr (reg) {
         // c.Pi.c and c.J = -(c.F)/2 for this pair's velocity
         R cpc = R(0);
@@ -1358,11 +1394,9 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
         if (cy(p) && cz(p)) cpc += R(2 * cy(p) * cz(p)) * Pyz;
         even += keep * W * R(4.5) * (cpc - trP * (R(1) / R(3)));
         odd += keep * W * R(-1.5) * cF;
-        bp = R(0);
-        bq = R(0);
       }
-      const R fsp = keep * bp + even + odd;
-      const R fsq = keep * bq + even - odd;
+      const R fsp = reg ? even + odd : keep * bp + even + odd;
+      const R fsq = reg ? even - odd : keep * bq + even - odd;
       if constexpr (Store<ST>::TWOSET) {
         const R seg = segamp * W * inv_norm<R>(p) * cg;
         const R fap = sA * fsp + seg;
@@ -1378,18 +1412,11 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
         const typename Store<ST>::E ep = encode<ST>(fsp, p), eq = encode<ST>(fsq, q);
         op[p * BLK] = ep;
         op[q * BLK] = eq;
-        // colour_split of p and of its opposite q: c_q.v = -(c_p.v) exactly,
-        // so the segregation term is formed once and negated (bit for bit
-        // what colour_split gives for q)
-        R cv = R(0);
-        if (cx(p)) cv += R(cx(p)) * R(svo.y);
-        if (cy(p)) cv += R(cy(p)) * R(svo.z);
-        if (cz(p)) cv += R(cz(p)) * R(svo.w);
-        const R seg = mul_rn(W * inv_norm<R>(p), cv);
-        const R dp = decode<ST>(ep, p), dq = decode<ST>(eq, q);
-        const R vap = fma_rn(R(svo.x), dp, seg), vaq = fma_rn(R(svo.x), dq, -seg);
-        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, p, vap, dp - vap);
-        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, q, vaq, dq - vaq);
+        // p and its opposite q: c_q.v = -(c_p.v) exactly, so the segregation term
+        // is formed once and negated (bit for bit what colour_split gives for q)
+        const float seg = split_seg(svo, p);
+        send_split<WALLFREE, L>(sw, e0, n, p, decode_scaled<ST>(ep, p), svo, seg);
+        send_split<WALLFREE, L>(sw, e0, n, q, decode_scaled<ST>(eq, q), svo, -seg);
       }
     }
   }

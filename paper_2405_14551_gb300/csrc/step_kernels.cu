@@ -115,7 +115,7 @@ cudaError_t launch_batched(int storage, const RunDesc* d_runs, const int* run_of
 
 int batched_tile(int storage, int tile, int halo, long long max_rows) {
   const unsigned long long plane = (unsigned long long)max_rows * BLK * (unsigned long long)state_arrays(storage) * elem_bytes(storage);
-  return halo >= 7 || plane >= (1ull << 32) ? 0 : tile;
+  return halo >= 6 || plane >= (1ull << 32) ? 0 : tile;
 }
 
 int sm_count_host() {

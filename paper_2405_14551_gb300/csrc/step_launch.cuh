@@ -33,12 +33,13 @@ inline bool fits_idx32(const Geo& g) {
   return row * (unsigned long long)g.ny < (1ull << 32);
 }
 
-// Calls f with the staging halo (1, 4 or 7) as a compile-time constant.
+// Calls f with the staging halo (1, 4, 6 or 7) as a compile-time constant.
 template <typename F>
 inline cudaError_t with_stage_halo(int halo, F&& f) {
   switch (halo) {
     case 1: return f(std::integral_constant<int, 1>{});
     case 4: return f(std::integral_constant<int, 4>{});
+    case 6: return f(std::integral_constant<int, 6>{});
     case 7: return f(std::integral_constant<int, 7>{});
   }
   return cudaErrorInvalidValue;
@@ -123,7 +124,7 @@ inline cudaError_t launch_step_tiles(int tile, const Geo& g, const Phys& p, cons
     constexpr int H = decltype(hc)::value;
 #define LBCG_TILE(TY, TZ, I32, MB) \
   launch_step_t<ST, LOADER, WS, WF, 32, TY, TZ, H, I32, MB, SC>(g, p, in, init, src, ab, out, phi, pg, fields, status, st)
-    if constexpr (LOADER == LOAD_PULL && WS && !WF && ST != 3 && H < 7 && !SC) {
+    if constexpr (LOADER == LOAD_PULL && WS && !WF && ST != 3 && H < 6 && !SC) {
       if (i32) {
         switch (tile) {
           case 1:
@@ -219,7 +220,7 @@ cudaError_t launch_batched_t(const RunDesc* d_runs, const int* run_of, long long
     constexpr int H = decltype(hc)::value;
 #define LBCG_TILE(TY, TZ, I32, MB) \
   launch_batched_step_t<ST, 32, TY, TZ, H, I32, MB>(d_runs, run_of, ntiles, parity, k, blocks, status, st)
-    if constexpr (H < 7) {
+    if constexpr (H < 6) {
       if (i32) {
         switch (tile) {
           case 1:
