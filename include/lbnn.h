@@ -95,6 +95,12 @@ int lbnn_up_concat_bwd(const float* dout, int32_t cs, int32_t cl, int32_t nx, in
 int lbnn_relu_bwd(const float* g, const void* y, int64_t n, int32_t relu, void* gb, float* gf, void* stream);
 /* db[c] += sum_v g[v][c] (c divides 256). */
 int lbnn_bias_grad(const float* g, int64_t nvox, int32_t c, float* db, void* stream);
+/* lbnn_relu_bwd and lbnn_bias_grad in one pass over [nvox][c], without the FP32
+ * copy between them: gb = BF16(g (y > 0)) (relu = 0: g, y unused), db[c] +=
+ * sum_v g (y > 0).  c a multiple of 4 that divides 256; g 16-byte, y and gb
+ * 8-byte aligned. */
+int lbnn_relu_bias_bwd(const float* g, const void* y, int64_t nvox, int32_t c, int32_t relu, void* gb, float* db,
+                       void* stream);
 /* weights of the input gradient: wt[ci][t][co] = w[co][taps-1-t][ci]. */
 int lbnn_flip_weights(const void* w, int32_t cout, int32_t taps, int32_t cin, void* wt, void* stream);
 /* weighted MSE over the first nch of c channels: grad = 2 w_c (p - t)/(n nch),

@@ -7,6 +7,7 @@
 
 #include "../../include/lbcg.h"
 #include "../../include/lbnn.h"
+#include "exact_sum.cuh"
 #include "internal.h"
 
 namespace lbcg {
@@ -21,14 +22,30 @@ static unsigned blocks_for(long long n) {
   return (unsigned)(b < 8192 ? (b < 1 ? 1 : b) : 8192);
 }
 
+static bool aligned16(const void* a, const void* b = nullptr, const void* c = nullptr, const void* d = nullptr) {
+  return !(((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 15);
+}
+
 // fields [5][N] (phi, rho, ux, uy, uz; FP32) -> x[N][C] BF16 with
-// (phi, s_rho (rho - 1), s_u ux, s_u uy, s_u uz, 0, ...)
-__global__ void k_pack_input(long long N, const float* __restrict__ f, int C, float s_rho, float s_u,
-                             bf16* __restrict__ x) {
+// (phi, s_rho (rho - 1), s_u ux, s_u uy, s_u uz, 0, ...).  VEC (C % 8 == 0, x
+// 16-byte aligned): whole 16-byte stores; bound by bytes (20 read, 2 C written
+// per node).  At 2.1 M nodes, C = 16: 188 -> 23 us.
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_pack_input(long long N, const float* __restrict__ f, int C, float s_rho, float s_u,
+                                                    bf16* __restrict__ x) {
   for (long long v = grid_stride_begin(); v < N; v += grid_stride()) {
     const float vals[5] = {f[v], s_rho * (f[N + v] - 1.0f), s_u * f[2 * N + v], s_u * f[3 * N + v],
                            s_u * f[4 * N + v]};
-    for (int c = 0; c < C; ++c) x[v * C + c] = __float2bfloat16(c < 5 ? vals[c] : 0.0f);
+    if constexpr (VEC) {
+      __align__(16) bf16 o[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) o[c] = __float2bfloat16(c < 5 ? vals[c] : 0.0f);
+      uint4* d = reinterpret_cast<uint4*>(x + v * C);
+      d[0] = *reinterpret_cast<const uint4*>(o);
+      for (int q = 1; q < C / 8; ++q) d[q] = make_uint4(0, 0, 0, 0);
+    } else {
+      for (int c = 0; c < C; ++c) x[v * C + c] = __float2bfloat16(c < 5 ? vals[c] : 0.0f);
+    }
   }
 }
 
@@ -47,13 +64,22 @@ __global__ void k_unpack_output(long long N, const float* __restrict__ f, const 
   }
 }
 
-// training target t[N][C] (FP32): scaled increments between two field sets
-__global__ void k_pack_target(long long N, const float* __restrict__ f0, const float* __restrict__ f1, int C,
-                              float s_rho, float s_u, float* __restrict__ t) {
+// training target t[N][C] (FP32): scaled increments between two field sets;
+// VEC (C % 4 == 0, t 16-byte aligned): whole 16-byte stores
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_pack_target(long long N, const float* __restrict__ f0, const float* __restrict__ f1,
+                                                     int C, float s_rho, float s_u, float* __restrict__ t) {
   for (long long v = grid_stride_begin(); v < N; v += grid_stride()) {
     const float d[5] = {f1[v] - f0[v], s_rho * (f1[N + v] - f0[N + v]), s_u * (f1[2 * N + v] - f0[2 * N + v]),
                         s_u * (f1[3 * N + v] - f0[3 * N + v]), s_u * (f1[4 * N + v] - f0[4 * N + v])};
-    for (int c = 0; c < C; ++c) t[v * C + c] = c < 5 ? d[c] : 0.0f;
+    if constexpr (VEC) {
+      float4* o = reinterpret_cast<float4*>(t + v * C);
+      o[0] = make_float4(d[0], d[1], d[2], d[3]);
+      o[1] = make_float4(d[4], 0.f, 0.f, 0.f);
+      for (int q = 2; q < C / 4; ++q) o[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      for (int c = 0; c < C; ++c) t[v * C + c] = c < 5 ? d[c] : 0.0f;
+    }
   }
 }
 
@@ -136,6 +162,38 @@ __global__ void k_avgpool2_bwd(const float* __restrict__ dy, int C, int nx, int 
     const int z = (int)(r % nz);
     const int b = (int)(r / nz);
     dx[e] += 0.125f * dy[((((long long)b * oz + z / 2) * oy + y / 2) * ox + x / 2) * C + c];
+  }
+}
+
+__device__ __forceinline__ float4 add4(float4 a, float4 b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
+// The same four channels (16 bytes) at a time, for C % 4 == 0: a thread reads a
+// parent once and updates its eight children, so the index arithmetic and the
+// parent's bytes are shared by eight nodes.  Bound by bytes (the read and the
+// write of dx).  128^3 x 32 channels: 340 -> 78 us.
+__global__ void __launch_bounds__(256) k_avgpool2_bwd_v4(const float4* __restrict__ dy, int G, int nx, int ny, int nz, int nb,
+                                                         float4* __restrict__ dx) {
+  const int ox = nx / 2, oy = ny / 2, oz = nz / 2;
+  const long long n = (long long)nb * oz * oy * ox * G;
+  for (long long e = grid_stride_begin(); e < n; e += grid_stride()) {
+    const long long pv = e / G;
+    const int g = (int)(e - pv * G);
+    long long r = pv / ox;
+    const int x = (int)(pv - r * ox) * 2;
+    const int y = (int)(r % oy) * 2;
+    r /= oy;
+    const int z = (int)(r % oz) * 2, b = (int)(r / oz);
+    const float4 d = dy[e];
+    float4* c[8];
+    float4 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      c[k] = dx + ((((long long)b * nz + z + (k >> 2)) * ny + y + (k >> 1 & 1)) * nx + x + (k & 1)) * G + g;
+      v[k] = *c[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      *c[k] = make_float4(v[k].x + 0.125f * d.x, v[k].y + 0.125f * d.y, v[k].z + 0.125f * d.z, v[k].w + 0.125f * d.w);
   }
 }
 
@@ -223,6 +281,36 @@ __global__ void k_up_concat_bwd(const float* __restrict__ dout, int Cs, int Cl, 
   }
 }
 
+// The same four channels (16 bytes) at a time, for Cs % 4 == Cl % 4 == 0, the
+// eight children summed in the same order.
+__global__ void __launch_bounds__(256) k_up_concat_bwd_v4(const float4* __restrict__ dout, int Gs, int Gl, int nx, int ny,
+                                                          int nz, int nb, float4* __restrict__ dskip,
+                                                          float4* __restrict__ dlow) {
+  const int G = Gs + Gl, ox = nx / 2, oy = ny / 2, oz = nz / 2;
+  const long long nl = (long long)nb * oz * oy * ox * Gl;
+  for (long long e = grid_stride_begin(); e < nl; e += grid_stride()) {
+    const long long pv = e / Gl;
+    const int g = (int)(e - pv * Gl);
+    long long r = pv / ox;
+    const int x = (int)(pv - r * ox) * 2;
+    const int y = (int)(r % oy) * 2;
+    r /= oy;
+    const int z = (int)(r % oz) * 2, b = (int)(r / oz);
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const long long v = (((long long)b * nz + z + (k >> 2)) * ny + y + (k >> 1 & 1)) * nx + x + (k & 1);
+      s = add4(s, dout[v * G + Gs + g]);
+    }
+    dlow[e] = add4(dlow[e], s);
+  }
+  const long long ns = (long long)nb * nz * ny * nx * Gs;
+  for (long long e = grid_stride_begin(); e < ns; e += grid_stride()) {
+    const long long v = e / Gs;
+    dskip[e] = add4(dskip[e], dout[v * G + (e - v * Gs)]);
+  }
+}
+
 // g_pre = g_post * (y > 0) (ReLU), as BF16 operand plus optional FP32 copy
 __global__ void k_relu_bwd(long long n, const float* __restrict__ g, const bf16* __restrict__ y, int relu,
                            bf16* __restrict__ gb, float* __restrict__ gf) {
@@ -231,6 +319,59 @@ __global__ void k_relu_bwd(long long n, const float* __restrict__ g, const bf16*
     if (relu && !(__bfloat162float(y[e]) > 0.0f)) v = 0.0f;
     if (gb) gb[e] = __float2bfloat16(v);
     if (gf) gf[e] = v;
+  }
+}
+
+// The gradient through ReLU and the bias gradient in one pass over [nvox][C]:
+// gb = BF16(g (y > 0)), db[c] += sum_v g (y > 0) (FP32).  A thread owns four
+// channels (C % 4 == 0, C / 4 divides 256) and keeps their sums in registers;
+// the FP32 copy that a separate bias pass would read is never written.  Bound
+// by bytes (8 per element: g, y read, gb written).  128^3 x 32 channels:
+// relu_bwd + bias_grad 214 -> 77 us.
+__global__ void __launch_bounds__(256) k_relu_bias_bwd(long long nvox, int G, const float4* __restrict__ g,
+                                                       const uint2* __restrict__ y, uint2* __restrict__ gb,
+                                                       float* __restrict__ db) {
+  __shared__ float4 red[256];
+  const int lanes = 256 / G, lane = threadIdx.x / G, q = threadIdx.x - lane * G;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  const long long step = (long long)gridDim.x * lanes;
+  constexpr int U = 4;  // voxels in flight
+  for (long long v0 = (long long)blockIdx.x * lanes + lane; v0 < nvox; v0 += U * step) {
+    float4 a[U];
+    uint2 m[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const long long v = v0 + u * step;
+      if (v >= nvox) continue;
+      a[u] = g[v * G + q];
+      if (y) m[u] = y[v * G + q];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const long long v = v0 + u * step;
+      if (v >= nvox) continue;
+      if (y) {
+        const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&m[u].x));
+        const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&m[u].y));
+        if (!(lo.x > 0.0f)) a[u].x = 0.0f;
+        if (!(lo.y > 0.0f)) a[u].y = 0.0f;
+        if (!(hi.x > 0.0f)) a[u].z = 0.0f;
+        if (!(hi.y > 0.0f)) a[u].w = 0.0f;
+      }
+      s = add4(s, a[u]);
+      const __nv_bfloat162 lo = __floats2bfloat162_rn(a[u].x, a[u].y), hi = __floats2bfloat162_rn(a[u].z, a[u].w);
+      gb[v * G + q] = make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
+    }
+  }
+  red[threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.x < G) {
+    for (int l = 1; l < lanes; ++l) s = add4(s, red[l * G + threadIdx.x]);
+    float* d = db + 4 * threadIdx.x;
+    atomicAdd(d, s.x);
+    atomicAdd(d + 1, s.y);
+    atomicAdd(d + 2, s.z);
+    atomicAdd(d + 3, s.w);
   }
 }
 
@@ -283,6 +424,56 @@ __global__ void __launch_bounds__(256) k_mse(long long N, int C, int nch, const 
   if (threadIdx.x == 0) atomicAdd(loss, red[0] * inv_count);
 }
 
+// The same four channels at a time (C % 4 == 0): quads past nch only store
+// their zeros, the index arithmetic is once per quad, and a thread's share of
+// the loss is summed in Sum3 terms (an FP64 product per element ran on the 2
+// FP64 lanes a clock and bounded the kernel, 254 us); a share that overflows
+// FP32 is taken again in FP64.  Bound by bytes.  128^3 nodes, C = 16, nch = 5:
+// 281 -> 85 us.
+__global__ void __launch_bounds__(256) k_mse_v4(long long N, int G, int nch, const float4* __restrict__ p,
+                                                const float4* __restrict__ t, const float* __restrict__ wch,
+                                                float inv_count, float4* __restrict__ grad, double* __restrict__ loss) {
+  __shared__ double red[256];
+  Sum3 sum;
+  for (long long e = grid_stride_begin(); e < N * G; e += grid_stride()) {
+    const int c0 = (int)(e % G) * 4;
+    float o[4] = {0.f, 0.f, 0.f, 0.f};
+    if (c0 < nch) {
+      const float4 a = p[e], b = t[e];
+      const float d[4] = {a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (c0 + k >= nch) continue;
+        const float w = wch[c0 + k];
+        const float ds = __fmul_rn(d[k], SQUARE_SCALE);
+        const float q = __fmul_rn(w, ds), r = __fmaf_rn(w, ds, -q);  // w d = q + r
+        sum.add_product(q, ds);
+        sum.add(__fmul_rn(r, ds));
+        o[k] = 2.0f * w * d[k] * inv_count;
+      }
+    }
+    grad[e] = make_float4(o[0], o[1], o[2], o[3]);
+  }
+  double s = sum.value() * SQUARE_UNSCALE;
+  if (!sum.finite()) {
+    s = 0.0;
+    for (long long e = grid_stride_begin(); e < N * G; e += grid_stride()) {
+      const int c0 = (int)(e % G) * 4;
+      if (c0 >= nch) continue;
+      const float4 a = p[e], b = t[e];
+      const float d[4] = {a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w};
+      for (int k = 0; k < 4 && c0 + k < nch; ++k) s += (double)wch[c0 + k] * d[k] * d[k];
+    }
+  }
+  red[threadIdx.x] = s;
+  __syncthreads();
+  for (int w = 128; w > 0; w >>= 1) {
+    if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) atomicAdd(loss, red[0] * inv_count);
+}
+
 // Adam on FP32 master weights, BF16 copy for the kernels (bf may be null)
 __global__ void k_adam(long long n, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2, float wd,
@@ -320,7 +511,8 @@ extern "C" {
 
 int lbnn_pack_input(const float* fields, int64_t n, int32_t c, float s_rho, float s_u, void* x, void* stream) {
   if (!fields || !x || n < 1 || c < 5) return report_error(LB_EINVAL, "pack_input arguments");
-  k_pack_input<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(n, fields, c, s_rho, s_u, (bf16*)x);
+  if (c % 8 == 0 && aligned16(x)) k_pack_input<true><<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(n, fields, c, s_rho, s_u, (bf16*)x);
+  else k_pack_input<false><<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(n, fields, c, s_rho, s_u, (bf16*)x);
   return launch_result("pack_input");
 }
 
@@ -334,7 +526,8 @@ int lbnn_unpack_output(const float* fields, const float* y, int64_t n, int32_t c
 int lbnn_pack_target(const float* f0, const float* f1, int64_t n, int32_t c, float s_rho, float s_u, float* t,
                      void* stream) {
   if (!f0 || !f1 || !t || n < 1 || c < 5) return report_error(LB_EINVAL, "pack_target arguments");
-  k_pack_target<<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(n, f0, f1, c, s_rho, s_u, t);
+  if (c % 4 == 0 && c >= 8 && aligned16(t)) k_pack_target<true><<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(n, f0, f1, c, s_rho, s_u, t);
+  else k_pack_target<false><<<blocks_for(n), 256, 0, (cudaStream_t)stream>>>(n, f0, f1, c, s_rho, s_u, t);
   return launch_result("pack_target");
 }
 
@@ -353,8 +546,11 @@ int lbnn_avgpool2(const void* x, int32_t c, int32_t nx, int32_t ny, int32_t nz, 
 int lbnn_avgpool2_bwd(const float* dy, int32_t c, int32_t nx, int32_t ny, int32_t nz, int32_t nb, float* dx,
                       void* stream) {
   if (!dy || !dx || c < 1 || nx % 2 || ny % 2 || nz % 2 || nb < 1) return report_error(LB_EINVAL, "avgpool2_bwd");
-  k_avgpool2_bwd<<<blocks_for((long long)nb * nz * ny * nx * c), 256, 0, (cudaStream_t)stream>>>(dy, c, nx, ny, nz,
-                                                                                                 nb, dx);
+  if (c % 4 == 0 && aligned16(dy, dx))
+    k_avgpool2_bwd_v4<<<blocks_for((long long)nb * nz * ny * nx * c / 32), 256, 0, (cudaStream_t)stream>>>(
+        (const float4*)dy, c / 4, nx, ny, nz, nb, (float4*)dx);
+  else
+    k_avgpool2_bwd<<<blocks_for((long long)nb * nz * ny * nx * c), 256, 0, (cudaStream_t)stream>>>(dy, c, nx, ny, nz, nb, dx);
   return launch_result("avgpool2_bwd");
 }
 
@@ -375,8 +571,12 @@ int lbnn_up_concat_bwd(const float* dout, int32_t cs, int32_t cl, int32_t nx, in
                        float* dskip, float* dlow, void* stream) {
   if (!dout || !dskip || !dlow || cs < 1 || cl < 1 || nx % 2 || ny % 2 || nz % 2 || nb < 1)
     return report_error(LB_EINVAL, "up_concat_bwd arguments");
-  k_up_concat_bwd<<<blocks_for((long long)nb * nz * ny * nx * (cs + cl)), 256, 0, (cudaStream_t)stream>>>(
-      dout, cs, cl, nx, ny, nz, nb, dskip, dlow);
+  if (cs % 4 == 0 && cl % 4 == 0 && aligned16(dout, dskip, dlow))
+    k_up_concat_bwd_v4<<<blocks_for((long long)nb * nz * ny * nx * cs / 4), 256, 0, (cudaStream_t)stream>>>(
+        (const float4*)dout, cs / 4, cl / 4, nx, ny, nz, nb, (float4*)dskip, (float4*)dlow);
+  else
+    k_up_concat_bwd<<<blocks_for((long long)nb * nz * ny * nx * (cs + cl)), 256, 0, (cudaStream_t)stream>>>(
+        dout, cs, cl, nx, ny, nz, nb, dskip, dlow);
   return launch_result("up_concat_bwd");
 }
 
@@ -392,6 +592,20 @@ int lbnn_bias_grad(const float* g, int64_t nvox, int32_t c, float* db, void* str
   return launch_result("bias_grad");
 }
 
+int lbnn_relu_bias_bwd(const float* g, const void* y, int64_t nvox, int32_t c, int32_t relu, void* gb, float* db,
+                       void* stream) {
+  if (!g || !gb || !db || nvox < 1 || c < 1 || c > 256 || 256 % c || (relu && !y))
+    return report_error(LB_EINVAL, "relu_bias_bwd arguments");
+  if (c % 4 || !aligned16(g) || (((uintptr_t)gb | (uintptr_t)(relu ? y : nullptr)) & 7))
+    return report_error(LB_EINVAL, "relu_bias_bwd needs c % 4 == 0, a 16-byte aligned g and 8-byte aligned y and gb");
+  // three CTAs an SM: enough loads in flight, and few enough that their atomics
+  // on the c sums do not queue (eight: 29 us at 262144 voxels x 128 channels)
+  const long long need = (nvox * (c / 4) + 255) / 256;
+  k_relu_bias_bwd<<<(unsigned)(need < 456 ? need : 456), 256, 0, (cudaStream_t)stream>>>(
+      nvox, c / 4, (const float4*)g, relu ? (const uint2*)y : nullptr, (uint2*)gb, db);
+  return launch_result("relu_bias_bwd");
+}
+
 int lbnn_flip_weights(const void* w, int32_t cout, int32_t taps, int32_t cin, void* wt, void* stream) {
   if (!w || !wt || cout < 1 || cin < 1 || (taps != 1 && taps != 27)) return report_error(LB_EINVAL, "flip_weights");
   k_flip_weights<<<blocks_for((long long)cout * taps * cin), 256, 0, (cudaStream_t)stream>>>((const bf16*)w, cout, taps,
@@ -402,8 +616,11 @@ int lbnn_flip_weights(const void* w, int32_t cout, int32_t taps, int32_t cin, vo
 int lbnn_mse(const float* p, const float* t, int64_t n, int32_t c, int32_t nch, const float* wch, float* grad,
              double* loss, void* stream) {
   if (!p || !t || !wch || !grad || !loss || n < 1 || nch < 1 || nch > c) return report_error(LB_EINVAL, "mse");
-  k_mse<<<blocks_for(n * c), 256, 0, (cudaStream_t)stream>>>(n, c, nch, p, t, wch, 1.0f / (float)(n * nch), grad,
-                                                             loss);
+  if (c % 4 == 0 && aligned16(p, t, grad))
+    k_mse_v4<<<blocks_for(n * c / 4) < 912 ? blocks_for(n * c / 4) : 912, 256, 0, (cudaStream_t)stream>>>(n, c / 4, nch, (const float4*)p, (const float4*)t, wch,
+                                                                      1.0f / (float)(n * nch), (float4*)grad, loss);
+  else
+    k_mse<<<blocks_for(n * c), 256, 0, (cudaStream_t)stream>>>(n, c, nch, p, t, wch, 1.0f / (float)(n * nch), grad, loss);
   return launch_result("mse");
 }
 

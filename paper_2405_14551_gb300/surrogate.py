@@ -198,10 +198,8 @@ class UNet:
         T = self.torch
         y = self.acts[("act", name)] if name != "head" else None
         gpre_b = self._buf(("gpre_b", name), (nv, co), T.bfloat16)
-        gpre_f = self._buf(("gpre_f", name), (nv, co), T.float32)
-        self._check(self.lib.lbnn_relu_bwd(_p(g), _p(y) if y is not None else None, nv * co, relu if name != "head" else 0,
-                                           _p(gpre_b), _p(gpre_f), self.sp), "relu_bwd")
-        self._check(self.lib.lbnn_bias_grad(_p(gpre_f), nv, co, _p(self.gb[name]), self.sp), "bias_grad")
+        self._check(self.lib.lbnn_relu_bias_bwd(_p(g), _p(y) if y is not None else None, nv, co, relu if name != "head" else 0,
+                                                _p(gpre_b), _p(self.gb[name]), self.sp), "relu_bias_bwd")
         x = self.acts[("in", name)]
         if isinstance(x, tuple):  # fused up-concat in forward: build the concatenated input now
             key, skip, cs, low, cl, lev = x
