@@ -20,6 +20,7 @@
 // up sets bit 4 of the status word.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <atomic>
 #include <string>
 
@@ -204,12 +205,18 @@ __global__ void __launch_bounds__(128, 1)
 // forward / input gradient, spatially tiled and pipelined (3x3x3 taps)
 // ---------------------------------------------------------------------------
 // Work item: an output block of 8 (x) x 16 (y) x TZ (z) voxels and CT output
-// channels (CT = Cout, or a slice of it when Cout is large and the grid
-// small).  Persistent CTAs walk the work items; warps have fixed roles:
+// channels (CT = Cout or a slice of it, pconv_choose).  Persistent CTAs walk the work items; warps have fixed roles:
 //   warps 0-3  epilogue: tensor memory -> bias, ReLU -> BF16 / FP32 stores
-//   warps 4-7  copies (cp.async, zero fill for padded voxels)
-//   warp 8     tensor-memory allocation; lane 0 issues the UMMAs
-// and hand buffers over through mbarriers only.
+//   the next 4 (8 without MERGE) weight copies, the next 8 input copies
+//              (cp.async, zero fill for padded voxels)
+//   last warp  tensor-memory allocation; one elected lane issues the UMMAs
+// and hand buffers over through mbarriers only.  A weight thread signals a slot
+// PCONV_LAG steps after filling it, so several steps are in flight; with one
+// group of 128 threads copying both operands in turn and 8 slots the UMMAs
+// waited for every halo.  Bound now: the copies (L2 to shared memory at 20 bytes
+// of sectors a cycle and SM) and the UMMAs' operand reads, about equally.
+// 128x128x256 voxels, 32 + 64 -> 32 channels: 1098 -> 835 us with the roles split
+// and the ring deeper, 760 with the issue from a converged warp.
 //
 // Per chunk of KC input channels the input block with a one-voxel halo
 // (10 x 18 x (TZ + 2) voxels) is staged once, in the layout
@@ -236,13 +243,19 @@ __global__ void __launch_bounds__(128, 1)
 // of one work item overlaps the UMMAs of the next.  Every wait is bounded; a
 // wait that gives up sets bit 4 of the status word and the CTA winds down.
 constexpr int PCONV_EPI = 128;     // epilogue threads (warps 0-3, one per tensor-memory lane quarter)
-constexpr int PCONV_THREADS = 288;
-constexpr int PCONV_PROD0 = 128;  // first copy thread
-constexpr int PCONV_NPROD = 128;  // copy threads
-constexpr int PCONV_MMA_WARP = 8;
-constexpr int PCONV_MAXWP = 8;    // weight pieces per copy thread and step (3 CT or CT rows x KC / 8 <= 1024)
-constexpr int PCONV_LAG = 5;      // steps a copy thread keeps in flight before it signals them
-constexpr int PCONV_NSW_MAX = 8;  // weight ring slots (at most)
+constexpr int PCONV_PROD0 = 128;   // first copy thread
+// Threads staging weights: warps 4-7 with MERGE (halo-heavy: few channels, deep
+// blocks), warps 4-11 without (weight-heavy: 128 or more output channels).
+constexpr int pconv_nwgt(bool merge) { return merge ? 128 : 256; }
+constexpr int PCONV_NHALO = 256;   // threads staging input halos (the next 8 warps)
+constexpr int pconv_threads(bool merge) { return PCONV_EPI + pconv_nwgt(merge) + PCONV_NHALO + 32; }
+constexpr int WCONV_NPROD = 256;   // copy threads of the weight gradient (all stage both operands)
+constexpr int WCONV_MMA_WARP = (PCONV_EPI + WCONV_NPROD) / 32;
+constexpr int WCONV_THREADS = PCONV_EPI + WCONV_NPROD + 32;
+constexpr int PCONV_MAXW = 1024;   // weight pieces per step (3 CT or CT rows x KC / 8)
+constexpr int PCONV_LAG = 2;       // steps a weight thread keeps in flight before it signals them
+constexpr int PCONV_NSW_MIN = 7;   // weight ring slots
+constexpr int PCONV_NSW_MAX = 16;
 
 __device__ __forceinline__ int wrap_or_pad(int c, int n, int periodic) {
   if (c >= 0 && c < n) return c;
@@ -262,6 +275,24 @@ __device__ __forceinline__ bool pconv_wait(uint64_t* bar, uint32_t parity, volat
   return false;
 }
 
+// The same for a whole warp, which stays converged.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, uint32_t limit) {
+  return __all_sync(0xffffffffu, pconv_wait(bar, parity, abort_flag, limit));
+}
+
+// 32 bytes at dst (16-byte aligned; wide: 32-byte aligned, one store)
+__device__ __forceinline__ void store32(void* dst, const uint32_t w[8], bool wide) {
+  if (wide) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                 "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+  } else {
+    uint4* p = reinterpret_cast<uint4*>(dst);
+    p[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    p[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
 struct PConvArgs {
   const __nv_bfloat16* X;   // input channels [0, cs): X[v][cs]
   const __nv_bfloat16* X2;  // input channels [cs, Cin), nearest x2 upsampled: X2[parent(v)][Cin - cs] (or null)
@@ -278,14 +309,15 @@ struct PConvArgs {
 };
 
 template <int TZ, bool MERGE>
-__global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P) {
+__global__ void __launch_bounds__(pconv_threads(MERGE), 1) k_conv_fwd_pipe(PConvArgs P) {
+  constexpr int NWGT = pconv_nwgt(MERGE), MMA_WARP = (PCONV_EPI + NWGT + PCONV_NHALO) / 32, MAXWP = PCONV_MAXW / NWGT;
   constexpr int SZH = TZ + 2;
   constexpr int HV = 10 * 18 * SZH;  // staged voxels
   constexpr int NBLK = MERGE ? 3 : 1;
   constexpr int SPC = MERGE ? 9 : 27;  // steps per chunk
   extern __shared__ __align__(1024) unsigned char smem[];
   const int t = threadIdx.x;
-  const int warp = t >> 5;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // uniform, also to the compiler
   const int KC = P.KC, CT = P.CT, Cin = P.Cin, nsw = P.nsw;
   const int NB = NBLK * CT;  // rows of a staged B operand
   const int cgs = KC / 8;
@@ -305,19 +337,19 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
   float* sbias = reinterpret_cast<float*>(tmem_slot + 4);  // Cout values (0 without bias)
   uint32_t ncols = 32;
   while ((int)ncols < 2 * TZ * CT) ncols <<= 1;
-  for (int c = t; c < P.Cout; c += PCONV_THREADS) sbias[c] = P.bias ? P.bias[c] : 0.0f;
+  for (int c = t; c < P.Cout; c += pconv_threads(MERGE)) sbias[c] = P.bias ? P.bias[c] : 0.0f;
 
-  if (warp == PCONV_MMA_WARP) {
+  if (warp == MMA_WARP) {
     tc::tmem_alloc(tmem_slot, ncols);
     tc::tmem_relinquish();
   }
   if (t == 0) {
     for (int k = 0; k < PCONV_NSW_MAX; ++k) {
-      tc::mbar_init(&w_full[k], PCONV_NPROD);
+      tc::mbar_init(&w_full[k], NWGT);
       tc::mbar_init(&w_empty[k], 1);
     }
     for (int k = 0; k < 2; ++k) {
-      tc::mbar_init(&h_full[k], PCONV_NPROD);
+      tc::mbar_init(&h_full[k], PCONV_NHALO);
       tc::mbar_init(&h_empty[k], 1);
       tc::mbar_init(&a_full[k], 1);
       tc::mbar_init(&a_empty[k], PCONV_EPI);
@@ -329,7 +361,7 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   const ConvGeo& g = P.g;
   const int bxs = g.nx / 8, bys = g.ny / 16, bzs = g.nz / TZ;
@@ -349,78 +381,50 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
     b = it / bzs;
   };
 
-  if (t >= PCONV_PROD0 && t < PCONV_PROD0 + PCONV_NPROD) {
-    // ------------------------------------------------------------ copies
+  if (t >= PCONV_PROD0 && t < PCONV_PROD0 + NWGT) {
+    // ------------------------------------------------------------ weight copies
     const int pt = t - PCONV_PROD0;
     const int nsteps = my_items * nchunks * SPC;
-    // Weight pieces: a copy thread stages the same (k group, row) positions
-    // of every step, so their offsets are set up once; a step only adds its
-    // tap and channel chunk.
-    int woff[PCONV_MAXWP];
-    uint32_t wdo[PCONV_MAXWP];
+    // A copy thread stages the same (k group, row) positions of every step, so
+    // their offsets are set up once; a step only adds its tap and channel chunk.
+    int woff[MAXWP];
+    uint32_t wdo[MAXWP];
 #pragma unroll
-    for (int i = 0; i < PCONV_MAXWP; ++i) {
-      const int p = pt + i * PCONV_NPROD;
+    for (int i = 0; i < MAXWP; ++i) {
+      const int p = pt + i * NWGT;
       const int kg = p % cgs, n = p / cgs;
       woff[i] = p < NB * cgs ? ((n % CT) * 27 + 9 * (n / CT)) * Cin + kg * 8 : -1;
       wdo[i] = (uint32_t)(kg * NB + n) * 16;
     }
-    // Input pieces: one staged row (zz, yy) holds 10 x voxels x cgs groups;
-    // a thread keeps its (xx, group) place in the row and walks the rows.
-    const int hl = 10 * cgs, hr = PCONV_NPROD / hl;
-    const bool hact = pt < hr * hl;
-    const int hq = (pt % hl) % cgs, hxx = (pt % hl) / cgs, hy0 = pt / hl;
     bool ok = true;
-    int gs = 0;
+    int gs = 0, slot = 0, hslot = 0;  // step, its slot, the slot of step gs - LAG
+    uint32_t ephase = 1;              // parity of the slot's last release
     for (int k = 0; k < my_items && ok; ++k) {
       int x0, y0, z0, b, n0;
       item_of(k, x0, y0, z0, b, n0);
-      const int gx = wrap_or_pad(x0 - 1 + hxx, g.nx, g.px);
-      const int cl = Cin - P.cs;
       const __nv_bfloat16* wbase = P.W + (size_t)n0 * 27 * Cin;
       for (int c = 0; c < nchunks && ok; ++c) {
         const int c0 = c * KC;
         for (int st = 0; st < SPC; ++st, ++gs) {
-          const int slot = gs % nsw;
-          if (gs >= nsw && !pconv_wait(&w_empty[slot], (uint32_t)(((gs / nsw) - 1) & 1), abort_flag, P.spin)) {
+          if (gs >= nsw && !pconv_wait(&w_empty[slot], ephase, abort_flag, P.spin)) {
             ok = false;
             break;
           }
           unsigned char* wdst = sW + (size_t)slot * w_bytes;
           const __nv_bfloat16* wsrc = wbase + st * Cin + c0;
 #pragma unroll
-          for (int i = 0; i < PCONV_MAXWP; ++i)
+          for (int i = 0; i < MAXWP; ++i)
             if (woff[i] >= 0) tc::cp_async16(wdst + wdo[i], wsrc + woff[i], true);
-          if (st == 0) {
-            const int cg = gs / SPC;
-            if (cg >= 2 && !pconv_wait(&h_empty[cg & 1], (uint32_t)(((cg >> 1) - 1) & 1), abort_flag, P.spin)) {
-              ok = false;
-              break;
-            }
-            if (hact) {
-              unsigned char* hdst = sH + (size_t)(cg & 1) * halo_bytes + ((size_t)hq * SZH * 180 + hxx) * 16;
-              // a chunk lies wholly in one source (KC divides cs); the second is read at the parent voxel
-              const bool up = c0 >= P.cs;
-              const __nv_bfloat16* hsrc = up ? P.X2 + (c0 - P.cs) + hq * 8 : P.X + c0 + hq * 8;
-              const int sh = up ? 1 : 0, ld = up ? cl : P.cs;
-              const int nyv = g.ny >> sh, nxv = g.nx >> sh, nzv = g.nz >> sh, gxv = gx >> sh;
-              for (int row = hy0; row < SZH * 18; row += hr) {
-                const int zz = row / 18, yy = row - 18 * zz;
-                const int gy = wrap_or_pad(y0 - 1 + yy, g.ny, g.py);
-                const int gz = wrap_or_pad(z0 - 1 + zz, g.nz, g.pz);
-                const bool in = gx >= 0 && gy >= 0 && gz >= 0;
-                const int v = in ? ((b * nzv + (gz >> sh)) * nyv + (gy >> sh)) * nxv + gxv : 0;
-                tc::cp_async16(hdst + (size_t)row * 160, hsrc + (long long)v * ld, in);
-              }
-            }
-          }
           tc::cp_async_commit();
+          if (++slot == nsw) {
+            slot = 0;
+            ephase ^= 1u;
+          }
           if (gs >= PCONV_LAG) {  // step gs - LAG has landed: hand it over
             tc::cp_async_wait<PCONV_LAG>();
             tc::fence_proxy_async_smem();
-            const int r = gs - PCONV_LAG;
-            tc::mbar_arrive(&w_full[r % nsw]);
-            if (r % SPC == 0) tc::mbar_arrive(&h_full[(r / SPC) & 1]);
+            tc::mbar_arrive(&w_full[hslot]);
+            if (++hslot == nsw) hslot = 0;
           }
         }
       }
@@ -429,16 +433,78 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
     tc::fence_proxy_async_smem();
     if (ok) {
       for (int r = nsteps > PCONV_LAG ? nsteps - PCONV_LAG : 0; r < nsteps; ++r) {
-        tc::mbar_arrive(&w_full[r % nsw]);
-        if (r % SPC == 0) tc::mbar_arrive(&h_full[(r / SPC) & 1]);
+        tc::mbar_arrive(&w_full[hslot]);
+        if (++hslot == nsw) hslot = 0;
       }
     } else {
       *abort_flag = 1;
       atomicOr(P.status, CONV_TIMEOUT);
     }
-  } else if (warp == PCONV_MMA_WARP) {
+  } else if (t >= PCONV_PROD0 + NWGT && t < PCONV_PROD0 + NWGT + PCONV_NHALO) {
+    // ------------------------------------------------------------ input copies
+    // One staged row (zz, yy) holds 10 x voxels x cgs groups; a thread keeps its
+    // (xx, group) place in the row and walks the rows.
+    const int pt = t - PCONV_PROD0 - NWGT;
+    // hr, the rows the group takes side by side, divides the 18 rows of a plane,
+    // so that a thread's rows keep their y in every plane.
+    const int hl = 10 * cgs, hmax = PCONV_NHALO / hl;
+    const int hr = hmax >= 18 ? 18 : (hmax >= 9 ? 9 : (hmax >= 6 ? 6 : 3));
+    const int nr = 18 / hr;  // rows of a plane per thread: 1 to 6
+    const bool hact = pt < hr * hl;
+    const int hq = (pt % hl) % cgs, hxx = (pt % hl) / cgs, hy0 = pt / hl;
+    const int cl = Cin - P.cs;
+    bool ok = true;
+    int cg = 0;
+    for (int k = 0; k < my_items && ok; ++k) {
+      int x0, y0, z0, b, n0;
+      item_of(k, x0, y0, z0, b, n0);
+      const int gx = wrap_or_pad(x0 - 1 + hxx, g.nx, g.px);
+      for (int c = 0; c < nchunks; ++c, ++cg) {
+        const int c0 = c * KC;
+        if (cg >= 2 && !pconv_wait(&h_empty[cg & 1], (uint32_t)(((cg >> 1) - 1) & 1), abort_flag, P.spin)) {
+          ok = false;
+          break;
+        }
+        if (hact) {
+          unsigned char* hdst = sH + (size_t)(cg & 1) * halo_bytes + ((size_t)hq * SZH * 180 + hy0 * 10 + hxx) * 16;
+          // a chunk lies wholly in one source (KC divides cs); the second is read at the parent voxel
+          const bool up = c0 >= P.cs;
+          const __nv_bfloat16* hsrc = up ? P.X2 + (c0 - P.cs) + hq * 8 : P.X + c0 + hq * 8;
+          const int sh = up ? 1 : 0, ld = up ? cl : P.cs;
+          const int nyv = g.ny >> sh, nxv = g.nx >> sh, nzv = g.nz >> sh;
+          int yo[6];  // voxel offset within a plane, -1 where padded
+#pragma unroll
+          for (int j = 0; j < 6; ++j) {
+            const int gy = j < nr ? wrap_or_pad(y0 - 1 + hy0 + j * hr, g.ny, g.py) : -1;
+            yo[j] = gx >= 0 && gy >= 0 ? (gy >> sh) * nxv + (gx >> sh) : -1;
+          }
+#pragma unroll 2
+          for (int zz = 0; zz < SZH; ++zz) {
+            const int gz = wrap_or_pad(z0 - 1 + zz, g.nz, g.pz);
+            const int zo = (b * nzv + (gz >> sh)) * nyv * nxv;
+#pragma unroll
+            for (int j = 0; j < 6; ++j) {
+              if (j >= nr) break;
+              const bool in = gz >= 0 && yo[j] >= 0;
+              tc::cp_async16(hdst + (size_t)(zz * 18 + j * hr) * 160, hsrc + (in ? (long long)(zo + yo[j]) * ld : 0ll), in);
+            }
+          }
+        }
+        tc::cp_async_commit();
+        tc::cp_async_wait<0>();
+        tc::fence_proxy_async_smem();
+        tc::mbar_arrive(&h_full[cg & 1]);
+      }
+    }
+    if (!ok) {
+      *abort_flag = 1;
+      atomicOr(P.status, CONV_TIMEOUT);
+    }
+  } else if (warp == MMA_WARP) {
     // ------------------------------------------------------------ UMMA issue
-    if ((t & 31) == 0) {
+    // All lanes walk the loop and one is elected at each UMMA, so that the
+    // descriptors stay in uniform registers.
+    {
       // descriptors: constant part + (shared address >> 4); every offset below is in 16-byte units
       const uint32_t a_lbo = (uint32_t)HV * 16, b_lbo = (uint32_t)NB * 16;
       const uint64_t adb = tc::smem_desc_base(a_lbo, 160), bdb = tc::smem_desc_base(b_lbo, 128);
@@ -452,7 +518,7 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
       uint32_t wphase = 0;
       for (int k = 0; k < my_items && ok; ++k) {
         const int ab = k & 1;
-        if (k >= 2 && !pconv_wait(&a_empty[ab], (uint32_t)(((k >> 1) - 1) & 1), abort_flag, P.spin)) {
+        if (k >= 2 && !warp_wait(&a_empty[ab], (uint32_t)(((k >> 1) - 1) & 1), abort_flag, P.spin)) {
           ok = false;
           break;
         }
@@ -460,13 +526,13 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
         const uint32_t acc = tmem + (uint32_t)(ab * TZ * CT);
         for (int c = 0; c < nchunks && ok; ++c) {
           const int cg = gs / SPC;
-          if (!pconv_wait(&h_full[cg & 1], (uint32_t)((cg >> 1) & 1), abort_flag, P.spin)) {
+          if (!warp_wait(&h_full[cg & 1], (uint32_t)((cg >> 1) & 1), abort_flag, P.spin)) {
             ok = false;
             break;
           }
           const uint32_t hb = tc::smem_u32(sH + (size_t)(cg & 1) * halo_bytes);
           for (int st = 0; st < SPC; ++st, ++gs) {
-            if (!pconv_wait(&w_full[slot], wphase, abort_flag, P.spin)) {
+            if (!warp_wait(&w_full[slot], wphase, abort_flag, P.spin)) {
               ok = false;
               break;
             }
@@ -484,7 +550,7 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
                     const int s = sb == 0 ? 1 : (sb == 1 ? 0 : 2);
 #pragma unroll
                     for (int q = 0; q < TZ; ++q)
-                      tc::mma_bf16(acc + (uint32_t)((TZ - 1 - q) * CT), aj + (uint64_t)((q + s) * 180),
+                      tc::mma_bf16_elect(acc + (uint32_t)((TZ - 1 - q) * CT), aj + (uint64_t)((q + s) * 180),
                                    bj + (uint64_t)(s * CT), id1, s == 1 ? 0u : 1u);
                   }
                 } else {
@@ -493,7 +559,7 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
                     const int s_lo = zz - (TZ - 1) > 0 ? zz - (TZ - 1) : 0;
                     const int s_hi = zz < 2 ? zz : 2;
                     const uint32_t id = s_hi - s_lo == 0 ? id1 : (s_hi - s_lo == 1 ? id2 : id3);
-                    tc::mma_bf16(acc + (uint32_t)((TZ - 1 - zz + s_lo) * CT), aj + (uint64_t)(zz * 180),
+                    tc::mma_bf16_elect(acc + (uint32_t)((TZ - 1 - zz + s_lo) * CT), aj + (uint64_t)(zz * 180),
                                  bj + (uint64_t)(s_lo * CT), id, 1u);
                   }
                 }
@@ -506,22 +572,22 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
                 const uint32_t accf = (c > 0 || st > 0 || j > 0) ? 1u : 0u;
 #pragma unroll
                 for (int q = 0; q < TZ; ++q)
-                  tc::mma_bf16(acc + (uint32_t)(q * CT), aj + (uint64_t)(q * 180), bj, id1, accf);
+                  tc::mma_bf16_elect(acc + (uint32_t)(q * CT), aj + (uint64_t)(q * 180), bj, id1, accf);
               }
             }
-            tc::mma_commit(&w_empty[slot]);
+            tc::mma_commit_elect(&w_empty[slot]);
             if (++slot == nsw) {
               slot = 0;
               wphase ^= 1u;
             }
           }
-          if (ok) tc::mma_commit(&h_empty[cg & 1]);
+          if (ok) tc::mma_commit_elect(&h_empty[cg & 1]);
         }
-        if (ok) tc::mma_commit(&a_full[ab]);
+        if (ok) tc::mma_commit_elect(&a_full[ab]);
       }
       // every UMMA issued so far has completed before the CTA winds down
-      tc::mma_commit(fin);
-      if (!tc::mbar_wait(fin, 0u, CONV_DRAIN_SPIN)) ok = false;
+      tc::mma_commit_elect(fin);
+      if (!__all_sync(0xffffffffu, tc::mbar_wait(fin, 0u, CONV_DRAIN_SPIN))) ok = false;
       if (!ok) {
         *abort_flag = 1;
         atomicOr(P.status, CONV_TIMEOUT);
@@ -531,6 +597,8 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
   } else if (warp < PCONV_EPI / 32) {
     // ------------------------------------------------------------ epilogue
     const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
+    // whole 32-byte sectors when the rows allow it
+    const bool wide = !(((uintptr_t)P.Y | (uintptr_t)P.Yf) & 31) && (P.ldy % 16 == 0 || (!P.Y && P.ldy % 8 == 0));
     const int r = t;  // accumulator row = output voxel (x0 + r % 8, y0 + r / 8)
     for (int k = 0; k < my_items; ++k) {
       const int ab = k & 1;
@@ -563,16 +631,19 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
             }
             const int c0 = n0 + col + 16 * h;
             if (P.Y) {
-              uint4* yp = reinterpret_cast<uint4*>(P.Y + v * P.ldy + c0);
-              yp[0] = make_uint4(pack_bf16(a[0], a[1]), pack_bf16(a[2], a[3]), pack_bf16(a[4], a[5]),
-                                 pack_bf16(a[6], a[7]));
-              yp[1] = make_uint4(pack_bf16(a[8], a[9]), pack_bf16(a[10], a[11]), pack_bf16(a[12], a[13]),
-                                 pack_bf16(a[14], a[15]));
+              uint32_t w[8];
+#pragma unroll
+              for (int e = 0; e < 8; ++e) w[e] = pack_bf16(a[2 * e], a[2 * e + 1]);
+              store32(P.Y + v * P.ldy + c0, w, wide);
             }
             if (P.Yf) {
-              float4* fp = reinterpret_cast<float4*>(P.Yf + v * P.ldy + c0);
 #pragma unroll
-              for (int e = 0; e < 4; ++e) fp[e] = make_float4(a[4 * e], a[4 * e + 1], a[4 * e + 2], a[4 * e + 3]);
+              for (int e = 0; e < 2; ++e) {
+                uint32_t w[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) w[i] = __float_as_uint(a[8 * e + i]);
+                store32(P.Yf + v * P.ldy + c0 + 8 * e, w, wide);
+              }
             }
           }
         }
@@ -583,7 +654,7 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == PCONV_MMA_WARP) tc::tmem_dealloc(tmem, ncols);
+  if (warp == MMA_WARP) tc::tmem_dealloc(tmem, ncols);
 }
 
 // ---------------------------------------------------------------------------
@@ -606,9 +677,8 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_fwd_pipe(PConvArgs P)
 // CTA accumulates its pass over its run of blocks in tensor memory and adds
 // the result to dW with FP32 atomics once.  Warp roles and bounded waits as
 // in the forward kernel; up to four staged blocks are in flight, and a copy
-// thread signals a block nst - 2 blocks after issuing it (nst = staged
-// slots: two with four, one with three, at once with two), so the slot it
-// refills next was handed over earlier.
+// thread signals a block one block after issuing it (at once with two slots), so
+// the slot it refills next was handed over earlier.
 constexpr int WCONV_HPLANE = 180 * 16;           // bytes of one staged halo plane
 constexpr int WCONV_HBYTES = 16 * WCONV_HPLANE;  // the 16 planes of an M block
 
@@ -623,10 +693,10 @@ struct WConvArgs {
   unsigned* status;
 };
 
-__global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_wgrad_pipe(WConvArgs P) {
+__global__ void __launch_bounds__(WCONV_THREADS, 1) k_conv_wgrad_pipe(WConvArgs P) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const int t = threadIdx.x;
-  const int warp = t >> 5;
+  const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // uniform, also to the compiler
   const int CN = P.CN;
   const size_t p_bytes = (size_t)128 * CN * 2, stage_bytes = WCONV_HBYTES + p_bytes;
   const int nst = P.nst;
@@ -654,13 +724,13 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_wgrad_pipe(WConvArgs 
   uint32_t ncols = 32;
   while ((int)ncols < ntap * CN) ncols <<= 1;
 
-  if (warp == PCONV_MMA_WARP) {
+  if (warp == WCONV_MMA_WARP) {
     tc::tmem_alloc(tmem_slot, ncols);
     tc::tmem_relinquish();
   }
   if (t == 0) {
     for (int k = 0; k < 4; ++k) {
-      tc::mbar_init(&full[k], PCONV_NPROD);
+      tc::mbar_init(&full[k], WCONV_NPROD);
       tc::mbar_init(&empty[k], 1);
     }
     tc::mbar_init(done, 1);
@@ -670,7 +740,7 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_wgrad_pipe(WConvArgs 
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   auto block_of = [&](long long bi, int& x0, int& y0, int& z, int& b) {
     x0 = (int)(bi % bxs) * 8;
     bi /= bxs;
@@ -680,14 +750,17 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_wgrad_pipe(WConvArgs 
     b = (int)(bi / g.nz);
   };
 
-  if (t >= PCONV_PROD0 && t < PCONV_PROD0 + PCONV_NPROD) {
+  if (t >= PCONV_PROD0 && t < PCONV_PROD0 + WCONV_NPROD) {
     // ------------------------------------------------------------ copies
     const int pt = t - PCONV_PROD0;
-    const int hrow0 = pt / 10, hxx = pt % 10;  // 12 halo rows per pass (120 threads)
-    const bool hact = pt < 120;
+    // a thread keeps one (xx, yy) place of the 10 x 18 halo and walks the planes,
+    // so that a block costs it three voxel offsets (z - 1, z, z + 1)
+    const int hyy = pt / 10, hxx = pt % 10;
+    const bool hact = pt < 180;
+    const int lp_end = min(16, nplanes - 16 * mj);  // rows of planes past the channels feed D rows nobody reads
     // blocks a copy thread keeps in flight before it signals them; the slot it
     // refills next must belong to a block whose UMMAs were already issued
-    const int lag = nst >= 3 ? nst - 2 : 0;
+    const int lag = nst >= 3 ? 1 : 0;
     bool ok = true;
     for (int i = 0; i < nmine && ok; ++i) {
       const int s = i % nst;
@@ -700,28 +773,29 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_wgrad_pipe(WConvArgs 
       unsigned char* sH = smem + (size_t)s * stage_bytes;
       unsigned char* sP = sH + WCONV_HBYTES;
       if (hact) {
-        const int gx = wrap_or_pad(x0 - 1 + hxx, g.nx, g.px);
-        for (int row = hrow0; row < 16 * 18; row += 12) {
-          const int lp = row / 18, yy = row - 18 * lp;
-          const int p = 16 * mj + lp;
-          if (p >= nplanes) break;  // rows of planes past the channels feed D rows nobody reads
-          const int hg = p / 3, zz = p - 3 * hg;
-          const int gy = wrap_or_pad(y0 - 1 + yy, g.ny, g.py);
-          const int gz = wrap_or_pad(z - 1 + zz, g.nz, g.pz);
-          const bool in = gx >= 0 && gy >= 0 && gz >= 0;
-          const long long v = in ? (((long long)b * g.nz + gz) * g.ny + gy) * g.nx + gx : 0;
-          tc::cp_async16(sH + (size_t)(row * 10 + hxx) * 16, P.H + v * P.CH + hg * 8, in);
+        const int gx = wrap_or_pad(x0 - 1 + hxx, g.nx, g.px), gy = wrap_or_pad(y0 - 1 + hyy, g.ny, g.py);
+        int vz[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          const int gz = wrap_or_pad(z - 1 + d, g.nz, g.pz);
+          vz[d] = gx >= 0 && gy >= 0 && gz >= 0 ? ((b * g.nz + gz) * g.ny + gy) * g.nx + gx : -1;
+        }
+        unsigned char* hdst = sH + (size_t)(hyy * 10 + hxx) * 16;
+#pragma unroll 4
+        for (int lp = 0; lp < lp_end; ++lp) {
+          const int p = 16 * mj + lp, hg = p / 3, zz = p - 3 * hg;
+          const int v = zz == 0 ? vz[0] : (zz == 1 ? vz[1] : vz[2]);
+          tc::cp_async16(hdst + (size_t)lp * WCONV_HPLANE, P.H + (long long)(v < 0 ? 0 : v) * P.CH + hg * 8, v >= 0);
         }
       }
       const long long vrow = (((long long)b * g.nz + z) * g.ny + y0) * g.nx + x0;
-      for (int q = pt; q < 128 * (CN / 8); q += PCONV_NPROD) {
+      for (int q = pt; q < 128 * (CN / 8); q += WCONV_NPROD) {
         const int x = q & 7, y = (q >> 3) & 15, pg = q >> 7;
         tc::cp_async16(sP + (size_t)q * 16, P.P + (vrow + (long long)y * g.nx + x) * P.CP + n0 + pg * 8, true);
       }
       tc::cp_async_commit();
       if (i >= lag) {
-        if (lag == 2) tc::cp_async_wait<2>();
-        else if (lag == 1) tc::cp_async_wait<1>();
+        if (lag == 1) tc::cp_async_wait<1>();
         else tc::cp_async_wait<0>();
         tc::fence_proxy_async_smem();
         tc::mbar_arrive(&full[(i - lag) % nst]);
@@ -735,14 +809,16 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_wgrad_pipe(WConvArgs 
       *abort_flag = 1;
       atomicOr(P.status, CONV_TIMEOUT);
     }
-  } else if (warp == PCONV_MMA_WARP) {
+  } else if (warp == WCONV_MMA_WARP) {
     // ------------------------------------------------------------ UMMA issue
-    if ((t & 31) == 0) {
+    // All lanes walk the loop and one is elected at each UMMA, so that the
+    // descriptors stay in uniform registers.
+    {
       const uint32_t idesc = tc::idesc_bf16(CONV_M, CN, true, true);
       bool ok = true;
       for (int i = 0; i < nmine; ++i) {
         const int s = i % nst;
-        if (!pconv_wait(&full[s], (uint32_t)((i / nst) & 1), abort_flag, P.spin)) {
+        if (!warp_wait(&full[s], (uint32_t)((i / nst) & 1), abort_flag, P.spin)) {
           ok = false;
           break;
         }
@@ -756,14 +832,14 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_wgrad_pipe(WConvArgs 
           const uint32_t d = tmem + (uint32_t)(tt * CN);
 #pragma unroll
           for (int k = 0; k < 8; ++k)  // k-step: two rows of 8 voxels (320 and 256 bytes on)
-            tc::mma_bf16(d, a0 + (uint64_t)(k * 20), bd0 + (uint64_t)(k * 16), idesc, (i > 0 || k > 0) ? 1u : 0u);
+            tc::mma_bf16_elect(d, a0 + (uint64_t)(k * 20), bd0 + (uint64_t)(k * 16), idesc, (i > 0 || k > 0) ? 1u : 0u);
         }
-        tc::mma_commit(&empty[s]);
+        tc::mma_commit_elect(&empty[s]);
       }
-      tc::mma_commit(done);  // every UMMA of this CTA, or none
+      tc::mma_commit_elect(done);  // every UMMA of this CTA, or none
       // drained here too, so that tensor memory outlives every committed UMMA
       // even when the epilogue's wait gives up
-      if (!tc::mbar_wait(done, 0u, CONV_DRAIN_SPIN)) ok = false;
+      if (!__all_sync(0xffffffffu, tc::mbar_wait(done, 0u, CONV_DRAIN_SPIN))) ok = false;
       if (!ok) {
         *abort_flag = 1;
         atomicOr(P.status, CONV_TIMEOUT);
@@ -805,7 +881,7 @@ __global__ void __launch_bounds__(PCONV_THREADS, 1) k_conv_wgrad_pipe(WConvArgs 
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == PCONV_MMA_WARP) tc::tmem_dealloc(tmem, ncols);
+  if (warp == WCONV_MMA_WARP) tc::tmem_dealloc(tmem, ncols);
 }
 
 // ---------------------------------------------------------------------------
@@ -865,6 +941,60 @@ __global__ void __launch_bounds__(128, 1)
   const uint32_t idesc = tc::idesc_bf16(CONV_M, Cout, true, true);
   bool ok = true;
   int issued = 0;  // chunks whose UMMAs were issued and committed
+  // 1x1x1: the column is the channel and the source voxel the voxel itself, and
+  // the columns past Cin are cleared once.  With at most PRE pieces a thread and
+  // chunk (the head), the pieces of the next two chunks wait in registers, so
+  // that a chunk costs its barriers and not its loads' latency.  128^3 voxels,
+  // 32 -> 16 channels: all 128 columns gathered per chunk by voxel coordinates
+  // 1130 us, without the coordinates 320, with the registers 172 us.
+  constexpr int PRE = 4;
+  const int ncg = min(CONV_M / 8, (ntot - col0) / 8), nbg = Cout / 8;  // column groups in use
+  const bool pre = NT == 1 && KV * (ncg + nbg) <= PRE * CONV_M;
+  uint4 held[2][PRE];
+  auto piece = [&](int i, int ch, int& kv, int& grp, bool& isb) {  // piece i of this thread in chunk ch: false past the end
+    int p = t + i * CONV_M;
+    isb = p >= KV * ncg;
+    if (isb) p -= KV * ncg;
+    const int n = isb ? nbg : ncg;
+    kv = p / n;
+    grp = p - kv * n;
+    return kv < KV;
+  };
+  auto fetch = [&](int ch, uint4 r[PRE]) {
+#pragma unroll
+    for (int i = 0; i < PRE; ++i) {
+      int kv, grp;
+      bool isb;
+      r[i] = make_uint4(0, 0, 0, 0);
+      if (!piece(i, ch, kv, grp, isb)) continue;
+      const long long vv = v_begin + (long long)ch * KV + kv;
+      if (vv < v_end)
+        r[i] = isb ? *reinterpret_cast<const uint4*>(dY + vv * Cout + grp * 8)
+                   : *reinterpret_cast<const uint4*>(X + vv * Cin + col0 + grp * 8);
+    }
+  };
+  auto put = [&](int buf, int ch, const uint4 r[PRE]) {
+#pragma unroll
+    for (int i = 0; i < PRE; ++i) {
+      int kv, grp;
+      bool isb;
+      if (!piece(i, ch, kv, grp, isb)) continue;
+      unsigned char* d = isb ? sB[buf] + (size_t)grp * b_mn + (size_t)(kv >> 3) * b_k : sA[buf] + (size_t)grp * a_mn + (size_t)(kv >> 3) * a_k;
+      *reinterpret_cast<uint4*>(d + (kv & 7) * 16) = r[i];
+    }
+  };
+  if constexpr (NT == 1) {
+    for (int p = t; p < 2 * KV * (CONV_M / 8); p += CONV_M) {
+      const int kv = p % KV, mg = p / KV % (CONV_M / 8);
+      if (mg >= ncg)
+        *reinterpret_cast<uint4*>(sA[p / (KV * (CONV_M / 8))] + (size_t)mg * a_mn + (size_t)(kv >> 3) * a_k + (kv & 7) * 16) =
+            make_uint4(0, 0, 0, 0);
+    }
+    if (pre) {
+      fetch(0, held[0]);
+      fetch(1, held[1]);
+    }
+  }
 
   for (int ch = 0; ch < nchunks; ++ch) {
     const int buf = ch & 1;
@@ -875,7 +1005,23 @@ __global__ void __launch_bounds__(128, 1)
     }
     const long long vb = v_begin + (long long)ch * KV;
     // A[(t,ci)][kv] = X[vb + kv + off_t][ci], 8 columns per 16-byte piece
-    for (int p = t; p < KV * (CONV_M / 8); p += CONV_M) {
+    if (pre) {
+      if (buf) {
+        put(1, ch, held[1]);
+        fetch(ch + 2, held[1]);
+      } else {
+        put(0, ch, held[0]);
+        fetch(ch + 2, held[0]);
+      }
+    } else if constexpr (NT == 1) {
+      for (int p = t; p < KV * ncg; p += CONV_M) {
+        const int kv = p / ncg, mg = p - kv * ncg;
+        const long long vv = vb + kv;
+        uint4 val = make_uint4(0, 0, 0, 0);
+        if (vv < v_end) val = *reinterpret_cast<const uint4*>(X + vv * Cin + col0 + mg * 8);
+        *reinterpret_cast<uint4*>(sA[buf] + (size_t)mg * a_mn + (size_t)(kv >> 3) * a_k + (kv & 7) * 16) = val;
+      }
+    } else for (int p = t; p < KV * (CONV_M / 8); p += CONV_M) {
       const int kv = p / (CONV_M / 8), mg = p % (CONV_M / 8);
       const int colg = col0 + mg * 8;
       const long long vv = vb + kv;
@@ -897,7 +1043,7 @@ __global__ void __launch_bounds__(128, 1)
       *reinterpret_cast<uint4*>(sA[buf] + (size_t)mg * a_mn + (size_t)(kv >> 3) * a_k + (kv & 7) * 16) = val;
     }
     // B[co][kv] = dY[vb + kv][co]
-    for (int p = t; p < KV * (Cout / 8); p += CONV_M) {
+    for (int p = t; !pre && p < KV * (Cout / 8); p += CONV_M) {
       const int kv = p / (Cout / 8), ng = p % (Cout / 8);
       const long long vv = vb + kv;
       uint4 val = make_uint4(0, 0, 0, 0);
@@ -980,8 +1126,13 @@ static size_t conv_wgrad_smem(int Cout) {
 constexpr size_t CONV_TILED_SMEM_MAX = 225 * 1024;
 static size_t pconv_smem_need(int tz, int KC, int CT, bool merge, int nsw) {
   const size_t halo = (size_t)10 * 18 * (tz + 2) * KC * 2;
-  return 2 * halo + (size_t)nsw * (merge ? 3 : 1) * CT * KC * 2 + 256 + 1024;  // + barriers, flags, bias
+  return 2 * halo + (size_t)nsw * (merge ? 3 : 1) * CT * KC * 2 + 512 + 1024;  // + barriers, flags, bias
 }
+
+// Bytes a cycle that the copy threads of one SM move from L2 (measured in both
+// tiled kernels: 9 to 11, twice that in sectors, as a 16-byte cp.async fetches
+// its whole sector).
+constexpr double COPY_RATE = 10.0;
 
 struct PConvCfg {
   int tz = 0, kc = 0, ct = 0, nsw = 0;
@@ -1016,9 +1167,9 @@ static PConvCfg pconv_choose(int cin, int cs, int cout, int nx, int ny, int nz, 
       for (int k = 0; k < 4; ++k) {
         const int kc = kcs[k];
         if (kc > cin || cin % kc || cs % kc) continue;
-        for (int nsw = PCONV_NSW_MAX; nsw >= PCONV_LAG + 2; --nsw) {
-          if (pconv_smem_need(tz, kc, ct, merge, nsw) > CONV_TILED_SMEM_MAX) continue;
-          if ((merge ? 3 : 1) * ct * (kc / 8) > PCONV_MAXWP * PCONV_NPROD || 10 * (kc / 8) > PCONV_NPROD) continue;
+        for (int nsw = PCONV_NSW_MAX; nsw >= PCONV_NSW_MIN; --nsw) {
+          if (pconv_smem_need(tz, kc, ct, merge, nsw) > CONV_TILED_SMEM_MAX + 256) continue;
+          if ((merge ? 3 : 1) * ct * (kc / 8) > PCONV_MAXW || 10 * (kc / 8) > PCONV_NHALO) continue;
           PConvCfg c;
           c.tz = tz;
           c.kc = kc;
@@ -1032,6 +1183,34 @@ static PConvCfg pconv_choose(int cin, int cs, int cout, int nx, int ny, int nz, 
       }
     }
   }
+  if (!best.tz) return best;
+  // KC and MERGE fix the order of every sum; the split into work items is free.
+  // Take the one with the least (waves) x (cycles a work item), the cycles being
+  // those of its UMMAs (N / 2 each, or the shared-memory reads of their operands)
+  // or of its copies at COPY_RATE, whichever is more.  384 -> 128 channels on 32^3:
+  // 256 items of one plane (two waves, each streaming all weights) 249 us, 128
+  // items of 64 channels and four planes 142 us; 64 -> 192 on 64^3 427 -> 252 us.
+  auto cost = [&](const PConvCfg& c) {
+    const int zs = c.merge ? c.tz + 2 : c.tz, steps = c.merge ? 9 : 27;
+    const double n = c.merge ? 3.0 * c.ct * c.tz / (c.tz + 2) : c.ct;  // columns of a UMMA
+    const double mma = c.kc / 16 * zs * std::max(n / 2, 32 + n / 4);
+    const double copy = 2.0 * c.kc * ((c.merge ? 3 : 1) * c.ct + 180.0 * (c.tz + 2) / steps) / COPY_RATE;
+    return (double)((c.items + nsm - 1) / nsm) * std::max(mma, copy);
+  };
+  const PConvCfg first = best;
+  for (int ns = 1; ns <= cout / 16; ++ns)
+    for (int tz = 8; tz >= 1; tz >>= 1) {
+      PConvCfg c = first;
+      c.ct = cout / ns;
+      c.tz = tz;
+      if (cout % ns || c.ct % 16 || nz % tz || 2 * tz * c.ct > 512 || (c.merge ? 3 * c.ct > 256 : tz > 4)) continue;
+      if ((c.merge ? 3 : 1) * c.ct * (c.kc / 8) > PCONV_MAXW) continue;
+      for (c.nsw = PCONV_NSW_MAX; c.nsw >= PCONV_NSW_MIN; --c.nsw)
+        if (pconv_smem_need(tz, c.kc, c.ct, c.merge, c.nsw) <= CONV_TILED_SMEM_MAX + 256) break;
+      if (c.nsw < PCONV_NSW_MIN) continue;
+      c.items = (long long)(nx / 8) * (ny / 16) * (nz / tz) * nb * ns;
+      if (cost(c) < cost(best)) best = c;
+    }
   return best;
 }
 
@@ -1048,15 +1227,16 @@ static int conv_fwd_pipe(const void* x, int cs, const void* x2, int cin, const v
   PConvArgs a{(const __nv_bfloat16*)x, (const __nv_bfloat16*)x2, cs, (const __nv_bfloat16*)w, bias,
               (__nv_bfloat16*)y, yf, cin, cout, ldy, c.kc, c.ct, c.nsw, g, relu, wait_limit(), status};
   cudaError_t e = cudaSuccess;
+  const int threads = pconv_threads(c.merge);
   auto launch = [&](auto kern) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return;
     int occ = 1;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, PCONV_THREADS, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, smem);
     if (e != cudaSuccess) return;
     const long long cap = (long long)nsm * (occ > 0 ? occ : 1);
     const unsigned blocks = (unsigned)(c.items < cap ? c.items : cap);
-    kern<<<blocks, PCONV_THREADS, smem, st>>>(a);
+    kern<<<blocks, threads, smem, st>>>(a);
     e = cudaGetLastError();
   };
   if (c.merge) {
@@ -1065,7 +1245,8 @@ static int conv_fwd_pipe(const void* x, int cs, const void* x2, int cin, const v
     else if (c.tz == 2) launch(k_conv_fwd_pipe<2, true>);
     else launch(k_conv_fwd_pipe<1, true>);
   } else {
-    if (c.tz == 2) launch(k_conv_fwd_pipe<2, false>);
+    if (c.tz == 4) launch(k_conv_fwd_pipe<4, false>);
+    else if (c.tz == 2) launch(k_conv_fwd_pipe<2, false>);
     else if (c.tz == 1) launch(k_conv_fwd_pipe<1, false>);
     else e = cudaErrorInvalidValue;
   }
@@ -1079,46 +1260,55 @@ static int conv_fwd_pipe(const void* x, int cs, const void* x2, int cin, const v
 // tensor memory, and enough voxel runs for every SM.
 static int conv_wgrad_pipe(const void* dy, int cout, const void* x, int cin, float* dw, const ConvGeo& g,
                            unsigned* status, cudaStream_t st) {
-  struct Or {
-    int o2, CH, CP, mblocks, nchunks, CN, ngroups, TG;
-    long long cost;
-  };
-  auto plan = [](int o2, int CH, int CP) {
-    Or o{o2, CH, CP, (3 * (CH / 8) + 15) / 16, 1, CP, 0, 0, 0};
-    while (o.CN > 256 || o.CP % o.nchunks || (o.CP / o.nchunks) % 16) {
-      ++o.nchunks;
-      o.CN = o.CP / o.nchunks;
-    }
-    o.CN = o.CP / o.nchunks;
-    const int fit = 512 / o.CN;  // taps whose accumulators fit tensor memory together
-    o.ngroups = (9 + fit - 1) / fit;
-    o.TG = (9 + o.ngroups - 1) / o.ngroups;
-    o.cost = (long long)o.mblocks * o.nchunks;
-    return o;
-  };
-  const Or a = plan(0, cin, cout), b = plan(1, cout, cin);
-  const Or o = b.cost < a.cost ? b : a;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const long long nblocks = (long long)(g.nx / 8) * (g.ny / 16) * g.nz * g.nb;
-  const int npass = o.mblocks * o.ngroups * o.nchunks;
-  long long slices = (nsm + npass - 1) / npass;
-  if (slices > nblocks) slices = nblocks;
-  if (slices < 1) slices = 1;
-  const long long per = (nblocks + slices - 1) / slices;
-  slices = (nblocks + per - 1) / per;
-  if (npass > 65535) return report_error(LB_EINVAL, "conv wgrad: too many passes");
+  struct Plan {
+    int o2, CH, CP, mblocks, nchunks, CN, ngroups, TG, npass;
+    long long slices, per;
+    double cost = 0;
+  };
+  Plan o{};
+  for (int o2 = 0; o2 < 2; ++o2)
+    for (int nchunks = 1; nchunks <= 16; ++nchunks) {
+      Plan q{};
+      q.o2 = o2;
+      q.CH = o2 ? cout : cin;
+      q.CP = o2 ? cin : cout;
+      q.nchunks = nchunks;
+      q.CN = q.CP / nchunks;
+      if (q.CP % nchunks || q.CN % 16 || q.CN > 256) continue;
+      const int planes = 3 * (q.CH / 8);
+      q.mblocks = (planes + 15) / 16;
+      const int fit = 512 / q.CN;  // taps whose accumulators fit tensor memory together
+      q.ngroups = (9 + fit - 1) / fit;
+      q.TG = (9 + q.ngroups - 1) / q.ngroups;
+      q.npass = q.mblocks * q.ngroups * nchunks;
+      if (q.npass > 65535) continue;
+      // one CTA fits an SM: never more of them than SMs when the passes allow it
+      q.slices = std::min(std::max((long long)(nsm / q.npass), 1ll), nblocks);
+      q.per = (nblocks + q.slices - 1) / q.slices;
+      q.slices = (nblocks + q.per - 1) / q.per;
+      const long long waves = (q.npass * q.slices + nsm - 1) / nsm;
+      // cycles a block: 8 UMMAs a tap of CN / 2 cycles (or their operands' shared-
+      // memory reads), against its copy at COPY_RATE
+      const double mma = q.TG * 8.0 * std::max(q.CN / 2.0, 32 + q.CN / 4.0);
+      const double copy = (2880.0 * planes / q.mblocks + 256.0 * q.CN) / COPY_RATE;
+      q.cost = (double)waves * (double)q.per * std::max(mma, copy);
+      if (o.cost == 0 || q.cost < o.cost) o = q;
+    }
+  if (o.cost == 0) return report_error(LB_EINVAL, "conv wgrad: too many passes");
   const size_t stage = (size_t)WCONV_HBYTES + (size_t)128 * o.CN * 2;
   int nst = (int)((CONV_TILED_SMEM_MAX - 128) / stage);
   nst = nst > 4 ? 4 : nst;
   if (nst < 2) return report_error(LB_EINVAL, "conv wgrad: staging does not fit shared memory");
   const size_t smem = conv_smem((size_t)nst * stage + 128, o.TG * o.CN);
   WConvArgs args{(const __nv_bfloat16*)(o.o2 ? dy : x), (const __nv_bfloat16*)(o.o2 ? x : dy), dw, o.CH, o.CP, cin,
-                 o.o2, o.CN, o.TG, o.ngroups, o.nchunks, (int)per, nst, g, wait_limit(), status};
+                 o.o2, o.CN, o.TG, o.ngroups, o.nchunks, (int)o.per, nst, g, wait_limit(), status};
   cudaError_t e = cudaFuncSetAttribute(k_conv_wgrad_pipe, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) {
-    k_conv_wgrad_pipe<<<dim3((unsigned)slices, (unsigned)npass), PCONV_THREADS, smem, st>>>(args);
+    k_conv_wgrad_pipe<<<dim3((unsigned)o.slices, (unsigned)o.npass), WCONV_THREADS, smem, st>>>(args);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess) return report_error(LB_ECUDA, std::string("conv wgrad (tiled): ") + cudaGetErrorString(e));
