@@ -205,18 +205,23 @@ __global__ void __launch_bounds__(128, 1)
 // forward / input gradient, spatially tiled and pipelined (3x3x3 taps)
 // ---------------------------------------------------------------------------
 // Work item: an output block of 8 (x) x 16 (y) x TZ (z) voxels and CT output
-// channels (CT = Cout or a slice of it, pconv_choose).  Persistent CTAs walk the work items; warps have fixed roles:
+// channels (CT = Cout or a slice of it, pconv_choose).  Persistent CTAs walk the
+// work items; warps have fixed roles:
 //   warps 0-3  epilogue: tensor memory -> bias, ReLU -> BF16 / FP32 stores
 //   the next 4 (8 without MERGE) weight copies, the next 8 input copies
 //              (cp.async, zero fill for padded voxels)
 //   last warp  tensor-memory allocation; one elected lane issues the UMMAs
-// and hand buffers over through mbarriers only.  A weight thread signals a slot
-// PCONV_LAG steps after filling it, so several steps are in flight; with one
-// group of 128 threads copying both operands in turn and 8 slots the UMMAs
-// waited for every halo.  Bound now: the copies (L2 to shared memory at 20 bytes
-// of sectors a cycle and SM) and the UMMAs' operand reads, about equally.
+// and hand buffers over through mbarriers only.  The weights of the three x taps
+// of a row are handed over together: a wait and a commit cost the issuing warp
+// 300 to 400 cycles, in which the tensor pipe runs dry (4 to 12 UMMAs of 40 to 96
+// cycles a tap).  A ring of fewer than 9 slots, two groups, would keep the copies
+// waiting instead and is handed over tap by tap (64 -> 64 channels on 64^3: 89 us
+// in groups, 71 by tap).  A weight thread signals one group (two taps) after
+// filling, so that several are in flight.  Bound now: the copies (16-byte pieces
+// that each fetch a 32-byte sector) and the UMMAs' operand reads, about equally.
 // 128x128x256 voxels, 32 + 64 -> 32 channels: 1098 -> 835 us with the roles split
-// and the ring deeper, 760 with the issue from a converged warp.
+// and the ring deeper, 760 with the issue from a converged warp, 603 with the
+// taps in groups.
 //
 // Per chunk of KC input channels the input block with a one-voxel halo
 // (10 x 18 x (TZ + 2) voxels) is staged once, in the layout
@@ -253,7 +258,6 @@ constexpr int WCONV_NPROD = 256;   // copy threads of the weight gradient (all s
 constexpr int WCONV_MMA_WARP = (PCONV_EPI + WCONV_NPROD) / 32;
 constexpr int WCONV_THREADS = PCONV_EPI + WCONV_NPROD + 32;
 constexpr int PCONV_MAXW = 1024;   // weight pieces per step (3 CT or CT rows x KC / 8)
-constexpr int PCONV_LAG = 2;       // steps a weight thread keeps in flight before it signals them
 constexpr int PCONV_NSW_MIN = 7;   // weight ring slots
 constexpr int PCONV_NSW_MAX = 16;
 
@@ -318,7 +322,8 @@ __global__ void __launch_bounds__(pconv_threads(MERGE), 1) k_conv_fwd_pipe(PConv
   extern __shared__ __align__(1024) unsigned char smem[];
   const int t = threadIdx.x;
   const int warp = __shfl_sync(0xffffffffu, t >> 5, 0);  // uniform, also to the compiler
-  const int KC = P.KC, CT = P.CT, Cin = P.Cin, nsw = P.nsw;
+  const int KC = P.KC, CT = P.CT, Cin = P.Cin;
+  const int gsz = P.nsw >= 9 ? 3 : 1, ngrp = P.nsw / gsz, nsw = gsz * ngrp;  // steps handed over together
   const int NB = NBLK * CT;  // rows of a staged B operand
   const int cgs = KC / 8;
   const size_t halo_bytes = (size_t)HV * KC * 2, w_bytes = (size_t)NB * KC * 2;
@@ -397,8 +402,8 @@ __global__ void __launch_bounds__(pconv_threads(MERGE), 1) k_conv_fwd_pipe(PConv
       wdo[i] = (uint32_t)(kg * NB + n) * 16;
     }
     bool ok = true;
-    int gs = 0, slot = 0, hslot = 0;  // step, its slot, the slot of step gs - LAG
-    uint32_t ephase = 1;              // parity of the slot's last release
+    int gs = 0, slot = 0, grp = 0, hgrp = 0;  // step, its slot and group, the group to hand over next
+    uint32_t ephase = 1;                      // parity of the group's last release
     for (int k = 0; k < my_items && ok; ++k) {
       int x0, y0, z0, b, n0;
       item_of(k, x0, y0, z0, b, n0);
@@ -406,7 +411,7 @@ __global__ void __launch_bounds__(pconv_threads(MERGE), 1) k_conv_fwd_pipe(PConv
       for (int c = 0; c < nchunks && ok; ++c) {
         const int c0 = c * KC;
         for (int st = 0; st < SPC; ++st, ++gs) {
-          if (gs >= nsw && !pconv_wait(&w_empty[slot], ephase, abort_flag, P.spin)) {
+          if (gs >= nsw && (gsz == 1 || st % 3 == 0) && !pconv_wait(&w_empty[grp], ephase, abort_flag, P.spin)) {
             ok = false;
             break;
           }
@@ -416,15 +421,20 @@ __global__ void __launch_bounds__(pconv_threads(MERGE), 1) k_conv_fwd_pipe(PConv
           for (int i = 0; i < MAXWP; ++i)
             if (woff[i] >= 0) tc::cp_async16(wdst + wdo[i], wsrc + woff[i], true);
           tc::cp_async_commit();
-          if (++slot == nsw) {
-            slot = 0;
-            ephase ^= 1u;
-          }
-          if (gs >= PCONV_LAG) {  // step gs - LAG has landed: hand it over
-            tc::cp_async_wait<PCONV_LAG>();
-            tc::fence_proxy_async_smem();
-            tc::mbar_arrive(&w_full[hslot]);
-            if (++hslot == nsw) hslot = 0;
+          if (++slot == nsw) slot = 0;
+          if (gsz == 1 || st % 3 == 2) {
+            if (++grp == ngrp) {
+              grp = 0;
+              ephase ^= 1u;
+            }
+            // the group before, or the step two before, has landed: hand it over
+            if (gs >= (gsz == 1 ? 2 : 3)) {
+              if (gsz == 1) tc::cp_async_wait<2>();
+              else tc::cp_async_wait<3>();
+              tc::fence_proxy_async_smem();
+              tc::mbar_arrive(&w_full[hgrp]);
+              if (++hgrp == ngrp) hgrp = 0;
+            }
           }
         }
       }
@@ -432,9 +442,9 @@ __global__ void __launch_bounds__(pconv_threads(MERGE), 1) k_conv_fwd_pipe(PConv
     tc::cp_async_wait<0>();
     tc::fence_proxy_async_smem();
     if (ok) {
-      for (int r = nsteps > PCONV_LAG ? nsteps - PCONV_LAG : 0; r < nsteps; ++r) {
-        tc::mbar_arrive(&w_full[hslot]);
-        if (++hslot == nsw) hslot = 0;
+      for (int r = min(nsteps, gsz == 1 ? 2 : 1); r > 0; --r) {
+        tc::mbar_arrive(&w_full[hgrp]);
+        if (++hgrp == ngrp) hgrp = 0;
       }
     } else {
       *abort_flag = 1;
@@ -514,7 +524,7 @@ __global__ void __launch_bounds__(pconv_threads(MERGE), 1) k_conv_fwd_pipe(PConv
       const uint32_t id3 = MERGE ? tc::idesc_bf16(CONV_M, 3 * CT, false, false) : id1;
       const int njs = KC / 16;
       bool ok = true;
-      int gs = 0, slot = 0;
+      int cg = 0, slot = 0, grp = 0;  // chunk, weight slot and group
       uint32_t wphase = 0;
       for (int k = 0; k < my_items && ok; ++k) {
         const int ab = k & 1;
@@ -524,61 +534,68 @@ __global__ void __launch_bounds__(pconv_threads(MERGE), 1) k_conv_fwd_pipe(PConv
         }
         tc::fence_after_sync();
         const uint32_t acc = tmem + (uint32_t)(ab * TZ * CT);
-        for (int c = 0; c < nchunks && ok; ++c) {
-          const int cg = gs / SPC;
+        for (int c = 0; c < nchunks && ok; ++c, ++cg) {
           if (!warp_wait(&h_full[cg & 1], (uint32_t)((cg >> 1) & 1), abort_flag, P.spin)) {
             ok = false;
             break;
           }
           const uint32_t hb = tc::smem_u32(sH + (size_t)(cg & 1) * halo_bytes);
-          for (int st = 0; st < SPC; ++st, ++gs) {
-            if (!warp_wait(&w_full[slot], wphase, abort_flag, P.spin)) {
-              ok = false;
-              break;
-            }
-            tc::fence_after_sync();
-            const uint64_t b0 = bdb + (tc::smem_u32(sW + (size_t)slot * w_bytes) >> 4);
-            if (MERGE) {
-              const int dxp = st % 3, dyp = st / 3;
-              const uint64_t a0 = adb + ((hb + (uint32_t)(dyp * 10 + dxp) * 16) >> 4);
-              for (int j = 0; j < njs; ++j) {
-                const uint64_t aj = a0 + (uint64_t)j * a_j, bj = b0 + (uint64_t)j * b_j;
-                if (c == 0 && st == 0 && j == 0) {
-                  // block 1 (dz = 0) initialises every plane, then blocks 0 and 2 accumulate
+          for (int sg = 0; sg < SPC / 3 && ok; ++sg) {
 #pragma unroll
-                  for (int sb = 0; sb < 3; ++sb) {
-                    const int s = sb == 0 ? 1 : (sb == 1 ? 0 : 2);
+            for (int dxp = 0; dxp < 3; ++dxp) {
+              if (dxp == 0 || gsz == 1) {
+                if (!warp_wait(&w_full[grp], wphase, abort_flag, P.spin)) {
+                  ok = false;
+                  break;
+                }
+                tc::fence_after_sync();
+              }
+              const uint64_t b0 = bdb + (tc::smem_u32(sW + (size_t)slot * w_bytes) >> 4);
+              const bool first = c == 0 && sg == 0 && dxp == 0;
+              if (MERGE) {
+                const uint64_t a0 = adb + ((hb + (uint32_t)(sg * 10 + dxp) * 16) >> 4);
+                for (int j = 0; j < njs; ++j) {
+                  const uint64_t aj = a0 + (uint64_t)j * a_j, bj = b0 + (uint64_t)j * b_j;
+                  if (first && j == 0) {
+                    // block 1 (dz = 0) initialises every plane, then blocks 0 and 2 accumulate
 #pragma unroll
-                    for (int q = 0; q < TZ; ++q)
-                      tc::mma_bf16_elect(acc + (uint32_t)((TZ - 1 - q) * CT), aj + (uint64_t)((q + s) * 180),
-                                   bj + (uint64_t)(s * CT), id1, s == 1 ? 0u : 1u);
-                  }
-                } else {
+                    for (int sb = 0; sb < 3; ++sb) {
+                      const int s = sb == 0 ? 1 : (sb == 1 ? 0 : 2);
 #pragma unroll
-                  for (int zz = 0; zz < SZH; ++zz) {
-                    const int s_lo = zz - (TZ - 1) > 0 ? zz - (TZ - 1) : 0;
-                    const int s_hi = zz < 2 ? zz : 2;
-                    const uint32_t id = s_hi - s_lo == 0 ? id1 : (s_hi - s_lo == 1 ? id2 : id3);
-                    tc::mma_bf16_elect(acc + (uint32_t)((TZ - 1 - zz + s_lo) * CT), aj + (uint64_t)(zz * 180),
-                                 bj + (uint64_t)(s_lo * CT), id, 1u);
+                      for (int q = 0; q < TZ; ++q)
+                        tc::mma_bf16_elect(acc + (uint32_t)((TZ - 1 - q) * CT), aj + (uint64_t)((q + s) * 180),
+                                           bj + (uint64_t)(s * CT), id1, s == 1 ? 0u : 1u);
+                    }
+                  } else {
+#pragma unroll
+                    for (int zz = 0; zz < SZH; ++zz) {
+                      const int s_lo = zz - (TZ - 1) > 0 ? zz - (TZ - 1) : 0;
+                      const int s_hi = zz < 2 ? zz : 2;
+                      const uint32_t id = s_hi - s_lo == 0 ? id1 : (s_hi - s_lo == 1 ? id2 : id3);
+                      tc::mma_bf16_elect(acc + (uint32_t)((TZ - 1 - zz + s_lo) * CT), aj + (uint64_t)(zz * 180),
+                                         bj + (uint64_t)(s_lo * CT), id, 1u);
+                    }
                   }
                 }
-              }
-            } else {
-              const int dxp = st % 3, dyp = (st / 3) % 3, dzp = st / 9;
-              const uint64_t a0 = adb + ((hb + (uint32_t)((dzp * 18 + dyp) * 10 + dxp) * 16) >> 4);
-              for (int j = 0; j < njs; ++j) {
-                const uint64_t aj = a0 + (uint64_t)j * a_j, bj = b0 + (uint64_t)j * b_j;
-                const uint32_t accf = (c > 0 || st > 0 || j > 0) ? 1u : 0u;
+              } else {
+                const int dyp = sg % 3, dzp = sg / 3;
+                const uint64_t a0 = adb + ((hb + (uint32_t)((dzp * 18 + dyp) * 10 + dxp) * 16) >> 4);
+                for (int j = 0; j < njs; ++j) {
+                  const uint64_t aj = a0 + (uint64_t)j * a_j, bj = b0 + (uint64_t)j * b_j;
+                  const uint32_t accf = !first || j > 0 ? 1u : 0u;
 #pragma unroll
-                for (int q = 0; q < TZ; ++q)
-                  tc::mma_bf16_elect(acc + (uint32_t)(q * CT), aj + (uint64_t)(q * 180), bj, id1, accf);
+                  for (int q = 0; q < TZ; ++q)
+                    tc::mma_bf16_elect(acc + (uint32_t)(q * CT), aj + (uint64_t)(q * 180), bj, id1, accf);
+                }
               }
-            }
-            tc::mma_commit_elect(&w_empty[slot]);
-            if (++slot == nsw) {
-              slot = 0;
-              wphase ^= 1u;
+              if (++slot == nsw) slot = 0;
+              if (dxp == 2 || gsz == 1) {
+                tc::mma_commit_elect(&w_empty[grp]);
+                if (++grp == ngrp) {
+                  grp = 0;
+                  wphase ^= 1u;
+                }
+              }
             }
           }
           if (ok) tc::mma_commit_elect(&h_empty[cg & 1]);
