@@ -187,8 +187,8 @@ int lb_init_fields(lb_handle* h, const float* phi, const float* rho, const float
  * Runs of 12 steps are replayed from a captured CUDA graph. */
 int lb_step(lb_handle* h, int64_t nsteps);
 
-/* Choose the tile shape of the step kernel (0..5: 32x8x4, 32x8x8, 32x8x2,
- * 32x8x1, 32x4x4 and, as 1, 32x8x8 nodes per CTA); used by autotuners.  Without
+/* Choose the tile shape of the step kernel (0..5: 32x8x4 for 0 and 2, 32x8x8 for
+ * 1, 3 and 5, 32x4x4 for 4, in nodes per CTA); used by autotuners.  Without
  * this call the step picks a shape by the lattice's size.  Results do not
  * depend on the tile (bit for bit).  The widest staging halo (h_max >= 4),
  * FP64 storage, the Shan-Chen model and lattices whose z planes exceed 32-bit

@@ -136,8 +136,9 @@ struct RunDesc {
 struct Tile {
   int tx, ty, tz;
 };
-constexpr int NUM_TILES = 6;
-extern const Tile kTiles[NUM_TILES];
+constexpr int NUM_TILES = 6;   // what lb_set_tile takes
+constexpr int NUM_SHAPES = 8;  // and two shallow shapes that only the choice by size takes
+extern const Tile kTiles[NUM_SHAPES];
 
 size_t elem_bytes(int storage);
 // population-like arrays of a state: 2 x 27 (two sets), 27 (single set) or

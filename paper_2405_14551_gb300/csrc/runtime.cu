@@ -342,7 +342,7 @@ AccBufs acc_bufs(const lb_handle* h) {
 // 2560 / 2660 / 2890 / 3350.
 int step_tile_of(const lb_handle* h) {
   if (h->tile_chosen) return h->tile;
-  const int order[4] = {1, 0, 2, 3};  // 32x8x8, x4, x2, x1
+  const int order[4] = {1, 0, 6, 7};  // 32x8x8, x4, x2, x1
   const long long sms = sm_count_host();
   for (int k = 0; k < 4; ++k) {
     const Tile& T = kTiles[order[k]];

@@ -109,8 +109,8 @@ inline cudaError_t launch_step_t(const Geo& g, const Phys& p, const StateBuf& in
                     reinterpret_cast<const R*>(phi), pg, g, phys_as<R>(p), fields, status);
 }
 
-// Tile shapes of the hot variant (pull, write state): 0..5 as kTiles; the
-// widest halo (7) only with tile 0.  Other variants, FP64, Shan-Chen and planes
+// Tile shapes of the hot variant (pull, write state): kTiles; the wide halos
+// (6, 7) only with tile 0.  Other variants, FP64, Shan-Chen and planes
 // that need 64-bit offsets use tile 0.
 template <int ST, int LOADER, bool WS, bool WF, bool SC>
 inline cudaError_t launch_step_tiles(int tile, const Geo& g, const Phys& p, const StateBuf& in, const InitBuf& init,
@@ -128,10 +128,11 @@ inline cudaError_t launch_step_tiles(int tile, const Geo& g, const Phys& p, cons
       if (i32) {
         switch (tile) {
           case 1:
+          case 3:
           case 5: return LBCG_TILE(8, 8, true, 2);
-          case 2: return LBCG_TILE(8, 2, true, 2);
-          case 3: return LBCG_TILE(8, 1, true, 2);
           case 4: return LBCG_TILE(4, 4, true, 4);
+          case 6: return LBCG_TILE(8, 2, true, 2);
+          case 7: return LBCG_TILE(8, 1, true, 2);
           default: break;
         }
       }
@@ -224,9 +225,8 @@ cudaError_t launch_batched_t(const RunDesc* d_runs, const int* run_of, long long
       if (i32) {
         switch (tile) {
           case 1:
+          case 3:
           case 5: return LBCG_TILE(8, 8, true, 2);
-          case 2: return LBCG_TILE(8, 2, true, 2);
-          case 3: return LBCG_TILE(8, 1, true, 2);
           case 4: return LBCG_TILE(4, 4, true, 4);
           default: break;
         }
