@@ -138,7 +138,9 @@ struct Tile {
 };
 constexpr int NUM_TILES = 6;   // what lb_set_tile takes
 constexpr int NUM_SHAPES = 8;  // and two shallow shapes that only the choice by size takes
-extern const Tile kTiles[NUM_SHAPES];
+extern const Tile kTiles[NUM_TILES];
+extern const Tile kShallow[NUM_SHAPES - NUM_TILES];
+inline const Tile& tile_shape(int shape) { return shape < NUM_TILES ? kTiles[shape] : kShallow[shape - NUM_TILES]; }
 
 size_t elem_bytes(int storage);
 // population-like arrays of a state: 2 x 27 (two sets), 27 (single set) or

@@ -345,7 +345,7 @@ int step_tile_of(const lb_handle* h) {
   const int order[4] = {1, 0, 6, 7};  // 32x8x8, x4, x2, x1
   const long long sms = sm_count_host();
   for (int k = 0; k < 4; ++k) {
-    const Tile& T = kTiles[order[k]];
+    const Tile& T = tile_shape(order[k]);
     const long long ctas = (long long)((h->g.nx + T.tx - 1) / T.tx) * ((h->g.ny + T.ty - 1) / T.ty) * ((h->g.nz + T.tz - 1) / T.tz);
     if (ctas >= (k == 0 ? 1 : 2) * sms) return order[k];
   }
@@ -1003,7 +1003,7 @@ int batch_descriptors(lb_batch* b) {
   b->max_rows = 0;
   for (lb_handle* h : b->runs) b->max_rows = std::max(b->max_rows, (long long)((h->g.nx + BLK - 1) / BLK) * h->g.ny);
   b->shape = batched_tile(b->storage, b->tile, b->halo, b->max_rows);
-  const Tile& T = kTiles[b->shape];
+  const Tile& T = tile_shape(b->shape);
   b->h_runs.resize(b->runs.size());
   for (size_t r = 0; r < b->runs.size(); ++r) {
     lb_handle* h = b->runs[r];

@@ -4,7 +4,8 @@
 
 namespace lbcg {
 
-const Tile kTiles[NUM_SHAPES] = {{32, 8, 4}, {32, 8, 8}, {32, 8, 4}, {32, 8, 8}, {32, 4, 4}, {32, 8, 8}, {32, 8, 2}, {32, 8, 1}};
+const Tile kTiles[NUM_TILES] = {{32, 8, 4}, {32, 8, 8}, {32, 8, 4}, {32, 8, 8}, {32, 4, 4}, {32, 8, 8}};
+const Tile kShallow[NUM_SHAPES - NUM_TILES] = {{32, 8, 2}, {32, 8, 1}};
 
 template <int ST>
 cudaError_t launch_phi_acc_t(const Geo& g, const StateBuf& in, unsigned long long* acc, cudaStream_t st);
