@@ -95,7 +95,7 @@ __device__ void block_tree(double (*s)[RED_THREADS], double v[NV]) {
 }
 
 // Sum over fluid nodes of (1 + phi)/2 from the sum of phi and the node count.
-__device__ __forceinline__ double volume_of(const Sum3& phi, int nodes) { return 0.5 * ((double)nodes + phi.value()); }
+__device__ __forceinline__ double volume_of(const Sum3& phi, int nodes) { return 0.5 * phi.plus(nodes); }
 // the kinetic term is formed from velocities scaled by SQUARE_SCALE
 constexpr double KE_UNSCALE = 0.5 * SQUARE_UNSCALE;
 
@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_partial(Geo g, const R* 
 
 // The same sums of FP32 fields, a thread's share in Sum3 terms, then FP64 for
 // the tree: the FP64 pipe (22 operations and conversions a node) bounded the
-// kernel above, 174 -> 86 us at 128x128x256.  A thread whose terms
-// overflow FP32 repeats its share in FP64.
+// kernel above, 174 -> 86 us at 128x128x256.  A thread whose terms leave
+// FP32's range repeats its share in FP64.
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_partial_f32(Geo g, const float* __restrict__ fl, double* partials) {
   __shared__ double s[8][RED_THREADS];
   const size_t N = (size_t)g.N;
@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_partial_f32(Geo g, const
   const long long end = beg + chunk < g.N ? beg + chunk : g.N;
   Sum3 a, b, j[3], ph, ke;
   int active = 0, nodes = 0;
+  bool moving = false;
   for (long long i = beg + threadIdx.x; i < end; i += RED_THREADS) {
     if (node_solid(g, i)) continue;
     ++nodes;
@@ -150,16 +151,15 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_partial_f32(Geo g, const
     for (int k = 0; k < 3; ++k) {
       const float p = __fmul_rn(rho, u[k]), e = __fmaf_rn(rho, u[k], -p);  // rho u = p + e
       j[k].add(p);
-      j[k].add(e);
-      const float w = __fmul_rn(u[k], SQUARE_SCALE);
-      const float ps = __fmul_rn(p, SQUARE_SCALE), es = __fmul_rn(e, SQUARE_SCALE);
-      ke.add_product(ps, w);
-      ke.add(__fmul_rn(es, w));
+      j[k].add_low(e);
+      ke.add_product(__fmul_rn(p, SQUARE_SCALE), __fmul_rn(e, SQUARE_SCALE), __fmul_rn(u[k], SQUARE_SCALE));
+      moving |= u[k] != 0.f;
     }
   }
   double v[8] = {a.value(),   b.value(),          j[0].value(),   j[1].value(),
                  j[2].value(), volume_of(ph, nodes), (double)active, KE_UNSCALE * ke.value()};
-  if (!(a.finite() && b.finite() && ph.finite() && j[0].finite() && j[1].finite() && j[2].finite() && ke.finite())) {
+  if (!(a.finite() && b.finite() && ph.finite() && j[0].finite() && j[1].finite() && j[2].finite() && ke.finite()) ||
+      (moving && ke.nearly_zero())) {
     for (int k = 0; k < 8; ++k) v[k] = 0.0;
     for (long long i = beg + threadIdx.x; i < end; i += RED_THREADS) {
       if (node_solid(g, i)) continue;

@@ -427,14 +427,15 @@ __global__ void __launch_bounds__(256) k_mse(long long N, int C, int nch, const 
 // The same four channels at a time (C % 4 == 0): quads past nch only store
 // their zeros, the index arithmetic is once per quad, and a thread's share of
 // the loss is summed in Sum3 terms (an FP64 product per element ran on the 2
-// FP64 lanes a clock and bounded the kernel, 254 us); a share that overflows
-// FP32 is taken again in FP64.  Bound by bytes.  128^3 nodes, C = 16, nch = 5:
+// FP64 lanes a clock and bounded the kernel, 254 us); a share that leaves FP32's
+// range is taken again in FP64.  Bound by bytes.  128^3 nodes, C = 16, nch = 5:
 // 281 -> 85 us.
 __global__ void __launch_bounds__(256) k_mse_v4(long long N, int G, int nch, const float4* __restrict__ p,
                                                 const float4* __restrict__ t, const float* __restrict__ wch,
                                                 float inv_count, float4* __restrict__ grad, double* __restrict__ loss) {
   __shared__ double red[256];
   Sum3 sum;
+  bool off = false;
   for (long long e = grid_stride_begin(); e < N * G; e += grid_stride()) {
     const int c0 = (int)(e % G) * 4;
     float o[4] = {0.f, 0.f, 0.f, 0.f};
@@ -447,15 +448,15 @@ __global__ void __launch_bounds__(256) k_mse_v4(long long N, int G, int nch, con
         const float w = wch[c0 + k];
         const float ds = __fmul_rn(d[k], SQUARE_SCALE);
         const float q = __fmul_rn(w, ds), r = __fmaf_rn(w, ds, -q);  // w d = q + r
-        sum.add_product(q, ds);
-        sum.add(__fmul_rn(r, ds));
+        sum.add_product(q, r, ds);
+        off |= w != 0.f && d[k] != 0.f;
         o[k] = 2.0f * w * d[k] * inv_count;
       }
     }
     grad[e] = make_float4(o[0], o[1], o[2], o[3]);
   }
   double s = sum.value() * SQUARE_UNSCALE;
-  if (!sum.finite()) {
+  if (!sum.finite() || (off && sum.nearly_zero())) {
     s = 0.0;
     for (long long e = grid_stride_begin(); e < N * G; e += grid_stride()) {
       const int c0 = (int)(e % G) * 4;
