@@ -170,6 +170,9 @@ cudaError_t launch_phi_acc(int storage, const Geo& g, const StateBuf& in, unsign
 cudaError_t launch_step(int storage, int loader, bool write_state, bool write_fields, int tile, const Geo& g,
                         const Phys& p, const StateBuf& in, const InitBuf& init, PhiSrc src, AccBufs ab, StateBuf out,
                         void* phi, int halo, const FieldOut& fields, unsigned* status, cudaStream_t st);
+// the density test of the current level alone (status bit 1; accin: its accumulator, null with LOAD_FIELDS)
+cudaError_t launch_density(int storage, int loader, const Geo& g, const Phys& p, const StateBuf& in, const InitBuf& init,
+                           const unsigned long long* accin, unsigned* status, cudaStream_t st);
 // phi of the current level into the padded array, nothing else
 cudaError_t launch_phi_only(int storage, const Geo& g, const Phys& p, const InitBuf& init, PhiSrc src, void* phi, int halo,
                             cudaStream_t st);

@@ -401,6 +401,16 @@ int ensure_fields(lb_handle* h) {
   return LB_OK;
 }
 
+// phi of the current level into the padded array, with the density test that a
+// pass over the populations makes.
+int padded_phi(lb_handle* h) {
+  LB_CUDA(launch_phi_only(h->storage, h->g, h->p, init_buf(h), phi_src(h), h->phi, h->halo, h->stream));
+  LB_CUDA(launch_density(h->storage, h->mode == 0 ? LOAD_FIELDS : LOAD_PULL, h->g, h->p, h->S[h->cur], init_buf(h),
+                         phi_src(h).acc, h->status, h->stream));
+  g_launches += 2;
+  return LB_OK;
+}
+
 // Write the fields of mask at the current time level: into the fields buffer
 // (field k at k N), or packed into dst (compute type).
 int compute_fields(lb_handle* h, uint32_t mask, void* dst = nullptr) {
@@ -410,14 +420,16 @@ int compute_fields(lb_handle* h, uint32_t mask, void* dst = nullptr) {
     if (rc) return rc;
   }
   if (dst && mask == LB_F_PHI) {  // no population enters phi
-    LB_CUDA(launch_phi_only(h->storage, h->g, h->p, init_buf(h), phi_src(h), h->phi, h->halo, h->stream));
+    const int rc = padded_phi(h);
+    if (rc) return rc;
     LB_CUDA(launch_phi_plain(h->storage, h->g, pad_geo(h->g, h->halo), h->phi, dst, h->stream));
+    g_launches += 1;
   } else {
     LB_CUDA(launch_step(h->storage, h->mode == 0 ? LOAD_FIELDS : LOAD_PULL, false, true, 0, h->g, h->p, h->S[h->cur],
                         init_buf(h), phi_src(h), AccBufs{nullptr, nullptr}, h->S[h->cur ^ 1], h->phi, h->halo,
                         field_out(dst ? dst : h->fields, mask, dst != nullptr), h->status, h->stream));
+    g_launches += 2;
   }
-  g_launches += 2;
   return LB_OK;
 }
 
@@ -796,9 +808,10 @@ int lb_droplet_count(lb_handle* h, int32_t* count) {
   if (!h->initialised) return set_err(LB_ESTATE, "handle not initialised");
   if (!h->labels && !(h->labels = (int*)dev_alloc(h, (size_t)h->g.N * sizeof(int))))
     return set_err(LB_ENOMEM, "label buffer allocation failed");
-  LB_CUDA(launch_phi_only(h->storage, h->g, h->p, init_buf(h), phi_src(h), h->phi, h->halo, h->stream));
+  const int rc = padded_phi(h);
+  if (rc) return rc;
   LB_CUDA(launch_cc(h->storage, h->g, h->phi, pad_geo(h->g, h->halo), h->labels, h->count, h->status, h->stream));
-  g_launches += 3;
+  g_launches += 2;
   int c = 0;
   unsigned st = 0;
   LB_CUDA(cudaMemcpyAsync(&c, h->count, sizeof(int), cudaMemcpyDeviceToHost, h->stream));

@@ -917,6 +917,48 @@ __global__ void __launch_bounds__(256) k_phi(PhiSrc src, InitBuf init, Geo g, Pa
     phi_row<R, SC>(src, init, g, pg, psi0, out, zero, (int)(row % g.ny), (int)(row / g.ny));
 }
 
+// The density test of the step and of the field pass (rho within (0, RHO_MAX),
+// or the run is marked unstable) by itself, for readouts of phi alone: k_phi's
+// sums are integers that a population which is not a number does not enter, so
+// the populations are pulled and summed as the step does it.  Initial fields
+// (LOAD_FIELDS) need phi and rho only, since fields_node's densities do not
+// depend on its populations.  One node per thread; bound by the population
+// bytes (half a step's), or 4 to 8 bytes a node.
+template <int ST, int LOADER>
+__global__ void __launch_bounds__(256) k_density(View<ST> S, InitBuf init, const unsigned long long* __restrict__ accin, Geo g,
+                                                 PhysR<typename Store<ST>::R> P, unsigned* __restrict__ status) {
+  using R = typename Store<ST>::R;
+  using E = typename Store<ST>::E;
+  bool bad = false;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < g.N; idx += stride) {
+    const int x = (int)(idx % g.nx);
+    const long long yz = idx / g.nx;
+    const int y = (int)(yz % g.ny), z = (int)(yz / g.ny);
+    if (is_solid(g, x, y, z)) continue;
+    Nbr n;
+    make_nbr(g, x, y, z, n);
+    R f[Q], rA, rB;
+    if constexpr (LOADER == LOAD_PULL) {
+      E ra[Q], rb[Q];
+      pull_walled<ST>(S, g, n, Lay<ST>::at(g, x, y, z), ra, rb, f);
+      if constexpr (!Store<ST>::MOMENT) pull_finish<ST>(ra, rb, f, rA, rB);
+      if constexpr (!Store<ST>::TWOSET) {
+        R rt = R(0);
+#pragma unroll
+        for (int i = 0; i < Q; ++i) rt += f[i];
+        Acc<R>::densities(accin, (size_t)idx, rA, rB);
+        rB = rt - rA;
+      }
+    } else {
+      fields_node<R, false>(init, g, P, n, idx, f, rA, rB, nullptr, nullptr);
+    }
+    const R rho = rA + rB;
+    bad |= !(rho > R(0) && rho < R(Acc<R>::RHO_MAX));
+  }
+  if (bad) atomicOr(status, 1u);
+}
+
 // ---------------------------------------------------------------------------
 // shared-memory layout of a tile
 // ---------------------------------------------------------------------------

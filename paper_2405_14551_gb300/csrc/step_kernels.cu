@@ -16,6 +16,9 @@ cudaError_t launch_step_s(int loader, bool ws, bool wf, int tile, const Geo& g, 
 template <int ST>
 cudaError_t launch_phi_s(const Geo& g, const Phys& p, const InitBuf& init, PhiSrc src, void* phi, int halo, cudaStream_t st);
 template <int ST>
+cudaError_t launch_density_t(int loader, const Geo& g, const Phys& p, const StateBuf& in, const InitBuf& init,
+                             const unsigned long long* accin, unsigned* status, cudaStream_t st);
+template <int ST>
 cudaError_t launch_batched_t(const RunDesc* d_runs, const int* run_of, long long ntiles, long long ngroups, int tile, int halo,
                              long long max_rows, int parity, int k, int blocks_per_sm, unsigned* status,
                              cudaStream_t st);
@@ -54,6 +57,18 @@ cudaError_t launch_phi_only(int storage, const Geo& g, const Phys& p, const Init
     case 2: return launch_phi_s<2>(g, p, init, src, phi, halo, st);
     case 3: return launch_phi_s<3>(g, p, init, src, phi, halo, st);
     case 4: return launch_phi_s<4>(g, p, init, src, phi, halo, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_density(int storage, int loader, const Geo& g, const Phys& p, const StateBuf& in, const InitBuf& init,
+                           const unsigned long long* accin, unsigned* status, cudaStream_t st) {
+  switch (storage) {
+    case 0: return launch_density_t<0>(loader, g, p, in, init, accin, status, st);
+    case 1: return launch_density_t<1>(loader, g, p, in, init, accin, status, st);
+    case 2: return launch_density_t<2>(loader, g, p, in, init, accin, status, st);
+    case 3: return launch_density_t<3>(loader, g, p, in, init, accin, status, st);
+    case 4: return launch_density_t<4>(loader, g, p, in, init, accin, status, st);
   }
   return cudaErrorInvalidValue;
 }
