@@ -91,10 +91,9 @@ __global__ void __launch_bounds__(256) k_phi_plain(Geo g, PadGeo pg, const R* __
   for (long long row = (long long)blockIdx.x * 8 + threadIdx.y; row < rows; row += (long long)gridDim.x * 8) {
     const long long y = row % g.ny, z = row / g.ny;
     const R* src = phi + pg.hx + (long long)pg.px * (pg.h + y + (long long)pg.py * (pg.h + z));
-    for (int x = threadIdx.x; x < g.nx; x += 32) {
-      const R v = src[x];
-      plain[row * g.nx + x] = v > R(0.5) * R(PHI_SOLID) ? R(0) : v;
-    }
+    const bool solid_row = (g.wy && (y == 0 || y == g.ny - 1)) || (g.wz && (z == 0 || z == g.nz - 1));
+    for (int x = threadIdx.x; x < g.nx; x += 32)  // by place, not by the marker: phi itself may be as large
+      plain[row * g.nx + x] = solid_row || (g.wx && (x == 0 || x == g.nx - 1)) ? R(0) : src[x];
   }
 }
 cudaError_t launch_phi_plain(int storage, const Geo& g, const PadGeo& pg, const void* phi, void* plain, cudaStream_t st) {

@@ -80,3 +80,28 @@ def test_density_of_a_stepped_level_is_reported(storage, model, how):
         read(s)
         assert _unstable(s) == bad, scale
         s.close()
+
+
+@pytest.mark.parametrize("storage", STORAGES)
+def test_phi_alone_equals_phi_among_others(storage):
+    """Also where phi is infinite, not a number or as large as the marker of
+    solid nodes."""
+    import torch
+
+    import paper_2405_14551_gb300.lbcg as L
+    f64 = storage == "twoset_f64"
+    for steps in (0, 3):
+        phi = _phi()
+        if steps == 0:
+            phi[2, 3, 4], phi[2, 3, 6], phi[5, 5, 5], phi[6, 5, 5] = np.inf, np.nan, 1e30, -np.inf
+        s = _sim(storage, 0b010)
+        s.init_fields(phi)
+        s.step(steps)
+        n = SHAPE[::-1]
+        one = torch.empty((1,) + n, dtype=torch.float64 if f64 else torch.float32, device="cuda")
+        two = torch.empty((2,) + n, dtype=one.dtype, device="cuda")
+        L.lb_fields(s.h, 0b1, one, True, f64=f64)
+        L.lb_fields(s.h, 0b11, two, True, f64=f64)
+        np.testing.assert_array_equal(one[0].cpu().numpy(), two[0].cpu().numpy())
+        assert not one[0, :, 0].any() and not one[0, :, -1].any()  # solid layers
+        s.close()
