@@ -44,8 +44,9 @@ extern "C" {
 /* ---- population storage formats ---------------------------------------- */
 /* Two population sets f^A, f^B in FP32; 432 B per node update.  (On the device
  * the populations of every storage but the moments lie in blocks of 32 nodes of
- * a row, [nz][ny][ceil(nx / 32)][comp * 27][32]; files and lb_get_populations
- * hold [comp][27][nz][ny][nx].) */
+ * a z plane, [nz][ceil(pitch ny / 32)][comp * 27][32], node x + pitch y of the
+ * plane, where pitch is nx rounded up to a multiple of 8 if that adds at most a
+ * sixteenth and nx itself otherwise; files and lb_get_populations hold [comp][27][nz][ny][nx].) */
 #define LB_STORAGE_TWOSET_F32 0
 /* Exact single-set form: total post-collision f* (27 x FP32) plus the colour
  * scalars s = rhoA/rho and v = beta rhoA rhoB/rho n (one float4); the pulling

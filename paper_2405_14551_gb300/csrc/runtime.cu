@@ -990,7 +990,7 @@ struct lb_batch {
   std::vector<RunDesc> h_runs;
   int* d_run_of = nullptr;  // run of every tile, then of every row group (owned by run 0)
   size_t run_of_cap = 0;
-  long long ntiles = 0, ngroups = 0, max_rows = 0, total_nodes = 0;
+  long long ntiles = 0, ngroups = 0, max_blocks = 0, total_nodes = 0;
   int halo = 1;  // staging halo of every run: the largest any of them needs
   int tile = 0;
   int shape = 0;  // the tile shape of the work list (batched_tile)
@@ -1013,9 +1013,9 @@ void batch_drop_graphs(lb_batch* b) {
 
 int batch_descriptors(lb_batch* b) {
   long long tb = 0, rb = 0;
-  b->max_rows = 0;
-  for (lb_handle* h : b->runs) b->max_rows = std::max(b->max_rows, (long long)((h->g.nx + BLK - 1) / BLK) * h->g.ny);
-  b->shape = batched_tile(b->storage, b->tile, b->halo, b->max_rows);
+  b->max_blocks = 0;
+  for (lb_handle* h : b->runs) b->max_blocks = std::max(b->max_blocks, (long long)plane_blocks(h->g));
+  b->shape = batched_tile(b->storage, b->tile, b->halo, b->max_blocks);
   const Tile& T = tile_shape(b->shape);
   b->h_runs.resize(b->runs.size());
   for (size_t r = 0; r < b->runs.size(); ++r) {
@@ -1060,7 +1060,7 @@ int batch_descriptors(lb_batch* b) {
 // one batched step from lattice parity `parity` and accumulator phase k
 int batch_issue(lb_batch* b, int parity, int k) {
   LB_CUDA(launch_batched(b->storage, b->d_runs, b->d_run_of, b->ntiles, b->ngroups, b->shape, b->halo,
-                         b->max_rows, parity, k, b->blocks_per_sm, b->runs[0]->status, b->stream));
+                         b->max_blocks, parity, k, b->blocks_per_sm, b->runs[0]->status, b->stream));
   g_launches += 2;
   return LB_OK;
 }

@@ -35,9 +35,9 @@
 // written once per step; the accumulators and the phase field add 8 B read,
 // 16 B atomically updated, 8 B zeroed and 4 B written and read per node (FP32
 // storages).
-// Populations lie in blocks of 32 nodes of a row, [z][y][x / 32][dir][32]
-// (Lay<ST>): for a fixed direction a warp reads one 128-byte line, and all
-// directions of a node are a constant offset apart.
+// Populations lie in blocks of 32 nodes of a z plane, [z][(x + pitch y) / 32][dir][32]
+// (Lay<ST>): for a fixed direction a warp reads 32 consecutive nodes of one or two
+// blocks, and all directions of a node are a constant offset apart.
 #include <cstdio>
 #include <cstdlib>
 #include <type_traits>
@@ -306,33 +306,36 @@ __device__ __forceinline__ bool region_walled(const Geo& g, int x0, int y0, int 
 }
 
 // Populations of a state (all storages but the moment records) are stored in
-// blocks of 32 nodes of a row: block (x / 32, y, z) holds its ND directions
-// one after the other, 32 values each.  A node's 27 (54) values then sit at
-// constant offsets from one address, and so do the values that one neighbour
-// row contributes, so that the pulls and stores of a node take their
-// direction from the instruction's immediate offset; a warp's store of a
-// whole node row is 32 x ND consecutive values.  With one array per direction
-// ([dir][z][y][x]) every access carried its own 64-bit address, some fifty
-// registers of them: 2.84 -> 2.57 ms per step of the 256x256x512 emulsion, 385
-// -> 358 us of Shan-Chen 128x128x256.
-// Rows are padded to whole blocks.
+// blocks of 32 nodes: the nodes of a z plane are counted x + pitch y, and block k
+// of the plane holds the ND directions of its 32 nodes one after the other, 32
+// values each.  A node's 27 (54) values then sit at constant offsets from one
+// address, and so do the values that one neighbour row contributes, so that the
+// pulls and stores of a node take their direction from the instruction's immediate
+// offset; with nx a multiple of 32 a warp's store of a whole node row is 32 x ND
+// consecutive values.  With one array per direction ([dir][z][y][x]) every access
+// carried its own 64-bit address, some fifty registers of them: 2.84 -> 2.57 ms per
+// step of the 256x256x512 emulsion, 385 -> 358 us of Shan-Chen 128x128x256.  Rows
+// that each began a block of their own cost nx = 33 1.94 times the memory, nx = 1 32
+// times, and their holes cost L2: 36x184x35, walls in y, 46.0 us a step against 38.7.
 template <int ST>
 struct Lay {
   using E = typename Store<ST>::E;
   static constexpr bool MOMENT = Store<ST>::MOMENT;
   static constexpr int ND = Store<ST>::TWOSET ? 2 * Q : Q;
   static constexpr int DS = MOMENT ? 1 : BLK;         // stride of the directions
-  // elements of one row, and element of node x of a row at direction 0 (moment
-  // storage: the node index)
-  __host__ __device__ __forceinline__ static size_t row(const Geo& g) {
-    return MOMENT ? (size_t)g.nx : (size_t)((g.nx + BLK - 1) / BLK) * (ND * BLK);
+  // nodes from one row to the next; elements of one z plane; the element of node n
+  // of a plane at direction 0 (moment storage: the node itself)
+  __host__ __device__ __forceinline__ static int pitch(const Geo& g) { return MOMENT ? g.nx : row_pitch(g.nx); }
+  __host__ __device__ __forceinline__ static size_t plane(const Geo& g) {
+    if constexpr (MOMENT) return (size_t)g.nx * (size_t)g.ny;
+    else return plane_blocks(g) * (ND * BLK);
   }
   template <typename I>
-  __host__ __device__ __forceinline__ static I in_row(I x) {
-    return MOMENT ? x : x / BLK * (I)(ND * BLK) + x % BLK;
+  __host__ __device__ __forceinline__ static I in_plane(I n) {
+    return MOMENT ? n : n / BLK * (I)(ND * BLK) + n % BLK;
   }
   __host__ __device__ __forceinline__ static size_t at(const Geo& g, int x, int y, int z) {
-    return row(g) * ((size_t)y + (size_t)g.ny * z) + in_row((size_t)x);
+    return plane(g) * (size_t)z + in_plane((size_t)x + (size_t)pitch(g) * (size_t)y);
   }
 };
 
@@ -501,7 +504,7 @@ template <int ST, bool IDX32>
 struct PlaneIdx {
   using I = typename std::conditional<IDX32, unsigned, size_t>::type;
   I o[3][3];  // [y + 1][x + 1] element offset within a plane (moment storage: node offset)
-  __device__ __forceinline__ static I at(const Geo& g, int x, int y) { return (I)Lay<ST>::row(g) * (I)y + Lay<ST>::in_row((I)x); }
+  __device__ __forceinline__ static I at(const Geo& g, int x, int y) { return Lay<ST>::in_plane((I)x + (I)Lay<ST>::pitch(g) * (I)y); }
   __device__ __forceinline__ void init(const Geo& g, int x, int y) {
     int xs[3], ys[3];
 #pragma unroll
@@ -528,7 +531,7 @@ template <int ST, bool IDX32>
 __device__ __forceinline__ void pull_plane(const View<ST>& S, const Geo& g, const PlaneIdx<ST, IDX32>& ix, const int zs[3],
                                            typename Store<ST>::E ra[Q], typename Store<ST>::E rb[Q]) {
   using E = typename Store<ST>::E;
-  const size_t plane = Lay<ST>::row(g) * (size_t)g.ny;
+  const size_t plane = Lay<ST>::plane(g);
   const E* zp[3] = {S.f + (size_t)zs[0] * plane, S.f + (size_t)zs[1] * plane, S.f + (size_t)zs[2] * plane};
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
@@ -1175,7 +1178,7 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
   if constexpr (WALLFREE) ix.init(g, x, y);
   else ix.o[1][1] = PI::at(g, x, y);
   const auto self_o = ix.o[1][1];
-  const size_t plane_e = Lay<ST>::row(g) * (size_t)g.ny;  // elements of a z plane
+  const size_t plane_e = Lay<ST>::plane(g);  // elements of a z plane
   int c = H * L::SXY + (ty + H) * L::SX + (tx + L::HX);
   int e0 = L::EXY + (ty + 1) * L::EX + (tx + 1);
   // gradient planes at z - 1 and z: a wall-free column takes one new plane a node
@@ -1524,7 +1527,7 @@ __device__ __forceinline__ void step_nodes_sc(const View<ST>& S, const View<ST>&
   if constexpr (WALLFREE) ix.init(g, x, y);
   else ix.o[1][1] = PI::at(g, x, y);
   const auto self_o = ix.o[1][1];
-  const size_t plane_e = Lay<ST>::row(g) * (size_t)g.ny;  // elements of a z plane
+  const size_t plane_e = Lay<ST>::plane(g);  // elements of a z plane
   int c = L::SXY + (ty + 1) * L::SX + (tx + L::HX);
   int e0 = L::EXY + (ty + 1) * L::EX + (tx + 1);
   GradPlane<R> alo, amid, blo, bmid;

@@ -20,7 +20,7 @@ cudaError_t launch_density_t(int loader, const Geo& g, const Phys& p, const Stat
                              const unsigned long long* accin, unsigned* status, cudaStream_t st);
 template <int ST>
 cudaError_t launch_batched_t(const RunDesc* d_runs, const int* run_of, long long ntiles, long long ngroups, int tile, int halo,
-                             long long max_rows, int parity, int k, int blocks_per_sm, unsigned* status,
+                             long long max_blocks, int parity, int k, int blocks_per_sm, unsigned* status,
                              cudaStream_t st);
 template <int ST>
 cudaError_t launch_export_t(int loader, const Geo& g, const Phys& p, const StateBuf& in, const InitBuf& init, int x0,
@@ -118,18 +118,18 @@ cudaError_t launch_export(int storage, int loader, const Geo& g, const Phys& p, 
 }
 
 cudaError_t launch_batched(int storage, const RunDesc* d_runs, const int* run_of, long long ntiles, long long ngroups, int tile,
-                           int halo, long long max_rows, int parity, int k, int blocks_per_sm, unsigned* status,
+                           int halo, long long max_blocks, int parity, int k, int blocks_per_sm, unsigned* status,
                            cudaStream_t st) {
   switch (storage) {
-    case 0: return launch_batched_t<0>(d_runs, run_of, ntiles, ngroups, tile, halo, max_rows, parity, k, blocks_per_sm, status, st);
-    case 1: return launch_batched_t<1>(d_runs, run_of, ntiles, ngroups, tile, halo, max_rows, parity, k, blocks_per_sm, status, st);
-    case 2: return launch_batched_t<2>(d_runs, run_of, ntiles, ngroups, tile, halo, max_rows, parity, k, blocks_per_sm, status, st);
+    case 0: return launch_batched_t<0>(d_runs, run_of, ntiles, ngroups, tile, halo, max_blocks, parity, k, blocks_per_sm, status, st);
+    case 1: return launch_batched_t<1>(d_runs, run_of, ntiles, ngroups, tile, halo, max_blocks, parity, k, blocks_per_sm, status, st);
+    case 2: return launch_batched_t<2>(d_runs, run_of, ntiles, ngroups, tile, halo, max_blocks, parity, k, blocks_per_sm, status, st);
   }
   return cudaErrorInvalidValue;  // no batched FP64 or moment instantiation
 }
 
-int batched_tile(int storage, int tile, int halo, long long max_rows) {
-  const unsigned long long plane = (unsigned long long)max_rows * BLK * (unsigned long long)state_arrays(storage) * elem_bytes(storage);
+int batched_tile(int storage, int tile, int halo, long long max_blocks) {
+  const unsigned long long plane = (unsigned long long)max_blocks * BLK * (unsigned long long)state_arrays(storage) * elem_bytes(storage);
   return halo >= 6 || plane >= (1ull << 32) ? 0 : tile;
 }
 
@@ -146,11 +146,11 @@ int sm_count_host() {
 
 template <typename E>
 __global__ void __launch_bounds__(256) k_direction(Geo g, E* __restrict__ f, int nd, int dir, E* __restrict__ plain, bool gather) {
-  const long long nbx = (g.nx + BLK - 1) / BLK;
+  const long long nb = (long long)plane_blocks(g);
+  const int pitch = row_pitch(g.nx);
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < g.N; i += (long long)gridDim.x * blockDim.x) {
-    const long long row = i / g.nx;
-    const int x = (int)(i - row * g.nx);
-    E& v = f[((row * nbx + x / BLK) * nd + dir) * BLK + x % BLK];
+    const long long row = i / g.nx, z = row / g.ny, n = (row - z * g.ny) * pitch + (i - row * g.nx);
+    E& v = f[((z * nb + n / BLK) * nd + dir) * BLK + n % BLK];
     if (gather) plain[i] = v;
     else v = plain[i];
   }
@@ -171,7 +171,7 @@ size_t elem_bytes(int storage) { return storage == 3 ? 8 : (storage == 2 ? 2 : 4
 int state_arrays(int storage) { return storage == 4 ? MOMENT_COEFS : (storage == 0 || storage == 3 ? 2 * Q : Q); }
 size_t state_elems(int storage, const Geo& g) {
   if (storage == 4) return (size_t)MOMENT_COEFS * (size_t)g.N;
-  return (size_t)((g.nx + BLK - 1) / BLK) * BLK * (size_t)g.ny * (size_t)g.nz * (size_t)state_arrays(storage);
+  return plane_blocks(g) * BLK * (size_t)g.nz * (size_t)state_arrays(storage);
 }
 bool storage_is_twoset(int storage) { return storage == 0 || storage == 3; }
 bool storage_is_f64(int storage) { return storage == 3; }

@@ -29,8 +29,7 @@ inline int resident_ctas(K kern, int threads, size_t smem) {
 // 32-bit byte offsets within a z plane of nx x ny nodes (moment storage: 16-byte records)
 template <int ST>
 inline bool fits_idx32(const Geo& g) {
-  const unsigned long long row = Lay<ST>::row(g) * (Store<ST>::MOMENT ? 16 : sizeof(typename Store<ST>::E));
-  return row * (unsigned long long)g.ny < (1ull << 32);
+  return (unsigned long long)Lay<ST>::plane(g) * (Store<ST>::MOMENT ? 16 : sizeof(typename Store<ST>::E)) < (1ull << 32);
 }
 
 // Calls f with the staging halo (1, 4, 6 or 7) as a compile-time constant.
@@ -219,7 +218,7 @@ inline cudaError_t launch_batched_step_t(const RunDesc* d_runs, const int* run_o
 
 template <int ST>
 cudaError_t launch_batched_t(const RunDesc* d_runs, const int* run_of, long long ntiles, long long ngroups, int tile, int halo,
-                             long long max_rows, int parity, int k, int blocks_per_sm, unsigned* status,
+                             long long max_blocks, int parity, int k, int blocks_per_sm, unsigned* status,
                              cudaStream_t st) {
   const long long cap = (long long)sm_count() * 8;
   const int pblocks = (int)(ngroups < cap ? ngroups : cap);
@@ -227,9 +226,9 @@ cudaError_t launch_batched_t(const RunDesc* d_runs, const int* run_of, long long
   cudaError_t e = launch_pdl(k_phi_batched<float>, dim3(pblocks), dim3(32, 8), 0, st, d_runs, run_of + ntiles, ngroups, k);
   if (e != cudaSuccess) return e;
   const int blocks = sm_count() * (blocks_per_sm > 0 ? blocks_per_sm : 2);
-  Geo wide{};  // a plane with as many nodes as the largest of the runs, a row to itself
+  Geo wide{};  // a plane with as many blocks as the largest of the runs
   wide.nx = BLK;
-  wide.ny = (int)max_rows;
+  wide.ny = (int)max_blocks;
   const bool i32 = fits_idx32<ST>(wide);
   return with_stage_halo(halo, [&](auto hc) -> cudaError_t {
     constexpr int H = decltype(hc)::value;
