@@ -162,9 +162,9 @@ __device__ __forceinline__ R eval_moment(const float4& qa, const float4& qb, con
 // Stored post-collision total population f*_dir of node src (single set
 // storages).  Reduced: the stored value.  Moment storage: the node's
 // quadratic form (eval_moment); only the records that c_i touches are read.
-template <int ST>
+template <int ST, typename I>
 __device__ __forceinline__ typename Store<ST>::R load_fs(const typename Store<ST>::E* __restrict__ f, size_t N, int dir,
-                                                         size_t src, int i, bool bb) {
+                                                         I src, int i, bool bb) {
   using R = typename Store<ST>::R;
   if constexpr (Store<ST>::MOMENT) {
     const float4 qa = reinterpret_cast<const float4*>(f)[src];
@@ -295,6 +295,26 @@ __device__ __forceinline__ bool is_solid(const Geo& g, int x, int y, int z) {
 __device__ __forceinline__ bool near_wall(const Geo& g, int x, int y, int z) {
   return (g.wx && (x <= 1 || x >= g.nx - 2)) || (g.wy && (y <= 1 || y >= g.ny - 2)) ||
          (g.wz && (z <= 1 || z >= g.nz - 2));
+}
+
+// Directions whose source x - c_i is solid, as bit i of a word: the x and y part of
+// a fluid node's column, and the z part of the node.  One bit test a direction
+// replaces three flags and their union, for the pull and (bit opp(i): x + c_i) for
+// the sends.
+__host__ __device__ constexpr unsigned dirs_along(int axis, int sign) {
+  unsigned m = 0;
+  for (int i = 0; i < Q; ++i)
+    if ((axis == 0 ? cx(i) : axis == 1 ? cy(i) : cz(i)) == sign) m |= 1u << i;
+  return m;
+}
+__device__ __forceinline__ unsigned axis_bits(int wall, int v, int n, unsigned lower, unsigned upper) {
+  return wall ? (v <= 1 ? lower : 0u) | (v >= n - 2 ? upper : 0u) : 0u;
+}
+__device__ __forceinline__ unsigned column_bits(const Geo& g, int x, int y) {
+  return axis_bits(g.wx, x, g.nx, dirs_along(0, 1), dirs_along(0, -1)) | axis_bits(g.wy, y, g.ny, dirs_along(1, 1), dirs_along(1, -1));
+}
+__device__ __forceinline__ unsigned node_bits(const Geo& g, int z) {
+  return axis_bits(g.wz, z, g.nz, dirs_along(2, 1), dirs_along(2, -1));
 }
 
 // Whether the box [x0 - d, x0 + TX - 1 + d] x ... (a tile and its halo of d
@@ -495,9 +515,9 @@ __device__ __forceinline__ T* uniform(T* p) {
   const unsigned lo = __reduce_or_sync(0xffffffffu, (unsigned)v), hi = __reduce_or_sync(0xffffffffu, (unsigned)(v >> 32));
   return reinterpret_cast<T*>(((unsigned long long)hi << 32) | lo);
 }
-// Where a node of a tile without solid neighbours (WALLFREE) reads its
-// neighbours' values.  The z plane of a source is the same for the whole CTA,
-// so a thread keeps nine offsets within a plane (3 x 3 neighbours in x and y)
+// Where a node reads its neighbours' values.  The z plane of a source is the
+// same for the whole CTA, so a thread keeps nine offsets within a plane (3 x 3
+// neighbours in x and y, wrapped; a fluid node of a walled axis never wraps)
 // for all its nodes; 27 addresses serve all pulls.  IDX32: the byte offsets
 // within one z plane fit in 32 bits.
 template <int ST, bool IDX32>
@@ -526,19 +546,28 @@ __device__ __forceinline__ T plane_ld(const T* __restrict__ base, I o) {
 }
 // The raw stored values a node pulls (both sets, or the single set's totals),
 // loaded before anything is decoded so that independent work (gradient, scan)
-// runs while they are in flight.
-template <int ST, bool IDX32>
+// runs while they are in flight.  Not WALLFREE: where wall has the direction's
+// bit, the opposite direction of the node itself (halfway bounce-back), as one
+// predicated load each way (selecting the address: 3 % slower at walls in x, single set).
+template <int ST, bool IDX32, bool WALLFREE>
 __device__ __forceinline__ void pull_plane(const View<ST>& S, const Geo& g, const PlaneIdx<ST, IDX32>& ix, const int zs[3],
-                                           typename Store<ST>::E ra[Q], typename Store<ST>::E rb[Q]) {
+                                           unsigned wall, typename Store<ST>::E ra[Q], typename Store<ST>::E rb[Q]) {
   using E = typename Store<ST>::E;
   const size_t plane = Lay<ST>::plane(g);
   const E* zp[3] = {S.f + (size_t)zs[0] * plane, S.f + (size_t)zs[1] * plane, S.f + (size_t)zs[2] * plane};
+  auto at = [](const E* z, auto o) { return reinterpret_cast<const E*>(reinterpret_cast<const char*>(z) + o * (unsigned)sizeof(E)); };
+  const E* self = at(zp[1], ix.o[1][1]);
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
-    const auto o = ix.o[1 - cy(i)][1 - cx(i)];
-    const E* p = reinterpret_cast<const E*>(reinterpret_cast<const char*>(zp[1 - cz(i)]) + o * (unsigned)sizeof(E));
-    ra[i] = p[i * BLK];
-    if constexpr (Store<ST>::TWOSET) rb[i] = p[(Q + i) * BLK];
+    const int a = 1 - cx(i), b = 1 - cy(i), c = 1 - cz(i);
+    const E* p = at(zp[c], ix.o[b][a]);
+    if (!WALLFREE && (wall >> i & 1u)) {
+      ra[i] = self[opp(i) * BLK];
+      if constexpr (Store<ST>::TWOSET) rb[i] = self[(Q + opp(i)) * BLK];
+    } else {
+      ra[i] = p[i * BLK];
+      if constexpr (Store<ST>::TWOSET) rb[i] = p[(Q + i) * BLK];
+    }
   }
 }
 // moment storage: the quadratic forms of the neighbours, evaluated
@@ -558,8 +587,25 @@ __device__ __forceinline__ void pull_plane_moment(const View<ST>& S, size_t N, s
     f[i] = eval_moment<R>(qa, qb, qc, i, false);
   }
 }
-// The same loads of a node with solid neighbours in reach (halfway
-// bounce-back from the node itself, Lay::at element self), any offset width.
+// The same with solid neighbours in reach, by node index (a lattice has fewer
+// than 2^31 nodes).
+template <int ST>
+__device__ __forceinline__ void pull_walled_moment(const View<ST>& S, const Geo& g, const Nbr& n, unsigned wall, int self,
+                                                   typename Store<ST>::R f[Q]) {
+  int row[3][3];
+#pragma unroll
+  for (int b = 0; b < 3; ++b)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) row[b][c] = g.nx * (n.ys[b] + g.ny * n.zs[c]);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const int a = 1 - cx(i), b = 1 - cy(i), c = 1 - cz(i);
+    const bool bb = wall >> i & 1u;
+    f[i] = load_fs<ST>(S.f, (size_t)g.N, i, (unsigned)(bb ? self : n.xs[a] + row[b][c]), i, bb);
+  }
+}
+// The same loads of any node (self: its Lay::at element), at any offset width,
+// outside the step.
 template <int ST>
 __device__ __forceinline__ void pull_walled(const View<ST>& S, const Geo& g, const Nbr& n, size_t self,
                                             typename Store<ST>::E ra[Q], typename Store<ST>::E rb[Q],
@@ -1112,16 +1158,16 @@ __device__ __forceinline__ void put_field(const FieldOut& o, int k, size_t N, si
 // accumulator index e0 to the node that pulls them: x + c_i, or the node
 // itself when x + c_i is solid (halfway bounce-back).
 template <bool WALLFREE, int EX, int EXY>
-__device__ __forceinline__ int send_to(int e0, const Nbr& n, int i) {
+__device__ __forceinline__ int send_to(int e0, unsigned wall, int i) {
   int e = e0 + cx(i) + EX * cy(i) + EXY * cz(i);
   if constexpr (!WALLFREE) {
-    if (n.sx[1 + cx(i)] | n.sy[1 + cy(i)] | n.sz[1 + cz(i)]) e = e0;
+    if (wall >> opp(i) & 1u) e = e0;
   }
   return e;
 }
 template <typename R, bool WALLFREE, int EX, int EXY, int E>
-__device__ __forceinline__ void send(unsigned long long* sw, int e0, const Nbr& n, int i, R a, R b) {
-  Acc<R>::send_shared(sw, E, send_to<WALLFREE, EX, EXY>(e0, n, i), a, b);
+__device__ __forceinline__ void send(unsigned long long* sw, int e0, unsigned wall, int i, R a, R b) {
+  Acc<R>::send_shared(sw, E, send_to<WALLFREE, EX, EXY>(e0, wall, i), a, b);
 }
 
 // Single-set storages: what colour_split gives the puller of the stored total
@@ -1131,10 +1177,10 @@ __device__ __forceinline__ void send(unsigned long long* sw, int e0, const Nbr& 
 // multiplications a direction fall away (bound by issue; FP16 storage at
 // 128x128x256: 329 -> 322 us a step).
 template <bool WALLFREE, typename L>
-__device__ __forceinline__ void send_split(unsigned long long* sw, int e0, const Nbr& n, int i, float fs, const float4& sv,
+__device__ __forceinline__ void send_split(unsigned long long* sw, int e0, unsigned wall, int i, float fs, const float4& sv,
                                            float seg) {
   const float va = fma_rn(sv.x, fs, seg);
-  Acc<float>::send_shared_scaled(sw, L::E, send_to<WALLFREE, L::EX, L::EXY>(e0, n, i), va, fs - va);
+  Acc<float>::send_shared_scaled(sw, L::E, send_to<WALLFREE, L::EX, L::EXY>(e0, wall, i), va, fs - va);
 }
 // the scaled segregation term w_i c_i.v/|c_i| of colour_split
 __device__ __forceinline__ float split_seg(const float4& sv, int i) {
@@ -1175,8 +1221,8 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
   if (x >= g.nx || y >= g.ny) return;
   using PI = PlaneIdx<ST, IDX32>;
   PI ix;
-  if constexpr (WALLFREE) ix.init(g, x, y);
-  else ix.o[1][1] = PI::at(g, x, y);
+  ix.init(g, x, y);
+  const unsigned wall_xy = WALLFREE ? 0u : column_bits(g, x, y);
   const auto self_o = ix.o[1][1];
   const size_t plane_e = Lay<ST>::plane(g);  // elements of a z plane
   int c = H * L::SXY + (ty + H) * L::SX + (tx + L::HX);
@@ -1199,17 +1245,15 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
       continue;
     }
     Nbr n;
-    if constexpr (!WALLFREE || LOADER != LOAD_PULL) make_nbr(g, x, y, z, n);
+    const unsigned wall = WALLFREE ? 0u : wall_xy | node_bits(g, z);
+    if constexpr (LOADER != LOAD_PULL || (Store<ST>::MOMENT && !WALLFREE)) make_nbr(g, x, y, z, n);
     R f[Q], rA, rB;
     E ra[Q], rb[Q];
     auto pull = [&]() {
-      if constexpr (WALLFREE) {
-        const int zs[3] = {z > 0 ? z - 1 : g.nz - 1, z, z + 1 < g.nz ? z + 1 : 0};
-        if constexpr (Store<ST>::MOMENT) pull_plane_moment<ST, IDX32>(S, N, plane, ix, zs, f);
-        else pull_plane<ST, IDX32>(S, g, ix, zs, ra, rb);
-      } else {
-        pull_walled<ST>(S, g, n, (size_t)z * plane_e + self_o, ra, rb, f);
-      }
+      const int zs[3] = {z > 0 ? z - 1 : g.nz - 1, z, z + 1 < g.nz ? z + 1 : 0};
+      if constexpr (Store<ST>::MOMENT && !WALLFREE) pull_walled_moment<ST>(S, g, n, wall, (int)self, f);
+      else if constexpr (Store<ST>::MOMENT) pull_plane_moment<ST, IDX32>(S, N, plane, ix, zs, f);
+      else pull_plane<ST, IDX32, WALLFREE>(S, g, ix, zs, wall, ra, rb);
     };
     if constexpr (LOADER == LOAD_PULL && EARLY) pull();
     const R phx = sp[c];
@@ -1396,7 +1440,7 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
         const float fs = mul_rn(eval_moment<R>(qa, qb, qc, i, false), Acc<float>::SCALE);
-        send_split<WALLFREE, L>(sw, e0, n, i, fs, svo, i == REST ? 0.f : split_seg(svo, i));
+        send_split<WALLFREE, L>(sw, e0, wall, i, fs, svo, i == REST ? 0.f : split_seg(svo, i));
       }
       continue;
     }
@@ -1410,11 +1454,11 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
         const R fb = fs - fa;
         op[REST * BLK] = encode<ST>(fa, REST);
         op[(Q + REST) * BLK] = encode<ST>(fb, REST);
-        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, REST, fa, fb);
+        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, wall, REST, fa, fb);
       } else {
         const typename Store<ST>::E enc = encode<ST>(fs, REST);
         op[REST * BLK] = enc;
-        send_split<WALLFREE, L>(sw, e0, n, REST, decode_scaled<ST>(enc, REST), svo, 0.f);
+        send_split<WALLFREE, L>(sw, e0, wall, REST, decode_scaled<ST>(enc, REST), svo, 0.f);
       }
     }
 #pragma unroll
@@ -1451,8 +1495,8 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
         op[q * BLK] = encode<ST>(faq, q);
         op[(Q + p) * BLK] = encode<ST>(fbp, p);
         op[(Q + q) * BLK] = encode<ST>(fbq, q);
-        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, p, fap, fbp);
-        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, q, faq, fbq);
+        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, wall, p, fap, fbp);
+        send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, wall, q, faq, fbq);
       } else {
         const typename Store<ST>::E ep = encode<ST>(fsp, p), eq = encode<ST>(fsq, q);
         op[p * BLK] = ep;
@@ -1460,8 +1504,8 @@ __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O,
         // p and its opposite q: c_q.v = -(c_p.v) exactly, so the segregation term
         // is formed once and negated (bit for bit what colour_split gives for q)
         const float seg = split_seg(svo, p);
-        send_split<WALLFREE, L>(sw, e0, n, p, decode_scaled<ST>(ep, p), svo, seg);
-        send_split<WALLFREE, L>(sw, e0, n, q, decode_scaled<ST>(eq, q), svo, -seg);
+        send_split<WALLFREE, L>(sw, e0, wall, p, decode_scaled<ST>(ep, p), svo, seg);
+        send_split<WALLFREE, L>(sw, e0, wall, q, decode_scaled<ST>(eq, q), svo, -seg);
       }
     }
   }
@@ -1524,8 +1568,8 @@ __device__ __forceinline__ void step_nodes_sc(const View<ST>& S, const View<ST>&
   if (x >= g.nx || y >= g.ny) return;
   using PI = PlaneIdx<ST, IDX32>;
   PI ix;
-  if constexpr (WALLFREE) ix.init(g, x, y);
-  else ix.o[1][1] = PI::at(g, x, y);
+  ix.init(g, x, y);
+  const unsigned wall_xy = WALLFREE ? 0u : column_bits(g, x, y);
   const auto self_o = ix.o[1][1];
   const size_t plane_e = Lay<ST>::plane(g);  // elements of a z plane
   int c = L::SXY + (ty + 1) * L::SX + (tx + L::HX);
@@ -1549,15 +1593,12 @@ __device__ __forceinline__ void step_nodes_sc(const View<ST>& S, const View<ST>&
       continue;
     }
     Nbr n;
-    if constexpr (!WALLFREE || LOADER != LOAD_PULL) make_nbr(g, x, y, z, n);
+    const unsigned wall = WALLFREE ? 0u : wall_xy | node_bits(g, z);
+    if constexpr (LOADER != LOAD_PULL) make_nbr(g, x, y, z, n);
     R fa[Q], fb[Q], rA = R(0), rB = R(0);
     if constexpr (LOADER == LOAD_PULL) {  // two-set storages: the stored values are the populations
-      if constexpr (WALLFREE) {
-        const int zs[3] = {z > 0 ? z - 1 : g.nz - 1, z, z + 1 < g.nz ? z + 1 : 0};
-        pull_plane<ST, IDX32>(S, g, ix, zs, fa, fb);
-      } else {
-        pull_walled<ST>(S, g, n, (size_t)z * plane_e + self_o, fa, fb, nullptr);
-      }
+      const int zs[3] = {z > 0 ? z - 1 : g.nz - 1, z, z + 1 < g.nz ? z + 1 : 0};
+      pull_plane<ST, IDX32, WALLFREE>(S, g, ix, zs, wall, fa, fb);
     }
     R gA[3], gB[3], gphi[3];
     if constexpr (WALLFREE) {
@@ -1663,7 +1704,7 @@ __device__ __forceinline__ void step_nodes_sc(const View<ST>& S, const View<ST>&
     auto put = [&](int i, R oa, R ob) {
       op[i * BLK] = encode<ST>(oa, i);
       op[(Q + i) * BLK] = encode<ST>(ob, i);
-      send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, n, i, oa, ob);
+      send<R, WALLFREE, L::EX, L::EXY, L::E>(sw, e0, wall, i, oa, ob);
     };
     put(REST, fma_rn(ka, fa[REST], mul_rn(wgt<R>(REST), qa.a)), fma_rn(kb, fb[REST], mul_rn(wgt<R>(REST), qb.a)));
     auto pairs = [&](auto cls) {
@@ -1711,9 +1752,11 @@ __device__ __forceinline__ void step_tile(const View<ST>& S, const View<ST>& O, 
   }
   cp_async_wait_all();
   __syncthreads();
-  // a tile whose one-node halo (with near contact: the scan's halo of K + 1
-  // nodes) holds no solid node needs no bounce-back or wall tests
-  const bool wallfree = !region_walled(g, x0, y0, z0, TX, TY, TZ, (H > 1 && P.A_h != R(0)) ? P.K + 1 : 1);
+  // A warp (a row of the tile) whose one-node halo (with near contact: the scan's
+  // halo of K + 1 nodes) holds no solid node needs no bounce-back or wall tests.
+  // Decided per warp: at a wall in y one row of eight takes the walled path.
+  const bool wallfree =
+      !region_walled(g, x0, uniform(y0 + (int)threadIdx.y), z0, TX, 1, TZ, (H > 1 && P.A_h != R(0)) ? P.K + 1 : 1);
   if constexpr (SC) {
     R* spa = sp + (NPH - 2) * L::NS;
     R* spb = spa + L::NS;
