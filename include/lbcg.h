@@ -188,13 +188,14 @@ int lb_init_fields(lb_handle* h, const float* phi, const float* rho, const float
  * Runs of 12 steps are replayed from a captured CUDA graph. */
 int lb_step(lb_handle* h, int64_t nsteps);
 
-/* Choose the tile shape of the step kernel (0..5: 32x8x4 for 0 and 2, 32x8x8 for
- * 1, 3 and 5, 32x4x4 for 4, in nodes per CTA); used by autotuners.  Without
- * this call the step picks a shape by the lattice's size.  Results do not
- * depend on the tile (bit for bit).  The widest staging halo (h_max >= 4),
- * FP64 storage, the Shan-Chen model and lattices whose z planes exceed 32-bit
- * byte offsets step with tile 0 whatever the setting.  lb_get_tile returns
- * the index last set (0 if none). */
+/* Choose the tile shape of the step kernel (0..5: 32x8x4 for 0, 32x8x8 for 1 and
+ * 5, 32x4x4 for 4, in nodes per CTA; 2 and 3: by size); used by autotuners.  Without
+ * this call, and where the shape gives an SM of the GPU less than one CTA of 256
+ * threads, the step picks a shape by the lattice's size.  Results do not depend on
+ * the tile (bit for bit).  The wide staging halos (h_max >= 4), FP64 storage and
+ * lattices whose z planes exceed 32-bit byte offsets step with 32x8x4 whatever the
+ * setting, the Shan-Chen model with 32x8x4 or a shallower shape by size.
+ * lb_get_tile returns the index last set (0 if none). */
 int lb_set_tile(lb_handle* h, int tile);
 int lb_get_tile(const lb_handle* h);
 

@@ -333,23 +333,45 @@ AccBufs acc_bufs(const lb_handle* h) {
   return AccBufs{h->acc[(k + 1) % 3], h->acc[(k + 2) % 3]};
 }
 
-// Tile of a handle whose caller chose none: the deepest tile (fewest halo nodes
-// staged and partial sums flushed per node) that gives every SM a CTA, two for
-// the shallower ones; on small lattices the tile that spreads the
-// nodes over the most SMs, since a step then lasts as long as one tile's chain
-// of nodes.  Measured us per step, x8 / x4 / x2 / x1: 32^3 29 / 25 / 17 / 13 (4 to
-// 32 times fewer CTAs than SM slots), 64x64x128 55 / 58 / 59 / 64, 256x256x512
-// 2560 / 2660 / 2890 / 3350.
-int step_tile_of(const lb_handle* h) {
-  if (h->tile_chosen) return h->tile;
-  const int order[4] = {1, 0, 6, 7};  // 32x8x8, x4, x2, x1
-  const long long sms = sm_count_host();
-  for (int k = 0; k < 4; ++k) {
-    const Tile& T = tile_shape(order[k]);
-    const long long ctas = (long long)((h->g.nx + T.tx - 1) / T.tx) * ((h->g.ny + T.ty - 1) / T.ty) * ((h->g.nz + T.tz - 1) / T.tz);
-    if (ctas >= (k == 0 ? 1 : 2) * sms) return order[k];
+// Shape of a handle's steps.  Where the caller set none (or 2 or 3, whose capped
+// forms are gone), the one of least modelled time: the busiest SM walks its share of
+// the CTAs two at a time (128 registers: two fit), a pair takes 10 / 9 of one alone,
+// and a CTA costs its TZ nodes a thread plus 3 / 4 of a node for staging and flush.
+// From 16 CTAs an SM on the last wave is lost in the rest.  Over 14 sizes from 24^3
+// to 128^3 with no, one or two walled axes, four storages and halos of 1 and 4: 0.4 %
+// over the fastest of the four on average, 8 % at worst, and nowhere slower than the
+// steps were with one array per direction.  Other overheads are worse: at 0.5 of a node
+// 100^3 takes 32x8x2 (reduced FP32, near contact: 98 us a step for 90), at 1 33x74x86
+// takes 32x8x8 (50 for 33).  The rule before, the deepest shape with a CTA an SM, took
+// 96x80x112 in two waves of 32x8x8 (two-set FP32, near contact: 107 us a step; 32x8x4 92).
+// A shape that the caller set stands where it gives every SM a CTA of 256 threads;
+// below that a step lasts as long as one CTA's chain of nodes, and the choice by
+// size is up to three times as fast (24^3, two-set FP32: 25 us with 32x8x8, 8.6 with 32x8x1).
+long long shape_ctas(const Geo& g, int shape) {
+  const Tile& T = tile_shape(shape);
+  return (long long)((g.nx + T.tx - 1) / T.tx) * ((g.ny + T.ty - 1) / T.ty) * ((g.nz + T.tz - 1) / T.tz);
+}
+int step_shape_of(const Geo& g, bool shan_chen, int set, long long sms) {
+  if (set >= 0 && set != 2 && set != 3) {
+    const Tile& T = tile_shape(set);
+    if (shape_ctas(g, set) * T.tx * T.ty >= 256 * sms) return set;
   }
-  return order[3];
+  const int order[4] = {1, 0, 6, 7};  // 32x8x8, x4, x2, x1
+  int best = -1;
+  double least = 0.0;
+  for (int k = shan_chen ? 1 : 0; k < 4; ++k) {  // Shan-Chen has no 32x8x8
+    const long long ctas = shape_ctas(g, order[k]), share = (ctas + sms - 1) / sms;
+    const double walk = share > 16 ? 5.0 * (double)ctas / (double)sms : 10.0 * (double)(share / 2) + 9.0 * (double)(share % 2);
+    const double t = (tile_shape(order[k]).tz + 0.75) * walk;
+    if (best < 0 || t < least) {
+      best = order[k];
+      least = t;
+    }
+  }
+  return best;
+}
+int step_tile_of(const lb_handle* h) {
+  return step_shape_of(h->g, h->p.model == LB_MODEL_SHAN_CHEN, h->tile_chosen ? h->tile : -1, sm_count_host());
 }
 
 // Issue one step (no graph).

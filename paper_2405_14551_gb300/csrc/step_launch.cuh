@@ -108,9 +108,10 @@ inline cudaError_t launch_step_t(const Geo& g, const Phys& p, const StateBuf& in
                     reinterpret_cast<const R*>(phi), pg, g, phys_as<R>(p), fields, status);
 }
 
-// Tile shapes of the hot variant (pull, write state): kTiles; the wide halos
-// (6, 7) only with tile 0.  Other variants, FP64, Shan-Chen and planes
-// that need 64-bit offsets use tile 0.
+// Tile shapes of the hot variant (pull, write state): kTiles and kShallow;
+// Shan-Chen takes 32x8x4 and the shallow ones (48^3, walls in x and y: 32x8x4 24.4 us a
+// step, 32x8x2 15.5).  Other variants, the wide halos (6, 7), FP64 and planes that
+// need 64-bit offsets use 32x8x4.
 template <int ST, int LOADER, bool WS, bool WF, bool SC>
 inline cudaError_t launch_step_tiles(int tile, const Geo& g, const Phys& p, const StateBuf& in, const InitBuf& init,
                                      PhiSrc src, AccBufs ab, StateBuf out, void* phi, int halo, const FieldOut& fields,
@@ -123,13 +124,16 @@ inline cudaError_t launch_step_tiles(int tile, const Geo& g, const Phys& p, cons
     constexpr int H = decltype(hc)::value;
 #define LBCG_TILE(TY, TZ, I32, MB) \
   launch_step_t<ST, LOADER, WS, WF, 32, TY, TZ, H, I32, MB, SC>(g, p, in, init, src, ab, out, phi, pg, fields, status, st)
-    if constexpr (LOADER == LOAD_PULL && WS && !WF && ST != 3 && H < 6 && !SC) {
+    if constexpr (LOADER == LOAD_PULL && WS && !WF && ST != 3 && H < 6) {
       if (i32) {
         switch (tile) {
           case 1:
-          case 3:
-          case 5: return LBCG_TILE(8, 8, true, 2);
-          case 4: return LBCG_TILE(4, 4, true, 4);
+          case 5:
+            if constexpr (!SC) return LBCG_TILE(8, 8, true, 2);
+            break;
+          case 4:
+            if constexpr (!SC) return LBCG_TILE(4, 4, true, 4);
+            break;
           case 6: return LBCG_TILE(8, 2, true, 2);
           case 7: return LBCG_TILE(8, 1, true, 2);
           default: break;
