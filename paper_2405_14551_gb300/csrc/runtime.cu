@@ -222,8 +222,9 @@ bool alloc_state(lb_handle* h, StateBuf& s) {
 }
 
 // Copy the current populations (and colour scalars) to or from a host buffer
-// in checkpoint order, one direction at a time through a buffer of N values.
-// Synchronises the stream.
+// in checkpoint order, one direction at a time through the other lattice of the
+// ping-pong pair, which the next step overwrites whole: a checkpoint needs no
+// device memory of its own.  Synchronises the stream.
 int copy_state_host(lb_handle* h, char* host, bool to_host) {
   const StateBuf& s = h->S[h->cur];
   const size_t N = (size_t)h->g.N, eb = elem_bytes(h->storage), nd = (size_t)state_arrays(h->storage);
@@ -232,8 +233,7 @@ int copy_state_host(lb_handle* h, char* host, bool to_host) {
   if (h->storage == LB_STORAGE_MOMENT_F32) {  // records, same order on the device
     e = to_host ? cudaMemcpyAsync(host, s.f, nd * N * eb, kind, h->stream) : cudaMemcpyAsync(s.f, host, nd * N * eb, kind, h->stream);
   } else {
-    void* tmp = dev_alloc(h, N * eb);
-    if (!tmp) return set_err(LB_ENOMEM, "checkpoint buffer allocation failed");
+    void* tmp = h->S[h->cur ^ 1].f;
     for (size_t d = 0; d < nd && e == cudaSuccess; ++d) {
       char* at = host + d * N * eb;
       if (!to_host) e = cudaMemcpyAsync(tmp, at, N * eb, kind, h->stream);
@@ -241,8 +241,6 @@ int copy_state_host(lb_handle* h, char* host, bool to_host) {
       g_launches += 1;
       if (to_host && e == cudaSuccess) e = cudaMemcpyAsync(at, tmp, N * eb, kind, h->stream);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    dev_free(h, tmp);
   }
   if (e == cudaSuccess && !storage_is_twoset(h->storage)) {
     char* at = host + nd * N * eb;

@@ -1,0 +1,61 @@
+"""What calls need beyond the memory of the handle: nothing for a checkpoint."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+STORAGES = ["twoset_f32", "reduced_f32", "reduced_f16", "twoset_f64", "moment_f32"]
+
+
+def _phi(shape, seed=1):
+    r = np.random.default_rng(seed)
+    return np.clip(r.standard_normal(shape[::-1]), -1, 1).astype(np.float32)
+
+
+class _Budget:
+    """Memory from PyTorch until `full` is set."""
+
+    def __new__(cls, device=0):
+        import paper_2405_14551_gb300.lbcg as L
+
+        class A(L.TorchAllocator):
+            full = False
+
+            def _alloc(self, ctx, nbytes):
+                return None if self.full else super()._alloc(ctx, nbytes)
+        return A(device)
+
+
+def _handle(shape, storage, seed=1):
+    import ctypes
+
+    import paper_2405_14551_gb300.lbcg as L
+    a = _Budget()
+    h = L.lb_create(L.make_grid(*shape), L.make_params(storage=storage, collision=int(storage == "moment_f32")), a)
+    L.lb_init_fields(h, _phi(shape, seed))
+    return h, a
+
+
+def _populations(h, shape):
+    import paper_2405_14551_gb300.lbcg as L
+    return L.lb_get_populations(h, (0, 0, 0) + shape)
+
+
+@pytest.mark.parametrize("storage", STORAGES)
+def test_checkpoints_need_no_device_memory(tmp_path, storage):
+    import paper_2405_14551_gb300.lbcg as L
+    shape, path = (37, 6, 5), str(tmp_path / "c.bin")
+    h, a = _handle(shape, storage)
+    k, b = _handle(shape, storage, 2)
+    for steps in (3, 4):  # both lattices of the pair as the current one
+        L.lb_step(h, steps)
+        a.full = b.full = True
+        L.lb_save(h, path)
+        L.lb_load(k, path)
+        L.lb_step(h, 2)
+        L.lb_step(k, 2)
+        a.full = b.full = False
+        for p, q in zip(_populations(h, shape), _populations(k, shape)):
+            np.testing.assert_array_equal(p, q)
+    L.lb_destroy(h)
+    L.lb_destroy(k)
