@@ -209,7 +209,9 @@ int64_t lb_time(const lb_handle* h);
 
 /* Write the selected fields at the current time level, [k][nz][ny][nx] float
  * in increasing bit order of mask, to dst (device or host pointer of
- * popcount(mask)*N floats, caller-owned).  Synchronises the stream when dst is
+ * popcount(mask)*N floats, caller-owned).  Kernels store straight into memory of
+ * the handle's GPU; a device destination of any other kind (another GPU's memory,
+ * pinned host memory) is filled by copies.  Synchronises the stream when dst is
  * on the host.  Solid nodes hold 0. */
 int lb_fields(lb_handle* h, uint32_t mask, float* dst, int dst_is_device);
 /* Same in double precision (fields of an FP64 handle keep full precision). */

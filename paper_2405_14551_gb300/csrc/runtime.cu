@@ -719,12 +719,24 @@ int lb_set_tile(lb_handle* h, int tile) {
 
 int lb_get_tile(const lb_handle* h) { return h ? h->tile : -1; }
 
+// Whether a kernel on the handle's device can store to p as to its own memory.
+// Another GPU's memory and host memory are reached by a copy, which the driver
+// routes without peer access and at the link's full rate.
+static bool stores_reach(const lb_handle* h, const void* p) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeManaged || (a.type == cudaMemoryTypeDevice && a.device == h->device);
+}
+
 static int fields_out(lb_handle* h, uint32_t mask, void* dst, int dst_is_device, bool dbl) {
   if (!h) return set_err(LB_EINVAL, "null handle");
   if (!dst) return set_err(LB_EINVAL, "dst is null");
   if (mask == 0 || (mask >> NFIELDS)) return set_err(LB_EINVAL, "field mask must select fields 0..13");
   const bool f64 = storage_is_f64(h->storage);
-  if (dst_is_device && f64 == dbl) return compute_fields(h, mask, dst);  // straight to the caller's array
+  if (dst_is_device && f64 == dbl && stores_reach(h, dst)) return compute_fields(h, mask, dst);  // straight to the caller's array
   int rc = compute_fields(h, mask);
   if (rc) return rc;
   const size_t N = (size_t)h->g.N;
@@ -747,7 +759,7 @@ static int fields_out(lb_handle* h, uint32_t mask, void* dst, int dst_is_device,
       g_launches += 1;
       from = tmp;
     }
-    cudaError_t e = cudaMemcpyAsync(d, from, N * ob, dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+    cudaError_t e = cudaMemcpyAsync(d, from, N * ob, dst_is_device ? cudaMemcpyDefault : cudaMemcpyDeviceToHost,
                                     h->stream);
     if (e != cudaSuccess) {
       if (tmp) dev_free(h, tmp);

@@ -236,8 +236,12 @@ def lb_set_stream(h, stream_ptr: int):
 def _used_by(h, *tensors):
     """Device tensors handed to a call on handle h: the caching allocator must
     not give their memory away before the handle's stream, which need not be
-    the tensors' own, has passed the call."""
+    the tensors' own, has passed the call.  (Host tensors, and arrays of another
+    kind, are not that allocator's.)"""
     import torch
+    tensors = [t for t in tensors if isinstance(t, torch.Tensor) and t.is_cuda]
+    if not tensors:
+        return
     s = torch.cuda.ExternalStream(load_library().lb_get_stream(h) or 0)
     for t in tensors:
         t.record_stream(s)

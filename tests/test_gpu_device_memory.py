@@ -1,4 +1,5 @@
-"""What calls need beyond the memory of the handle: nothing for a checkpoint."""
+"""What calls need beyond the memory of the handle: nothing for a checkpoint; and
+the destinations that a field readout takes."""
 import numpy as np
 import pytest
 
@@ -59,3 +60,32 @@ def test_checkpoints_need_no_device_memory(tmp_path, storage):
             np.testing.assert_array_equal(p, q)
     L.lb_destroy(h)
     L.lb_destroy(k)
+
+
+@pytest.mark.parametrize("storage,mask", [("twoset_f32", 0b1), ("reduced_f16", 0b10011), ("twoset_f64", 0b101)])
+def test_device_destination_that_is_not_this_gpus_memory(storage, mask):
+    """Pinned host memory, as a tensor and as a bare pointer, passed as a device
+    destination."""
+    import torch
+
+    import paper_2405_14551_gb300.lbcg as L
+    shape = (37, 6, 5)
+    s = L.Sim(*shape, storage=storage)
+    s.init_fields(_phi(shape))
+    s.step(4)
+    n = bin(mask).count("1")
+    for f64 in (False, True):
+        dt = torch.float64 if f64 else torch.float32
+        want = torch.empty((n,) + shape[::-1], dtype=dt, device="cuda")
+        L.lb_fields(s.h, mask, want, True, f64=f64)
+        pinned = torch.zeros(want.shape, dtype=dt, pin_memory=True)
+
+        class Bare:
+            def data_ptr(self):
+                return pinned.data_ptr()
+        for dst in (pinned, Bare()):
+            pinned.zero_()
+            L.lb_fields(s.h, mask, dst, True, f64=f64)
+            torch.cuda.synchronize()
+            assert torch.equal(pinned, want.cpu())
+    s.close()
