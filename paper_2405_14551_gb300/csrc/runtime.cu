@@ -1020,8 +1020,7 @@ struct lb_batch {
   int device = 0;
   RunDesc* d_runs = nullptr;
   std::vector<RunDesc> h_runs;
-  int* d_run_of = nullptr;  // run of every tile, then of every row group (owned by run 0)
-  size_t run_of_cap = 0;
+  int* d_run_of = nullptr;  // run of every tile, then of every row group (owned by run 0; room for the smallest tiles)
   long long ntiles = 0, ngroups = 0, max_blocks = 0, total_nodes = 0;
   int halo = 1;  // staging halo of every run: the largest any of them needs
   int tile = 0;
@@ -1043,12 +1042,14 @@ void batch_drop_graphs(lb_batch* b) {
   }
 }
 
+// work items of k_phi_batched
+long long row_groups(const Geo& g) { return ((long long)g.ny * g.nz + 7) / 8; }
+
 int batch_descriptors(lb_batch* b) {
   long long tb = 0, rb = 0;
   b->max_blocks = 0;
   for (lb_handle* h : b->runs) b->max_blocks = std::max(b->max_blocks, (long long)plane_blocks(h->g));
   b->shape = batched_tile(b->storage, b->tile, b->halo, b->max_blocks);
-  const Tile& T = tile_shape(b->shape);
   b->h_runs.resize(b->runs.size());
   for (size_t r = 0; r < b->runs.size(); ++r) {
     lb_handle* h = b->runs[r];
@@ -1062,8 +1063,8 @@ int batch_descriptors(lb_batch* b) {
     d.pg = pad_geo(h->g, h->halo);
     d.tile_begin = tb;
     d.row_begin = rb;
-    tb += (long long)((h->g.nx + T.tx - 1) / T.tx) * ((h->g.ny + T.ty - 1) / T.ty) * ((h->g.nz + T.tz - 1) / T.tz);
-    rb += ((long long)h->g.ny * h->g.nz + 7) / 8;
+    tb += shape_ctas(h->g, b->shape);
+    rb += row_groups(h->g);
   }
   b->ntiles = tb;
   b->ngroups = rb;
@@ -1072,14 +1073,6 @@ int batch_descriptors(lb_batch* b) {
     const bool last = r + 1 == b->h_runs.size();
     std::fill(run_of.begin() + b->h_runs[r].tile_begin, run_of.begin() + (last ? tb : b->h_runs[r + 1].tile_begin), (int)r);
     std::fill(run_of.begin() + tb + b->h_runs[r].row_begin, run_of.begin() + tb + (last ? rb : b->h_runs[r + 1].row_begin), (int)r);
-  }
-  if (run_of.size() > b->run_of_cap) {
-    LB_CUDA(cudaStreamSynchronize(b->stream));  // steps in flight read the old table
-    dev_free(b->runs[0], b->d_run_of);
-    b->run_of_cap = 0;
-    b->d_run_of = (int*)dev_alloc(b->runs[0], run_of.size() * sizeof(int));
-    if (!b->d_run_of) return set_err(LB_ENOMEM, "work list allocation failed");
-    b->run_of_cap = run_of.size();
   }
   LB_CUDA(cudaMemcpyAsync(b->d_run_of, run_of.data(), run_of.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
   LB_CUDA(cudaMemcpyAsync(b->d_runs, b->h_runs.data(), sizeof(RunDesc) * b->h_runs.size(), cudaMemcpyHostToDevice,
@@ -1220,7 +1213,10 @@ int lb_batch_create(int32_t nruns, const lb_grid* grids, const lb_params* params
     b->total_nodes += h->g.N;
   }
   b->d_runs = (RunDesc*)dev_alloc(b->runs[0], sizeof(RunDesc) * (size_t)nruns);
-  if (!b->d_runs) {
+  long long items = 0;  // with the smallest tiles, 32x4x4
+  for (lb_handle* h : b->runs) items += shape_ctas(h->g, 4) + row_groups(h->g);
+  b->d_run_of = (int*)dev_alloc(b->runs[0], (size_t)items * sizeof(int));
+  if (!b->d_runs || !b->d_run_of) {
     lb_batch_destroy(b);
     return set_err(LB_ENOMEM, "descriptor allocation failed");
   }

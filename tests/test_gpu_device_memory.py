@@ -1,5 +1,5 @@
-"""What calls need beyond the memory of the handle: nothing for a checkpoint; and
-the destinations that a field readout takes."""
+"""What calls need beyond the memory of the handle: nothing for a checkpoint or a
+batch's steps; and the destinations that a field readout takes."""
 import numpy as np
 import pytest
 
@@ -60,6 +60,22 @@ def test_checkpoints_need_no_device_memory(tmp_path, storage):
             np.testing.assert_array_equal(p, q)
     L.lb_destroy(h)
     L.lb_destroy(k)
+
+
+def test_batched_steps_need_no_device_memory():
+    import paper_2405_14551_gb300.lbcg as L
+    shapes = [(33, 17, 9), (8, 40, 3), (64, 4, 4)]
+    a = _Budget()
+    b = L.lb_batch_create([L.make_grid(*s) for s in shapes], [L.make_params(A_h=0.1 * (k % 2)) for k in range(3)], a)
+    for k, s in enumerate(shapes):
+        L.lb_init_fields(L.lb_batch_run(b, k), _phi(s, k))
+    a.full = True
+    for tile in range(L.NUM_TILES):
+        L.lb_batch_set_tile(b, tile, 2)
+        L.lb_batch_step(b, 13)
+    L.lb_batch_check(b)
+    a.full = False
+    L.lb_batch_destroy(b)
 
 
 @pytest.mark.parametrize("storage,mask", [("twoset_f32", 0b1), ("reduced_f16", 0b10011), ("twoset_f64", 0b101)])
