@@ -342,8 +342,8 @@ int lb_batch_set_tile(lb_batch* b, int tile, int blocks_per_sm);
 /* Autotuner: time `steps` batched steps for every tile shape and CTAs-per-SM
  * in {1, 2, 4}, keep the fastest.  Needs freshly initialised runs (step 0)
  * and returns every run to its initial state afterwards.  With use_cache, a result stored for the same
- * GPU, storage and set of run shapes is reused.  Results are appended to the
- * file named by LBCG_TUNE_CACHE (default $HOME/.cache/lbcg_tune.txt).
+ * GPU, storage, set of run shapes and revision of the tile table is reused.
+ * Results are appended to the file named by LBCG_TUNE_CACHE (default $HOME/.cache/lbcg_tune.txt).
  * result (host, 4 doubles): tile, blocks_per_sm, ms per step, 1 if cached. */
 int lb_batch_autotune(lb_batch* b, int32_t steps, int use_cache, double* result);
 

@@ -1150,6 +1150,11 @@ std::string tune_cache_path() {
   return std::string(home ? home : "/tmp") + "/.cache/lbcg_tune.txt";
 }
 
+// What a tile index launches and what was timed: raised whenever a tile shape, the
+// meaning of an index or the batched kernel changes, so that the choice and the
+// time of another build are not taken for this one's.
+constexpr int TUNE_REVISION = 2;
+
 std::string batch_key(const lb_batch* b) {
   cudaDeviceProp prop{};
   int dev = 0;
@@ -1166,7 +1171,7 @@ std::string batch_key(const lb_batch* b) {
   std::string name = prop.name;
   for (char& c : name)
     if (c == ' ') c = '_';
-  key << name << "|st" << b->storage << "|";
+  key << "rev" << TUNE_REVISION << "|" << name << "|st" << b->storage << "|";
   for (auto& sh : shapes) key << sh << ",";
   return key.str();
 }
