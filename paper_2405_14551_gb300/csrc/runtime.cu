@@ -1378,6 +1378,15 @@ int batch_tune(lb_batch* b, int32_t steps, int use_cache, double* result) {
   LB_CUDA(cudaEventCreate(&e0));
   LB_CUDA(cudaEventCreate(&e1));
   for (int tile = 0; tile < NUM_TILES; ++tile) {
+    // an index that launches a shape already timed (0 = 2, 1 = 3 = 5; all of them with a wide scan) is skipped
+    auto same = [&](int other) {
+      const Tile &s = tile_shape(batched_tile(b->storage, tile, b->halo, b->max_blocks)),
+                 &t = tile_shape(batched_tile(b->storage, other, b->halo, b->max_blocks));
+      return s.tx == t.tx && s.ty == t.ty && s.tz == t.tz;
+    };
+    bool timed = false;
+    for (int other = 0; other < tile; ++other) timed |= same(other);
+    if (timed) continue;
     for (int bps : bps_opts) {
       if ((rc = lb_batch_set_tile(b, tile, bps)) || (rc = batch_prepare(b))) break;
       for (int k = 0; k < 2 && rc == LB_OK; ++k) {

@@ -1,4 +1,4 @@
-"""The batch autotuner's cache file."""
+"""The batch autotuner: its cache file and what it times."""
 import numpy as np
 import pytest
 
@@ -27,3 +27,16 @@ def test_entries_of_another_revision_are_not_used(tmp_path, monkeypatch):
         path.write_text(f"{old} 3 1 0.000001\n")
         _, _, t, cached = _batch().autotune(steps=1)
         assert cached == 0 and t > 1e-5
+
+
+@pytest.mark.parametrize("h_max,shapes", [(3.0, 3), (5.0, 1)])
+def test_each_shape_is_timed_once(tmp_path, monkeypatch, h_max, shapes):
+    """Indexes that launch the same shape are timed once: per shape and number of
+    CTAs an SM two warm-up steps and one timed, of two launches each; one step more
+    for each run that has not begun."""
+    import paper_2405_14551_gb300.lbcg as L
+    monkeypatch.setenv("LBCG_TUNE_CACHE", str(tmp_path / "tune.txt"))
+    b = _batch(h_max)
+    before = L.lb_launch_count()
+    b.autotune(steps=1, use_cache=False)
+    assert L.lb_launch_count() - before == 2 * 3 + shapes * 3 * 3 * 2
