@@ -845,7 +845,7 @@ def main():
                        "l2": "state far larger than L2, no flush", "parallelism": f"replicas x{world}"},
             "roofline": {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak, "unit": "GB/s",
                          "frac": round(achieved / peak, 4), "traffic": traffic,
-                         "kernel": "k_step (the whole step: one launch)",
+                         "kernel": "k_phi + k_step (the whole step: two launches)",
                          "peak_kind": peak_kind, "kernel_ms": round(step_ms, 4),
                          "bytes_per_node": bpn, "whole_step_frac": round(step_frac, 4)},
             "cpu_baseline": cpu,

@@ -172,10 +172,10 @@ bool storage_is_f64(int storage);
 // two-set 339 against 430).  6 instead of 7 for K <= 5: 315 -> 303 us a step
 // of the reduced storage there.
 inline int stage_halo(const Phys& p) { return p.A_h == 0.0 ? 1 : (p.K <= 3 ? 4 : p.K <= 5 ? 6 : 7); }
-// rebuild the accumulator of the current time level from the populations of in
 // one direction of a state (not the moment storage) from its blocks to a plain
 // [z][y][x] array (gather) or back
 cudaError_t launch_direction(int storage, const Geo& g, void* f, int dir, void* plain, bool gather, cudaStream_t st);
+// rebuild the accumulator of the current time level from the populations of in
 cudaError_t launch_phi_acc(int storage, const Geo& g, const StateBuf& in, unsigned long long* acc, cudaStream_t st);
 // one step (write_state) or the fields of the current level (write_fields): two
 // launches, k_phi into the padded array phi (for a halo of `halo` nodes), then

@@ -5,6 +5,8 @@
 
 #include <string>
 
+#include <algorithm>
+
 #include "../../include/lbcg.h"
 #include "../../include/lbnn.h"
 #include "exact_sum.cuh"
@@ -601,8 +603,8 @@ int lbnn_relu_bias_bwd(const float* g, const void* y, int64_t nvox, int32_t c, i
     return report_error(LB_EINVAL, "relu_bias_bwd needs c % 4 == 0, a 16-byte aligned g and 8-byte aligned y and gb");
   // three CTAs an SM: enough loads in flight, and few enough that their atomics
   // on the c sums do not queue (eight: 29 us at 262144 voxels x 128 channels)
-  const long long need = (nvox * (c / 4) + 255) / 256;
-  k_relu_bias_bwd<<<(unsigned)(need < 456 ? need : 456), 256, 0, (cudaStream_t)stream>>>(
+  const long long need = (nvox * (c / 4) + 255) / 256, cap = 3ll * sm_count_host();
+  k_relu_bias_bwd<<<(unsigned)(need < cap ? need : cap), 256, 0, (cudaStream_t)stream>>>(
       nvox, c / 4, (const float4*)g, relu ? (const uint2*)y : nullptr, (uint2*)gb, db);
   return launch_result("relu_bias_bwd");
 }
@@ -618,7 +620,7 @@ int lbnn_mse(const float* p, const float* t, int64_t n, int32_t c, int32_t nch, 
              double* loss, void* stream) {
   if (!p || !t || !wch || !grad || !loss || n < 1 || nch < 1 || nch > c) return report_error(LB_EINVAL, "mse");
   if (c % 4 == 0 && aligned16(p, t, grad))
-    k_mse_v4<<<blocks_for(n * c / 4) < 912 ? blocks_for(n * c / 4) : 912, 256, 0, (cudaStream_t)stream>>>(n, c / 4, nch, (const float4*)p, (const float4*)t, wch,
+    k_mse_v4<<<std::min(blocks_for(n * c / 4), (unsigned)(6 * sm_count_host())), 256, 0, (cudaStream_t)stream>>>(n, c / 4, nch, (const float4*)p, (const float4*)t, wch,
                                                                       1.0f / (float)(n * nch), (float4*)grad, loss);
   else
     k_mse<<<blocks_for(n * c), 256, 0, (cudaStream_t)stream>>>(n, c, nch, p, t, wch, 1.0f / (float)(n * nch), grad, loss);

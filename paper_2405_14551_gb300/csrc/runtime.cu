@@ -453,7 +453,7 @@ int compute_fields(lb_handle* h, uint32_t mask, void* dst = nullptr) {
   return LB_OK;
 }
 
-// lb_create with a staging halo of at least min_halo (1, 4 or 7) nodes.
+// lb_create with a staging halo of at least min_halo (1, 4, 6 or 7) nodes.
 int create_handle(const lb_grid* grid, const lb_params* params, const lb_alloc* alloc, int min_halo, lb_handle** out) {
   if (!out) return set_err(LB_EINVAL, "out is null");
   *out = nullptr;

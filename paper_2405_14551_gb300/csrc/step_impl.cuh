@@ -3,24 +3,22 @@
 // (arXiv 2405.14551, Sec. III.B-III.D) for sm_103a.
 //
 // A step is two kernels.  k_phi decodes the phase field of the current level
-// from the component densities that the step before accumulated (item 4), once
+// from the component densities that the step before accumulated (item 3), once
 // per node, into an array padded by the staging halo, and zeroes the
 // accumulator two steps ahead.  k_step works on CTA tiles of TX x TY x TZ nodes
 // (TX x TY threads, TZ nodes per thread):
 //   1. stage phi(t) of the tile plus a halo of H nodes in shared memory
 //      (16-byte asynchronous copies from k_phi's array);
-//   2. with near contact (A_h != 0, halo H > K): every interface node of the
-//      tile scans along its outward normal (Eqs. stress_jump,
-//      near_cont_force); the distance h stays in shared memory.  The
-//      in-loop tile (INL) scans each interface node in item 3 instead,
-//      while the node's population loads are in flight;
-//   3. every thread pulls the 27 (x2) populations of its nodes (periodic
-//      wrap, halfway bounce-back at solid neighbours, Sec. III.D), takes the
-//      moments, the colour gradient from the staged tile, the repulsion from
-//      h, the Guo-shifted velocity, relaxes the total populations (BGK), adds
-//      the perturbation Omega^(2) and the forcing source, recolours (Eqs.
-//      ome3_1/2) and stores the post-collision state once;
-//   4. each post-collision component population f*^k_i(x) is also what the
+//   2. every thread walks its column of nodes.  Per node it issues the loads of
+//      the 27 (x2) populations (periodic wrap, halfway bounce-back at solid
+//      neighbours, Sec. III.D), takes the colour gradient from the staged tile
+//      and, at an interface node with near contact (A_h != 0, halo H > K), scans
+//      along its outward normal (Eqs. stress_jump, near_cont_force) while the
+//      loads are in flight; then the moments, the repulsion from the distance h,
+//      the Guo-shifted velocity, the relaxation of the total populations (BGK),
+//      the perturbation Omega^(2) and the forcing source, the recolouring (Eqs.
+//      ome3_1/2), and the post-collision state is stored once;
+//   3. each post-collision component population f*^k_i(x) is also what the
 //      node x + c_i pulls at the next step (x itself, as direction opp(i),
 //      when x + c_i is solid), so it is x's contribution to rho_k there.  The
 //      CTA sums the contributions over its tile plus a one-node ring in
@@ -656,11 +654,11 @@ __device__ __forceinline__ void pull_finish(const typename Store<ST>::E ra[Q], c
 // half, two's complement), so one atomic adds both.  FP64: SHIFT = 56 (sums
 // within +-128, step 1.4e-17), two 64-bit words per node.  RHO_MAX bounds the
 // density that the status check accepts, so that no sum leaves its range.
-// The accumulator words are staged, zeroed and updated by every step while
-// the population state streams through L2; their loads, stores and
-// reductions carry an evict-last L2 policy, so that more of them are still
-// in L2 when the next access comes (measured: 3.24 -> 3.17 ms per step on
-// the 256x256x512 emulsion).
+// The accumulator words are read, zeroed and updated by every step while the
+// population state streams through L2; their stores and reductions carry an
+// evict-last L2 policy, so that more of them are still in L2 when the next
+// access comes (256x256x512 emulsion, 3.24 -> 3.17 ms per step when it came in,
+// before k_phi).
 __device__ __forceinline__ unsigned long long acc_policy() {
   unsigned long long pol;
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
@@ -676,14 +674,6 @@ __device__ __forceinline__ void acc_st(unsigned long long* p, unsigned long long
                "l"(acc_policy())
                : "memory");
 }
-__device__ __forceinline__ ulonglong2 acc_ld2(const unsigned long long* p) {
-  ulonglong2 v;
-  asm volatile("ld.global.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"
-               : "=l"(v.x), "=l"(v.y)
-               : "l"(__cvta_generic_to_global(p)), "l"(acc_policy()));
-  return v;
-}
-
 template <typename R>
 struct Acc;
 template <>
@@ -872,8 +862,8 @@ __device__ __forceinline__ R sc_psi(R r, R psi0) {
 // start filling free SMs once all its own CTAs run, and touches global memory
 // only after its predecessor has completed.  That hides the launch latency,
 // the larger part of a step on small lattices.  Together with k_phi reading each
-// word once: 58.1 -> 54.5 us per step at 64x64x128, 2.57 -> 2.50 ms at
-// 256x256x512.
+// word once: 58.1 -> 54.5 us per step at 64x64x128 (an event after every step; 44.7
+// when 12 steps replay from a graph), 2.57 -> 2.50 ms at 256x256x512.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_primary() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
