@@ -335,13 +335,15 @@ AccBufs acc_bufs(const lb_handle* h) {
 // forms are gone), the one of least modelled time: the busiest SM walks its share of
 // the CTAs two at a time (128 registers: two fit), a pair takes 10 / 9 of one alone,
 // and a CTA costs its TZ nodes a thread plus 3 / 4 of a node for staging and flush.
-// From 16 CTAs an SM on the last wave is lost in the rest.  Over 14 sizes from 24^3
-// to 128^3 with no, one or two walled axes, four storages and halos of 1 and 4: 0.4 %
-// over the fastest of the four on average, 8 % at worst, and nowhere slower than the
-// steps were with one array per direction.  Other overheads are worse: at 0.5 of a node
-// 100^3 takes 32x8x2 (reduced FP32, near contact: 98 us a step for 90), at 1 33x74x86
-// takes 32x8x8 (50 for 33).  The rule before, the deepest shape with a CTA an SM, took
-// 96x80x112 in two waves of 32x8x8 (two-set FP32, near contact: 107 us a step; 32x8x4 92).
+// Beyond 8 CTAs an SM the CTAs have drifted apart and the last wave is lost in the
+// rest (184x128x160, FP16 without near contact: 32x8x8 at 12.6 CTAs an SM 209 us a
+// step, 32x8x4 227).  Over 20 sizes from 24^3 to 244x128x128 with no, one or two walled
+// axes, four storages and halos of 1 and 4: 0.3 % over the fastest of the four on
+// average, 9 % at worst, and nowhere slower than the steps were with one array per
+// direction.  Overheads from 0.5 to 0.9 of a node choose alike; at 1 33x74x86 takes
+// 32x8x8 (reduced FP32, near contact, walls in x and y: 50 us a step for 33).  The rule
+// before, the deepest shape with a CTA an SM, took 96x80x112 in two waves of 32x8x8
+// (two-set FP32, near contact: 107 us a step; 32x8x4 92).
 // A shape that the caller set stands where it gives every SM a CTA of 256 threads;
 // below that a step lasts as long as one CTA's chain of nodes, and the choice by
 // size is up to three times as fast (24^3, two-set FP32: 25 us with 32x8x8, 8.6 with 32x8x1).
@@ -359,7 +361,7 @@ int step_shape_of(const Geo& g, bool shan_chen, int set, long long sms) {
   double least = 0.0;
   for (int k = shan_chen ? 1 : 0; k < 4; ++k) {  // Shan-Chen has no 32x8x8
     const long long ctas = shape_ctas(g, order[k]), share = (ctas + sms - 1) / sms;
-    const double walk = share > 16 ? 5.0 * (double)ctas / (double)sms : 10.0 * (double)(share / 2) + 9.0 * (double)(share % 2);
+    const double walk = share > 8 ? 5.0 * (double)ctas / (double)sms : 10.0 * (double)(share / 2) + 9.0 * (double)(share % 2);
     const double t = (tile_shape(order[k]).tz + 0.75) * walk;
     if (best < 0 || t < least) {
       best = order[k];
