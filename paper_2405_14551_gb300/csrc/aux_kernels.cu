@@ -127,9 +127,10 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_partial(Geo g, const R* 
 
 // The same sums of FP32 fields, a thread's share in Sum3 terms, then FP64 for
 // the tree: the FP64 pipe (22 operations and conversions a node) bounded the
-// kernel above, 174 -> 86 us at 128x128x256.  A thread whose terms leave
+// kernel above, 174 -> 78 us at 128x128x256.  Four CTAs an SM cap it at 64 registers
+// (80 without the cap: three CTAs, 178 us).  A thread whose terms leave
 // FP32's range repeats its share in FP64.
-__global__ void __launch_bounds__(RED_THREADS) k_reduce_partial_f32(Geo g, const float* __restrict__ fl, double* partials) {
+__global__ void __launch_bounds__(RED_THREADS, 4) k_reduce_partial_f32(Geo g, const float* __restrict__ fl, double* partials) {
   __shared__ double s[8][RED_THREADS];
   const size_t N = (size_t)g.N;
   const long long chunk = (g.N + gridDim.x - 1) / gridDim.x;
