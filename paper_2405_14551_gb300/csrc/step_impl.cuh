@@ -961,39 +961,42 @@ __global__ void __launch_bounds__(256) k_phi(PhiSrc src, InitBuf init, Geo g, Pa
 // sums are integers that a population which is not a number does not enter, so
 // the populations are pulled and summed as the step does it.  Initial fields
 // (LOAD_FIELDS) need phi and rho only, since fields_node's densities do not
-// depend on its populations.  One node per thread; bound by the population
-// bytes (half a step's), or 4 to 8 bytes a node.
+// depend on its populations.  A warp takes a row; bound by the population bytes
+// (half a step's), or 4 to 8 bytes a node: two-set FP32, 128x128x256, 151 us pulled
+// (133 at the copy rate), 13 us of initial fields (about 100 with a thread per node
+// and its two 64-bit divisions).
 template <int ST, int LOADER>
 __global__ void __launch_bounds__(256) k_density(View<ST> S, InitBuf init, const unsigned long long* __restrict__ accin, Geo g,
                                                  PhysR<typename Store<ST>::R> P, unsigned* __restrict__ status) {
   using R = typename Store<ST>::R;
   using E = typename Store<ST>::E;
   bool bad = false;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < g.N; idx += stride) {
-    const int x = (int)(idx % g.nx);
-    const long long yz = idx / g.nx;
-    const int y = (int)(yz % g.ny), z = (int)(yz / g.ny);
-    if (is_solid(g, x, y, z)) continue;
-    Nbr n;
-    make_nbr(g, x, y, z, n);
-    R f[Q], rA, rB;
-    if constexpr (LOADER == LOAD_PULL) {
-      E ra[Q], rb[Q];
-      pull_walled<ST>(S, g, n, Lay<ST>::at(g, x, y, z), ra, rb, f);
-      if constexpr (!Store<ST>::MOMENT) pull_finish<ST>(ra, rb, f, rA, rB);
-      if constexpr (!Store<ST>::TWOSET) {
-        R rt = R(0);
+  const long long rows = (long long)g.ny * g.nz;
+  for (long long row = (long long)blockIdx.x * 8 + threadIdx.y; row < rows; row += (long long)gridDim.x * 8) {
+    const int z = (int)((unsigned)row / (unsigned)g.ny), y = (int)row - z * g.ny;  // rows <= nodes < 2^31
+    for (int x = threadIdx.x; x < g.nx; x += 32) {
+      if (is_solid(g, x, y, z)) continue;
+      const long long idx = row * g.nx + x;
+      Nbr n;
+      make_nbr(g, x, y, z, n);
+      R f[Q], rA, rB;
+      if constexpr (LOADER == LOAD_PULL) {
+        E ra[Q], rb[Q];
+        pull_walled<ST>(S, g, n, Lay<ST>::at(g, x, y, z), ra, rb, f);
+        if constexpr (!Store<ST>::MOMENT) pull_finish<ST>(ra, rb, f, rA, rB);
+        if constexpr (!Store<ST>::TWOSET) {
+          R rt = R(0);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) rt += f[i];
-        Acc<R>::densities(accin, (size_t)idx, rA, rB);
-        rB = rt - rA;
+          for (int i = 0; i < Q; ++i) rt += f[i];
+          Acc<R>::densities(accin, (size_t)idx, rA, rB);
+          rB = rt - rA;
+        }
+      } else {
+        fields_node<R, false>(init, g, P, n, idx, f, rA, rB, nullptr, nullptr);
       }
-    } else {
-      fields_node<R, false>(init, g, P, n, idx, f, rA, rB, nullptr, nullptr);
+      const R rho = rA + rB;
+      bad |= !(rho > R(0) && rho < R(Acc<R>::RHO_MAX));
     }
-    const R rho = rA + rB;
-    bad |= !(rho > R(0) && rho < R(Acc<R>::RHO_MAX));
   }
   if (bad) atomicOr(status, 1u);
 }
@@ -1191,8 +1194,9 @@ __device__ __forceinline__ float decode_scaled(typename Store<ST>::E v, int i) {
 // sp holds phi of the tile and its halo (Layout), accin the accumulator of the
 // current level (null: the densities come from phi).  The near-contact scan of
 // an interface node runs between the loads and the sums of its pull, while
-// the loads are in flight (EARLY), or before the loads in the tiles whose
-// registers cannot hold a node's raw values through it.
+// the loads are in flight (EARLY), or before the loads where the registers cannot
+// hold a node's raw values through it: two-set batches, whose run parameters are
+// loaded (12 runs of 48^3 to 96^3, near contact: 502 us a step early, 484 late).
 template <int ST, int LOADER, bool WS, bool WF, int TX, int TY, int TZ, int H, bool WALLFREE, bool IDX32, bool REG, bool EARLY>
 __device__ __forceinline__ void step_nodes(const View<ST>& S, const View<ST>& O, const InitBuf& init, const Geo& g,
                                            const PhysR<typename Store<ST>::R>& P,

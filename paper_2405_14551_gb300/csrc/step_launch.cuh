@@ -158,10 +158,10 @@ template <int ST>
 cudaError_t launch_density_t(int loader, const Geo& g, const Phys& p, const StateBuf& in, const InitBuf& init,
                              const unsigned long long* accin, unsigned* status, cudaStream_t st) {
   auto run = [&](auto kern) {
-    const long long need = (g.N + 255) / 256, cap = (long long)sm_count() * 8;
+    const long long need = ((long long)g.ny * g.nz + 7) / 8, cap = (long long)sm_count() * 8;
     const int blocks = (int)(need < cap ? need : cap);
-    trace_kernel("k_density", kern, dim3(blocks), dim3(256), 0);
-    kern<<<blocks, 256, 0, st>>>(view<ST>(in), init, accin, g, phys_as<typename Store<ST>::R>(p), status);
+    trace_kernel("k_density", kern, dim3(blocks), dim3(32, 8), 0);
+    kern<<<blocks, dim3(32, 8), 0, st>>>(view<ST>(in), init, accin, g, phys_as<typename Store<ST>::R>(p), status);
     return cudaGetLastError();
   };
   return loader == LOAD_PULL ? run(k_density<ST, LOAD_PULL>) : run(k_density<ST, LOAD_FIELDS>);
