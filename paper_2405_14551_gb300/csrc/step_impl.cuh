@@ -1765,7 +1765,9 @@ __device__ __forceinline__ void step_tile(const View<ST>& S, const View<ST>& O, 
       step_nodes<ST, LOADER, WS, WF, TX, TY, TZ, H, decltype(wf)::value, IDX32, decltype(reg)::value, EARLY>(
           S, O, init, g, P, fields, status, sp, sw, accin, x0, y0, z0);
     };
-    if (P.collision == 1) {  // regularised collision
+    // (the moment storage holds the regularised collision only; a BGK copy of its
+    // loop, which nothing reached, cost it 3 to 5 % in registers)
+    if (Store<ST>::MOMENT || P.collision == 1) {  // regularised collision
       if (wallfree) nodes(std::true_type{}, std::true_type{});
       else nodes(std::false_type{}, std::true_type{});
     } else {
