@@ -202,13 +202,14 @@ class ClockSampler:
                 "power_w_max": max((float(r[3]) for r in rows if r[3].replace(".", "").isdigit()), default=None)}
 
 
-# DRAM bytes per node of one step launch, read from an ncu capture
-# (dram__bytes_read.sum + dram__bytes_write.sum of k_step on the dense emulsion
-# 128x128x256 with the given tile, divided by its nodes; the kernel's traffic
-# grows with the node count) together with a digest of the kernel sources it
-# was taken on: a changed kernel reports null until it is captured again.
-K_STEP_TRAFFIC = {  # storage -> (bytes per node, source digest, tile)
-    "twoset_f32": (451.8, "437add262738ef64", 5),  # mean of 2 launches: 1892.1 / 1897.8 MB per 4194304 nodes
+# DRAM bytes per node of one step, read from an ncu capture
+# (dram__bytes_read.sum + dram__bytes_write.sum of k_phi and k_step on the dense
+# emulsion 128x128x256, divided by its nodes; the traffic grows with the node
+# count), with a digest of the kernel sources it was taken on (a changed kernel
+# reports null until it is captured again) and the tile indexes that launch the
+# captured shape at that size and at the workload's.
+K_STEP_TRAFFIC = {  # storage -> (bytes per node, source digest, tiles)
+    "twoset_f32": (440.4, "454e90064bb09d40", (1, 2, 3, 5)),
 }
 
 
@@ -804,7 +805,7 @@ def main():
     bpn = L.BYTES_PER_NODE[stid]
     achieved = bpn * nodes / (step_ms / 1e3) / 1e9
     tr = K_STEP_TRAFFIC.get(storage)
-    traffic = round(tr[0] * nodes) if (tr and tr[1] == kernel_digest() and best_tile == tr[2]) else None
+    traffic = round(tr[0] * nodes) if (tr and tr[1] == kernel_digest() and best_tile in tr[2]) else None
     step_frac = bpn * value * 1e6 / world / 1e9 / peak
 
     e2e = None if args.no_e2e else end_to_end(args, L, sim, wl, nodes, world, barrier, maxall)
