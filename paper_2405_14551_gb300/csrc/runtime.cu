@@ -722,8 +722,8 @@ int lb_set_tile(lb_handle* h, int tile) {
 int lb_get_tile(const lb_handle* h) { return h ? h->tile : -1; }
 
 // Whether a kernel on the handle's device can store to p as to its own memory.
-// Another GPU's memory and host memory are reached by a copy, which the driver
-// routes without peer access and at the link's full rate.
+// Another GPU's memory and host memory are reached by a copy, which CUDA routes
+// without peer access and at the link's full rate.
 static bool stores_reach(const lb_handle* h, const void* p) {
   cudaPointerAttributes a{};
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {

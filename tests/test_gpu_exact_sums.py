@@ -53,7 +53,7 @@ def test_single_nodes_keep_fp64_precision():
 
 # a thread's share is at most 12 nodes here; summed in FP64 a node rounds 6 times, and
 # the trees over 256 threads and over the blocks add at most 8 levels each
-@pytest.mark.parametrize("kind", ["plain", "cancelling", "beyond", "tiny", "far"])
+@pytest.mark.parametrize("kind", ["plain", "cancelling", "beyond", "beyond_phi", "tiny", "far"])
 def test_sums_cancelling_and_out_of_range(kind):
     shape = (16, 16, 12)
     n = 16 * 16 * 12
@@ -64,6 +64,8 @@ def test_sums_cancelling_and_out_of_range(kind):
         f[RHO, 1::2] = f[RHO, ::2]
     elif kind == "beyond":  # squares above FP32's range: the share is summed in FP64
         f[UX, 7] = 3e25
+    elif kind == "beyond_phi":  # two values of one share whose FP32 sum overflows
+        f[PHI, [5, 261]] = 3e38
     elif kind == "tiny":  # all squares below it
         f[UX:UZ + 1] *= np.float32(1e-24)
     elif kind == "far":  # a large term beside the round-off of the others
@@ -73,6 +75,26 @@ def test_sums_cancelling_and_out_of_range(kind):
     mag[5] = ref[5]  # a sum of non-negative terms 1 + phi
     for k in range(8):
         assert abs(Fr(float(got[k])) - ref[k]) <= (12 + 6 + 16) * mag[k] * Fr(1, 2**53), k
+
+
+@pytest.mark.parametrize("big", [1.0, 3e38])
+def test_volume_of_a_phase_field(big):
+    """lb_phi_monitor's volume, also where a share overflows FP32: the sum that
+    lb_reduce_f64 gives, bit for bit."""
+    import torch
+
+    import paper_2405_14551_gb300.lbcg as L
+    shape = (16, 16, 12)
+    f = _fields(16 * 16 * 12, 9)
+    f[PHI, [5, 261]] = big
+    s = L.Sim(*shape)
+    d = torch.from_numpy(f[PHI].copy()).cuda()
+    torch.cuda.synchronize()
+    _, volume = L.lb_phi_monitor(s.h, d)
+    s.close()
+    assert volume == _reduce(f, shape)[5]
+    ref = _exact(f)[5]
+    assert abs(Fr(volume) - ref) <= (12 + 6 + 16) * ref * Fr(1, 2**53)
 
 
 @pytest.mark.parametrize("c,nch", [(4, 1), (4, 3), (8, 5)])
